@@ -158,11 +158,18 @@ struct Ctx {
     // for the batched driver, where problems share the GPU.
     bool dataflow = true;
     int flow_ctas = 0;
-    // two-level factorisation with emulated FP64 tensor-core trailing updates; with it the
-    // Grams and the FP64-accuracy products of the split path (its loss, the learned step's
-    // trial losses) also run as emulated FP64 products
-    bool emulated = false;
+    // factorisation in fixed-point blocks (ldl_fix.cu), or in dataflow panels, with tensor-core
+    // trailing updates
+    bool fixed = false, two_level = false;
+    FixWs fix;
     OzWs oz;
+    // FP64-accurate products on the tensor cores for the FP64 path (and every FP64 Gram and
+    // loss): the digits of the constant operands are cut once per call (rows of Z and of its
+    // transpose, rows of X_k and of its transpose), those of W o W, W o Y and of a factor's
+    // columns into dP / dA as they are formed.
+    bool ozp = false;
+    OzMat dZ[2], dX[2], dXT[2], dP, dA;
+    bool have_dZ[2] = {}, have_dX[2] = {}, have_dXT[2] = {};
     double* part = nullptr;
     size_t part_cap = 0;
     double* red = nullptr;
@@ -207,16 +214,43 @@ struct Ctx {
     }
 };
 
-enum : unsigned { NEED_ALS = 1, NEED_NORM = 2, NEED_SAFE = 4, NEED_BATCHED = 8 };
+// The same for a call that ran products only.
+thc_cpd_status product_errors(const Ctx& c) {
+    if (c.prec != THC_CPD_FP64) {
+        if (int e = mixed_take_error())
+            return set_err(THC_CPD_ERR_TIMEOUT, "tensor-core kernel wait gave up (code %d)", e);
+    }
+    if (c.ozp || c.fixed || c.two_level) {
+        if (int e = oz_take_error())
+            return set_err(THC_CPD_ERR_TIMEOUT, "emulated-product kernel wait gave up (code %d)", e);
+    }
+    return THC_CPD_OK;
+}
 
-// Whether a single problem's LDL^T runs in panels with emulated tensor-core updates: on
-// request, and by default from R = 1024 on (measured on GB300, BF16x3 sweeps: emulated vs
-// dataflow 334 vs 395 sweeps/s at R = 720, 211 vs 207 at 1080, 104 vs 59 at 1800), within
-// the panel plans' range.
+// What a call needs of the context: the sweeps' buffers, ||G||^2, the Grams, and whether several
+// problems run side by side.
+enum : unsigned { NEED_ALS = 1, NEED_NORM = 2, NEED_GRAM = 4, NEED_BATCHED = 8 };
+
+// The factorisation of an R x R normal matrix for the `ldl` option.
+enum class Ldl { kBlocked, kDataflow, kTwoLevel, kFixed };
 constexpr int kEmulatedMinR = 1024;
-bool use_emulated_ldl(int ldl, int R, int nmax) {
-    const bool fits = R > kOzPanel && R <= 4096 && cdiv((long)R + nmax - kOzPanel, 16) <= 256;
-    return fits && (ldl == THC_CPD_LDL_EMULATED || (ldl == THC_CPD_LDL_AUTO && R >= kEmulatedMinR));
+constexpr int kFixedMinR = 48, kFixedMaxR = 128;
+constexpr int kFixedBatchedMinR = 400;
+// On its own, a problem takes the fixed-point kernel (ldl_fix.cu) while it is a single block of some
+// tiles (48 to 128 columns), the dataflow kernel up to 1024 and from there dataflow panels with emulated trailing updates (within
+// their plans' range). Side by side, problems of 400 columns and more take fixed-point blocks,
+// which leave the FP64 pipes to the others, smaller ones the blocked FP64 kernels.
+Ldl ldl_route(int ldl, int R, int nmax, bool batched) {
+    const bool two = R > kOzPanel && R <= 4096 && cdiv((long)R + nmax - kOzPanel, 16) <= 256;
+    switch (ldl) {
+        case THC_CPD_LDL_BLOCKED: return Ldl::kBlocked;
+        case THC_CPD_LDL_DATAFLOW: return Ldl::kDataflow;
+        case THC_CPD_LDL_EMULATED: return two ? Ldl::kTwoLevel : Ldl::kBlocked;
+        default: break;
+    }
+    if (two && R >= kEmulatedMinR) return Ldl::kTwoLevel;
+    if ((batched ? R >= kFixedBatchedMinR : R >= kFixedMinR && R <= kFixedMaxR) && ldl_fix_prepare()) return Ldl::kFixed;
+    return batched ? Ldl::kBlocked : Ldl::kDataflow;
 }
 
 // grid cap of the dataflow factorisation when the batched driver is asked for it
@@ -234,71 +268,104 @@ thc_cpd_status ctx_init(Ctx& c, const Shape& s, const double* Xo, const double* 
     c.prec = opts ? opts->precision : THC_CPD_FP64;
     set_wait_limit(opts);
     const int Rt = s.Rt, R = s.R, nmax = s.nmax;
-    size_t pc = 0;
+    const bool als = need & NEED_ALS, norm = need & NEED_NORM, gram = als || (need & NEED_GRAM);
+    const bool mixed = c.prec != THC_CPD_FP64;
+    const bool tf32 = c.prec == THC_CPD_TF32X3;
+    const bool fp64 = !mixed || als || gram;  // FP64 projections (MTTKRP, or a split run's loss)
+    // FP64 products that go to the tensor cores: room for the operands' digits and split sums
+    const bool w_z = fp64 && oz_worth(Rt, R, Rt, false), w_n = norm && oz_worth(Rt, Rt, Rt, false);
+    c.ozp = oz_available() && (w_z || w_n || (fp64 && oz_worth(Rt, R, nmax, false)) ||
+                               (gram && oz_worth(R, R, nmax, true)));
+    const bool ozp = c.ozp;
+    // FP64-pipe products: split-K partial sums of those that stay there
+    size_t pc = 1;
+    auto pipe = [&](int M, int N, int K, bool symm) {
+        if (!(ozp && oz_worth(M, N, K, symm))) pc = std::max(pc, dgemm_part_need(M, N, K));
+    };
     for (int k = 0; k < 2; ++k) {
         const int n = s.n[k];
-        pc = std::max(pc, dgemm_part_need(Rt, R, n));
-        pc = std::max(pc, dgemm_part_need(n, R, Rt));
-        pc = std::max(pc, dgemm_part_need(R, R, n));
-        pc = std::max(pc, dgemm_part_need(Rt, Rt, n));
+        pipe(Rt, R, n, false);
+        pipe(n, R, Rt, false);
+        if (gram) pipe(R, R, n, true);
+        if (norm) pc = std::max(pc, dgemm_part_need(Rt, Rt, n));
     }
-    pc = std::max(pc, dgemm_part_need(Rt, R, Rt));
-    if (need & NEED_NORM) pc = std::max(pc, dgemm_part_need(Rt, Rt, Rt));
-    if (need & NEED_SAFE) pc = std::max(pc, dgemm_part_need(nmax, R, R));
+    pipe(Rt, R, Rt, false);
+    if (norm) pipe(Rt, Rt, Rt, false);
     c.part_cap = pc;
+    const int ldl = opts ? opts->ldl : THC_CPD_LDL_AUTO;
+    Ldl route = als ? ldl_route(ldl, R, nmax, need & NEED_BATCHED) : Ldl::kDataflow;
+    if (route == Ldl::kTwoLevel && !(oz_prepare(R, s.o) && oz_prepare(R, s.v)))
+        route = (need & NEED_BATCHED) ? Ldl::kBlocked : Ldl::kDataflow;
+    c.fixed = als && route == Ldl::kFixed;
+    c.two_level = als && route == Ldl::kTwoLevel;
     size_t bytes = 0;
     const size_t RtR = (size_t)Rt * R, RR = (size_t)R * R;
-    bytes += 4 * Arena::need<double>(RtR);                 // W
-    bytes += 4 * Arena::need<double>(RR);                  // G
-    bytes += Arena::need<double>(RtR);                     // Y
-    bytes += Arena::need<double>((size_t)(R + nmax) * R);  // Haug
-    bytes += Arena::need<double>(RR + R);                  // X = L D and D^{-1}
-    bytes += Arena::need<int>(cdiv(R, 32));               // arrival counters of the LDL^T
-    bytes += Arena::need<int>(flow_sync_ints(R, nmax));   // dataflow LDL^T progress
-    bytes += Arena::need<int>(bsolve_sync_ints(nmax));    // sliced backward solve progress
+    if (fp64) bytes += 5 * Arena::need<double>(RtR);      // W, Y
+    if (gram) bytes += 4 * Arena::need<double>(RR);       // G
+    if (als) {
+        bytes += Arena::need<double>((size_t)(R + nmax) * R);         // Haug
+        bytes += Arena::need<double>((c.fixed ? 0 : RR) + R);         // X = L D and D^{-1}
+        bytes += Arena::need<int>(cdiv(R, 32));                       // arrival counters of the LDL^T
+        bytes += Arena::need<int>(c.fixed ? 1 : flow_sync_ints(R, nmax));  // dataflow LDL^T progress
+        bytes += Arena::need<int>(bsolve_sync_ints(nmax));            // sliced backward solve progress
+        if (c.fixed) bytes += ldl_fix_ws_bytes(R, nmax);
+    }
     bytes += Arena::need<double>(pc);
     bytes += Arena::need<double>(loss_red_need() + 2 * kReduceBlocks);
     bytes += Arena::need<double>(R);
     bytes += 2 * Arena::need<DevScalars>(1);
-    if (need & NEED_ALS) {  // two rollback snapshots (pipelined runs alternate)
+    if (als) {  // two rollback snapshots (pipelined runs alternate)
         bytes += Arena::need<DevScalars>(1);
         bytes += 2 * (2 * Arena::need<double>((size_t)s.o * R) + 2 * Arena::need<double>((size_t)s.v * R));
         bytes += 2 * Arena::need<double>(R);
     }
-    if (need & NEED_NORM) bytes += 3 * Arena::need<double>((size_t)Rt * Rt);
-    const bool mixed = c.prec != THC_CPD_FP64;
-    const bool tf32 = c.prec == THC_CPD_TF32X3;
+    if (norm) bytes += 3 * Arena::need<double>((size_t)Rt * Rt);
     if (mixed) bytes += mixed_ws_bytes(tf32, s.o, s.v, Rt, R);
-    // the factorisation: plans (host task lists, uploaded once per shape) are prepared here,
-    // never inside a capture
-    const int ldl = opts ? opts->ldl : THC_CPD_LDL_AUTO;
-    c.emulated = use_emulated_ldl(ldl, R, nmax) && oz_prepare(R, s.o) && oz_prepare(R, s.v);
-    int oz_ra = std::max(R + nmax, Rt), oz_rb = R;
+    int oz_ra = 1, oz_rb = 1;
     size_t oz_part = 0;
-    if (c.emulated) bsolve_ws_rows(R, nmax, &oz_ra, &oz_rb, &oz_part);
-    if (c.emulated) oz_ldl_ws_rows(R, nmax, &oz_ra, &oz_rb);
-    if (c.emulated) bytes += oz_ws_bytes(oz_ra, oz_rb, oz_part);
+    const bool ozl = c.fixed || c.two_level;
+    if (ozl) bsolve_ws_rows(R, nmax, &oz_ra, &oz_rb, &oz_part);
+    if (c.two_level) oz_ldl_ws_rows(R, nmax, &oz_ra, &oz_rb);
+    if (ozp) {
+        if (fp64) {
+            for (int k = 0; k < 2; ++k) {
+                oz_product_ws(s.n[k], R, Rt, &oz_ra, &oz_rb, &oz_part);
+                oz_product_ws(Rt, R, s.n[k], &oz_ra, &oz_rb, &oz_part);
+            }
+            oz_product_ws(Rt, R, Rt, &oz_ra, &oz_rb, &oz_part);
+        }
+        if (norm) oz_product_ws(Rt, Rt, Rt, &oz_ra, &oz_rb, &oz_part);
+        bytes += 2 * ozmat_bytes(Rt, Rt) + ozmat_bytes(R, Rt) + ozmat_bytes(R, nmax);
+        for (int k = 0; k < 2; ++k) bytes += ozmat_bytes(s.n[k], Rt) + ozmat_bytes(Rt, s.n[k]);
+    }
+    if (ozl || ozp) bytes += oz_ws_bytes(oz_ra, oz_rb, oz_part);
     CK(cudaMallocAsync(&c.block, bytes, c.st));
     Arena ar;
     ar.base = (char*)c.block;
     ar.cap = bytes;
-    for (int k = 0; k < 4; ++k) c.W[k] = ar.take<double>(RtR);
-    for (int k = 0; k < 4; ++k) c.G[k] = ar.take<double>(RR);
-    c.Y = ar.take<double>(RtR);
-    c.Haug = ar.take<double>((size_t)(R + nmax) * R);
-    c.LinvD = ar.take<double>(RR + R);
-    c.counters = ar.take<int>(cdiv(R, 32));
-    c.flow_sync = ar.take<int>(flow_sync_ints(R, nmax));
-    c.bs_sync = ar.take<int>(bsolve_sync_ints(nmax));
-    // zero once: every launch that uses them leaves them zero again
-    CK(cudaMemsetAsync(c.flow_sync, 0, sizeof(int) * flow_sync_ints(R, nmax), c.st));
-    CK(cudaMemsetAsync(c.bs_sync, 0, sizeof(int) * bsolve_sync_ints(nmax), c.st));
+    if (fp64) {
+        for (int k = 0; k < 4; ++k) c.W[k] = ar.take<double>(RtR);
+        c.Y = ar.take<double>(RtR);
+    }
+    if (gram)
+        for (int k = 0; k < 4; ++k) c.G[k] = ar.take<double>(RR);
+    if (als) {
+        c.Haug = ar.take<double>((size_t)(R + nmax) * R);
+        c.LinvD = ar.take<double>((c.fixed ? 0 : RR) + R);
+        c.counters = ar.take<int>(cdiv(R, 32));
+        c.flow_sync = ar.take<int>(c.fixed ? 1 : flow_sync_ints(R, nmax));
+        c.bs_sync = ar.take<int>(bsolve_sync_ints(nmax));
+        if (c.fixed) ldl_fix_carve(c.fix, ar, R, nmax);
+        // zero once: every launch that uses them leaves them zero again
+        if (!c.fixed) CK(cudaMemsetAsync(c.flow_sync, 0, sizeof(int) * flow_sync_ints(R, nmax), c.st));
+        CK(cudaMemsetAsync(c.bs_sync, 0, sizeof(int) * bsolve_sync_ints(nmax), c.st));
+    }
     c.part = ar.take<double>(pc);
     c.red = ar.take<double>(loss_red_need() + 2 * kReduceBlocks);
     c.ones = ar.take<double>(R);
     c.sc = ar.take<DevScalars>(1);
     c.sc_snap = ar.take<DevScalars>(1);
-    if (need & NEED_ALS) {
+    if (als) {
         c.sc_slot[0] = c.sc_snap;
         c.sc_slot[1] = ar.take<DevScalars>(1);
         for (int b = 0; b < 2; ++b) {
@@ -308,7 +375,7 @@ thc_cpd_status ctx_init(Ctx& c, const Shape& s, const double* Xo, const double* 
         for (int k = 0; k < 4; ++k) c.Asnap[k] = c.Asnap_slot[0][k];
         c.lamsnap = c.lamsnap_slot[0];
     }
-    if (need & NEED_NORM) {
+    if (norm) {
         c.S = ar.take<double>((size_t)Rt * Rt);
         c.T = ar.take<double>((size_t)Rt * Rt);
         c.U = ar.take<double>((size_t)Rt * Rt);
@@ -317,14 +384,25 @@ thc_cpd_status ctx_init(Ctx& c, const Shape& s, const double* Xo, const double* 
         mixed_ws_carve(c.mx, ar, tf32, s.o, s.v, Rt, R);
         CK(mixed_setup(c.mx, c.st, Xo, Xv, Z));
     }
-    if (c.emulated) oz_ws_carve(c.oz, ar, oz_ra, oz_rb, oz_part);
-    fill(c.st, c.ones, R, 1.0);
-    c.dataflow = c.emulated || ldl == THC_CPD_LDL_DATAFLOW ||
-                 (ldl == THC_CPD_LDL_AUTO && !(need & NEED_BATCHED));
-    c.flow_ctas = (need & NEED_BATCHED) ? kBatchedFlowCtas : 0;
-    if (c.dataflow) {
-        flow_prepare(R, s.o);
-        flow_prepare(R, s.v);
+    if (ozp) {
+        for (int h = 0; h < 2; ++h) ozmat_carve(c.dZ[h], ar, Rt, Rt);
+        for (int k = 0; k < 2; ++k) {
+            ozmat_carve(c.dX[k], ar, s.n[k], Rt);
+            ozmat_carve(c.dXT[k], ar, Rt, s.n[k]);
+        }
+        ozmat_carve(c.dP, ar, R, Rt);
+        ozmat_carve(c.dA, ar, R, nmax);
+    }
+    if (ozl || ozp) oz_ws_carve(c.oz, ar, oz_ra, oz_rb, oz_part);
+    if (gram) fill(c.st, c.ones, R, 1.0);
+    if (als && !c.fixed) {
+        c.dataflow = route != Ldl::kBlocked;
+        c.flow_ctas = (need & NEED_BATCHED) ? kBatchedFlowCtas : 0;
+        if (route == Ldl::kDataflow) {
+            // plans (host task lists, uploaded once per shape) are prepared here, never inside a capture
+            flow_prepare(R, s.o);
+            flow_prepare(R, s.v);
+        }
     }
     CK(cudaGetLastError());
     return THC_CPD_OK;
@@ -353,12 +431,69 @@ thc_cpd_status ctx_safe_buffers(Ctx& c) {
 }
 
 // ---- building blocks -----------------------------------------------------------------
+// The FP64-accurate products run on the tensor cores (oz_gemm.cu) from a size on (oz_worth),
+// on the FP64 pipes below it. Digits of a constant operand, cut on first use:
+const OzMat& digits_Z(Ctx& c, int half) {  // half 0: rows of Z, 1: rows of Z^T
+    if (!c.have_dZ[half]) {
+        if (half == 0)
+            oz_split_rows(c.st, c.Z, c.s.Rt, c.dZ[0]);
+        else
+            oz_split_cols(c.st, c.Z, nullptr, c.s.Rt, c.dZ[1]);
+        c.have_dZ[half] = true;
+    }
+    return c.dZ[half];
+}
+
+const OzMat& digits_X(Ctx& c, int k) {  // rows of X_k
+    if (!c.have_dX[k]) {
+        oz_split_rows(c.st, c.X[k], c.s.Rt, c.dX[k]);
+        c.have_dX[k] = true;
+    }
+    return c.dX[k];
+}
+
+const OzMat& digits_XT(Ctx& c, int k) {  // rows of X_k^T
+    if (!c.have_dXT[k]) {
+        oz_split_cols(c.st, c.X[k], nullptr, c.s.Rt, c.dXT[k]);
+        c.have_dXT[k] = true;
+    }
+    return c.dXT[k];
+}
+
+void mul_digits(Ctx& c, const OzMat& A, const OzMat& B, double* C, int ldc, bool symm) {
+    ProfScope prof(c.st, KC_OZ, (symm ? 1.0 : 2.0) * A.rows * (double)B.rows * A.K);
+    oz_mul(c.st, A, B, C, ldc, 1.0, symm ? OZ_SYMM : 0, c.oz.part, c.oz.part_cap);
+}
+
+// An FP64-accuracy product of operands that are used once
 void gemm64(Ctx& c, bool trans_a, int M, int N, int K, const double* A, int lda, const double* B,
-            const double* B2, int ldb, double* C, int ldc, bool symm);
+            const double* B2, int ldb, double* C, int ldc, bool symm) {
+    if (c.ozp && oz_worth(M, N, K, symm) && M <= c.oz.rowsA && N <= c.oz.rowsB)
+        oz_dgemm(c.st, trans_a, M, N, K, A, lda, B, B2, ldb, C, ldc, symm, c.oz);
+    else
+        dgemm(c.st, trans_a, M, N, K, A, lda, B, B2, ldb, C, ldc, nullptr, symm, c.part, c.part_cap);
+}
 
 void compute_normG2(Ctx& c) {
     const int o = c.s.o, v = c.s.v, Rt = c.s.Rt;
     // S = (Xo^T Xo) o (Xv^T Xv); U = S Z S; ||G||^2 = sum Z o U
+    if (c.ozp && oz_worth(Rt, Rt, Rt, false)) {
+        mul_digits(c, digits_XT(c, 0), digits_XT(c, 0), c.T, Rt, true);
+        mul_digits(c, digits_XT(c, 1), digits_XT(c, 1), c.S, Rt, true);
+        // S is symmetric: its columns, cut from the two Grams, serve as left and right operand
+        OzMat s, t;
+        s.d = c.oz.sB;
+        s.e = c.oz.eB;
+        t.d = c.oz.sA;
+        t.e = c.oz.eA;
+        s.rows = s.K = t.rows = t.K = Rt;
+        oz_split_cols(c.st, c.T, c.S, Rt, s);
+        mul_digits(c, s, digits_Z(c, 1), c.U, Rt, false);  // S Z
+        oz_split_rows(c.st, c.U, Rt, t);
+        mul_digits(c, t, s, c.T, Rt, false);                // (S Z) S
+        sum_hadamard_normG2(c.st, (long)Rt * Rt, c.Z, c.T, c.red, c.sc);
+        return;
+    }
     dgemm(c.st, true, Rt, Rt, o, c.X[0], Rt, c.X[0], nullptr, Rt, c.T, Rt, nullptr, true, c.part, c.part_cap);
     dgemm(c.st, true, Rt, Rt, v, c.X[1], Rt, c.X[1], nullptr, Rt, c.S, Rt, c.T, true, c.part, c.part_cap);
     gemm64(c, false, Rt, Rt, Rt, c.S, Rt, c.Z, nullptr, Rt, c.T, Rt, false);
@@ -366,58 +501,49 @@ void compute_normG2(Ctx& c) {
     sum_hadamard_normG2(c.st, (long)Rt * Rt, c.Z, c.U, c.red, c.sc);
 }
 
-// An FP64-accuracy product: emulated on the tensor cores when the context has the
-// emulated path (same result up to rounding), else on the FP64 pipes.
-void gemm64(Ctx& c, bool trans_a, int M, int N, int K, const double* A, int lda, const double* B,
-            const double* B2, int ldb, double* C, int ldc, bool symm) {
-    if (c.emulated && M <= c.oz.rowsA && N <= c.oz.rowsB)
-        oz_dgemm(c.st, trans_a, M, N, K, A, lda, B, B2, ldb, C, ldc, nullptr, symm, c.oz);
-    else
-        dgemm(c.st, trans_a, M, N, K, A, lda, B, B2, ldb, C, ldc, nullptr, symm, c.part, c.part_cap);
-}
-
-// W_k = X_k^T A_k; emu: as an emulated product (the split path's FP64 loss), else on the
-// FP64 pipes (the FP64 path's MTTKRP)
-void project_fp64(Ctx& c, int k, const double* Ak, bool emu = false) {
-    if (emu) {
-        gemm64(c, true, c.s.Rt, c.s.R, c.s.n[k], c.X[k], c.s.Rt, Ak, nullptr, c.s.R, c.W[k], c.s.R, false);
-        return;
-    }
-    dgemm(c.st, true, c.s.Rt, c.s.R, c.s.n[k], c.X[k], c.s.Rt, Ak, nullptr, c.s.R, c.W[k], c.s.R,
-          nullptr, false, c.part, c.part_cap);
-}
-
-void gram_fp64(Ctx& c, int k, const double* Ak) {
-    if (c.emulated) {
-        gemm64(c, true, c.s.R, c.s.R, c.s.n[k], Ak, c.s.R, Ak, nullptr, c.s.R, c.G[k], c.s.R, true);
-        return;
-    }
-    dgemm(c.st, true, c.s.R, c.s.R, c.s.n[k], Ak, c.s.R, Ak, nullptr, c.s.R, c.G[k], c.s.R, nullptr,
-          true, c.part, c.part_cap);
+// What follows from a factor: its Gram G_k = A_k^T A_k and its projection W_k = X_k^T A_k (either
+// or both); on the tensor cores from one cut of its columns.
+void factor_products(Ctx& c, int k, const double* Ak, bool gram, bool proj) {
+    const int n = c.s.n[k], R = c.s.R, Rt = c.s.Rt;
+    const bool og = c.ozp && gram && oz_worth(R, R, n, true), op = c.ozp && proj && oz_worth(Rt, R, n, false);
+    OzMat a = c.dA;
+    a.K = n;
+    if (og || op) oz_split_cols(c.st, Ak, nullptr, R, a);
+    if (og)
+        mul_digits(c, a, a, c.G[k], R, true);
+    else if (gram)
+        dgemm(c.st, true, R, R, n, Ak, R, Ak, nullptr, R, c.G[k], R, nullptr, true, c.part, c.part_cap);
+    if (op)
+        mul_digits(c, digits_XT(c, k & 1), a, c.W[k], R, false);
+    else if (proj)
+        dgemm(c.st, true, Rt, R, n, c.X[k], Rt, Ak, nullptr, R, c.W[k], R, nullptr, false, c.part, c.part_cap);
 }
 
 // Y = Z (W3 o W4) for modes 0,1 and Y = Z^T (W1 o W2) for modes 2,3
-void zgemm_fp64(Ctx& c, int half, bool emu = false) {
+void zgemm_fp64(Ctx& c, int half) {
     const int Rt = c.s.Rt, R = c.s.R;
-    if (emu) {
-        if (half == 0)
-            gemm64(c, false, Rt, R, Rt, c.Z, Rt, c.W[2], c.W[3], R, c.Y, R, false);
-        else
-            gemm64(c, true, Rt, R, Rt, c.Z, Rt, c.W[0], c.W[1], R, c.Y, R, false);
+    const double *a = c.W[half == 0 ? 2 : 0], *b = c.W[half == 0 ? 3 : 1];
+    if (c.ozp && oz_worth(Rt, R, Rt, false)) {
+        const OzMat& z = digits_Z(c, half);
+        oz_split_cols(c.st, a, b, R, c.dP);
+        mul_digits(c, z, c.dP, c.Y, R, false);
         return;
     }
-    if (half == 0)
-        dgemm(c.st, false, Rt, R, Rt, c.Z, Rt, c.W[2], c.W[3], R, c.Y, R, nullptr, false, c.part, c.part_cap);
-    else
-        dgemm(c.st, true, Rt, R, Rt, c.Z, Rt, c.W[0], c.W[1], R, c.Y, R, nullptr, false, c.part, c.part_cap);
+    dgemm(c.st, half == 1, Rt, R, Rt, c.Z, Rt, a, b, R, c.Y, R, nullptr, false, c.part, c.part_cap);
 }
 
 int partner_of(int k) { return k == 0 ? 1 : k == 1 ? 0 : k == 2 ? 3 : 2; }
 
 // M_k = X_k (W_partner o Y)
 void backproject_fp64(Ctx& c, int k, double* M) {
-    dgemm(c.st, false, c.s.n[k], c.s.R, c.s.Rt, c.X[k], c.s.Rt, c.W[partner_of(k)], c.Y, c.s.R, M,
-          c.s.R, nullptr, false, c.part, c.part_cap);
+    const int n = c.s.n[k], Rt = c.s.Rt, R = c.s.R;
+    if (c.ozp && oz_worth(n, R, Rt, false)) {
+        const OzMat& x = digits_X(c, k & 1);
+        oz_split_cols(c.st, c.W[partner_of(k)], c.Y, R, c.dP);
+        mul_digits(c, x, c.dP, M, R, false);
+        return;
+    }
+    dgemm(c.st, false, n, R, Rt, c.X[k], Rt, c.W[partner_of(k)], c.Y, R, M, R, nullptr, false, c.part, c.part_cap);
 }
 
 void others(int k, int* a, int* b, int* d) {
@@ -429,14 +555,29 @@ void others(int k, int* a, int* b, int* d) {
     *d = t[2];
 }
 
+// The digits that a sweep reads are cut here, before any sweep is captured (a cut recorded in a
+// graph would run again with every replay).
+void prepare_digits(Ctx& c) {
+    if (!c.ozp) return;
+    const int Rt = c.s.Rt, R = c.s.R;
+    const bool fp64 = c.prec == THC_CPD_FP64;
+    for (int k = 0; k < 2; ++k) {
+        if (oz_worth(Rt, R, c.s.n[k], false)) digits_XT(c, k);
+        if (fp64 && oz_worth(c.s.n[k], R, Rt, false)) digits_X(c, k);
+    }
+    if (oz_worth(Rt, R, Rt, false)) {
+        if (fp64) digits_Z(c, 0);
+        digits_Z(c, 1);
+    }
+}
+
 // W_k and G_k for every mode from the current factors (start of a run / after rollback)
 void refresh_state(Ctx& c, const double* const A[4]) {
+    prepare_digits(c);
     for (int k = 0; k < 4; ++k) {
-        if (c.prec == THC_CPD_FP64)
-            project_fp64(c, k, A[k]);
-        else
-            mixed_project(c.mx, c.st, k, A[k], false);
-        gram_fp64(c, k, A[k]);
+        const bool fp64 = c.prec == THC_CPD_FP64;
+        factor_products(c, k, A[k], true, fp64);
+        if (!fp64) mixed_project(c.mx, c.st, k, A[k], false);
     }
 }
 
@@ -457,8 +598,9 @@ thc_cpd_status mode_update(Ctx& c, double* const A[4], double* lam, int k, bool 
         CK(cudaMemcpyAsync(Mrows, c.Msave, sizeof(double) * n * R, cudaMemcpyDeviceToDevice, c.st));
         CK(cudaMemcpyAsync(c.Haug, c.Hsave, sizeof(double) * R * R, cudaMemcpyDeviceToDevice, c.st));
     }
-    chol_solve(c.st, R, n, c.Haug, A[k], c.LinvD, c.LinvD + (size_t)R * R, c.sc, k, c.counters,
-               c.dataflow ? c.flow_sync : nullptr, c.flow_ctas, c.bs_sync, c.emulated ? &c.oz : nullptr);
+    chol_solve(c.st, R, n, c.Haug, A[k], c.LinvD, c.LinvD + (c.fixed ? 0 : (size_t)R * R), c.sc, k, c.counters,
+               c.dataflow ? c.flow_sync : nullptr, c.flow_ctas, c.bs_sync, c.fixed ? &c.fix : nullptr,
+               c.fixed || c.two_level ? &c.oz : nullptr, c.two_level);
     if (safe) {
         DevScalars* h = host_scalars();
         if (!h) return set_err(THC_CPD_ERR_ALLOC, "pinned host buffer allocation failed");
@@ -474,11 +616,9 @@ thc_cpd_status mode_update(Ctx& c, double* const A[4], double* lam, int k, bool 
         }
     }
     normalise_columns(c.st, n, R, A[k], lam, c.LinvD);  // panel buffer is free after the solve
-    gram_fp64(c, k, A[k]);
-    if (c.prec == THC_CPD_FP64)
-        project_fp64(c, k, A[k]);
-    else
-        CK(mixed_project(c.mx, c.st, k, A[k], true));
+    const bool fp64 = c.prec == THC_CPD_FP64;
+    factor_products(c, k, A[k], true, fp64);
+    if (!fp64) CK(mixed_project(c.mx, c.st, k, A[k], true));
     CK(cudaGetLastError());
     return THC_CPD_OK;
 }
@@ -501,8 +641,8 @@ thc_cpd_status sweep(Ctx& c, double* const A[4], double* lam, bool safe, bool ev
             loss_eval(c.st, c.s.Rt, c.s.R, c.Y, c.W[2], c.W[3], lam, c.G, c.red, c.sc, tol);
         } else {
             // the loss is a cancelling difference: FP64 projections and Z product
-            for (int k = 0; k < 4; ++k) project_fp64(c, k, A[k], true);
-            zgemm_fp64(c, 1, true);
+            for (int k = 0; k < 4; ++k) factor_products(c, k, A[k], false, true);
+            zgemm_fp64(c, 1);
             loss_eval(c.st, c.s.Rt, c.s.R, c.Y, c.W[2], c.W[3], lam, c.G, c.red, c.sc, tol);
         }
     }
@@ -1223,7 +1363,8 @@ thc_cpd_status thc_cpd_thc_norm2(int o, int v, int Rt, const double* Xo, const d
     o2.precision = THC_CPD_FP64;
     Ctx c;
     CKS(ctx_init(c, s, Xo, Xv, Z, &o2, NEED_NORM));
-    return obtain_norm(c, 0.0, normG2_host);
+    CKS(obtain_norm(c, 0.0, normG2_host));
+    return product_errors(c);
 }
 
 thc_cpd_status thc_cpd_mttkrp(int o, int v, int Rt, int R, const double* Xo, const double* Xv,
@@ -1238,7 +1379,7 @@ thc_cpd_status thc_cpd_mttkrp(int o, int v, int Rt, int R, const double* Xo, con
     CKS(ctx_init(c, s, Xo, Xv, Z, opts, 0));
     if (c.prec == THC_CPD_FP64) {
         for (int k = 0; k < 4; ++k)
-            if (k != mode) project_fp64(c, k, A[k]);
+            if (k != mode) factor_products(c, k, A[k], false, true);
         zgemm_fp64(c, mode / 2);
         backproject_fp64(c, mode, M);
     } else {
@@ -1257,9 +1398,7 @@ thc_cpd_status thc_cpd_mttkrp(int o, int v, int Rt, int R, const double* Xo, con
     }
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(c.st));
-    if (int e = mixed_take_error())
-        return set_err(THC_CPD_ERR_TIMEOUT, "tensor-core kernel wait gave up (code %d)", e);
-    return THC_CPD_OK;
+    return product_errors(c);
 }
 
 thc_cpd_status thc_cpd_split_gemm(int M, int N, int K, const double* A, const double* B, double* C,
@@ -1313,19 +1452,17 @@ thc_cpd_status thc_cpd_loss(int o, int v, int Rt, int R, const double* Xo, const
     thc_cpd_opts o2 = opts ? *opts : thc_cpd_opts{};
     o2.precision = THC_CPD_FP64;  // the loss is always evaluated in FP64
     Ctx c;
-    CKS(ctx_init(c, s, Xo, Xv, Z, &o2, normG2 > 0.0 ? 0u : NEED_NORM));
+    CKS(ctx_init(c, s, Xo, Xv, Z, &o2, NEED_GRAM | (normG2 > 0.0 ? 0u : NEED_NORM)));
     double nG2;
     CKS(obtain_norm(c, normG2, &nG2));
-    for (int k = 0; k < 4; ++k) {
-        project_fp64(c, k, A[k]);
-        gram_fp64(c, k, A[k]);
-    }
+    for (int k = 0; k < 4; ++k) factor_products(c, k, A[k], true, true);
     zgemm_fp64(c, 1);
     loss_eval(c.st, Rt, R, c.Y, c.W[2], c.W[3], lam ? lam : c.ones, c.G, c.red, c.sc, 0.0);
     DevScalars h;
     CKS(read_scalars(c, &h));
     if (loss_host) *loss_host = h.loss;
     if (fit_host) *fit_host = h.fit;
+    CKS(product_errors(c));
     if (!isfinite(h.loss)) return set_err(THC_CPD_ERR_NONFINITE, "loss is not finite");
     return THC_CPD_OK;
 }
@@ -1374,10 +1511,9 @@ extern "C" thc_cpd_status thc_cpd_emulated_gemm(int M, int N, int K, const doubl
     if (!oz_available())
         return set_err(THC_CPD_ERR_UNSUPPORTED, "the emulated product needs an sm_103 device");
     cudaStream_t st = stream_of(opts);
-    // room for every K chunk's digits (one update launch) unless that would pass 65536 rows
-    const long nch = cdiv(K, kOzPanel);
-    const bool all = nch * (M + N) <= 65536;
-    const int rowsA = all ? (int)(nch * M) : M, rowsB = all ? (int)(nch * N) : N;
+    // room for every K chunk's digits (one launch) unless that would pass 65536 digit rows a side
+    const long nch = std::min<long>(cdiv(K, kOzPanel), std::max<long>(1, 65536 / std::max(M, N)));
+    const int rowsA = (int)(nch * M), rowsB = (int)(nch * N);
     const size_t bytes = oz_ws_bytes(rowsA, rowsB);
     struct Ws {
         void* p = nullptr;
@@ -1406,18 +1542,23 @@ namespace thc {
 int spd_solve(cudaStream_t st, int R, int n, const double* H, const double* M, double* A,
               const short* tasks, int ntasks, int* used_pinv, int ldl) {
     if (used_pinv) *used_pinv = 0;
-    if (!flow_prepare(R, n)) return set_err(THC_CPD_ERR_UNSUPPORTED, "no dataflow schedule for R=%d n=%d", R, n);
+    Ldl route = tasks || ldl == THC_CPD_LDL_BLOCKED ? Ldl::kDataflow : ldl_route(ldl, R, n, false);
+    if (route == Ldl::kBlocked) route = Ldl::kDataflow;  // (a solve alone has no blocked variant)
+    if (route == Ldl::kTwoLevel && !oz_prepare(R, n)) route = Ldl::kDataflow;
+    const bool fixed = route == Ldl::kFixed, two = route == Ldl::kTwoLevel, ozl = fixed || two;
+    if (!ozl && !flow_prepare(R, n))
+        return set_err(THC_CPD_ERR_UNSUPPORTED, "no dataflow schedule for R=%d n=%d", R, n);
     const size_t RR = (size_t)R * R, nR = (size_t)n * R;
-    const bool emu = use_emulated_ldl(ldl, R, n) && !tasks &&
-                     oz_prepare(R, n);
-    int oz_ra = R + n, oz_rb = R;
+    int oz_ra = 1, oz_rb = 1;
     size_t oz_part = 0;
-    if (emu) bsolve_ws_rows(R, n, &oz_ra, &oz_rb, &oz_part);
-    if (emu) oz_ldl_ws_rows(R, n, &oz_ra, &oz_rb);
-    size_t bytes = (emu ? oz_ws_bytes(oz_ra, oz_rb, oz_part) : 0) + Arena::need<double>(RR + nR) + 3 * Arena::need<double>(RR) + Arena::need<double>(R) +
+    if (ozl) bsolve_ws_rows(R, n, &oz_ra, &oz_rb, &oz_part);
+    if (two) oz_ldl_ws_rows(R, n, &oz_ra, &oz_rb);
+    size_t bytes = Arena::need<double>(RR + nR) + 3 * Arena::need<double>(RR) + Arena::need<double>(R) +
                    Arena::need<double>(std::max(RR, nR)) + Arena::need<double>(R) +
                    Arena::need<int>(flow_sync_ints(R, n)) + Arena::need<int>(bsolve_sync_ints(n)) +
                    Arena::need<DevScalars>(1) + Arena::need<short>(4 * (size_t)std::max(ntasks, 1));
+    if (ozl) bytes += oz_ws_bytes(oz_ra, oz_rb, oz_part);
+    if (fixed) bytes += ldl_fix_ws_bytes(R, n);
     struct Ws {
         void* p = nullptr;
         cudaStream_t st;
@@ -1442,23 +1583,27 @@ int spd_solve(cudaStream_t st, int R, int n, const double* H, const double* M, d
     DevScalars* sc = ar.take<DevScalars>(1);
     void* dtasks = ar.take<short>(4 * (size_t)std::max(ntasks, 1));
     OzWs oz;
-    if (emu) oz_ws_carve(oz, ar, oz_ra, oz_rb, oz_part);
+    FixWs fix;
+    if (ozl) oz_ws_carve(oz, ar, oz_ra, oz_rb, oz_part);
+    if (fixed) ldl_fix_carve(fix, ar, R, n);
     CK(cudaMemsetAsync(fsync, 0, sizeof(int) * flow_sync_ints(R, n), st));
     CK(cudaMemsetAsync(bsync, 0, sizeof(int) * bsolve_sync_ints(n), st));
     scalars_init(st, sc, 0.0);
     copy_with_maxdiag(st, R, H, Haug, sc);
     CK(cudaMemcpyAsync(Hsave, H, sizeof(double) * RR, cudaMemcpyDeviceToDevice, st));
     CK(cudaMemcpyAsync(Haug + RR, M, sizeof(double) * nR, cudaMemcpyDeviceToDevice, st));
-    {
+    if (fixed) {
+        CK(ldl_fix(st, R, n, Haug, dinv, sc, 0, fix));
+    } else if (two) {
+        CK(ldl_oz(st, R, n, Haug, P, dinv, sc, 0, fsync, oz));
+    } else {
         ProfScope prof(st, KC_CHOL, (double)R * R * R / 3.0 + (double)n * R * R);
         if (tasks)
             CK(ldl_flow_tasks(st, R, n, Haug, P, dinv, sc, 0, fsync, tasks, ntasks, dtasks));
-        else if (emu)
-            CK(ldl_oz(st, R, n, Haug, P, dinv, sc, 0, fsync, oz));
         else
             CK(ldl_flow(st, R, n, Haug, P, dinv, sc, 0, fsync));
     }
-    backward_solve(st, R, n, Haug, A, bsync, emu ? &oz : nullptr);
+    backward_solve(st, R, n, Haug, A, bsync, ozl ? &oz : nullptr);
     CK(cudaGetLastError());
     DevScalars* h = host_scalars();
     if (!h) return set_err(THC_CPD_ERR_ALLOC, "pinned host buffer allocation failed");

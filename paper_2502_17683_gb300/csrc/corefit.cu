@@ -119,7 +119,10 @@ extern "C" thc_cpd_status thc_cpd_core_fit(int o, int v, int Rt, int naux, const
     if (used_pinv) *used_pinv = 0;
     cudaStream_t st = opts ? (cudaStream_t)opts->stream : (cudaStream_t)0;
     const int ldl = opts ? opts->ldl : THC_CPD_LDL_AUTO;
-    const bool emu = ldl == THC_CPD_LDL_EMULATED && oz_available();
+    // products from digits on the tensor cores: all on request, else those that are faster there
+    const bool all = ldl == THC_CPD_LDL_EMULATED && oz_available();
+    const bool emu = oz_available() && (all || oz_worth(std::min(naux * o, 8192), Rt, v, false) ||
+                                        oz_worth(Rt, Rt, std::max(v, naux), true));
     if (opts) {
         const double lim = opts->wait_limit_s;
         flow_set_wait_ns(lim > 0.0 ? (unsigned long long)(lim * 1e9) : 0ull);
@@ -134,12 +137,17 @@ extern "C" thc_cpd_status thc_cpd_core_fit(int o, int v, int Rt, int naux, const
     size_t bytes = Arena::need<double>((size_t)rows_t * Rt) + 2 * Arena::need<double>((size_t)naux * Rt) +
                    3 * Arena::need<double>(RR) + Arena::need<double>(part_cap) + Arena::need<double>(3 * CF_BLOCKS + 3);
     if (loss) bytes += Arena::need<double>(ov * naux) + Arena::need<double>((size_t)naux * naux) + 2 * Arena::need<double>(RR);
-    int rowsA = std::max(rows_t, Rt), rowsB = Rt;
-    if (loss) {
-        rowsA = std::max(rowsA, naux);
-        rowsB = std::max(rowsB, naux);
+    int rowsA = 1, rowsB = 1;
+    size_t oz_part = 0;
+    if (emu) {
+        oz_product_ws(rows_t, Rt, v, &rowsA, &rowsB, &oz_part);
+        oz_product_ws(Rt, Rt, std::max(std::max(o, v), naux), &rowsA, &rowsB, &oz_part);
+        if (loss) {
+            oz_product_ws(naux, naux, std::min<size_t>(ov, 8 * kOzPanel), &rowsA, &rowsB, nullptr);
+            oz_product_ws(Rt, Rt, Rt, &rowsA, &rowsB, &oz_part);
+        }
+        bytes += oz_ws_bytes(rowsA, rowsB, oz_part);
     }
-    if (emu) bytes += oz_ws_bytes(rowsA, rowsB);
     void* block = nullptr;
     if (cudaMallocAsync(&block, bytes, st) != cudaSuccess) return cerr(THC_CPD_ERR_ALLOC, "workspace allocation failed");
     struct Free {
@@ -166,11 +174,11 @@ extern "C" thc_cpd_status thc_cpd_core_fit(int o, int v, int Rt, int naux, const
         W2 = ar.take<double>(RR);
     }
     OzWs oz;
-    if (emu) oz_ws_carve(oz, ar, rowsA, rowsB);
+    if (emu) oz_ws_carve(oz, ar, rowsA, rowsB, oz_part);
     auto gemm = [&](bool ta, int M, int N, int K, const double* A, int lda, const double* Bp, int ldb, double* C,
                     int ldc, bool symm) {
-        if (emu)
-            return oz_dgemm(st, ta, M, N, K, A, lda, Bp, nullptr, ldb, C, ldc, nullptr, symm, oz);
+        if (all || (emu && oz_worth(std::min(M, 8192), N, K, symm)))
+            return oz_dgemm(st, ta, M, N, K, A, lda, Bp, nullptr, ldb, C, ldc, symm, oz);
         dgemm(st, ta, M, N, K, A, lda, Bp, nullptr, ldb, C, ldc, nullptr, symm, gpart, part_cap);
         return cudaGetLastError();
     };

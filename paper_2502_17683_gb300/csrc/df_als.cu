@@ -88,7 +88,7 @@ thc_cpd_status derr(thc_cpd_status s, const char* fmt, ...) {
 struct DfCtx {
     cudaStream_t st;
     int o, v, naux, R, ldl;
-    bool emu;
+    bool all, emu;  // every product from digits on the tensor cores / those that are faster there
     const double* B;
     double *Bp, *T, *V12, *V34, *ones, *H, *M, *lamtmp, *gpart, *red;
     double* G[4];
@@ -102,8 +102,8 @@ struct DfCtx {
     }
     void gemm(bool ta, int M_, int N_, int K_, const double* A, int lda, const double* Bm, int ldb, double* C,
               int ldc, bool symm) {
-        if (emu)
-            ck(oz_dgemm(st, ta, M_, N_, K_, A, lda, Bm, nullptr, ldb, C, ldc, nullptr, symm, oz));
+        if (all || (emu && oz_worth(std::min(M_, 8192), N_, K_, symm)))
+            ck(oz_dgemm(st, ta, M_, N_, K_, A, lda, Bm, nullptr, ldb, C, ldc, symm, oz));
         else
             dgemm(st, ta, M_, N_, K_, A, lda, Bm, nullptr, ldb, C, ldc, nullptr, symm, gpart, part_cap);
     }
@@ -153,7 +153,8 @@ extern "C" thc_cpd_status thc_cpd_df_als(int o, int v, int naux, int R, const do
     c.naux = naux;
     c.R = R;
     c.ldl = opts ? opts->ldl : THC_CPD_LDL_AUTO;
-    c.emu = c.ldl == THC_CPD_LDL_EMULATED && oz_available();
+    c.all = c.ldl == THC_CPD_LDL_EMULATED && oz_available();
+    c.emu = c.all || (oz_available() && oz_worth((int)std::min<long>(naux * std::max(o, v), 8192), R, std::max(o, v), false));
     c.B = B;
     if (opts) {
         const double lim = opts->wait_limit_s;
@@ -162,12 +163,19 @@ extern "C" thc_cpd_status thc_cpd_df_als(int o, int v, int naux, int R, const do
     const size_t RR = (size_t)R * R, ov = (size_t)o * v, nR = (size_t)naux * R;
     c.part_cap = std::max(dgemm_part_need((int)(naux * nmax), R, (int)nmax), dgemm_part_need(R, R, (int)nmax));
     c.part_cap = std::max(c.part_cap, dgemm_part_need(naux, naux, (int)ov));
-    const int rowsA = (int)std::max<long>(naux * nmax, R), rowsB = std::max(R, naux);
+    int rowsA = 1, rowsB = 1;
+    size_t oz_part = 0;
+    if (c.emu) {
+        oz_product_ws(naux * o, R, v, &rowsA, &rowsB, &oz_part);
+        oz_product_ws(naux * v, R, o, &rowsA, &rowsB, &oz_part);
+        oz_product_ws(R, R, (int)nmax, &rowsA, &rowsB, nullptr);
+        oz_product_ws(naux, naux, (int)std::min<size_t>(ov, 8 * kOzPanel), &rowsA, &rowsB, nullptr);
+    }
     size_t bytes = Arena::need<double>(ov * naux) * 2 + Arena::need<double>((size_t)naux * nmax * R) +
                    3 * Arena::need<double>(nR) + 5 * Arena::need<double>(RR) + Arena::need<double>(nmax * R) +
                    Arena::need<double>(R) + Arena::need<double>(c.part_cap) + Arena::need<double>(loss_red_need()) +
                    Arena::need<double>((size_t)naux * naux) + Arena::need<DevScalars>(1);
-    if (c.emu) bytes += oz_ws_bytes(rowsA, rowsB);
+    if (c.emu) bytes += oz_ws_bytes(rowsA, rowsB, oz_part);
     void* block = nullptr;
     if (cudaMallocAsync(&block, bytes, c.st) != cudaSuccess) return derr(THC_CPD_ERR_ALLOC, "workspace allocation failed");
     struct Free {
@@ -192,7 +200,7 @@ extern "C" thc_cpd_status thc_cpd_df_als(int o, int v, int naux, int R, const do
     c.red = ar.take<double>(loss_red_need());
     double* Q = ar.take<double>((size_t)naux * naux);
     c.sc = ar.take<DevScalars>(1);
-    if (c.emu) oz_ws_carve(c.oz, ar, rowsA, rowsB);
+    if (c.emu) oz_ws_carve(c.oz, ar, rowsA, rowsB, oz_part);
     cudaStream_t st = c.st;
 
     // set-up: permuted B, ||G_DF||^2 = ||D D^T||^2, Grams, V34 of the start factors

@@ -115,7 +115,14 @@ extern "C" thc_cpd_status thc_cpd_exchange(int o, int v, int Rt, int R, int nalp
     if (chk != THC_CPD_OK) return (thc_cpd_status)chk;
     if (nalpha < 1 || nalpha > 1024) return xerr(THC_CPD_ERR_SHAPE, "need 1 <= nalpha <= 1024");
     if (!lam || !Lam || !Gam) return xerr(THC_CPD_ERR_ARG, "lam, Lam and Gam must be non-null");
-    const bool emu = opts && opts->ldl == THC_CPD_LDL_EMULATED && oz_available() && Rt <= 8192 && R <= 8192;
+    // the products that are faster from digits (all of them on request) run on the tensor cores; the
+    // digits of the factors' columns are cut once for all points, those of Lam o X and Gam o X once per point
+    const bool ozd = oz_available() && Rt <= 8192 && R <= 8192 && std::max(o, v) <= 8192;
+    const bool all = ozd && opts && opts->ldl == THC_CPD_LDL_EMULATED;
+    auto on_tc = [&](int M, int N, int K, bool symm) { return all || (ozd && oz_worth(M, N, K, symm)); };
+    const bool tc_z = on_tc(Rt, R, Rt, false), tc_u[2] = {on_tc(Rt, R, o, false), on_tc(Rt, R, v, false)};
+    const bool tc_m = on_tc(R, R, o, true), tc_n = on_tc(R, R, v, false);
+    const bool emu = tc_z || tc_u[0] || tc_u[1] || tc_m || tc_n;
     cudaStream_t st = opts ? (cudaStream_t)opts->stream : (cudaStream_t)0;
     const size_t RtR = (size_t)Rt * R, RR = (size_t)R * R;
     const int nmax = std::max(o, v);
@@ -125,7 +132,15 @@ extern "C" thc_cpd_status thc_cpd_exchange(int o, int v, int Rt, int R, int nalp
                    5 * Arena::need<double>(RtR) + 3 * Arena::need<double>((size_t)nmax * R) +
                    3 * Arena::need<double>(RR) + Arena::need<double>(XR_BLOCKS) +
                    Arena::need<double>(2 * (size_t)nalpha) + Arena::need<double>(part_cap);
-    if (emu) bytes += oz_ws_bytes(std::max(Rt, R), R);
+    int oz_ra = 1, oz_rb = 1;
+    size_t oz_part = 0;
+    if (emu) {
+        oz_product_ws(Rt, R, Rt, &oz_ra, &oz_rb, &oz_part);
+        oz_product_ws(Rt, R, nmax, &oz_ra, &oz_rb, &oz_part);
+        oz_product_ws(R, R, nmax, &oz_ra, &oz_rb, &oz_part);
+        bytes += oz_ws_bytes(oz_ra, oz_rb, oz_part) + 2 * ozmat_bytes(R, o) + 2 * ozmat_bytes(R, v) +
+                 ozmat_bytes(Rt, o) + ozmat_bytes(Rt, v) + ozmat_bytes(Rt, Rt) + ozmat_bytes(R, Rt) + ozmat_bytes(R, nmax);
+    }
     void* block = nullptr;
     if (cudaMallocAsync(&block, bytes, st) != cudaSuccess) return xerr(THC_CPD_ERR_ALLOC, "workspace allocation failed");
     Arena ar;
@@ -146,13 +161,25 @@ extern "C" thc_cpd_status thc_cpd_exchange(int o, int v, int Rt, int R, int nalp
     double* res = ar.take<double>(2 * (size_t)nalpha);
     double* gpart = ar.take<double>(part_cap);
     OzWs oz;
-    if (emu) oz_ws_carve(oz, ar, std::max(Rt, R), R);
+    OzMat dA[4], dXo, dXv, dZ, dP, dS;
+    if (emu) {
+        oz_ws_carve(oz, ar, oz_ra, oz_rb, oz_part);
+        for (int k = 0; k < 4; ++k) ozmat_carve(dA[k], ar, R, (k & 1) ? v : o);
+        ozmat_carve(dXo, ar, Rt, o);
+        ozmat_carve(dXv, ar, Rt, v);
+        ozmat_carve(dZ, ar, Rt, Rt);
+        ozmat_carve(dP, ar, R, Rt);
+        ozmat_carve(dS, ar, R, nmax);
+        for (int k = 0; k < 4; ++k)
+            if (tc_u[k & 1] || ((k & 1) ? (tc_n && k == 1) : tc_m)) oz_split_cols(st, A[k], nullptr, R, dA[k]);
+        if (tc_z) oz_split_rows(st, Z, Rt, dZ);
+    }
     auto gemm = [&](bool ta, int M, int Nn, int K, const double* Ap, int lda, const double* Bp,
                     const double* B2, int ldb, double* C, int ldc) {
-        if (emu)
-            oz_dgemm(st, ta, M, Nn, K, Ap, lda, Bp, B2, ldb, C, ldc, nullptr, false, oz);
-        else
-            dgemm(st, ta, M, Nn, K, Ap, lda, Bp, B2, ldb, C, ldc, nullptr, false, gpart, part_cap);
+        dgemm(st, ta, M, Nn, K, Ap, lda, Bp, B2, ldb, C, ldc, nullptr, false, gpart, part_cap);
+    };
+    auto mul = [&](const OzMat& a, const OzMat& b, double* C, bool symm) {
+        oz_mul(st, a, b, C, R, 1.0, symm ? OZ_SYMM : 0, oz.part, oz.part_cap);
     };
     auto scale = [&](int rows, int n, const double* s, const double* X, double* out) {
         const long total = (long)rows * n;
@@ -166,22 +193,53 @@ extern "C" thc_cpd_status thc_cpd_exchange(int o, int v, int Rt, int R, int nalp
             const double* lA = Lam + (size_t)al * o;
             const double* gA = Gam + (size_t)al * v;
             // single CPD
-            scale(o, Rt, lA, Xo, XoL);
-            scale(v, Rt, gA, Xv, XvG);
-            gemm(true, Rt, R, o, XoL, Rt, A[0], nullptr, R, U[0], R);
-            gemm(true, Rt, R, o, XoL, Rt, A[2], nullptr, R, U[2], R);
-            gemm(true, Rt, R, v, XvG, Rt, A[1], nullptr, R, U[1], R);
-            gemm(true, Rt, R, v, XvG, Rt, A[3], nullptr, R, U[3], R);
-            gemm(false, Rt, R, Rt, Z, Rt, U[2], U[1], R, Y, R);  // Z (U3 o U2)
+            if (tc_u[0]) {
+                oz_split_cols(st, Xo, nullptr, Rt, dXo, lA);
+                mul(dXo, dA[0], U[0], false);
+                mul(dXo, dA[2], U[2], false);
+            } else {
+                scale(o, Rt, lA, Xo, XoL);
+                gemm(true, Rt, R, o, XoL, Rt, A[0], nullptr, R, U[0], R);
+                gemm(true, Rt, R, o, XoL, Rt, A[2], nullptr, R, U[2], R);
+            }
+            if (tc_u[1]) {
+                oz_split_cols(st, Xv, nullptr, Rt, dXv, gA);
+                mul(dXv, dA[1], U[1], false);
+                mul(dXv, dA[3], U[3], false);
+            } else {
+                scale(v, Rt, gA, Xv, XvG);
+                gemm(true, Rt, R, v, XvG, Rt, A[1], nullptr, R, U[1], R);
+                gemm(true, Rt, R, v, XvG, Rt, A[3], nullptr, R, U[3], R);
+            }
+            if (tc_z) {  // Z (U3 o U2)
+                oz_split_cols(st, U[2], U[1], R, dP);
+                mul(dZ, dP, Y, false);
+            } else {
+                gemm(false, Rt, R, Rt, Z, Rt, U[2], U[1], R, Y, R);
+            }
             k_single_partials<<<XR_BLOCKS, XR_THREADS, 0, st>>>((long)RtR, R, U[0], U[3], Y, lam, part);
             k_neg_final<<<1, XR_THREADS, 0, st>>>(part, XR_BLOCKS, res + 2 * al);
             // double CPD
-            scale(o, R, lA, A[0], A1L);
-            scale(o, R, lA, A[2], A3L);
-            scale(v, R, gA, A[3], A4G);
-            gemm(true, R, R, o, A[0], R, A1L, nullptr, R, M1, R);
-            gemm(true, R, R, o, A[2], R, A3L, nullptr, R, M3, R);
-            gemm(true, R, R, v, A[1], R, A4G, nullptr, R, N, R);
+            if (tc_m) {  // A^T diag(Lam) A is symmetric
+                dS.K = o;
+                oz_split_cols(st, A[0], nullptr, R, dS, lA);
+                mul(dA[0], dS, M1, true);
+                oz_split_cols(st, A[2], nullptr, R, dS, lA);
+                mul(dA[2], dS, M3, true);
+            } else {
+                scale(o, R, lA, A[0], A1L);
+                scale(o, R, lA, A[2], A3L);
+                gemm(true, R, R, o, A[0], R, A1L, nullptr, R, M1, R);
+                gemm(true, R, R, o, A[2], R, A3L, nullptr, R, M3, R);
+            }
+            if (tc_n) {
+                dS.K = v;
+                oz_split_cols(st, A[3], nullptr, R, dS, gA);
+                mul(dA[1], dS, N, false);
+            } else {
+                scale(v, R, gA, A[3], A4G);
+                gemm(true, R, R, v, A[1], R, A4G, nullptr, R, N, R);
+            }
             k_double_partials<<<XR_BLOCKS, XR_THREADS, 0, st>>>(R, M1, N, M3, lam, part);
             k_neg_final<<<1, XR_THREADS, 0, st>>>(part, XR_BLOCKS, res + 2 * al + 1);
             count_launch(4);

@@ -26,21 +26,24 @@ void hadamard3(cudaStream_t st, int R, const double* Ga, const double* Gb, const
 //   A pivot <= R * eps * sc->maxdiag sets bit `mode` of sc->fail_mask (the result is then
 //   garbage and the caller replays the mode with the pseudo-inverse).
 //   counters: cdiv(R, 32) ints (arrival counters of the update kernels, cleared inside).
+//   fix: with it the factorisation runs in fixed-point blocks of 128 columns with tensor-core
+//   trailing updates (ldl_fix.cu); else
 //   flow_sync: flow_sync_ints(R, n) ints, zero before the first use (each launch leaves
 //   them zero), or null: with it (and a plan for (R, n)) the factorisation runs as one
-//   persistent dataflow launch (P is then R x R), else as one launch per block step.
+//   persistent dataflow launch (P is then R x R), or (two_level) in dataflow panels with
+//   emulated trailing updates (ldl_oz, oz.cuh), else as one launch per block step.
 //   flow_ctas: 0 = the dataflow kernel takes one CTA per SM; > 0 = at most that many CTAs
 //   with only the shared memory they use (problems running side by side).
 //   bs_sync: bsolve_sync_ints(n) ints, the progress counters of the backward solve (by
 //   column slices, ldl_flow.cu); zero before the first use, left zero by each launch.
-//   oz: with it (and flow_sync) the factorisation runs in 256- (below R = 1536: 128-) column panels with emulated
-//   FP64 tensor-core trailing updates (ldl_oz, oz.cuh).
+//   oz: workspace of the split backward solve's products, or null.
 struct OzWs;
+struct FixWs;
 void chol_solve(cudaStream_t st, int R, int n, double* Haug, double* A, double* P, double* dinv,
                 DevScalars* sc, int mode, int* counters, int* flow_sync, int flow_ctas,
-                int* bs_sync, const OzWs* oz = nullptr);
-// The backward solve A L = Y of a factorised Haug (Y in its rows R..R+n): with an emulated
-// factorisation's workspace (oz) and n >= 128, a block of >= 768 columns is split at a
+                int* bs_sync, const FixWs* fix = nullptr, const OzWs* oz = nullptr, bool two_level = false);
+// The backward solve A L = Y of a factorised Haug (Y in its rows R..R+n): with a product
+// workspace (oz) and n >= 128, a block of >= 768 columns is split at a
 // column h0: the trailing block first, the coupling Y1 -= A2 L21 as an emulated product,
 // then the leading block, each of them split again by the same rule.
 void backward_solve(cudaStream_t st, int R, int n, double* Haug, double* A, int* bs_sync,

@@ -579,11 +579,13 @@ int bsolve_split_point(int m, int n) {
 
 void chol_solve(cudaStream_t st, int R, int n, double* Haug, double* A, double* P, double* dinv,
                 DevScalars* sc, int mode, int* counters, int* flow_sync, int flow_ctas,
-                int* bs_sync, const OzWs* oz) {
+                int* bs_sync, const FixWs* fix, const OzWs* oz, bool two_level) {
     NvtxRange nvtx_range("thc_cpd LDL^T and solve");
     const int nrows = R + n;
     const int nJ = cdiv(R, NB);
-    if (oz && flow_sync) {
+    if (fix) {
+        ldl_fix(st, R, n, Haug, dinv, sc, mode, *fix);
+    } else if (two_level && oz && flow_sync) {
         ldl_oz(st, R, n, Haug, P, dinv, sc, mode, flow_sync, *oz, flow_ctas);
     } else if (flow_sync && flow_prepare(R, n)) {
         ProfScope prof(st, KC_CHOL, (double)R * R * R / 3.0 + (double)n * R * R);

@@ -59,7 +59,7 @@ struct NdCtx {
     cudaStream_t st;
     int d, dL, Rt, R, nmax, ldl;
     int n[ND_MAX];
-    bool emu;
+    bool all, emu;  // every product from digits on the tensor cores / those that are faster there
     const double* X[ND_MAX];
     const double* Z;
     double *W[ND_MAX], *G[ND_MAX];
@@ -74,8 +74,8 @@ struct NdCtx {
     }
     void gemm(bool ta, int M_, int N_, int K_, const double* A, int lda, const double* B, int ldb, double* C,
               int ldc, bool symm) {
-        if (emu)
-            ck(oz_dgemm(st, ta, M_, N_, K_, A, lda, B, nullptr, ldb, C, ldc, nullptr, symm, oz));
+        if (all || (emu && oz_worth(M_, N_, K_, symm)))
+            ck(oz_dgemm(st, ta, M_, N_, K_, A, lda, B, nullptr, ldb, C, ldc, symm, oz));
         else
             dgemm(st, ta, M_, N_, K_, A, lda, B, nullptr, ldb, C, ldc, nullptr, symm, gpart, part_cap);
     }
@@ -149,18 +149,31 @@ thc_cpd_status nd_alloc(NdCtx& c, int d, int dL, const int* dims, int Rt, int R,
     }
     c.Z = Z;
     c.ldl = opts ? opts->ldl : THC_CPD_LDL_AUTO;
-    c.emu = c.ldl == THC_CPD_LDL_EMULATED && oz_available();
+    c.all = c.ldl == THC_CPD_LDL_EMULATED && oz_available();
+    c.emu = c.all || (oz_available() && (oz_worth(Rt, R, Rt, false) || oz_worth(Rt, R, c.nmax, false) ||
+                                         oz_worth(R, R, c.nmax, true) || (setup && oz_worth(Rt, Rt, Rt, false))));
     const size_t RtR = (size_t)Rt * R, RR = (size_t)R * R, RtRt = (size_t)Rt * Rt;
     c.part_cap = std::max(dgemm_part_need(Rt, R, c.nmax), dgemm_part_need(Rt, R, Rt));
     c.part_cap = std::max(c.part_cap, std::max(dgemm_part_need(c.nmax, R, Rt), dgemm_part_need(R, R, c.nmax)));
     if (setup) c.part_cap = std::max(c.part_cap, std::max(dgemm_part_need(Rt, Rt, c.nmax), dgemm_part_need(Rt, Rt, Rt)));
-    const int rowsA = std::max(std::max(c.nmax, Rt), R), rowsB = std::max(R, Rt);
+    int rowsA = 1, rowsB = 1;
+    size_t oz_part = 0;
+    if (c.emu) {
+        for (int k = 0; k < d; ++k) {
+            oz_product_ws(Rt, R, c.n[k], &rowsA, &rowsB, &oz_part);
+            oz_product_ws(c.n[k], R, Rt, &rowsA, &rowsB, &oz_part);
+            oz_product_ws(R, R, c.n[k], &rowsA, &rowsB, nullptr);
+            if (setup) oz_product_ws(Rt, Rt, c.n[k], &rowsA, &rowsB, nullptr);
+        }
+        oz_product_ws(Rt, R, Rt, &rowsA, &rowsB, &oz_part);
+        if (setup) oz_product_ws(Rt, Rt, Rt, &rowsA, &rowsB, &oz_part);
+    }
     size_t bytes = (size_t)d * (Arena::need<double>(RtR) + Arena::need<double>(RR)) + 3 * Arena::need<double>(RtR) +
                    Arena::need<double>((size_t)c.nmax * R) + 2 * Arena::need<double>(RR) +
                    Arena::need<double>(std::max(RtR, RR)) + Arena::need<double>(R) + Arena::need<double>(c.part_cap) +
                    Arena::need<double>(loss_red_need()) + Arena::need<DevScalars>(1);
     if (setup) bytes += 3 * Arena::need<double>(RtRt);
-    if (c.emu) bytes += oz_ws_bytes(rowsA, rowsB);
+    if (c.emu) bytes += oz_ws_bytes(rowsA, rowsB, oz_part);
     if (cudaMallocAsync(block, bytes, c.st) != cudaSuccess) return nerr(THC_CPD_ERR_ALLOC, "workspace allocation failed");
     Arena ar;
     ar.base = (char*)*block;
@@ -186,7 +199,7 @@ thc_cpd_status nd_alloc(NdCtx& c, int d, int dL, const int* dims, int Rt, int R,
         c.SR = ar.take<double>(RtRt);
         c.U = ar.take<double>(RtRt);
     }
-    if (c.emu) oz_ws_carve(c.oz, ar, rowsA, rowsB);
+    if (c.emu) oz_ws_carve(c.oz, ar, rowsA, rowsB, oz_part);
     return THC_CPD_OK;
 }
 
