@@ -31,10 +31,10 @@ __device__ __forceinline__ long long fixed62(double x, int e) {
         m |= 1LL << 52;
     else
         ex = 1;
-    const int sh = (ex - 1022) - e + 9;  // <= 9
+    const int sh = (ex - 1022) - e + 9;  // <= 9 for a normal x (a subnormal m has fewer bits)
     long long X = 0;
     if (sh >= 0)
-        X = m << min(sh, 10);
+        X = (long long)((unsigned long long)m << min(sh, 62));
     else if (sh > -54)
         X = (m + (1LL << (-sh - 1))) >> (-sh);
     return b < 0 ? -X : X;
