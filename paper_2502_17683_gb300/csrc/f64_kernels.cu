@@ -180,6 +180,73 @@ k_dsyrk32(int N, int K, const double* __restrict__ A, const double* __restrict__
     }
 }
 
+// The same product on T x T tiles (T = 8, 16, 32; 64 threads) for outputs that give the 64-wide
+// tiles too few CTAs: an SM takes T^2 K / 2 clocks per tile on its FP64 pipe, so a 60 x 80 x 5
+// product on two 64 x 64 tiles (K padded to 16) costs 16 us and on 80 of 8 x 8 under 2 us. K is
+// not split and not padded; with T = 8 a K of 64 is loaded at once. SYMM: lower tiles only, mirrored.
+template <int T, bool TA, bool HADB, bool SYMM>
+__global__ void __launch_bounds__(64)
+k_dgemm_small(int M, int N, int K, const double* __restrict__ A, int lda, const double* __restrict__ B,
+              const double* __restrict__ B2, int ldb, double* __restrict__ C, int ldc) {
+    constexpr int BK = 512 / T, Q = T / 8;  // Q x Q outputs per thread
+    constexpr int PER = T * BK / 64;        // elements of each operand tile per thread
+    __shared__ double As[BK][T + 1];
+    __shared__ double Bs[BK][T + 1];
+    const int bx = blockIdx.x, by = blockIdx.y;
+    if (SYMM && by < bx) return;
+    const int m0 = by * T, n0 = bx * T, tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+    double acc[Q][Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i)
+#pragma unroll
+        for (int j = 0; j < Q; ++j) acc[i][j] = 0.0;
+    for (int k0 = 0; k0 < K; k0 += BK) {
+        const int kn = min(BK, K - k0);
+        double av[PER], bv[PER];
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            const int idx = tid + 64 * u;
+            const int r = TA ? idx % T : idx / BK, c = TA ? idx / T : idx % BK;
+            const int m = m0 + r;
+            av[u] = (m < M && c < kn) ? (TA ? A[(size_t)(k0 + c) * lda + m] : A[(size_t)m * lda + k0 + c]) : 0.0;
+            const int rb = idx % T, cb = idx / T, n = n0 + rb;
+            bv[u] = 0.0;
+            if (n < N && cb < kn) {
+                const size_t o = (size_t)(k0 + cb) * ldb + n;
+                bv[u] = HADB ? B[o] * B2[o] : B[o];
+            }
+        }
+        if (k0) __syncthreads();
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            const int idx = tid + 64 * u;
+            As[TA ? idx / T : idx % BK][TA ? idx % T : idx / BK] = av[u];
+            Bs[idx / T][idx % T] = bv[u];
+        }
+        __syncthreads();
+        for (int kk = 0; kk < kn; ++kk) {
+            double a[Q], b[Q];
+#pragma unroll
+            for (int i = 0; i < Q; ++i) a[i] = As[kk][ty + 8 * i];
+#pragma unroll
+            for (int j = 0; j < Q; ++j) b[j] = Bs[kk][tx + 8 * j];
+#pragma unroll
+            for (int i = 0; i < Q; ++i)
+#pragma unroll
+                for (int j = 0; j < Q; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < Q; ++i)
+#pragma unroll
+        for (int j = 0; j < Q; ++j) {
+            const int m = m0 + ty + 8 * i, n = n0 + tx + 8 * j;
+            if (m >= M || n >= N) continue;
+            C[(size_t)m * ldc + n] = acc[i][j];
+            if (SYMM) C[(size_t)n * ldc + m] = acc[i][j];
+        }
+}
+
 namespace {
 struct GemmPlan {
     int BM, BN, splits, kchunk, tiles;
@@ -247,6 +314,54 @@ void dispatch_gemm(cudaStream_t st, const GemmPlan& p, bool ta, bool hadb, bool 
     THC_G(false, false, true)
 #undef THC_G
 }
+
+// Tile of the small-tile kernel for a product, or 0 when the large tiles (splits of K included) are
+// estimated faster: clocks of the busiest SM, T^2 / 2 per step of K and tile on the FP64 pipe (32 x
+// 32 and 64 x 64 tiles run their K in steps of 16, padded), ~800 per loaded chunk of K (latency) and
+// ~6000 for the second launch of a split.
+int small_tile(int M, int N, int K, bool symm, bool trans_a, const GemmPlan& p) {
+    if (K < 1) return 0;
+    auto waves = [&](long tiles) { return (double)cdiv(tiles, num_sms()); };
+    double best;
+    if (symm && trans_a) {
+        const long t = cdiv(N, SYT);
+        best = waves(t * (t + 1) / 2) * (cdiv(K, 16) * (800.0 + 16 * SYT * SYT / 2.0));
+    } else {
+        best = waves((long)p.tiles * p.splits) * (cdiv(p.kchunk, 16) * (800.0 + 16 * p.BM * 64 / 2.0)) +
+               (p.splits > 1 ? 6000.0 : 0.0);
+    }
+    int tile = 0;
+    for (int T : {32, 16, 8}) {
+        const long tm = cdiv(M, T), tn = cdiv(N, T);
+        const int bk = 512 / T;
+        const double c = waves(symm ? tm * (tm + 1) / 2 : tm * tn) * (cdiv(K, bk) * 800.0 + K * T * T / 2.0);
+        if (c < 0.9 * best) {
+            best = c;
+            tile = T;
+        }
+    }
+    return tile;
+}
+
+template <int T>
+bool launch_small(cudaStream_t st, bool ta, bool hadb, bool symm, int M, int N, int K, const double* A, int lda,
+                  const double* B, const double* B2, int ldb, double* C, int ldc) {
+    const dim3 grid(cdiv(N, T), cdiv(M, T));
+    if (grid.y > 65535) return false;
+#define THC_S(TA_, HB_, SY_)                                                                             \
+    if (ta == TA_ && hadb == HB_ && symm == SY_) {                                                       \
+        k_dgemm_small<T, TA_, HB_, SY_><<<grid, 64, 0, st>>>(M, N, K, A, lda, B, B2, ldb, C, ldc);       \
+        return true;                                                                                     \
+    }
+    THC_S(false, false, false)
+    THC_S(false, true, false)
+    THC_S(true, false, false)
+    THC_S(true, true, false)
+    THC_S(true, false, true)
+    THC_S(false, false, true)
+#undef THC_S
+    return false;
+}
 }  // namespace
 
 size_t dgemm_part_need(int M, int N, int K) {
@@ -272,6 +387,17 @@ void dgemm(cudaStream_t st, bool trans_a, int M, int N, int K, const double* A, 
     }
     const bool hadb = B2 != nullptr;
     ProfScope prof(st, KC_DGEMM, (symm ? 1.0 : 2.0) * M * (double)N * K);
+    if (!E) {
+        const int T = small_tile(M, N, K, symm, trans_a, p);
+        const bool done =
+            T == 8 ? launch_small<8>(st, trans_a, hadb, symm, M, N, K, A, lda, B, B2, ldb, C, ldc)
+            : T == 16 ? launch_small<16>(st, trans_a, hadb, symm, M, N, K, A, lda, B, B2, ldb, C, ldc)
+            : T == 32 ? launch_small<32>(st, trans_a, hadb, symm, M, N, K, A, lda, B, B2, ldb, C, ldc) : false;
+        if (done) {
+            count_launch();
+            return;
+        }
+    }
     if (symm && trans_a && !hadb && !E && M == N && lda == ldb && K > 0) {
         const int nt = cdiv(N, SYT);
         count_launch();
