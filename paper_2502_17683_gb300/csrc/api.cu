@@ -234,12 +234,11 @@ enum : unsigned { NEED_ALS = 1, NEED_NORM = 2, NEED_GRAM = 4, NEED_BATCHED = 8 }
 // The factorisation of an R x R normal matrix for the `ldl` option.
 enum class Ldl { kBlocked, kDataflow, kTwoLevel, kFixed };
 constexpr int kEmulatedMinR = 1024;
-constexpr int kFixedMinR = 48, kFixedMaxR = 128;
 constexpr int kFixedBatchedMinR = 400;
-// On its own, a problem takes the fixed-point kernel (ldl_fix.cu) while it is a single block of some
-// tiles (48 to 128 columns), the dataflow kernel up to 1024 and from there dataflow panels with emulated trailing updates (within
-// their plans' range). Side by side, problems of 400 columns and more take fixed-point blocks,
-// which leave the FP64 pipes to the others, smaller ones the blocked FP64 kernels.
+// On its own, a problem takes the dataflow kernel up to 1024 columns and from there dataflow panels
+// with emulated trailing updates (within their plans' range). Side by side, problems of 400 columns
+// and more take fixed-point blocks (ldl_fix.cu), which leave the FP64 pipes to the others, smaller
+// ones the blocked FP64 kernels.
 Ldl ldl_route(int ldl, int R, int nmax, bool batched) {
     const bool two = R > kOzPanel && R <= 4096 && cdiv((long)R + nmax - kOzPanel, 16) <= 256;
     switch (ldl) {
@@ -249,7 +248,7 @@ Ldl ldl_route(int ldl, int R, int nmax, bool batched) {
         default: break;
     }
     if (two && R >= kEmulatedMinR) return Ldl::kTwoLevel;
-    if ((batched ? R >= kFixedBatchedMinR : R >= kFixedMinR && R <= kFixedMaxR) && ldl_fix_prepare()) return Ldl::kFixed;
+    if (batched && R >= kFixedBatchedMinR && ldl_fix_prepare()) return Ldl::kFixed;
     return batched ? Ldl::kBlocked : Ldl::kDataflow;
 }
 

@@ -10,9 +10,9 @@
 // warp), runs beside the FP64 work of others, and a one-CTA kernel of it carries a pivot column in
 // ~500 clocks (a dataflow panel ~1300 on its four kinds of CTA, ldl_flow.cu). Measured: 12 problems
 // of R = 144 .. 1080, two sweeps: 35.6 ms with the blocked FP64 kernels, 22.8 ms with these from
-// R = 400 on; alone, R = 80 with 15 rows: 59 us against 83 us of the dataflow kernel, but 1.3 ms
-// against 1.2 ms of emulated dataflow panels at R = 1080: the chain of one CTA (67 us per 128
-// columns, half of it the trailing update of the block itself) bounds it there.
+// R = 400 on. Alone, a solve takes 155 us at R = 80 (15 rows; the dataflow kernel 149) and 1.33 ms at
+// R = 1080 (dataflow panels with emulated updates 1.21): the chain of one CTA (67 us per 128
+// columns, half of it the block's own trailing update) bounds it, so it runs in batches only.
 // Accuracy: the block is scaled symmetrically by powers of two so that its diagonal lies in
 // [1/4, 1): every entry of a positive definite matrix and of its Schur complements is then below 1
 // in magnitude. All quantities are held with 62 fraction bits (l = x' / d' <= 2: 61); each product

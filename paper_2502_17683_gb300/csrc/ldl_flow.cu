@@ -913,10 +913,11 @@ const Plan* get_plan(int R, int n) {
     int nsm = 152;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     // every SM (measured: 152 CTAs beat 120 and 80 at R = 720; the chain's waits for
-    // workers shrink), fewer only when there are fewer tasks than worker groups
-    p.grid = (int)std::min<long>(nsm, 1 + std::max<long>(1, ((long)p.nmain + kGroups - 1) / kGroups));
-    // four critical CTAs on a full grid (seven critical tasks per chain step), else one
-    p.ncrit = p.ntasks > p.nmain ? (p.grid >= 16 ? 4 : 1) : 0;
+    // workers shrink), fewer only when there are fewer main tasks than CTAs: a CTA's four
+    // groups share its SM's FP64 pipe, so few tasks are spread one per SM
+    p.grid = (int)std::min<long>(nsm, 1 + std::max<long>(1, p.nmain));
+    // four critical CTAs (seven critical tasks per chain step) on a grid of some size, else one
+    p.ncrit = p.ntasks > p.nmain ? (p.grid >= 8 ? 4 : 1) : 0;
     p.grid = std::min(nsm, p.grid + p.ncrit);
     if (p.grid < 1 + p.ncrit + (p.nmain > 0 ? 1 : 0)) return nullptr;
     if (cudaFuncSetAttribute(k_ldl_flow, cudaFuncAttributeMaxDynamicSharedMemorySize, kFlowSmem) !=
