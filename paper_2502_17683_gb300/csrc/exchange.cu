@@ -7,8 +7,13 @@
 //   double CPD:  M1 = A1^T diag(Lam) A1, M3 = A3^T diag(Lam) A3, N = A2^T diag(Gam) A4,
 //       E_double = - lam^T (M1 o N o M3 o N^T) lam                       O(N R^2)
 //   robust (Eq. rob_K):  E_robust = 2 E_single - E_double (no first-order CPD error).
-// The products run as FP64 GEMMs, on the FP64 pipes or, on request, as the FP64-accurate
-// emulated products of the BF16 tensor cores (oz_dgemm); the reductions are fixed-order.
+// The quadrature points are independent, so a group of them (as many as 1 GB of intermediates
+// holds) goes through every step as one product over the stacked points, (alpha, P) as rows of U and
+// (alpha, r) as columns of Y, M1, M3 and N: 20 launches for all points instead of 20 for each. At
+// (o, v, R_thc, R_cp) = (20, 100, 480, 720) with 12 points a product per point fills a fraction of
+// the SMs (12 us for 14 to 70 MFLOP).
+// The products run on the FP64 pipes or, from a size on (oz_worth, of a whole group) or on request,
+// as the FP64-accurate products of the BF16 tensor cores; the reductions are fixed-order.
 #include <math.h>
 #include <stdio.h>
 
@@ -40,33 +45,50 @@ __device__ double xr_block_sum(double v, double* sh) {
     return v;
 }
 
-// out[r * n + c] = s[r] * X[r * n + c]   (rows scaled by the quadrature factors)
-__global__ void k_scale_rows(int rows, int n, const double* __restrict__ s, const double* __restrict__ X,
+// out[r][al n + c] = s[al rows + r] X[r][c] for al < g: the rows scaled by the factors of g points,
+// the points' results side by side
+__global__ void k_scale_rows(int rows, int n, int g, const double* __restrict__ s, const double* __restrict__ X,
                              double* __restrict__ out) {
-    const long total = (long)rows * n;
-    for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total; e += (long)gridDim.x * blockDim.x)
-        out[e] = s[e / n] * X[e];
+    const long total = (long)rows * g * n;
+    for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total; e += (long)gridDim.x * blockDim.x) {
+        const int c = (int)(e % n);
+        const long t = e / n;
+        const int al = (int)(t % g), r = (int)(t / g);
+        out[e] = s[(size_t)al * rows + r] * X[(size_t)r * n + c];
+    }
 }
 
-// partial sums of lam_r U1 U4 Y over the Rt x R grid (one per block, fixed order)
+// partial sums of lam_r U1 U4 Y over the Rt x R grid of point blockIdx.y (U: its Rt x R block, Y: its
+// R columns of g R; one per block, fixed order)
 __global__ void __launch_bounds__(XR_THREADS)
-k_single_partials(long n, int R, const double* __restrict__ U1, const double* __restrict__ U4,
+k_single_partials(int Rt, int R, int g, const double* __restrict__ U1, const double* __restrict__ U4,
                   const double* __restrict__ Y, const double* __restrict__ lam, double* __restrict__ part) {
     __shared__ double sh[32];
+    const long n = (long)Rt * R;
+    const size_t off = (size_t)blockIdx.y * n, gR = (size_t)g * R;
+    U1 += off;
+    U4 += off;
+    Y += (size_t)blockIdx.y * R;
     double s = 0.0;
-    for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < n; e += (long)gridDim.x * blockDim.x)
-        s = fma(lam[e % R] * U1[e], U4[e] * Y[e], s);
+    for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < n; e += (long)gridDim.x * blockDim.x) {
+        const int P = (int)(e / R), r = (int)(e % R);
+        s = fma(lam[r] * U1[e], U4[e] * Y[P * gR + r], s);
+    }
     s = xr_block_sum(s, sh);
-    if (threadIdx.x == 0) part[blockIdx.x] = s;
+    if (threadIdx.x == 0) part[(size_t)blockIdx.y * XR_BLOCKS + blockIdx.x] = s;
 }
 
-// partial sums of lam_r lam_s M1[r,s] N[r,s] M3[r,s] N[s,r] over 32 x 32 tiles (N^T through
-// shared memory so that both reads are coalesced)
+// partial sums of lam_r lam_s M1[r,s] N[r,s] M3[r,s] N[s,r] of point blockIdx.y (its R columns of
+// g R) over 32 x 32 tiles (N^T through shared memory so that both reads are coalesced)
 __global__ void __launch_bounds__(XR_THREADS)
-k_double_partials(int R, const double* __restrict__ M1, const double* __restrict__ N,
+k_double_partials(int R, int g, const double* __restrict__ M1, const double* __restrict__ N,
                   const double* __restrict__ M3, const double* __restrict__ lam, double* __restrict__ part) {
     __shared__ double nt[32][33];
     __shared__ double sh[32];
+    const size_t ld = (size_t)g * R, off = (size_t)blockIdx.y * R;
+    M1 += off;
+    M3 += off;
+    N += off;
     const int tiles = (R + 31) / 32;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8
     double s = 0.0;
@@ -75,29 +97,30 @@ k_double_partials(int R, const double* __restrict__ M1, const double* __restrict
         __syncthreads();
         for (int k = ty; k < 32; k += 8) {  // nt[k][tx] = N[c0 + k][r0 + tx]
             const int rr = c0 + k, cc = r0 + tx;
-            nt[k][tx] = (rr < R && cc < R) ? N[(size_t)rr * R + cc] : 0.0;
+            nt[k][tx] = (rr < R && cc < R) ? N[rr * ld + cc] : 0.0;
         }
         __syncthreads();
         for (int k = ty; k < 32; k += 8) {
             const int r = r0 + k, c = c0 + tx;
             if (r < R && c < R) {
-                const size_t e = (size_t)r * R + c;
+                const size_t e = r * ld + c;
                 s = fma(lam[r] * lam[c], M1[e] * N[e] * M3[e] * nt[tx][k], s);
             }
         }
     }
     s = xr_block_sum(s, sh);
-    if (threadIdx.x == 0) part[blockIdx.x] = s;
+    if (threadIdx.x == 0) part[(size_t)blockIdx.y * XR_BLOCKS + blockIdx.x] = s;
 }
 
-// out[slot] = -sum of the partials (one block, fixed order)
+// out[2 al + slot] = -sum of point al's partials (block al, fixed order)
 __global__ void __launch_bounds__(XR_THREADS)
 k_neg_final(const double* __restrict__ part, int nb, double* __restrict__ out) {
     __shared__ double sh[32];
+    part += (size_t)blockIdx.x * nb;
     double s = 0.0;
     for (int i = threadIdx.x; i < nb; i += blockDim.x) s += part[i];
     s = xr_block_sum(s, sh);
-    if (threadIdx.x == 0) *out = -s;
+    if (threadIdx.x == 0) out[2 * blockIdx.x] = -s;
 }
 
 thc_cpd_status xerr(thc_cpd_status s, const char* m) { return (thc_cpd_status)set_error(s, m); }
@@ -115,140 +138,129 @@ extern "C" thc_cpd_status thc_cpd_exchange(int o, int v, int Rt, int R, int nalp
     if (chk != THC_CPD_OK) return (thc_cpd_status)chk;
     if (nalpha < 1 || nalpha > 1024) return xerr(THC_CPD_ERR_SHAPE, "need 1 <= nalpha <= 1024");
     if (!lam || !Lam || !Gam) return xerr(THC_CPD_ERR_ARG, "lam, Lam and Gam must be non-null");
-    // the products that are faster from digits (all of them on request) run on the tensor cores; the
-    // digits of the factors' columns are cut once for all points, those of Lam o X and Gam o X once per point
-    const bool ozd = oz_available() && Rt <= 8192 && R <= 8192 && std::max(o, v) <= 8192;
-    const bool all = ozd && opts && opts->ldl == THC_CPD_LDL_EMULATED;
-    auto on_tc = [&](int M, int N, int K, bool symm) { return all || (ozd && oz_worth(M, N, K, symm)); };
-    const bool tc_z = on_tc(Rt, R, Rt, false), tc_u[2] = {on_tc(Rt, R, o, false), on_tc(Rt, R, v, false)};
-    const bool tc_m = on_tc(R, R, o, true), tc_n = on_tc(R, R, v, false);
-    const bool emu = tc_z || tc_u[0] || tc_u[1] || tc_m || tc_n;
     cudaStream_t st = opts ? (cudaStream_t)opts->stream : (cudaStream_t)0;
     const size_t RtR = (size_t)Rt * R, RR = (size_t)R * R;
     const int nmax = std::max(o, v);
+    // points per group: at most 1 GB of intermediates, and 32-bit extents of the stacked products
+    const size_t per = 8 * (5 * RtR + 3 * RR + (size_t)(o + v) * (Rt + R) + (size_t)o * R) + 16 * ((size_t)cdiv(Rt, 128) * 128 * R);
+    int g = (int)std::min<size_t>(nalpha, std::max<size_t>(1, (size_t(1) << 30) / per));
+    while (g > 1 && ((long)g * std::max(Rt, R) * std::max(std::max(Rt, R), nmax) >= 0x7fffffffL)) --g;
+    // products from digits: all on request, else those of a group that are faster there
+    const bool ozd = oz_available() && Rt <= 8192 && R <= 8192 && nmax <= 8192;
+    const bool all = ozd && opts && opts->ldl == THC_CPD_LDL_EMULATED;
+    auto on_tc = [&](int M, int N, int K) { return all || (ozd && oz_worth_flops(2.0 * g * M * (double)N * K)); };
+    const bool tc_z = on_tc(Rt, R, Rt), tc_u[2] = {on_tc(Rt, R, o), on_tc(Rt, R, v)};
+    const bool tc_m = on_tc(R, R, o), tc_n = on_tc(R, R, v);
+    const bool emu = tc_z || tc_u[0] || tc_u[1] || tc_m || tc_n;
     const size_t part_cap = std::max(dgemm_part_need(Rt, R, Rt),
-                                     std::max(dgemm_part_need(Rt, R, nmax), dgemm_part_need(R, R, nmax)));
-    size_t bytes = Arena::need<double>((size_t)o * Rt) + Arena::need<double>((size_t)v * Rt) +
-                   5 * Arena::need<double>(RtR) + 3 * Arena::need<double>((size_t)nmax * R) +
-                   3 * Arena::need<double>(RR) + Arena::need<double>(XR_BLOCKS) +
-                   Arena::need<double>(2 * (size_t)nalpha) + Arena::need<double>(part_cap);
-    int oz_ra = 1, oz_rb = 1;
-    size_t oz_part = 0;
-    if (emu) {
-        oz_product_ws(Rt, R, Rt, &oz_ra, &oz_rb, &oz_part);
-        oz_product_ws(Rt, R, nmax, &oz_ra, &oz_rb, &oz_part);
-        oz_product_ws(R, R, nmax, &oz_ra, &oz_rb, &oz_part);
-        bytes += oz_ws_bytes(oz_ra, oz_rb, oz_part) + 2 * ozmat_bytes(R, o) + 2 * ozmat_bytes(R, v) +
-                 ozmat_bytes(Rt, o) + ozmat_bytes(Rt, v) + ozmat_bytes(Rt, Rt) + ozmat_bytes(R, Rt) + ozmat_bytes(R, nmax);
-    }
+                                     std::max(dgemm_part_need(g * Rt, R, nmax), dgemm_part_need(R, g * R, nmax)));
+    size_t bytes = Arena::need<double>((size_t)o * g * Rt) + Arena::need<double>((size_t)v * g * Rt) +
+                   5 * Arena::need<double>(g * RtR) + 2 * Arena::need<double>((size_t)o * g * R) +
+                   Arena::need<double>((size_t)v * g * R) + 3 * Arena::need<double>(g * RR) +
+                   Arena::need<double>((size_t)XR_BLOCKS * g) + Arena::need<double>(2 * (size_t)nalpha) +
+                   Arena::need<double>(part_cap);
+    if (emu)
+        bytes += 2 * ozmat_bytes(R, o) + 2 * ozmat_bytes(R, v) + ozmat_bytes(g * Rt, o) + ozmat_bytes(g * Rt, v) +
+                 ozmat_bytes(Rt, Rt) + ozmat_bytes(g * R, Rt) + ozmat_bytes(g * R, nmax);
     void* block = nullptr;
     if (cudaMallocAsync(&block, bytes, st) != cudaSuccess) return xerr(THC_CPD_ERR_ALLOC, "workspace allocation failed");
     Arena ar;
     ar.base = (char*)block;
     ar.cap = bytes;
-    double* XoL = ar.take<double>((size_t)o * Rt);
-    double* XvG = ar.take<double>((size_t)v * Rt);
+    double* XoL = ar.take<double>((size_t)o * g * Rt);
+    double* XvG = ar.take<double>((size_t)v * g * Rt);
     double* U[4];
-    for (int k = 0; k < 4; ++k) U[k] = ar.take<double>(RtR);
-    double* Y = ar.take<double>(RtR);
-    double* A1L = ar.take<double>((size_t)nmax * R);
-    double* A3L = ar.take<double>((size_t)nmax * R);
-    double* A4G = ar.take<double>((size_t)nmax * R);
-    double* M1 = ar.take<double>(RR);
-    double* M3 = ar.take<double>(RR);
-    double* N = ar.take<double>(RR);
-    double* part = ar.take<double>(XR_BLOCKS);
+    for (int k = 0; k < 4; ++k) U[k] = ar.take<double>(g * RtR);
+    double* Y = ar.take<double>(g * RtR);
+    double* A1L = ar.take<double>((size_t)o * g * R);
+    double* A3L = ar.take<double>((size_t)o * g * R);
+    double* A4G = ar.take<double>((size_t)v * g * R);
+    double* M1 = ar.take<double>(g * RR);
+    double* M3 = ar.take<double>(g * RR);
+    double* N = ar.take<double>(g * RR);
+    double* part = ar.take<double>((size_t)XR_BLOCKS * g);
     double* res = ar.take<double>(2 * (size_t)nalpha);
     double* gpart = ar.take<double>(part_cap);
-    OzWs oz;
-    OzMat dA[4], dXo, dXv, dZ, dP, dS;
+    OzMat dA[4], dX[2], dZ, dP, dS;
     if (emu) {
-        oz_ws_carve(oz, ar, oz_ra, oz_rb, oz_part);
         for (int k = 0; k < 4; ++k) ozmat_carve(dA[k], ar, R, (k & 1) ? v : o);
-        ozmat_carve(dXo, ar, Rt, o);
-        ozmat_carve(dXv, ar, Rt, v);
+        ozmat_carve(dX[0], ar, g * Rt, o);
+        ozmat_carve(dX[1], ar, g * Rt, v);
         ozmat_carve(dZ, ar, Rt, Rt);
-        ozmat_carve(dP, ar, R, Rt);
-        ozmat_carve(dS, ar, R, nmax);
+        ozmat_carve(dP, ar, g * R, Rt);
+        ozmat_carve(dS, ar, g * R, nmax);
+        // the digits of what no point changes
         for (int k = 0; k < 4; ++k)
             if (tc_u[k & 1] || ((k & 1) ? (tc_n && k == 1) : tc_m)) oz_split_cols(st, A[k], nullptr, R, dA[k]);
         if (tc_z) oz_split_rows(st, Z, Rt, dZ);
     }
-    auto gemm = [&](bool ta, int M, int Nn, int K, const double* Ap, int lda, const double* Bp,
-                    const double* B2, int ldb, double* C, int ldc) {
-        dgemm(st, ta, M, Nn, K, Ap, lda, Bp, B2, ldb, C, ldc, nullptr, false, gpart, part_cap);
-    };
-    auto mul = [&](const OzMat& a, const OzMat& b, double* C, bool symm) {
-        oz_mul(st, a, b, C, R, 1.0, symm ? OZ_SYMM : 0, oz.part, oz.part_cap);
-    };
-    auto scale = [&](int rows, int n, const double* s, const double* X, double* out) {
-        const long total = (long)rows * n;
-        k_scale_rows<<<(int)std::min<long>(cdiv(total, 256), 4L * num_sms()), 256, 0, st>>>(rows, n, s, X, out);
+    auto scale = [&](int rows, int n, int gg, const double* s, const double* X, double* out) {
+        const long total = (long)rows * n * gg;
+        k_scale_rows<<<(int)std::min<long>(cdiv(total, 256), 4L * num_sms()), 256, 0, st>>>(rows, n, gg, s, X, out);
         count_launch();
     };
     {
         ProfScope prof(st, emu ? KC_OZ : KC_DGEMM,
                        (double)nalpha * (4.0 * (o + v) * RtR + 2.0 * Rt * RtR + (4.0 * o + 2.0 * v) * RR));
-        for (int al = 0; al < nalpha; ++al) {
-            const double* lA = Lam + (size_t)al * o;
-            const double* gA = Gam + (size_t)al * v;
-            // single CPD
-            if (tc_u[0]) {
-                oz_split_cols(st, Xo, nullptr, Rt, dXo, lA);
-                mul(dXo, dA[0], U[0], false);
-                mul(dXo, dA[2], U[2], false);
-            } else {
-                scale(o, Rt, lA, Xo, XoL);
-                gemm(true, Rt, R, o, XoL, Rt, A[0], nullptr, R, U[0], R);
-                gemm(true, Rt, R, o, XoL, Rt, A[2], nullptr, R, U[2], R);
+        for (int a0 = 0; a0 < nalpha; a0 += g) {
+            const int gg = std::min(g, nalpha - a0), gRt = gg * Rt, gR = gg * R;
+            const double* lA = Lam + (size_t)a0 * o;
+            const double* gA = Gam + (size_t)a0 * v;
+            // single CPD: U1, U3 from Lam o Xo, U2, U4 from Gam o Xv, Y = Z (U3 o U2)
+            for (int h = 0; h < 2; ++h) {
+                const int n = h ? v : o;
+                double* XS = h ? XvG : XoL;
+                scale(n, Rt, gg, h ? gA : lA, h ? Xv : Xo, XS);
+                OzMat d = dX[h];
+                d.rows = gRt;
+                if (tc_u[h]) oz_split_cols(st, XS, nullptr, gRt, d);
+                for (int k = h; k < 4; k += 2) {
+                    if (tc_u[h])
+                        oz_mul(st, d, dA[k], U[k], R, 1.0, 0);
+                    else
+                        dgemm(st, true, gRt, R, n, XS, gRt, A[k], nullptr, R, U[k], R, nullptr, false, gpart, part_cap);
+                }
             }
-            if (tc_u[1]) {
-                oz_split_cols(st, Xv, nullptr, Rt, dXv, gA);
-                mul(dXv, dA[1], U[1], false);
-                mul(dXv, dA[3], U[3], false);
+            if (tc_z) {
+                OzMat d = dP;
+                d.rows = gR;
+                oz_split_cols_stack(st, U[2], U[1], R, R, gg, d);
+                oz_mul(st, dZ, d, Y, gR, 1.0, 0);
             } else {
-                scale(v, Rt, gA, Xv, XvG);
-                gemm(true, Rt, R, v, XvG, Rt, A[1], nullptr, R, U[1], R);
-                gemm(true, Rt, R, v, XvG, Rt, A[3], nullptr, R, U[3], R);
+                for (int al = 0; al < gg; ++al)
+                    dgemm(st, false, Rt, R, Rt, Z, Rt, U[2] + al * RtR, U[1] + al * RtR, R, Y + (size_t)al * R, gR,
+                          nullptr, false, gpart, part_cap);
             }
-            if (tc_z) {  // Z (U3 o U2)
-                oz_split_cols(st, U[2], U[1], R, dP);
-                mul(dZ, dP, Y, false);
-            } else {
-                gemm(false, Rt, R, Rt, Z, Rt, U[2], U[1], R, Y, R);
-            }
-            k_single_partials<<<XR_BLOCKS, XR_THREADS, 0, st>>>((long)RtR, R, U[0], U[3], Y, lam, part);
-            k_neg_final<<<1, XR_THREADS, 0, st>>>(part, XR_BLOCKS, res + 2 * al);
-            // double CPD
-            if (tc_m) {  // A^T diag(Lam) A is symmetric
-                dS.K = o;
-                oz_split_cols(st, A[0], nullptr, R, dS, lA);
-                mul(dA[0], dS, M1, true);
-                oz_split_cols(st, A[2], nullptr, R, dS, lA);
-                mul(dA[2], dS, M3, true);
-            } else {
-                scale(o, R, lA, A[0], A1L);
-                scale(o, R, lA, A[2], A3L);
-                gemm(true, R, R, o, A[0], R, A1L, nullptr, R, M1, R);
-                gemm(true, R, R, o, A[2], R, A3L, nullptr, R, M3, R);
-            }
-            if (tc_n) {
-                dS.K = v;
-                oz_split_cols(st, A[3], nullptr, R, dS, gA);
-                mul(dA[1], dS, N, false);
-            } else {
-                scale(v, R, gA, A[3], A4G);
-                gemm(true, R, R, v, A[1], R, A4G, nullptr, R, N, R);
-            }
-            k_double_partials<<<XR_BLOCKS, XR_THREADS, 0, st>>>(R, M1, N, M3, lam, part);
-            k_neg_final<<<1, XR_THREADS, 0, st>>>(part, XR_BLOCKS, res + 2 * al + 1);
+            k_single_partials<<<dim3(XR_BLOCKS, gg), XR_THREADS, 0, st>>>(Rt, R, gg, U[0], U[3], Y, lam, part);
+            k_neg_final<<<gg, XR_THREADS, 0, st>>>(part, XR_BLOCKS, res + 2 * a0);
+            // double CPD: M1 = A1^T (Lam o A1), M3 = A3^T (Lam o A3), N = A2^T (Gam o A4)
+            auto pair = [&](const double* Al, const OzMat& dl, const double* As, const double* s, int n, double* AS,
+                            double* out, bool tc) {
+                scale(n, R, gg, s, As, AS);
+                if (tc) {
+                    OzMat d = dS;
+                    d.rows = gR;
+                    d.K = n;
+                    oz_split_cols(st, AS, nullptr, gR, d);
+                    oz_mul(st, dl, d, out, gR, 1.0, 0);
+                } else {
+                    dgemm(st, true, R, gR, n, Al, R, AS, nullptr, gR, out, gR, nullptr, false, gpart, part_cap);
+                }
+            };
+            pair(A[0], dA[0], A[0], lA, o, A1L, M1, tc_m);
+            pair(A[2], dA[2], A[2], lA, o, A3L, M3, tc_m);
+            pair(A[1], dA[1], A[3], gA, v, A4G, N, tc_n);
+            k_double_partials<<<dim3(XR_BLOCKS, gg), XR_THREADS, 0, st>>>(R, gg, M1, N, M3, lam, part);
+            k_neg_final<<<gg, XR_THREADS, 0, st>>>(part, XR_BLOCKS, res + 2 * a0 + 1);
             count_launch(4);
         }
     }
     std::vector<double> h(2 * (size_t)nalpha);
     cudaError_t e = cudaMemcpyAsync(h.data(), res, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, st);
-    cudaFreeAsync(block, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    // freed after the synchronisation, which gives what the pool holds unused back to the device: the
+    // next call finds the block in the pool (mapping 650 MB anew took 1.9 ms)
+    cudaFreeAsync(block, st);
     if (e != cudaSuccess) {
         char msg[256];
         snprintf(msg, sizeof msg, "exchange energy failed: %s", cudaGetErrorString(e));

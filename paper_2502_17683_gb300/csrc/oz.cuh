@@ -46,10 +46,11 @@ void ozmat_carve(OzMat& m, Arena& ar, int rows, int K);
 
 // Digits of the rows of src (rows x K, row-major, ld).
 void oz_split_rows(cudaStream_t st, const double* src, int ld, OzMat& out);
-// Digits of the columns of S (K x rows, row-major, ld), times S2 element by element and row k of S
-// times rs[k] when given.
-void oz_split_cols(cudaStream_t st, const double* S, const double* S2, int ld, OzMat& out,
-                   const double* rs = nullptr);
+// Digits of the columns of S (K x rows, row-major, ld), times S2 element by element when given.
+void oz_split_cols(cudaStream_t st, const double* S, const double* S2, int ld, OzMat& out);
+// The same of g matrices of n columns stored one below the other (K rows each): rows al n + c of out
+// (out.rows = g n) are the columns of matrix al.
+void oz_split_cols_stack(cudaStream_t st, const double* S, const double* S2, int ld, int n, int g, OzMat& out);
 
 // Device workspace of emulated products: digits of both operands and split-K partial sums.
 struct OzWs {
@@ -80,6 +81,7 @@ cudaError_t oz_mul(cudaStream_t st, const OzMat& A, const OzMat& B, double* C, i
 // Whether an M x N x K product (symm: only its lower triangle) is faster from digits than on the
 // FP64 pipes.
 bool oz_worth(int M, int N, int K, bool symm);
+bool oz_worth_flops(double flops);  // by its flops alone
 
 // The tensor-core kernels can run on the current device (sm_103, enough shared memory).
 bool oz_available();

@@ -129,11 +129,10 @@ k_oz_split_rows(const double* __restrict__ src, int ld, int rows, int K, uint16_
 constexpr int COLS_PER_BLOCK = 8;   // output rows (source columns) per block, one warp each
 constexpr int kColsMaxK = 3072;     // K of one slab of the column split (its shared memory: 193 KB)
 
-// Exponents of the columns of S (K x N, ld), times S2 and row k times rs[k] when given (only for
-// K > kColsMaxK).
+// Exponents of the columns of S (K x N, ld), times S2 when given (only for K > kColsMaxK).
 __global__ void __launch_bounds__(256)
-k_oz_col_exps(const double* __restrict__ S1, const double* __restrict__ S2, const double* __restrict__ rs,
-              int ld, int N, int K, int* __restrict__ exps) {
+k_oz_col_exps(const double* __restrict__ S1, const double* __restrict__ S2, int ld, int N, int K,
+              int* __restrict__ exps) {
     __shared__ int sh[8][32];
     const int n = blockIdx.x * 32 + (threadIdx.x & 31), w = threadIdx.x >> 5;
     int e = kZeroExp;
@@ -141,7 +140,6 @@ k_oz_col_exps(const double* __restrict__ S1, const double* __restrict__ S2, cons
         for (int k = w; k < K; k += 8) {
             double v = S1[(size_t)k * ld + n];
             if (S2) v *= S2[(size_t)k * ld + n];
-            if (rs) v *= rs[k];
             e = max(e, dbl_exp(v));
         }
     sh[w][threadIdx.x & 31] = e;
@@ -153,15 +151,19 @@ k_oz_col_exps(const double* __restrict__ S1, const double* __restrict__ S2, cons
 }
 
 // Digits of the columns of S1 (K x N row-major, ld), times S2 element by element when given (a
-// Hadamard operand) and its row k times rs[k] when given: a block brings a K x 8 slab into shared memory once (64-byte row pieces),
+// Hadamard operand): a block brings a K x 8 slab into shared memory once (64-byte row pieces),
 // finds its columns' exponents on the way and then cuts one column per warp. blockIdx.y: slab of
-// kColsMaxK rows; with several (have_exp) the exponents come from k_oz_col_exps.
+// kColsMaxK rows; with several (have_exp) the exponents come from k_oz_col_exps. blockIdx.z: matrix of a
+// stack (K ld apart), N of the `rows` output rows each.
 __global__ void __launch_bounds__(256)
-k_oz_split_cols(const double* __restrict__ S1, const double* __restrict__ S2, const double* __restrict__ rs,
-                int ld, int N, int K, uint16_t* __restrict__ out, int* __restrict__ exps, int have_exp) {
+k_oz_split_cols(const double* __restrict__ S1, const double* __restrict__ S2, int ld, int N, int K, int rows,
+                uint16_t* __restrict__ out, int* __restrict__ exps, int have_exp) {
     extern __shared__ __align__(16) double slab[];  // [8][pitch]: column n at n * pitch
     __shared__ int sh[8][COLS_PER_BLOCK];
     const int n0 = blockIdx.x * COLS_PER_BLOCK, k0 = blockIdx.y * kColsMaxK;
+    S1 += (size_t)blockIdx.z * K * ld;
+    if (S2) S2 += (size_t)blockIdx.z * K * ld;
+    exps += (size_t)blockIdx.z * N;
     const int kn = min(K - k0, kColsMaxK), kpad = (kn + KP - 1) / KP * KP;
     const int pitch = kpad + 4;  // = 4 mod 16 doubles: the 8 x 4 pieces of a warp's stores miss each other's banks
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -177,7 +179,6 @@ k_oz_split_cols(const double* __restrict__ S1, const double* __restrict__ S2, co
             if (live && k < kn) {
                 v = p1[(size_t)k * ld];
                 if (p2) v *= p2[(size_t)k * ld];
-                if (rs) v *= rs[k0 + k];
             }
             e = max(e, dbl_exp(v));
             slab[nn * pitch + k] = v;
@@ -199,8 +200,8 @@ k_oz_split_cols(const double* __restrict__ S1, const double* __restrict__ S2, co
         if (e == kZeroExp) e = 0;
         if (lane == 0) exps[n] = e;
     }
-    const size_t stride = (size_t)N * KP;
-    uint16_t* o = out + (size_t)(k0 / KP) * S * stride + (size_t)n * KP + 4 * lane;
+    const size_t stride = (size_t)rows * KP;
+    uint16_t* o = out + (size_t)(k0 / KP) * S * stride + ((size_t)blockIdx.z * N + n) * KP + 4 * lane;
     for (int k = 4 * lane; k < kpad; k += KP, o += S * stride) {
         const double2 a = *reinterpret_cast<const double2*>(&slab[w * pitch + k]);
         const double2 b = *reinterpret_cast<const double2*>(&slab[w * pitch + k + 2]);
@@ -556,6 +557,10 @@ PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
 std::once_flag g_once;
 bool g_ready = false;
 int g_num_sm = 148;
+// From 1e7 flops on, products run from digits. An MTTKRP at (o, v, R_thc, R_cp) in us with the line at
+// 4e6 / 8e6 / 1.6e7 / 3e7 / never: (6,30,144,216) 183 / 187 / 167 / 172 / 172, (8,40,192,288)
+// 172 / 188 / 185 / 188 / 190, (14,70,336,504) 207 / 203 / 202 / 252 / 337, (20,100,480,720)
+// 230 / 232 / 248 / 252 / 691, (30,150,720,1080) 328 / 334 / 328 / 330 / 1761.
 constexpr double kWorthFlops = 1.0e7;
 constexpr int kColsSmem = COLS_PER_BLOCK * (kColsMaxK + 4) * (int)sizeof(double);
 
@@ -683,18 +688,25 @@ void oz_split_rows(cudaStream_t st, const double* src, int ld, OzMat& m) {
     count_launch();
 }
 
-void oz_split_cols(cudaStream_t st, const double* S1, const double* S2, int ld, OzMat& m, const double* rs) {
-    if (m.rows <= 0) return;
+void oz_split_cols_stack(cudaStream_t st, const double* S1, const double* S2, int ld, int n, int g, OzMat& m) {
+    if (n <= 0 || g <= 0) return;
     const int parts = cdiv(m.K, kColsMaxK);
     if (parts > 1) {
-        k_oz_col_exps<<<cdiv(m.rows, 32), 256, 0, st>>>(S1, S2, rs, ld, m.rows, m.K, m.e);
-        count_launch();
+        for (int al = 0; al < g; ++al) {
+            const size_t off = (size_t)al * m.K * ld;
+            k_oz_col_exps<<<cdiv(n, 32), 256, 0, st>>>(S1 + off, S2 ? S2 + off : nullptr, ld, n, m.K, m.e + (size_t)al * n);
+        }
+        count_launch(g);
     }
     const int kpad = cdiv(std::min(m.K, kColsMaxK), KP) * KP;
-    k_oz_split_cols<<<dim3(cdiv(m.rows, COLS_PER_BLOCK), parts), 256,
-                      COLS_PER_BLOCK * (kpad + 4) * sizeof(double), st>>>(S1, S2, rs, ld, m.rows, m.K, m.d, m.e,
+    k_oz_split_cols<<<dim3(cdiv(n, COLS_PER_BLOCK), parts, g), 256,
+                      COLS_PER_BLOCK * (kpad + 4) * sizeof(double), st>>>(S1, S2, ld, n, m.K, m.rows, m.d, m.e,
                                                                            parts > 1 ? 1 : 0);
     count_launch();
+}
+
+void oz_split_cols(cudaStream_t st, const double* S1, const double* S2, int ld, OzMat& m) {
+    oz_split_cols_stack(st, S1, S2, ld, m.rows, 1, m);
 }
 
 cudaError_t oz_mul(cudaStream_t st, const OzMat& A, const OzMat& B, double* C, int ldc, double sign,
@@ -729,9 +741,10 @@ size_t oz_ws_bytes(int rowsA, int rowsB, size_t part_doubles) {
 
 bool oz_available() { return oz_init(); }
 
+bool oz_worth_flops(double flops) { return flops >= kWorthFlops; }
+
 bool oz_worth(int M, int N, int K, bool symm) {
-    const double fl = (symm ? 1.0 : 2.0) * M * (double)N * K;
-    return fl >= kWorthFlops && M <= 8192 && N <= 8192 && K <= kOzMaxChunks * KP;
+    return oz_worth_flops((symm ? 1.0 : 2.0) * M * (double)N * K) && M <= 8192 && N <= 8192 && K <= kOzMaxChunks * KP;
 }
 
 void oz_ws_carve(OzWs& w, Arena& ar, int rowsA, int rowsB, size_t part_doubles) {
