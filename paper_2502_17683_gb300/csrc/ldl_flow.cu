@@ -115,6 +115,9 @@ __device__ __forceinline__ int ld_acquire(const int* p) {
     return v;
 }
 
+// Cumulative: what other threads of the CTA wrote before a barrier that this thread has passed is
+// ordered before the store as well, so no fence goes with it (a fence beside it doubles its latency,
+// which every hop from one task to the next pays).
 __device__ __forceinline__ void st_release(int* p, int v) {
     asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
@@ -207,20 +210,27 @@ __device__ bool smem_wait(const volatile int* p, int v, int* abort_flag, unsigne
 }
 
 // LDL^T of the jb x jb tile in S.D (lower triangle) into S.L (strictly lower), S.D's
-// diagonal and S.dinv. Threads 0..127 compute with a barrier of their own per column.
+// diagonal and S.dinv. Threads 0..159 compute with a barrier of their own per column.
 // Thread 0 carries only the pivot chain, one column ahead: d(c+1) = a(c+1, c+1) -
 // a(c+1, c)^2 / d(c) and its reciprocal, with 1/d(c) in a register and a(c+1, c)^2 formed,
 // one column earlier, by the thread that finished a(c+1, c). (Each FP64 instruction of a
-// warp costs tens of clocks of issue on this part, so the chain thread issues four per
-// column and nothing else.) Warps 1-3 apply column c to the rest of the tile over the
-// packed pair list, at most two pairs per thread whose operands are all read before
-// either is written. A pivot <= tau sets S.bad and continues with 1 (the caller then
-// replays the mode with the pseudo-inverse). Ends with a barrier of the chain's threads
-// 0..255.
+// warp costs 64 clocks of issue on this part, so the chain thread issues four per
+// column and nothing else.) Warps 1-4 hold the entries (r, s), 1 <= s <= r, one per thread in a
+// register over the whole tile, the later columns' in the lower threads; a column takes a
+// multiplication and an FMA of the warps that still have entries past it (one shared-memory
+// read of the column, two FP64 instructions), and only what the next column reads goes back to
+// shared memory: its entries, L, and the pivot after next. Columns took 606 clocks with two entries
+// per thread read and written through shared memory. A pivot <= tau sets S.bad and continues with 1
+// (the caller then replays the mode with the pseudo-inverse). Ends with a barrier of the chain's
+// threads 0..255.
 __device__ void factor_tile(ChainSmem& S, int jb, double tau) {
     const int tid = threadIdx.x;
-    if (tid < 128) {
+    if (tid < 160) {
         double inv = 0.0;  // thread 0: 1/d(c) of the current column
+        // this thread's entry (r, s)
+        const int e = tid - 32;
+        int r = FB, s = -1;
+        double z = 0.0;
         if (tid == 0) {
             S.bad = 0;
             double d = S.D[0][0];
@@ -235,60 +245,40 @@ __device__ void factor_tile(ChainSmem& S, int jb, double tau) {
                 const double x = S.D[1][0];
                 S.x2[1] = x * x;
             }
+        } else if (e >= 0 && e < FB * (FB - 1) / 2) {
+            const int rs = S.pairs[e];
+            r = rs >> 8;
+            s = r < jb ? rs & 0xFF : -1;
+            if (s >= 0) z = S.D[r][s];
         }
         for (int c = 0; c < jb; ++c) {
-            asm volatile("bar.sync 1, 128;" ::: "memory");  // dinv[c] and column c are final
+            asm volatile("bar.sync 1, 160;" ::: "memory");  // dinv[c] and column c are final
             if (tid == 0) {
                 if (c + 1 < jb) {
                     double d1 = fma(-S.x2[c + 1], inv, S.D[c + 1][c + 1]);
                     // the check runs beside the reciprocal, off the chain
                     const bool ok = pivot_ok(d1, tau);
-                    double r = recip_nr(d1);
+                    double rc = recip_nr(d1);
                     if (!ok) {
                         S.bad = 1;
                         d1 = 1.0;
-                        r = 1.0;
+                        rc = 1.0;
                     }
                     S.D[c + 1][c + 1] = d1;
-                    S.dinv[c + 1] = r;
-                    inv = r;
+                    S.dinv[c + 1] = rc;
+                    inv = rc;
                 }
-            } else if (tid >= 32) {
-                // pair (r, s), c < s <= r: L(r, c) = a(r, c) / d(c) when s = c + 1, and
-                // a(r, s) -= L(r, c) a(s, c) except for the pivot (c+1, c+1), thread 0's.
-                // Column c is read-only in this step and every pair writes its own entry.
-                const double inv_c = S.dinv[c];
-                const int hi = FB - 1 - c;
-                const int npair = hi * (hi + 1) / 2;
-                int r[2], ss[2];
-                double x[2], y[2], z[2];
-#pragma unroll
-                for (int k = 0; k < 2; ++k) {
-                    const int e = tid - 32 + 96 * k;
-                    r[k] = FB;
-                    ss[k] = 0;
-                    if (e < npair) {
-                        const int rs = S.pairs[e];
-                        r[k] = rs >> 8;
-                        ss[k] = rs & 0xFF;
-                    }
-                    x[k] = y[k] = z[k] = 0.0;
-                    if (r[k] < jb) {
-                        x[k] = S.D[r[k]][c];
-                        y[k] = S.D[ss[k]][c];
-                        if (r[k] != c + 1) z[k] = S.D[r[k]][ss[k]];
-                    }
-                }
-                const double l0 = x[0] * inv_c, l1 = x[1] * inv_c;
-#pragma unroll
-                for (int k = 0; k < 2; ++k) {
-                    if (r[k] >= jb) continue;
-                    const double l = k ? l1 : l0;
-                    if (ss[k] == c + 1) S.L[r[k]][c] = l;
-                    if (r[k] == c + 1) continue;
-                    const double a = fma(-l, y[k], z[k]);
-                    S.D[r[k]][ss[k]] = a;
-                    if (r[k] == c + 2 && ss[k] == c + 1) S.x2[r[k]] = a * a;
+            } else if (s > c) {
+                // L(r, c) = a(r, c) / d(c); a(r, s) -= L(r, c) a(s, c). Column c is read-only in this
+                // step; the pivot (c+1, c+1) is thread 0's.
+                const double l = S.D[r][c] * S.dinv[c];
+                z = fma(-l, S.D[s][c], z);
+                if (s == c + 1) {
+                    S.L[r][c] = l;
+                    if (r != s) S.D[r][s] = z;
+                    if (r == c + 2) S.x2[r] = z * z;
+                } else if (s == c + 2 && r == s) {
+                    S.D[r][r] = z;
                 }
             }
         }
@@ -445,13 +435,11 @@ __device__ void flow_publisher(const FlowArgs& a, ChainSmem& S) {
         if (s > 0) {
             asm volatile("bar.sync 7, 288;" ::: "memory");
             if (lane == 0 && S.live) {
-                __threadfence();
                 st_release(&sdone[s], s);
             }
         }
         asm volatile("bar.sync 8, 288;" ::: "memory");
         if (lane == 0 && S.live) {
-            __threadfence();
             st_release(fdone, s + 1);
         }
         if (lane == 0) S.pub = s + 1;  // both barriers of step s passed
@@ -515,7 +503,6 @@ __device__ void task_S(const FlowArgs& a, WorkerSmem& W, int gt, int bar, int t,
     }
     group_sync(bar);
     if (gt == 0) {
-        __threadfence();
         st_release(&sdone[t], k + 1);
     }
 }
@@ -562,14 +549,15 @@ __device__ void task_U(const FlowArgs& a, WorkerSmem& W, int gt, int bar, int t,
     if (v1) a.H[(size_t)row1 * ld + col] = h1 - (u0 + u1);
     group_sync(bar);
     if (gt == 0) {
-        __threadfence();
         st_release(&cnt[t * a.nT + j], k + 1);
     }
 }
 
-// Worker group loop over tickets [0, count) of `list`, handed out by `counter` in order.
+// Worker group loop over tickets [0, count) of `list`, handed out by `counter` in order. reserve:
+// claim the next ticket while one runs. The critical groups do not: a ticket in reserve waits for
+// its group's current task, whose inputs may come a chain step later.
 __device__ void flow_worker(const FlowArgs& a, WorkerSmem& W, int g, const FlowTask* list,
-                            int count, int* counter) {
+                            int count, int* counter, bool reserve) {
     const int gt = threadIdx.x & 127, bar = 1 + g;
     if (gt == 0) W.ticket = atomicAdd(counter, 1);
     group_sync(bar);
@@ -579,13 +567,13 @@ __device__ void flow_worker(const FlowArgs& a, WorkerSmem& W, int g, const FlowT
         // claim the next ticket while this one runs (holding one in reserve keeps the
         // lowest unfinished ticket runnable: a group works on its lower ticket first)
         int nxt = 0;
-        if (gt == 0) nxt = atomicAdd(counter, 1);
+        if (gt == 0 && reserve) nxt = atomicAdd(counter, 1);
         const FlowTask tk = list[ti];
         if (tk.type == 0)
             task_S(a, W, gt, bar, tk.t, tk.k);
         else
             task_U(a, W, gt, bar, tk.t, tk.j, tk.k);
-        if (gt == 0) W.ticket = nxt;
+        if (gt == 0) W.ticket = reserve ? nxt : atomicAdd(counter, 1);
         group_sync(bar);
     }
 }
@@ -620,9 +608,9 @@ __global__ void __launch_bounds__(kFlowThreads, 1) k_ldl_flow(FlowArgs a) {
         if (role <= a.ncrit) {
             // a critical CTA: one group, alone on its SM
             if (g == 0)
-                flow_worker(a, ws[0], 0, a.tasks + a.nmain, a.ntasks - a.nmain, a.sync + 4);
+                flow_worker(a, ws[0], 0, a.tasks + a.nmain, a.ntasks - a.nmain, a.sync + 4, false);
         } else {
-            flow_worker(a, ws[g], g, a.tasks, a.nmain, a.sync);
+            flow_worker(a, ws[g], g, a.tasks, a.nmain, a.sync, true);
         }
     }
     // the last CTA out clears this launch's counters for the next one (no memset node)
@@ -755,7 +743,6 @@ __global__ void __launch_bounds__(kBsThreads) k_bsolve_slices(BsArgs a) {
             __syncthreads();
             if (mine) {
                 if (lane == 0) {
-                    __threadfence();
                     st_release(&prog[r], a.nJ - J);
                 }
             } else if (qv && q < c0) {
@@ -916,8 +903,9 @@ const Plan* get_plan(int R, int n) {
     // workers shrink), fewer only when there are fewer main tasks than CTAs: a CTA's four
     // groups share its SM's FP64 pipe, so few tasks are spread one per SM
     p.grid = (int)std::min<long>(nsm, 1 + std::max<long>(1, p.nmain));
-    // four critical CTAs (seven critical tasks per chain step) on a grid of some size, else one
-    p.ncrit = p.ntasks > p.nmain ? (p.grid >= 8 ? 4 : 1) : 0;
+    // critical CTAs: seven critical tasks per chain step, those of the next step claimed while they
+    // wait; fewer on small grids
+    p.ncrit = p.ntasks > p.nmain ? (p.grid >= 64 ? 12 : p.grid >= 24 ? 8 : p.grid >= 8 ? 4 : 1) : 0;
     p.grid = std::min(nsm, p.grid + p.ncrit);
     if (p.grid < 1 + p.ncrit + (p.nmain > 0 ? 1 : 0)) return nullptr;
     if (cudaFuncSetAttribute(k_ldl_flow, cudaFuncAttributeMaxDynamicSharedMemorySize, kFlowSmem) !=
