@@ -68,16 +68,20 @@ constexpr int kMaxTiles = 256;             // largest schedule the host builds
 constexpr int kFlowMaxTiles = 128;
 
 struct FlowTask {
-    short type, t, j, k;                   // type 0: S(t, k); 1: U(t, j, k)
+    short type, t, j, k;                   // type 0: S(t, k); 1: U(t, j, k); 2: S(t, k), then U(t, k + 1, k)
 };
 
-// The tasks on the two panels just behind chain step s in row tile s: S(s, s-2),
-// U(s, s-1, s-2), U(s, s, s-2), which feed step s directly, and S(s, s-3), U(s, j, s-3)
-// (j = s-2, s-1, s), which feed those. They are served by worker groups of their own that
-// run alone on their SMs, so that the FP64 pipes they issue to are not shared with three
-// other groups (which makes a task several times slower and, here, holds up the chain).
-__host__ __device__ __forceinline__ bool critical_task(const FlowTask& x, int nT) {
-    return x.t < nT && x.k >= x.t - 3;
+// The tasks on the three panels just behind chain step s in row tile s: S(s, s-2),
+// U(s, s-1, s-2), U(s, s, s-2), which feed step s directly, S(s, s-3), U(s, j, s-3)
+// (j = s-2, s-1, s), which feed those, and panel s-4's, which feed these. They are served by
+// worker groups of their own that run alone on their SMs, so that the FP64 pipes they issue
+// to are not shared with three other groups (which makes a task several times slower and,
+// here, holds up the chain: a step whose panel s-4 came late took 18 us to the chain's inputs,
+// one whose panel did not 9 us). Two panels and three, with S and its first U in one task:
+// 720 x 20 solves 597 -> 585 us, 1080 x 150 1137 -> 1112, 1800 x 50 1799 -> 1770; four and
+// five panels measured the same as three.
+bool critical_task(const FlowTask& x, int nT) {
+    return x.t < nT && x.k >= x.t - 4;
 }
 
 struct ChainSmem {
@@ -209,6 +213,22 @@ __device__ bool smem_wait(const volatile int* p, int v, int* abort_flag, unsigne
     return true;
 }
 
+// Barriers of factor_tile: warp 0 is the pivot side, warps 1-4 the entries' side; column c uses the
+// ones of its parity. Arriving without waiting is safe with two of a kind: the pivot side reaches its
+// arrival for column c + 2 after it has waited for the entries of column c, which those arrive
+// with after their wait for pivot c; and the entries reach their arrival for column c + 2 after pivot
+// c + 2, which the pivot side arrives with after its wait for column c's entries.
+__device__ __forceinline__ void f_arrive_pivot(int c) {
+    __syncwarp();
+    asm volatile("bar.arrive %0, 160;" ::"r"(c & 1 ? 14 : 11) : "memory");
+}
+__device__ __forceinline__ void f_wait_pivot(int c) { asm volatile("bar.sync %0, 160;" ::"r"(c & 1 ? 14 : 11) : "memory"); }
+__device__ __forceinline__ void f_arrive_column(int c) { asm volatile("bar.arrive %0, 160;" ::"r"(c & 1 ? 15 : 12) : "memory"); }
+__device__ __forceinline__ void f_wait_column(int c) {
+    asm volatile("bar.sync %0, 160;" ::"r"(c & 1 ? 15 : 12) : "memory");
+}
+__device__ __forceinline__ void f_sync_entries() { asm volatile("bar.sync 13, 128;" ::: "memory"); }
+
 // LDL^T of the jb x jb tile in S.D (lower triangle) into S.L (strictly lower), S.D's
 // diagonal and S.dinv. Threads 0..159 compute with a barrier of their own per column.
 // Thread 0 carries only the pivot chain, one column ahead: d(c+1) = a(c+1, c+1) -
@@ -219,8 +239,11 @@ __device__ bool smem_wait(const volatile int* p, int v, int* abort_flag, unsigne
 // register over the whole tile, the later columns' in the lower threads; a column takes a
 // multiplication and an FMA of the warps that still have entries past it (one shared-memory
 // read of the column, two FP64 instructions), and only what the next column reads goes back to
-// shared memory: its entries, L, and the pivot after next. Columns took 606 clocks with two entries
-// per thread read and written through shared memory. A pivot <= tau sets S.bad and continues with 1
+// shared memory: its entries, L, and the pivot after next. The two sides hand over through
+// barriers of their own, arriving
+// without waiting, so that neither stands still while the other works: the entries of column c and
+// pivot c + 1 are formed side by side. Columns took 606 clocks with two entries per thread read and
+// written through shared memory and one barrier for all. A pivot <= tau sets S.bad and continues with 1
 // (the caller then replays the mode with the pseudo-inverse). Ends with a barrier of the chain's
 // threads 0..255.
 __device__ void factor_tile(ChainSmem& S, int jb, double tau) {
@@ -251,34 +274,44 @@ __device__ void factor_tile(ChainSmem& S, int jb, double tau) {
             s = r < jb ? rs & 0xFF : -1;
             if (s >= 0) z = S.D[r][s];
         }
-        for (int c = 0; c < jb; ++c) {
-            asm volatile("bar.sync 1, 160;" ::: "memory");  // dinv[c] and column c are final
-            if (tid == 0) {
-                if (c + 1 < jb) {
+        if (tid < 32) {
+            // the pivot chain
+            f_arrive_pivot(0);
+            for (int c = 0; c + 1 < jb; ++c) {
+                if (c) f_wait_column(c - 1);  // x2[c + 1] and the pivot's entry, column c - 1 applied
+                if (tid == 0) {
                     double d1 = fma(-S.x2[c + 1], inv, S.D[c + 1][c + 1]);
                     // the check runs beside the reciprocal, off the chain
                     const bool ok = pivot_ok(d1, tau);
-                    double rc = recip_nr(d1);
-                    if (!ok) {
-                        S.bad = 1;
-                        d1 = 1.0;
-                        rc = 1.0;
-                    }
-                    S.D[c + 1][c + 1] = d1;
-                    S.dinv[c + 1] = rc;
-                    inv = rc;
+                    const double rc = recip_nr(d1);
+                    inv = ok ? rc : 1.0;
+                    S.dinv[c + 1] = inv;
+                    S.D[c + 1][c + 1] = ok ? d1 : 1.0;
+                    if (!ok) S.bad = 1;
                 }
-            } else if (s > c) {
-                // L(r, c) = a(r, c) / d(c); a(r, s) -= L(r, c) a(s, c). Column c is read-only in this
-                // step; the pivot (c+1, c+1) is thread 0's.
-                const double l = S.D[r][c] * S.dinv[c];
-                z = fma(-l, S.D[s][c], z);
-                if (s == c + 1) {
-                    S.L[r][c] = l;
-                    if (r != s) S.D[r][s] = z;
-                    if (r == c + 2) S.x2[r] = z * z;
-                } else if (s == c + 2 && r == s) {
-                    S.D[r][r] = z;
+                f_arrive_pivot(c + 1);
+            }
+            if (jb > 1) f_wait_column(jb - 2);  // (the last arrival of the entries)
+        } else {
+            for (int c = 0; c < jb; ++c) {
+                const bool on = s > c;
+                const double x = on ? S.D[r][c] : 0.0, y = on ? S.D[s][c] : 0.0;
+                f_wait_pivot(c);  // dinv[c]
+                if (on) {
+                    // L(r, c) = a(r, c) / d(c); a(r, s) -= L(r, c) a(s, c). The pivot (c+1, c+1) is thread 0's.
+                    const double l = x * S.dinv[c];
+                    z = fma(-l, y, z);
+                    if (s == c + 1) {
+                        S.L[r][c] = l;
+                        if (r != s) S.D[r][s] = z;
+                        if (r == c + 2) S.x2[r] = z * z;
+                    } else if (s == c + 2 && r == s) {
+                        S.D[r][r] = z;
+                    }
+                }
+                if (c + 1 < jb) {
+                    f_arrive_column(c);
+                    f_sync_entries();  // column c + 1 is complete for the next step's reads
                 }
             }
         }
@@ -457,8 +490,42 @@ __device__ __forceinline__ void tile_rows(const FlowArgs& a, int t, int& r0, int
     }
 }
 
-// S(t, k) by one worker group: thread gt owns column c of rows rr and rr + 8.
-__device__ void task_S(const FlowArgs& a, WorkerSmem& W, int gt, int bar, int t, int k) {
+// Tile (t, j) -= A X(j, k)^T for A (L(t, k)) in W.A, by one worker group; ready when the caller's
+// barrier has covered W.A. Waits for X(j, k) and the tile's previous panel, publishes cnt[t][j].
+__device__ void update_tile(const FlowArgs& a, WorkerSmem& W, int gt, int bar, int t, int j, int k, int r0, int rlim) {
+    const int R = a.R;
+    const size_t ld = a.ld;
+    const int k0 = k * FB, kb = min(FB, R - k0), c0 = j * FB;
+    const int c = gt & 15, rr = gt >> 4;
+    const int row0 = r0 + rr, row1 = r0 + rr + 8, col = c0 + c;
+    const bool cv = c < kb;
+    W.B[rr][c] = (cv && c0 + rr < R) ? __ldcg(a.P + (size_t)(c0 + rr) * ld + k0 + c) : 0.0;
+    W.B[rr + 8][c] = (cv && c0 + rr + 8 < R) ? __ldcg(a.P + (size_t)(c0 + rr + 8) * ld + k0 + c) : 0.0;
+    const bool diag = t == j;
+    const bool v0 = row0 < rlim && col < R && !(diag && c > rr);
+    const bool v1 = row1 < rlim && col < R && !(diag && c > rr + 8);
+    const double h0 = v0 ? __ldcg(a.H + (size_t)row0 * ld + col) : 0.0;
+    const double h1 = v1 ? __ldcg(a.H + (size_t)row1 * ld + col) : 0.0;
+    group_sync(bar);
+    double s0 = 0.0, s1 = 0.0, u0 = 0.0, u1 = 0.0;
+#pragma unroll
+    for (int q = 0; q < FB; q += 2) {
+        const double b0 = W.B[c][q], b1 = W.B[c][q + 1];
+        s0 = fma(W.A[rr][q], b0, s0);
+        s1 = fma(W.A[rr][q + 1], b1, s1);
+        u0 = fma(W.A[rr + 8][q], b0, u0);
+        u1 = fma(W.A[rr + 8][q + 1], b1, u1);
+    }
+    if (v0) a.H[(size_t)row0 * ld + col] = h0 - (s0 + s1);
+    if (v1) a.H[(size_t)row1 * ld + col] = h1 - (u0 + u1);
+    group_sync(bar);
+    if (gt == 0) st_release(&cnt_of(a)[t * a.nT + j], k + 1);
+}
+
+// S(t, k) by one worker group: thread gt owns column c of rows rr and rr + 8. then_U: U(t, k + 1, k)
+// follows at once from the registers' L(t, k) (the next link of the row's chain of tasks, without
+// the hop through its flag and a second read).
+__device__ void task_S(const FlowArgs& a, WorkerSmem& W, int gt, int bar, int t, int k, bool then_U) {
     const int R = a.R;
     const size_t ld = a.ld;
     int* sdone = sdone_of(a);
@@ -501,20 +568,31 @@ __device__ void task_S(const FlowArgs& a, WorkerSmem& W, int gt, int bar, int t,
         a.H[(size_t)row1 * ld + k0 + c] = b1 * di;
         if (hrow) a.P[(size_t)row1 * ld + k0 + c] = b1;
     }
+    if (then_U) {
+        W.A[rr][c] = (cv && row0 < rlim) ? b0 * di : 0.0;
+        W.A[rr + 8][c] = (cv && row1 < rlim) ? b1 * di : 0.0;
+    }
     group_sync(bar);
     if (gt == 0) {
         st_release(&sdone[t], k + 1);
     }
+    if (!then_U) return;
+    const int j = k + 1;
+    if (gt == 0) {
+        const int* const pc[2] = {&sdone[j], &cnt_of(a)[t * a.nT + j]};
+        const int vc[2] = {k + 1, k};
+        W.ok = flow_wait(pc, vc, a.sync + 3, a.wait_ns);
+    }
+    group_sync(bar);
+    if (!W.ok) return;
+    update_tile(a, W, gt, bar, t, j, k, r0, rlim);
 }
 
 // U(t, j, k) by one worker group: tile (t, j) -= L(t, k) X(j, k)^T.
 __device__ void task_U(const FlowArgs& a, WorkerSmem& W, int gt, int bar, int t, int j, int k) {
-    const int R = a.R;
-    const size_t ld = a.ld;
     int* sdone = sdone_of(a);
-    int* cnt = cnt_of(a);
     if (gt == 0) {
-        const int* const pc[3] = {&sdone[t], &sdone[j], &cnt[t * a.nT + j]};
+        const int* const pc[3] = {&sdone[t], &sdone[j], &cnt_of(a)[t * a.nT + j]};
         const int vc[3] = {k + 1, k + 1, k};
         W.ok = flow_wait(pc, vc, a.sync + 3, a.wait_ns);
     }
@@ -522,35 +600,11 @@ __device__ void task_U(const FlowArgs& a, WorkerSmem& W, int gt, int bar, int t,
     if (!W.ok) return;
     int r0, rlim;
     tile_rows(a, t, r0, rlim);
-    const int k0 = k * FB, kb = min(FB, R - k0), c0 = j * FB;
-    const int c = gt & 15, rr = gt >> 4;
-    const int row0 = r0 + rr, row1 = r0 + rr + 8, col = c0 + c;
-    const bool cv = c < kb;
-    W.A[rr][c] = (cv && row0 < rlim) ? __ldcg(a.H + (size_t)row0 * ld + k0 + c) : 0.0;
-    W.A[rr + 8][c] = (cv && row1 < rlim) ? __ldcg(a.H + (size_t)row1 * ld + k0 + c) : 0.0;
-    W.B[rr][c] = (cv && c0 + rr < R) ? __ldcg(a.P + (size_t)(c0 + rr) * ld + k0 + c) : 0.0;
-    W.B[rr + 8][c] = (cv && c0 + rr + 8 < R) ? __ldcg(a.P + (size_t)(c0 + rr + 8) * ld + k0 + c) : 0.0;
-    const bool diag = t == j;
-    const bool v0 = row0 < rlim && col < R && !(diag && c > rr);
-    const bool v1 = row1 < rlim && col < R && !(diag && c > rr + 8);
-    const double h0 = v0 ? __ldcg(a.H + (size_t)row0 * ld + col) : 0.0;
-    const double h1 = v1 ? __ldcg(a.H + (size_t)row1 * ld + col) : 0.0;
-    group_sync(bar);
-    double s0 = 0.0, s1 = 0.0, u0 = 0.0, u1 = 0.0;
-#pragma unroll
-    for (int q = 0; q < FB; q += 2) {
-        const double b0 = W.B[c][q], b1 = W.B[c][q + 1];
-        s0 = fma(W.A[rr][q], b0, s0);
-        s1 = fma(W.A[rr][q + 1], b1, s1);
-        u0 = fma(W.A[rr + 8][q], b0, u0);
-        u1 = fma(W.A[rr + 8][q + 1], b1, u1);
-    }
-    if (v0) a.H[(size_t)row0 * ld + col] = h0 - (s0 + s1);
-    if (v1) a.H[(size_t)row1 * ld + col] = h1 - (u0 + u1);
-    group_sync(bar);
-    if (gt == 0) {
-        st_release(&cnt[t * a.nT + j], k + 1);
-    }
+    const int k0 = k * FB, kb = min(FB, a.R - k0), c = gt & 15, rr = gt >> 4;
+    const double* L = a.H + (size_t)(r0 + rr) * a.ld + k0 + c;
+    W.A[rr][c] = (c < kb && r0 + rr < rlim) ? __ldcg(L) : 0.0;
+    W.A[rr + 8][c] = (c < kb && r0 + rr + 8 < rlim) ? __ldcg(L + 8 * (size_t)a.ld) : 0.0;
+    update_tile(a, W, gt, bar, t, j, k, r0, rlim);
 }
 
 // Worker group loop over tickets [0, count) of `list`, handed out by `counter` in order. reserve:
@@ -569,8 +623,8 @@ __device__ void flow_worker(const FlowArgs& a, WorkerSmem& W, int g, const FlowT
         int nxt = 0;
         if (gt == 0 && reserve) nxt = atomicAdd(counter, 1);
         const FlowTask tk = list[ti];
-        if (tk.type == 0)
-            task_S(a, W, gt, bar, tk.t, tk.k);
+        if (tk.type != 1)
+            task_S(a, W, gt, bar, tk.t, tk.k, tk.type == 2);
         else
             task_U(a, W, gt, bar, tk.t, tk.j, tk.k);
         if (gt == 0) W.ticket = reserve ? nxt : atomicAdd(counter, 1);
@@ -861,6 +915,31 @@ bool build_tasks(int R, int n, std::vector<FlowTask>& out, int& nT, int& nM) {
     return true;
 }
 
+// The device's lists from one in list order: the main tasks, then the critical ones, each in list
+// order, with every critical U(t, k + 1, k) folded into its S(t, k) (all it waits for sorts before
+// that S: keys up to 2k against 2k + 1). Returns the number of main tasks.
+int device_lists(std::vector<FlowTask>& h, int nT) {
+    std::stable_partition(h.begin(), h.end(), [&](const FlowTask& x) { return !critical_task(x, nT); });
+    int nmain = 0;
+    while (nmain < (int)h.size() && !critical_task(h[nmain], nT)) ++nmain;
+    std::vector<char> has_S((size_t)nT * nT, 0), has_U((size_t)nT * nT, 0);
+    for (size_t i = nmain; i < h.size(); ++i) {
+        const FlowTask& x = h[i];
+        if (x.type == 0) has_S[(size_t)x.t * nT + x.k] = 1;
+        if (x.type == 1 && x.j == x.k + 1) has_U[(size_t)x.t * nT + x.k] = 1;
+    }
+    size_t w = nmain;
+    for (size_t i = nmain; i < h.size(); ++i) {
+        FlowTask x = h[i];
+        const size_t at = (size_t)x.t * nT + x.k;
+        if (x.type == 1 && x.j == x.k + 1 && has_S[at]) continue;
+        if (x.type == 0 && has_U[at]) x.type = 2;
+        h[w++] = x;
+    }
+    h.resize(w);
+    return nmain;
+}
+
 struct Plan {
     FlowTask* tasks = nullptr;  // main tasks, then the critical ones, each in list order
     int ntasks = 0, nmain = 0, nT = 0, nM = 0, grid = 0, ncrit = 0;
@@ -883,14 +962,11 @@ const Plan* get_plan(int R, int n) {
     if (cdiv(R, FB) > kFlowMaxTiles || cdiv(n, FB) > kMaxTiles) return nullptr;
     std::vector<FlowTask> h;
     if (!build_tasks(R, n, h, p.nT, p.nM)) return nullptr;
-    p.ntasks = (int)h.size();
     // split the list into the main and the critical subsequences; each keeps the list
     // order, so the argument for progress (every task comes after all it waits for; a
     // group works on its lower ticket first) holds for each, given one group serves it
-    std::stable_partition(h.begin(), h.end(),
-                          [&](const FlowTask& x) { return !critical_task(x, p.nT); });
-    p.nmain = 0;
-    while (p.nmain < p.ntasks && !critical_task(h[p.nmain], p.nT)) ++p.nmain;
+    p.nmain = device_lists(h, p.nT);
+    p.ntasks = (int)h.size();
     if (p.ntasks > 0) {
         if (cudaMalloc(&p.tasks, sizeof(FlowTask) * h.size()) != cudaSuccess) return nullptr;
         if (cudaMemcpy(p.tasks, h.data(), sizeof(FlowTask) * h.size(), cudaMemcpyHostToDevice) !=
@@ -951,10 +1027,8 @@ cudaError_t ldl_flow_tasks(cudaStream_t st, int R, int n, double* Haug, double* 
     for (int i = 0; i < ntasks; ++i)
         h[i] = FlowTask{host_tasks[4 * i], host_tasks[4 * i + 1], host_tasks[4 * i + 2],
                         host_tasks[4 * i + 3]};
-    std::stable_partition(h.begin(), h.end(),
-                          [&](const FlowTask& x) { return !critical_task(x, p->nT); });
-    int nmain = 0;
-    while (nmain < ntasks && !critical_task(h[nmain], p->nT)) ++nmain;
+    const int nmain = device_lists(h, p->nT);
+    ntasks = (int)h.size();
     if (ntasks > 0) {
         const cudaError_t e = cudaMemcpyAsync(dev_tasks, h.data(), sizeof(FlowTask) * h.size(),
                                               cudaMemcpyHostToDevice, st);
