@@ -50,7 +50,7 @@
 
 namespace thc {
 
-__device__ int g_flow_error = 0;
+__device__ __managed__ int g_flow_error = 0;  // in managed memory: see take_error_word
 
 namespace {
 
@@ -1091,12 +1091,7 @@ cudaError_t bsolve_slices(cudaStream_t st, int R, int n, const double* Yf, doubl
     return cudaGetLastError();
 }
 
-int flow_take_error() {
-    int h = 0, z = 0;
-    cudaMemcpyFromSymbol(&h, g_flow_error, sizeof(int));
-    if (h) cudaMemcpyToSymbol(g_flow_error, &z, sizeof(int));
-    return h;
-}
+int flow_take_error() { return take_error_word(&g_flow_error); }
 
 }  // namespace thc
 

@@ -13,7 +13,7 @@
 
 namespace thc {
 
-__device__ int g_oz_error = 0;
+__device__ __managed__ int g_oz_error = 0;  // in managed memory: see take_error_word
 
 namespace {
 
@@ -902,11 +902,6 @@ cudaError_t oz_gemm_sub(cudaStream_t st, int M, int N, int K, const double* A, i
     return product(st, M, N, K, A, lda, false, B, nullptr, ldb, true, C, ldc, -1.0, OZ_ACC, ws);
 }
 
-int oz_take_error() {
-    int h = 0, z = 0;
-    cudaMemcpyFromSymbol(&h, g_oz_error, sizeof(int));
-    if (h) cudaMemcpyToSymbol(g_oz_error, &z, sizeof(int));
-    return h;
-}
+int oz_take_error() { return take_error_word(&g_oz_error); }
 
 }  // namespace thc

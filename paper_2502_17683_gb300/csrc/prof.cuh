@@ -21,6 +21,14 @@ struct ProfScope {
     ~ProfScope();
 };
 
+// A kernel family's error word, read and cleared once the stream has drained (0: no wait gave up).
+// The words lie in managed memory and no kernel touches them unless a bounded wait gives up, so
+// their page stays with the host and a call that ends well reads plain memory; a copy from a device
+// symbol blocked the host for 10 us a word, two or three words a call.
+inline int take_error_word(int* word) {
+    return __atomic_load_n(word, __ATOMIC_RELAXED) ? __atomic_exchange_n(word, 0, __ATOMIC_RELAXED) : 0;
+}
+
 // A named range on the host timeline (NVTX v3, header-only): shown by profilers that record
 // NVTX (nsys timelines, ncu's --nvtx-include filters), a no-op when none is attached.
 struct NvtxRange {

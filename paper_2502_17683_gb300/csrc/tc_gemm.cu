@@ -14,7 +14,7 @@
 
 namespace thc {
 
-__device__ int g_tc_error = 0;
+__device__ __managed__ int g_tc_error = 0;  // in managed memory: see take_error_word
 
 namespace {
 
@@ -383,12 +383,7 @@ bool tc_available() {
     return load_encode();
 }
 
-int tc_take_error() {
-    int h = 0, z = 0;
-    cudaMemcpyFromSymbol(&h, g_tc_error, sizeof(int));
-    if (h) cudaMemcpyToSymbol(g_tc_error, &z, sizeof(int));
-    return h;
-}
+int tc_take_error() { return take_error_word(&g_tc_error); }
 
 namespace {
 
