@@ -381,7 +381,7 @@ thc_cpd_status ctx_init(Ctx& c, const Shape& s, const double* Xo, const double* 
     }
     if (mixed) {
         mixed_ws_carve(c.mx, ar, tf32, s.o, s.v, Rt, R);
-        CK(mixed_setup(c.mx, c.st, Xo, Xv, Z));
+        if (als) CK(mixed_setup(c.mx, c.st, Xo, Xv, Z));  // a single MTTKRP splits what its mode takes
     }
     if (ozp) {
         for (int h = 0; h < 2; ++h) ozmat_carve(c.dZ[h], ar, Rt, Rt);
@@ -573,10 +573,11 @@ void prepare_digits(Ctx& c) {
 // W_k and G_k for every mode from the current factors (start of a run / after rollback)
 void refresh_state(Ctx& c, const double* const A[4]) {
     prepare_digits(c);
+    const bool fp64 = c.prec == THC_CPD_FP64;
+    if (!fp64) mixed_split_factors(c.mx, c.st, A);
     for (int k = 0; k < 4; ++k) {
-        const bool fp64 = c.prec == THC_CPD_FP64;
         factor_products(c, k, A[k], true, fp64);
-        if (!fp64) mixed_project(c.mx, c.st, k, A[k], false);
+        if (!fp64) mixed_project(c.mx, c.st, k, false);
     }
 }
 
@@ -617,7 +618,12 @@ thc_cpd_status mode_update(Ctx& c, double* const A[4], double* lam, int k, bool 
     normalise_columns(c.st, n, R, A[k], lam, c.LinvD);  // panel buffer is free after the solve
     const bool fp64 = c.prec == THC_CPD_FP64;
     factor_products(c, k, A[k], true, fp64);
-    if (!fp64) CK(mixed_project(c.mx, c.st, k, A[k], true));
+    if (!fp64) {
+        const double* one[4] = {};
+        one[k] = A[k];
+        mixed_split_factors(c.mx, c.st, one);
+        CK(mixed_project(c.mx, c.st, k, true));
+    }
     CK(cudaGetLastError());
     return THC_CPD_OK;
 }
@@ -1091,8 +1097,10 @@ thc_cpd_status run_als(int o, int v, int Rt, int R, const double* Xo, const doub
                                                    cudaMemcpyDeviceToDevice, c.st));
                         }
                         CK(cudaMemcpyAsync(lam, L.lamT, sizeof(double) * R, cudaMemcpyDeviceToDevice, c.st));
-                        if (c.prec != THC_CPD_FP64)
-                            for (int k = 0; k < 4; ++k) CK(mixed_project(c.mx, c.st, k, A[k], false));
+                        if (c.prec != THC_CPD_FP64) {
+                            mixed_split_factors(c.mx, c.st, A);
+                            for (int k = 0; k < 4; ++k) CK(mixed_project(c.mx, c.st, k, false));
+                        }
                         CK(cudaMemcpyAsync(c.sc, L.sc, sizeof(DevScalars), cudaMemcpyDeviceToDevice, c.st));
                         DevScalars* hs = host_scalars();
                         CK(cudaMemcpyAsync(hs, L.sc, sizeof(DevScalars), cudaMemcpyDeviceToHost, c.st));
@@ -1387,9 +1395,10 @@ thc_cpd_status thc_cpd_mttkrp(int o, int v, int Rt, int R, const double* Xo, con
         // the Hadamard operand P of the wanted half must be written last:
         // half 0 needs P34 (from mode 3), half 1 needs P12 (from mode 1)
         static const int order[2][4] = {{0, 1, 2, 3}, {3, 0, 1, 2}};
+        CK(mixed_setup(c.mx, c.st, Xo, Xv, Z, A, mode));
         for (int i = 0; i < 4; ++i) {
             const int k = order[mode / 2][i];
-            if (k != mode) CK(mixed_project(c.mx, c.st, k, A[k], false));
+            if (k != mode) CK(mixed_project(c.mx, c.st, k, false));
         }
         CK(mixed_zgemm(c.mx, c.st, mode / 2));
         if (mode == 1 || mode == 3) CK(mixed_partner(c.mx, c.st, mode));
@@ -1426,8 +1435,10 @@ thc_cpd_status thc_cpd_split_gemm(int M, int N, int K, const double* A, const do
     sa.rows = M; sb.rows = N;
     sa.cols = sb.cols = K;
     sa.pitch = sb.pitch = pitch;
-    split_rows(st, tf32, A, K, M, K, sa);
-    split_rows(st, tf32, B, K, N, K, sb);
+    SplitJobs js;
+    split_add(js, A, K, M, K, false, sa);
+    split_add(js, B, K, N, K, false, sb);
+    split_run(st, tf32, js);
     TcEpilogue ep;
     ep.out_f64t = C;  // D'[n][m] = B[n] . A[m] stored transposed: C[m][n]
     ep.ld_f64t = N;

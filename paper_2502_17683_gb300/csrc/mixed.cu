@@ -61,21 +61,32 @@ void mixed_ws_carve(MixedWs& mx, Arena& ar, bool tf32, int o, int v, int Rt, int
 }
 
 cudaError_t mixed_setup(MixedWs& mx, cudaStream_t st, const double* Xo, const double* Xv,
-                        const double* Z) {
-    const bool t = mx.tf32;
+                        const double* Z, const double* const A[4], int mode) {
     const int Rt = mx.Rt;
-    split_rows(st, t, Z, Rt, Rt, Rt, mx.Zs);
-    split_transpose(st, t, Z, Rt, Rt, Rt, mx.ZTs);
-    split_transpose(st, t, Xo, Rt, mx.o, Rt, mx.XT[0]);
-    split_transpose(st, t, Xv, Rt, mx.v, Rt, mx.XT[1]);
-    split_rows(st, t, Xo, Rt, mx.o, Rt, mx.Xs[0]);
-    split_rows(st, t, Xv, Rt, mx.v, Rt, mx.Xs[1]);
+    const double* X[2] = {Xo, Xv};
+    SplitJobs js;
+    if (mode < 0 || mode / 2 == 0) split_add(js, Z, Rt, Rt, Rt, false, mx.Zs);
+    if (mode < 0 || mode / 2 == 1) split_add(js, Z, Rt, Rt, Rt, true, mx.ZTs);
+    for (int k = 0; k < 2; ++k) {
+        const int n = k == 0 ? mx.o : mx.v;
+        split_add(js, X[k], Rt, n, Rt, true, mx.XT[k]);
+        if (mode < 0 || mode % 2 == k) split_add(js, X[k], Rt, n, Rt, false, mx.Xs[k]);
+    }
+    for (int k = 0; k < 4 && A; ++k)
+        if (k != mode) split_add(js, A[k], mx.R, k % 2 == 0 ? mx.o : mx.v, mx.R, true, mx.At[k]);
+    split_run(st, mx.tf32, js);
     return cudaGetLastError();
 }
 
-cudaError_t mixed_project(MixedWs& mx, cudaStream_t st, int k, const double* Ak, bool in_sweep) {
+void mixed_split_factors(MixedWs& mx, cudaStream_t st, const double* const A[4]) {
+    SplitJobs js;
+    for (int k = 0; k < 4; ++k)
+        if (A[k]) split_add(js, A[k], mx.R, k % 2 == 0 ? mx.o : mx.v, mx.R, true, mx.At[k]);
+    split_run(st, mx.tf32, js);
+}
+
+cudaError_t mixed_project(MixedWs& mx, cudaStream_t st, int k, bool in_sweep) {
     const int n = (k % 2 == 0) ? mx.o : mx.v;
-    split_transpose(st, mx.tf32, Ak, mx.R, n, mx.R, mx.At[k]);
     TcEpilogue ep;
     ep.out_f32 = mx.Wt[k];
     ep.ld_f32 = mx.Rt;

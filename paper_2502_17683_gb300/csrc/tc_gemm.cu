@@ -555,48 +555,89 @@ int split_pitch(bool tf32, int cols) {
     return std::max(kb, ((cols + kb - 1) / kb) * kb);
 }
 
+// Split of two neighbours of a row (the second only if `two`), idx even: stored as pairs.
 template <bool TF32>
-__device__ __forceinline__ void store_split_d(void* hi, void* lo, size_t idx, double x) {
+__device__ __forceinline__ void store_split_pair(void* hi, void* lo, size_t idx, double x0, double x1, bool two) {
     if (TF32) {
-        const float xf = (float)x;
-        const uint32_t u = __float_as_uint(xf);
-        const float h = __uint_as_float((u + 0x1000u) & 0xFFFFE000u);
-        const float r = (float)(x - (double)h);
-        const float l = __uint_as_float((__float_as_uint(r) + 0x1000u) & 0xFFFFE000u);
-        ((float*)hi)[idx] = h;
-        ((float*)lo)[idx] = l;
+        float h[2], l[2];
+        const double x[2] = {x0, x1};
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const uint32_t u = __float_as_uint((float)x[i]);
+            h[i] = __uint_as_float((u + 0x1000u) & 0xFFFFE000u);
+            const float r = (float)(x[i] - (double)h[i]);
+            l[i] = __uint_as_float((__float_as_uint(r) + 0x1000u) & 0xFFFFE000u);
+        }
+        if (two) {
+            *(float2*)((float*)hi + idx) = make_float2(h[0], h[1]);
+            *(float2*)((float*)lo + idx) = make_float2(l[0], l[1]);
+        } else {
+            ((float*)hi)[idx] = h[0];
+            ((float*)lo)[idx] = l[0];
+        }
     } else {
-        const __nv_bfloat16 h = __double2bfloat16(x);
-        const __nv_bfloat16 l = __double2bfloat16(x - (double)__bfloat162float(h));
-        ((__nv_bfloat16*)hi)[idx] = h;
-        ((__nv_bfloat16*)lo)[idx] = l;
+        __nv_bfloat162 h, l;
+        h.x = __double2bfloat16(x0);
+        h.y = __double2bfloat16(x1);
+        l.x = __double2bfloat16(x0 - (double)__bfloat162float(h.x));
+        l.y = __double2bfloat16(x1 - (double)__bfloat162float(h.y));
+        if (two) {
+            *(__nv_bfloat162*)((__nv_bfloat16*)hi + idx) = h;
+            *(__nv_bfloat162*)((__nv_bfloat16*)lo + idx) = l;
+        } else {
+            ((__nv_bfloat16*)hi)[idx] = h.x;
+            ((__nv_bfloat16*)lo)[idx] = l.x;
+        }
     }
 }
 
+// Every operand that a step needs split, in one launch: each block takes one 2048-entry tile of
+// one job. The work is reading FP64 once (16 MB for the largest configuration's operands, 3 us of
+// traffic), so what a launch of its own for each of six or seven small matrices costs, and how many
+// loads a thread has in flight, decide: 8 loads a thread are issued before the first is used, and
+// entries are written in pairs (128 bytes a warp). The nine launches of a BF16x3 MTTKRP at (o, v, R_thc,
+// R_cp) = (50, 250, 1200, 1800) took 66 us of its 199; it takes 148 with this one. As given: 32 x 64 tiles straight through.
+// Transposed: 64 x 32 tiles through shared memory, so that reads and writes are both coalesced.
 template <bool TF32>
-__global__ void k_split_rows(const double* __restrict__ src, int ld, int rows, int cols, void* hi,
-                             void* lo, int pitch) {
-    const long n = (long)rows * cols;
-    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-        const int r = (int)(i / cols), c = (int)(i % cols);
-        store_split_d<TF32>(hi, lo, (size_t)r * pitch + c, src[(size_t)r * ld + c]);
+__global__ void __launch_bounds__(256) k_split_jobs(const __grid_constant__ SplitJobs js) {
+    __shared__ double t[64][33];
+    int i0 = 0;
+    while (i0 + 1 < js.n && (int)blockIdx.x >= js.job[i0 + 1].tile0) ++i0;
+    const SplitJob& J = js.job[i0];
+    const int tile = blockIdx.x - J.tile0, tr = tile / J.tiles_c, tc = tile % J.tiles_c;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (!J.transposed) {
+        const int r0 = tr * 32 + w, c = tc * 64 + 2 * lane;
+        double x[4][2];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const double* p = J.src + (size_t)(r0 + 8 * i) * J.ld + c;
+            x[i][0] = (r0 + 8 * i < J.rows && c < J.cols) ? p[0] : 0.0;
+            x[i][1] = (r0 + 8 * i < J.rows && c + 1 < J.cols) ? p[1] : 0.0;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (r0 + 8 * i < J.rows && c < J.cols)
+                store_split_pair<TF32>(J.hi, J.lo, (size_t)(r0 + 8 * i) * J.pitch + c, x[i][0], x[i][1],
+                                       c + 1 < J.cols);
+        return;
     }
-}
-
-// 32 x 32 tiles through shared memory so that reads and writes are both coalesced
-template <bool TF32>
-__global__ void k_split_transpose(const double* __restrict__ src, int ld, int rows, int cols,
-                                  void* hi, void* lo, int pitch) {
-    __shared__ double t[32][33];
-    const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int r = r0 + i, c = c0 + threadIdx.x;
-        t[i][threadIdx.x] = (r < rows && c < cols) ? src[(size_t)r * ld + c] : 0.0;
+    const int r0 = tr * 64, c0 = tc * 32;
+    double x[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int r = r0 + w + 8 * i;
+        x[i] = (r < J.rows && c0 + lane < J.cols) ? J.src[(size_t)r * J.ld + c0 + lane] : 0.0;
     }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) t[w + 8 * i][lane] = x[i];
     __syncthreads();
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int c = c0 + i, r = r0 + threadIdx.x;
-        if (c < cols && r < rows) store_split_d<TF32>(hi, lo, (size_t)c * pitch + r, t[threadIdx.x][i]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int c = c0 + w + 8 * i, r = r0 + 2 * lane;
+        if (c < J.cols && r < J.rows)
+            store_split_pair<TF32>(J.hi, J.lo, (size_t)c * J.pitch + r, t[2 * lane][w + 8 * i],
+                                   t[2 * lane + 1][w + 8 * i], r + 1 < J.rows);
     }
 }
 
@@ -611,25 +652,19 @@ __global__ void k_split_hadamard(const float* __restrict__ a, const float* __res
     }
 }
 
-void split_rows(cudaStream_t st, bool tf32, const double* src, int ld, int rows, int cols,
-                SplitMat& d) {
-    const long n = (long)rows * cols;
-    const int blocks = (int)std::min<long>(cdiv(n, 256), 4L * num_sms());
-    count_launch();
-    if (tf32)
-        k_split_rows<true><<<blocks, 256, 0, st>>>(src, ld, rows, cols, d.hi, d.lo, d.pitch);
-    else
-        k_split_rows<false><<<blocks, 256, 0, st>>>(src, ld, rows, cols, d.hi, d.lo, d.pitch);
+void split_add(SplitJobs& js, const double* src, int ld, int rows, int cols, bool transposed, SplitMat& d) {
+    SplitJob& J = js.job[js.n++];
+    J = SplitJob{src, d.hi, d.lo, ld, rows, cols, d.pitch, transposed, cdiv(cols, transposed ? 32 : 64), js.tiles};
+    js.tiles += J.tiles_c * cdiv(rows, transposed ? 64 : 32);
 }
 
-void split_transpose(cudaStream_t st, bool tf32, const double* src, int ld, int rows, int cols,
-                     SplitMat& d) {
-    dim3 grid(cdiv(cols, 32), cdiv(rows, 32)), block(32, 8);
+void split_run(cudaStream_t st, bool tf32, const SplitJobs& js) {
+    if (js.tiles == 0) return;
     count_launch();
     if (tf32)
-        k_split_transpose<true><<<grid, block, 0, st>>>(src, ld, rows, cols, d.hi, d.lo, d.pitch);
+        k_split_jobs<true><<<js.tiles, 256, 0, st>>>(js);
     else
-        k_split_transpose<false><<<grid, block, 0, st>>>(src, ld, rows, cols, d.hi, d.lo, d.pitch);
+        k_split_jobs<false><<<js.tiles, 256, 0, st>>>(js);
 }
 
 void split_hadamard(cudaStream_t st, bool tf32, const float* a, const float* b, int ld, int rows,

@@ -50,12 +50,20 @@ int tc_take_error();
 // Conversions into split operands (elements per 128-byte K block: 64 BF16 or 32 TF32).
 int split_kblock(bool tf32);
 int split_pitch(bool tf32, int cols);
-// dst[r][c] = split(src[r * ld + c]) for r < rows, c < cols
-void split_rows(cudaStream_t st, bool tf32, const double* src, int ld, int rows, int cols,
-                SplitMat& dst);
-// dst[c][r] = split(src[r * ld + c]) (transposed)
-void split_transpose(cudaStream_t st, bool tf32, const double* src, int ld, int rows, int cols,
-                     SplitMat& dst);
+// A list of FP64 matrices to split in one launch (tile0, tiles_c: its share of the grid).
+struct SplitJob {
+    const double* src;
+    void *hi, *lo;
+    int ld, rows, cols, pitch;
+    int transposed, tiles_c, tile0;
+};
+struct SplitJobs {
+    SplitJob job[12];  // Z both ways, X_k both ways, four factors, two to spare
+    int n = 0, tiles = 0;
+};
+// dst[r][c] = split(src[r * ld + c]) for r < rows, c < cols, or dst[c][r] if transposed
+void split_add(SplitJobs& js, const double* src, int ld, int rows, int cols, bool transposed, SplitMat& dst);
+void split_run(cudaStream_t st, bool tf32, const SplitJobs& js);
 // dst[r][c] = split(a[r][c] * b[r][c]) for FP32 operands with leading dimension ld
 void split_hadamard(cudaStream_t st, bool tf32, const float* a, const float* b, int ld, int rows,
                     int cols, SplitMat& dst);

@@ -154,3 +154,36 @@ def test_batched_fixed_point_blocks(api):
     for p, r in zip(ps, res):
         ref = O.als(p.Xo, p.Xv, p.Z, p.A, 3)
         assert abs(r["fit"] - ref["fits"][-1]) <= 1e-10
+
+
+# One launch splits several matrices, as given in 32 x 64 tiles and transposed in 64 x 32 ones:
+# one row or column, one short of a tile, a tile, one more. Bound: a split keeps 16 bits (2^-17
+# each operand, 2^-17 for the dropped lo x lo term), FP32 accumulation adds K 2^-23.
+@pytest.mark.parametrize("M,N,K", [(1, 1, 1), (31, 33, 63), (32, 64, 64), (33, 65, 65), (129, 17, 191)])
+def test_split_gemm_tiles(api, M, N, K):
+    g = torch.Generator(device="cuda").manual_seed(M * 1000 + K)
+    A = torch.randn(M, K, generator=g, device="cuda", dtype=torch.float64)
+    B = torch.randn(N, K, generator=g, device="cuda", dtype=torch.float64)
+    C = api.thc_cpd_split_gemm(A, B, precision="bf16x3")
+    lim = (2.0 ** -15 + K * 2.0 ** -23) * (A.abs() @ B.abs().T)
+    assert ((C - A @ B.T).abs() <= lim).all()
+
+
+@pytest.mark.parametrize("mode", [0, 1, 2, 3])
+@pytest.mark.parametrize("o,v,Rt,R", [(1, 2, 8, 8), (3, 33, 63, 65), (31, 64, 129, 97)])
+def test_split_mttkrp_operands(api, o, v, Rt, R, mode):
+    g = torch.Generator(device="cuda").manual_seed(o * 100 + Rt)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda", dtype=torch.float64)
+    X, Z = [rnd(o, Rt), rnd(v, Rt)], rnd(Rt, Rt)
+    A = [rnd(n, R) for n in (o, v, o, v)]
+
+    def mttkrp(X, Z, A):
+        W = [X[k % 2].T @ A[k] for k in range(4)]
+        Y = Z @ (W[2] * W[3]) if mode < 2 else Z.T @ (W[0] * W[1])
+        return X[mode % 2] @ (W[mode ^ 1] * Y)
+
+    M = api.thc_cpd_mttkrp(X[0], X[1], Z, A, mode, precision="bf16x3")
+    # three products deep, each split and accumulated as above, on absolute values
+    lim = (6 * 2.0 ** -15 + (max(o, v) * 3 + 2 * Rt) * 2.0 ** -23) * mttkrp(
+        [x.abs() for x in X], Z.abs(), [a.abs() for a in A])
+    assert ((M - mttkrp(X, Z, A)).abs() <= lim).all()
