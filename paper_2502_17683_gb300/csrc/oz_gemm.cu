@@ -83,15 +83,20 @@ __device__ __forceinline__ double scaled_sum(long long hi, long long lo, int e, 
 
 constexpr int ROWS_PER_BLOCK = 4;  // one warp per row
 
-// Digits of the rows of src (rows x K, ld): a warp finds its row's exponent, then cuts four
-// consecutive values per lane (8-byte stores, a 256-byte line per slice and chunk). The second
-// read of the row comes from L1 / L2. VEC: 16-byte loads (even ld, aligned base).
+// Digits of the rows of src (rows x K, ld): wpr warps of a block of four take a row, a chunk of
+// KP values at a time each; they find the row's exponent, then cut four consecutive values per
+// lane (8-byte stores, a 256-byte line per slice and chunk). The second read of the row comes from
+// L1 / L2. VEC: 16-byte loads (even ld, aligned base). Few rows leave an SM a handful of warps, so
+// the time is that of one warp's chain of reads and cuts: several warps to a long row shorten it
+// (713 x 713: 8.0 -> 5.5 us).
 template <bool VEC>
 __global__ void __launch_bounds__(32 * ROWS_PER_BLOCK)
 k_oz_split_rows(const double* __restrict__ src, int ld, int rows, int K, uint16_t* __restrict__ out,
-                int* __restrict__ exps) {
-    const int lane = threadIdx.x & 31, r = blockIdx.x * ROWS_PER_BLOCK + (threadIdx.x >> 5);
-    if (r >= rows) return;
+                int* __restrict__ exps, int wpr) {
+    __shared__ int sh[ROWS_PER_BLOCK];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, part = w % wpr;
+    const int r = blockIdx.x * (ROWS_PER_BLOCK / wpr) + w / wpr;
+    const bool live = r < rows;
     const double* p = src + (size_t)r * ld;
     auto load4 = [&](int k, double (&v)[4]) {
         if (VEC && k + 3 < K) {
@@ -107,19 +112,26 @@ k_oz_split_rows(const double* __restrict__ src, int ld, int rows, int K, uint16_
         }
     };
     int e = kZeroExp;
-#pragma unroll 4
-    for (int k = 4 * lane; k < K; k += KP) {
+    const int step = wpr * KP;
+#pragma unroll 2
+    for (int k = part * KP + 4 * lane; live && k < K; k += step) {
         double v[4];
         load4(k, v);
 #pragma unroll
         for (int i = 0; i < 4; ++i) e = max(e, dbl_exp(v[i]));
     }
     e = __reduce_max_sync(0xffffffffu, e);
+    if (wpr > 1) {
+        if (lane == 0) sh[w] = e;
+        __syncthreads();
+        for (int i = 0; i < wpr; ++i) e = max(e, sh[w - part + i]);
+    }
+    if (!live) return;
     if (e == kZeroExp) e = 0;
-    if (lane == 0) exps[r] = e;
+    if (lane == 0 && part == 0) exps[r] = e;
     const size_t stride = (size_t)rows * KP;
-    uint16_t* o = out + (size_t)r * KP + 4 * lane;
-    for (int k = 4 * lane; k - 4 * lane < K; k += KP, o += S * stride) {
+    uint16_t* o = out + (size_t)part * S * stride + (size_t)r * KP + 4 * lane;
+    for (int k = part * KP + 4 * lane; k - 4 * lane < K; k += step, o += wpr * S * stride) {
         double v[4];
         load4(k, v);
         store_digits4(v, e, o, stride);
@@ -152,14 +164,19 @@ k_oz_col_exps(const double* __restrict__ S1, const double* __restrict__ S2, int 
 
 // Digits of the columns of S1 (K x N row-major, ld), times S2 element by element when given (a
 // Hadamard operand): a block brings a K x 8 slab into shared memory once (64-byte row pieces),
-// finds its columns' exponents on the way and then cuts one column per warp. blockIdx.y: slab of
-// kColsMaxK rows; with several (have_exp) the exponents come from k_oz_col_exps. blockIdx.z: matrix of a
-// stack (K ld apart), N of the `rows` output rows each.
-__global__ void __launch_bounds__(256)
+// finds its columns' exponents on the way and then cuts a column's chunks on blockDim / 256 warps.
+// blockIdx.y: slab of kColsMaxK rows; with several (have_exp) the exponents come from k_oz_col_exps.
+// blockIdx.z: matrix of a stack (K ld apart), N of the `rows` output rows each.
+// With no more blocks than SMs the time is one block's chain of loads and cuts, not the traffic:
+// eight loads a thread (of each operand) are issued before the first is used, whatever K, and a
+// block has 256 threads per chunk up to 1024 (713 x 713 times a second matrix: 19.9 -> 9.3 us,
+// 713 x 1061: 16.1 -> 9.4, 480 x 720: 10.2 -> 7).
+__global__ void __launch_bounds__(1024)
 k_oz_split_cols(const double* __restrict__ S1, const double* __restrict__ S2, int ld, int N, int K, int rows,
                 uint16_t* __restrict__ out, int* __restrict__ exps, int have_exp) {
     extern __shared__ __align__(16) double slab[];  // [8][pitch]: column n at n * pitch
-    __shared__ int sh[8][COLS_PER_BLOCK];
+    __shared__ int sh[32][COLS_PER_BLOCK];
+    const int nw = blockDim.x >> 5, cparts = nw / COLS_PER_BLOCK;
     const int n0 = blockIdx.x * COLS_PER_BLOCK, k0 = blockIdx.y * kColsMaxK;
     S1 += (size_t)blockIdx.z * K * ld;
     if (S2) S2 += (size_t)blockIdx.z * K * ld;
@@ -173,38 +190,45 @@ k_oz_split_cols(const double* __restrict__ S1, const double* __restrict__ S2, in
         const double* p1 = S1 + (size_t)k0 * ld + n;
         const double* p2 = S2 ? S2 + (size_t)k0 * ld + n : nullptr;
         int e = kZeroExp;
-#pragma unroll 8
-        for (int k = tid >> 3; k < kpad; k += 32) {
-            double v = 0.0;
-            if (live && k < kn) {
-                v = p1[(size_t)k * ld];
-                if (p2) v *= p2[(size_t)k * ld];
+        const int step = blockDim.x >> 3;
+        for (int kb = tid >> 3; kb < kpad; kb += 8 * step) {
+            double v[8], v2[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int k = kb + u * step;
+                const bool in = live && k < kn;
+                v[u] = in ? p1[(size_t)k * ld] : 0.0;
+                v2[u] = in && p2 ? p2[(size_t)k * ld] : 1.0;
             }
-            e = max(e, dbl_exp(v));
-            slab[nn * pitch + k] = v;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int k = kb + u * step;
+                if (p2) v[u] *= v2[u];
+                e = max(e, dbl_exp(v[u]));
+                if (k < kpad) slab[nn * pitch + k] = v[u];
+            }
         }
         e = max(e, __shfl_xor_sync(0xffffffffu, e, 8));
         e = max(e, __shfl_xor_sync(0xffffffffu, e, 16));
         if (lane < 8) sh[w][lane] = e;
     }
     __syncthreads();
-    const int n = n0 + w;
+    const int col = w % COLS_PER_BLOCK, part = w / COLS_PER_BLOCK, n = n0 + col;
     if (n >= N) return;
     int e;
     if (have_exp) {
         e = exps[n];
     } else {
         e = kZeroExp;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) e = max(e, sh[i][w]);
+        for (int i = 0; i < nw; ++i) e = max(e, sh[i][col]);
         if (e == kZeroExp) e = 0;
-        if (lane == 0) exps[n] = e;
+        if (lane == 0 && part == 0) exps[n] = e;
     }
     const size_t stride = (size_t)rows * KP;
-    uint16_t* o = out + (size_t)(k0 / KP) * S * stride + ((size_t)blockIdx.z * N + n) * KP + 4 * lane;
-    for (int k = 4 * lane; k < kpad; k += KP, o += S * stride) {
-        const double2 a = *reinterpret_cast<const double2*>(&slab[w * pitch + k]);
-        const double2 b = *reinterpret_cast<const double2*>(&slab[w * pitch + k + 2]);
+    uint16_t* o = out + (size_t)(k0 / KP + part) * S * stride + ((size_t)blockIdx.z * N + n) * KP + 4 * lane;
+    for (int k = part * KP + 4 * lane; k < kpad; k += cparts * KP, o += cparts * S * stride) {
+        const double2 a = *reinterpret_cast<const double2*>(&slab[col * pitch + k]);
+        const double2 b = *reinterpret_cast<const double2*>(&slab[col * pitch + k + 2]);
         const double v[4] = {a.x, a.y, b.x, b.y};
         store_digits4(v, e, o, stride);
     }
@@ -680,11 +704,12 @@ void ozmat_carve(OzMat& m, Arena& ar, int rows, int K) {
 
 void oz_split_rows(cudaStream_t st, const double* src, int ld, OzMat& m) {
     if (m.rows <= 0) return;
-    const int grid = cdiv(m.rows, ROWS_PER_BLOCK);
+    // up to eight rows per SM, more warps to a row (see the kernel); beyond, the rows fill the chip
+    const int wpr = m.rows > 8 * g_num_sm ? 1 : m.K > 2 * KP ? 4 : m.K > KP ? 2 : 1, grid = cdiv(m.rows, ROWS_PER_BLOCK / wpr);
     if (ld % 2 == 0 && ((uintptr_t)src & 15) == 0)
-        k_oz_split_rows<true><<<grid, 32 * ROWS_PER_BLOCK, 0, st>>>(src, ld, m.rows, m.K, m.d, m.e);
+        k_oz_split_rows<true><<<grid, 32 * ROWS_PER_BLOCK, 0, st>>>(src, ld, m.rows, m.K, m.d, m.e, wpr);
     else
-        k_oz_split_rows<false><<<grid, 32 * ROWS_PER_BLOCK, 0, st>>>(src, ld, m.rows, m.K, m.d, m.e);
+        k_oz_split_rows<false><<<grid, 32 * ROWS_PER_BLOCK, 0, st>>>(src, ld, m.rows, m.K, m.d, m.e, wpr);
     count_launch();
 }
 
@@ -699,7 +724,12 @@ void oz_split_cols_stack(cudaStream_t st, const double* S1, const double* S2, in
         count_launch(g);
     }
     const int kpad = cdiv(std::min(m.K, kColsMaxK), KP) * KP;
-    k_oz_split_cols<<<dim3(cdiv(n, COLS_PER_BLOCK), parts, g), 256,
+    // up to two blocks per SM, more threads to a block (see the kernel); beyond, blocks of 256 hide
+    // each other's latency better (twelve 480 x 720 matrices in a stack: the exchange energies took
+    // 920 us with 1024 threads, 892 with 256)
+    const long blocks = (long)cdiv(n, COLS_PER_BLOCK) * parts * g;
+    const int threads = blocks > 2L * g_num_sm ? 256 : 256 * std::min(4, kpad / KP);
+    k_oz_split_cols<<<dim3(cdiv(n, COLS_PER_BLOCK), parts, g), threads,
                       COLS_PER_BLOCK * (kpad + 4) * sizeof(double), st>>>(S1, S2, ld, n, m.K, m.rows, m.d, m.e,
                                                                            parts > 1 ? 1 : 0);
     count_launch();

@@ -187,3 +187,30 @@ def test_split_mttkrp_operands(api, o, v, Rt, R, mode):
     lim = (6 * 2.0 ** -15 + (max(o, v) * 3 + 2 * Rt) * 2.0 ** -23) * mttkrp(
         [x.abs() for x in X], Z.abs(), [a.abs() for a in A])
     assert ((M - mttkrp(X, Z, A)).abs() <= lim).all()
+
+
+# The digit cuts take several warps to a row up to 8 rows per SM, and up to 1024 threads to 8 columns
+# up to two blocks per SM: one size on either side of both lines, for 148 to 160 SMs.
+@pytest.mark.parametrize("shape", [(1150, 33, 300), (1300, 31, 257)])
+def test_emulated_product_rows(api, shape):
+    test_emulated_product_edges(api, shape)
+
+
+# bound: FP64 sums of n, Rt and Rt terms on either side, on absolute values
+@pytest.mark.parametrize("R", [2360, 2600])
+@pytest.mark.parametrize("mode", [0, 3])
+def test_fp64_mttkrp_many_columns(api, R, mode):
+    o, v, Rt = 9, 17, 290
+    g = torch.Generator(device="cuda").manual_seed(R + mode)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda", dtype=torch.float64)
+    X, Z = [rnd(o, Rt), rnd(v, Rt)], rnd(Rt, Rt)
+    A = [rnd(n, R) for n in (o, v, o, v)]
+
+    def mttkrp(X, Z, A):
+        W = [X[k % 2].T @ A[k] for k in range(4)]
+        Y = Z @ (W[2] * W[3]) if mode < 2 else Z.T @ (W[0] * W[1])
+        return X[mode % 2] @ (W[mode ^ 1] * Y)
+
+    M = api.thc_cpd_mttkrp(X[0], X[1], Z, A, mode)
+    lim = 2 * (3 * v + 2 * Rt) * U * mttkrp([x.abs() for x in X], Z.abs(), [a.abs() for a in A])
+    assert ((M - mttkrp(X, Z, A)).abs() <= lim).all()
