@@ -252,12 +252,12 @@ void thc_cpd_profile(int enable);
 int thc_cpd_profile_read(thc_cpd_kstat* out, int max_classes);
 
 /* C (M x N) = A (M x K) B (N x K)^T to FP64 accuracy on the BF16 tensor cores (the
- * contraction behind THC_CPD_LDL_EMULATED, exposed for testing and reuse; the paper's
- * solves are FP64, Sec. 2.1 and 3). Every row of A and of B is scaled by a power of two and
- * cut into 7 signed 8-bit integer digits (an error-free splitting after Ozaki, Ogita, Oishi
+ * contraction behind the FP64 path's products and THC_CPD_LDL_EMULATED, exposed for testing
+ * and reuse; the paper is FP64, Sec. 2.1 and 3). Every row of A and of B is scaled by a power of
+ * two and cut into 8 signed 8-bit integer digits (an error-free splitting after Ozaki, Ogita, Oishi
  * and Rump, Numer. Algorithms 59, 2012); the digit products are exact on the tensor cores
  * (FP32 accumulation of integers below 2^24, K in chunks of 128) and are recombined exactly
- * in 64-bit integers, then rounded once to FP64. Error: about 2^-53 |C| + 2^-55 K
+ * in 64-bit integers over all of K, then rounded once to FP64. Error: about 2^-53 |C| + 2^-61 K
  * max_k |A_ik| max_k |B_jk|. Row-major FP64 device arrays (lda, ldb, ldc in elements).
  * Shapes: 1 <= M, N <= 4096, K >= 1. Synchronises. */
 thc_cpd_status thc_cpd_emulated_gemm(int M, int N, int K, const double* A, int lda, const double* B,
@@ -272,9 +272,9 @@ thc_cpd_status thc_cpd_emulated_gemm(int M, int N, int K, const double* A, int l
  *   e_robust = 2 e_single - e_double (Eq. rob_K; no error of first order in G - Gt),
  * G the THC block (Eq. THC) and Gt = sum_r lam_r A1 A2 A3 A4 (Eq. cp4). Device inputs as for
  * thc_cpd_loss (lam may not be NULL); the three energies are returned in host memory (each
- * pointer may be NULL). The contractions are FP64 GEMMs on the FP64 pipes, or with
- * opts->ldl = THC_CPD_LDL_EMULATED the FP64-accurate emulated products of the tensor cores;
- * the reductions run in a fixed order. 1 <= nalpha <= 1024. Synchronises. */
+ * pointer may be NULL). Contractions of 1e7 flops or more (over a group of points) run as
+ * FP64-accurate products on the tensor cores, smaller ones on the FP64 pipes; with
+ * opts->ldl = THC_CPD_LDL_EMULATED all run on the tensor cores. The reductions run in a fixed order. 1 <= nalpha <= 1024. Synchronises. */
 thc_cpd_status thc_cpd_exchange(int o, int v, int Rt, int R, int nalpha, const double* Xo,
                                 const double* Xv, const double* Z, const double* const A[4],
                                 const double* lam, const double* Lam, const double* Gam,
@@ -289,9 +289,10 @@ thc_cpd_status thc_cpd_exchange(int o, int v, int Rt, int R, int nalpha, const d
  * S, pseudo-inverse of S when a pivot fails: *used_pinv = 1). The result is symmetric.
  * Xo (o x Rt), Xv (v x Rt), B (naux x o x v, row-major), Z (Rt x Rt, written): device FP64.
  * loss: NULL, or host double receiving ||G_DF - G_THC(Z)||^2 (no 1/2) in factor form.
- * 1 <= R_thc <= 2048; o * v, naux * o, naux * R_thc and naux^2 below 2^31. The GEMMs run on the
- * FP64 pipes, or with opts->ldl = THC_CPD_LDL_EMULATED as the FP64-accurate emulated products
- * of the tensor cores (the solve then uses the emulated two-level LDL^T as well).
+ * 1 <= R_thc <= 2048; o * v, naux * o, naux * R_thc and naux^2 below 2^31. GEMMs of
+ * 1e7 flops or more run as FP64-accurate products on the tensor cores, smaller ones on the FP64
+ * pipes; with opts->ldl = THC_CPD_LDL_EMULATED all run on the tensor cores (and the solve uses
+ * the emulated two-level LDL^T).
  * Allocates its workspace (about 256 MiB plus 2 naux R_thc doubles, plus naux o v and naux^2
  * doubles with loss) with cudaMallocAsync on opts->stream. Synchronises. */
 thc_cpd_status thc_cpd_core_fit(int o, int v, int Rt, int naux, const double* Xo, const double* Xv,
@@ -304,8 +305,8 @@ thc_cpd_status thc_cpd_core_fit(int o, int v, int Rt, int naux, const double* Xo
  * GEMMs of 2 naux o v R flop per sweep), the same normal-equation solve, normalisation, loss
  * and stopping rule as thc_cpd_als: A[4] (o x R, v x R, o x R, v x R) start factors in, final
  * unit-column factors out; lam (R) out; sweeps_done and fit_host (host) out, each may be NULL.
- * opts->precision must be THC_CPD_FP64; opts->ldl = THC_CPD_LDL_EMULATED runs the GEMMs and the
- * solve on the emulated FP64 tensor-core path. opts->history: NULL or 2 * max_sweeps host
+ * opts->precision must be THC_CPD_FP64; GEMMs as for thc_cpd_core_fit, opts->ldl =
+ * THC_CPD_LDL_EMULATED runs them all and the solve on the FP64-accurate tensor-core path. opts->history: NULL or 2 * max_sweeps host
  * doubles (loss, fit per sweep). opts->flags_out bit 0: a pseudo-inverse solve was used.
  * Workspace: about (2 o v + max(o, v) R + 3 R) naux + naux^2 + 5 R^2 doubles (cudaMallocAsync).
  * 1 <= R <= 2048, 1 <= o, v <= 4096. Synchronises once per sweep. */
@@ -319,8 +320,8 @@ thc_cpd_status thc_cpd_df_als(int o, int v, int naux, int R, const double* B, do
  * CPD Gt = sum_r lam_r prod_k A_k[i_k,r]. dims: host array of the d mode sizes; X, A: host
  * arrays of d device pointers (X_k dims[k] x Rt, A_k dims[k] x R, row-major FP64); Z: device
  * Rt x Rt (need not be symmetric). 2 <= d <= 8, 1 <= dL <= d - 1, 1 <= dims[k] <= 4096,
- * 1 <= R <= 2048. Precision FP64 only; opts->ldl = THC_CPD_LDL_EMULATED runs the GEMMs and the
- * solve on the emulated FP64 tensor-core path.
+ * 1 <= R <= 2048. Precision FP64 only; GEMMs as for thc_cpd_core_fit, opts->ldl =
+ * THC_CPD_LDL_EMULATED runs them all and the solve on the FP64-accurate tensor-core path.
  * thc_cpd_nd_mttkrp: M (dims[mode] x R, device) = the mode-`mode` MTTKRP (lam not applied).
  * thc_cpd_nd_als: A in/out (unit columns out), lam out, sweeps_done / fit_host host (may be
  * NULL); solve, normalisation, loss, stopping rule, history and flags_out as thc_cpd_df_als.

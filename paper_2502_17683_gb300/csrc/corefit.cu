@@ -14,8 +14,8 @@
 //   Z          = F^T F                         symmetric GEMM
 // and, on request, the loss ||G_DF - G_THC(Z)||^2 = ||D D^T||^2 - 2 <E^T E, Z> + <Z, S Z S>
 // (D[X,(i,a)] = B[X,i,a]) with three fixed-order dot products.
-// The GEMMs run on the FP64 pipes, or as the FP64-accurate emulated products of the BF16
-// tensor cores (oz_dgemm) when opts->ldl is THC_CPD_LDL_EMULATED.
+// The GEMMs run as FP64-accurate products on the BF16 tensor cores (oz_dgemm) from 1e7 flops
+// on (oz_worth; all of them with THC_CPD_LDL_EMULATED), smaller ones on the FP64 pipes.
 #include <math.h>
 #include <stdarg.h>
 #include <stdio.h>

@@ -16,9 +16,9 @@
 // single GEMMs over all X. The normal equations, their solve (LDL^T, pseudo-inverse on a
 // failed pivot), the column normalisation and the factor-form loss are those of the
 // THC-driven path; only the MTTKRP and ||G_DF||^2 = ||D D^T||_F^2 (D = B as naux x o v)
-// differ. GEMMs on the FP64 pipes, or the FP64-accurate emulated products of the tensor
-// cores with opts->ldl = THC_CPD_LDL_EMULATED (the solve then uses the emulated two-level
-// LDL^T too).
+// differ. GEMMs as FP64-accurate products on the tensor cores from 1e7 flops on (oz_worth),
+// smaller ones on the FP64 pipes; with THC_CPD_LDL_EMULATED all of them on the tensor cores,
+// and the solve uses the emulated two-level LDL^T too.
 #include <math.h>
 #include <stdarg.h>
 #include <stdio.h>

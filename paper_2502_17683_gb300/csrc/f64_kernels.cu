@@ -767,7 +767,7 @@ void coupling_rows(int m, int n, long* ra, long* rb, long* part) {
     const long nch = cdiv(m - h, kOzPanel);
     *ra = std::max(*ra, nch * n);
     *rb = std::max(*rb, nch * h);
-    // the K groups oz_gemm_sub forms for an n x h product (128 x 32 tiles)
+    // the most K groups that an n x h product takes (of 128 x 32 tiles)
     const long tiles = (long)cdiv(n, 128) * cdiv(h, 32);
     const long groups = std::min<long>(nch, std::max<long>(1, num_sms() / tiles));
     *part = std::max(*part, (groups - 1) * n * (long)h);

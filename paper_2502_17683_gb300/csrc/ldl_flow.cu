@@ -17,7 +17,7 @@
 // Chain step s runs S(s, s-1), U(s, s, s-1), F(s) back to back in shared memory (warps 0-7
 // of the chain CTA; warps 8-14 prefetch its next two tiles, warp 15 publishes its
 // progress). The other tasks form one list in a fixed order, split into the critical
-// tasks (row tile s on panels s-2, s-3), served by CTAs of their own, and the rest; worker
+// tasks (row tile s on panels s-2 .. s-4), served by CTAs of their own, and the rest; worker
 // groups (128 threads) claim entries with an atomic ticket and wait for their inputs on
 // per-tile progress counters:
 //   sdone[t] = k + 1 once S(t, k) is stored; cnt[t][j] = number of panels applied to tile
@@ -979,7 +979,7 @@ const Plan* get_plan(int R, int n) {
     // workers shrink), fewer only when there are fewer main tasks than CTAs: a CTA's four
     // groups share its SM's FP64 pipe, so few tasks are spread one per SM
     p.grid = (int)std::min<long>(nsm, 1 + std::max<long>(1, p.nmain));
-    // critical CTAs: seven critical tasks per chain step, those of the next step claimed while they
+    // critical CTAs: nine critical tasks per chain step, those of the next step claimed while they
     // wait; fewer on small grids
     p.ncrit = p.ntasks > p.nmain ? (p.grid >= 64 ? 12 : p.grid >= 24 ? 8 : p.grid >= 8 ? 4 : 1) : 0;
     p.grid = std::min(nsm, p.grid + p.ncrit);

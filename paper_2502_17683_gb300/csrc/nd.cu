@@ -12,8 +12,9 @@
 // their solve, the normalisation and the factor-form loss
 //     ||G||^2 = sum Z o (S_L Z S_R),  <G, Gt> = sum_r lam_r sum_Q (Z^T P_L)[Q,r] P_R[Q,r],
 //     ||Gt||^2 = lam^T (o_k Gram_k) lam
-// are those of the order-4 path. GEMMs on the FP64 pipes, or the FP64-accurate emulated
-// tensor-core products with opts->ldl = THC_CPD_LDL_EMULATED.
+// are those of the order-4 path. GEMMs as FP64-accurate tensor-core
+// products from 1e7 flops on (oz_worth; all of them with THC_CPD_LDL_EMULATED), smaller ones on
+// the FP64 pipes.
 #include <math.h>
 #include <stdarg.h>
 #include <stdio.h>
