@@ -502,7 +502,7 @@ void compute_normG2(Ctx& c) {
 
 // What follows from a factor: its Gram G_k = A_k^T A_k and its projection W_k = X_k^T A_k (either
 // or both); on the tensor cores from one cut of its columns.
-void factor_products(Ctx& c, int k, const double* Ak, bool gram, bool proj) {
+void factor_products(Ctx& c, int k, const double* Ak, bool gram, bool proj, SmallJobs& small) {
     const int n = c.s.n[k], R = c.s.R, Rt = c.s.Rt;
     const bool og = c.ozp && gram && oz_worth(R, R, n, true), op = c.ozp && proj && oz_worth(Rt, R, n, false);
     OzMat a = c.dA;
@@ -510,11 +510,11 @@ void factor_products(Ctx& c, int k, const double* Ak, bool gram, bool proj) {
     if (og || op) oz_split_cols(c.st, Ak, nullptr, R, a);
     if (og)
         mul_digits(c, a, a, c.G[k], R, true);
-    else if (gram)
+    else if (gram && !dgemm_small_add(small, true, R, R, n, Ak, R, Ak, R, c.G[k]))
         dgemm(c.st, true, R, R, n, Ak, R, Ak, nullptr, R, c.G[k], R, nullptr, true, c.part, c.part_cap);
     if (op)
         mul_digits(c, digits_XT(c, k & 1), a, c.W[k], R, false);
-    else if (proj)
+    else if (proj && !dgemm_small_add(small, false, Rt, R, n, c.X[k], Rt, Ak, R, c.W[k]))
         dgemm(c.st, true, Rt, R, n, c.X[k], Rt, Ak, nullptr, R, c.W[k], R, nullptr, false, c.part, c.part_cap);
 }
 
@@ -575,10 +575,12 @@ void refresh_state(Ctx& c, const double* const A[4]) {
     prepare_digits(c);
     const bool fp64 = c.prec == THC_CPD_FP64;
     if (!fp64) mixed_split_factors(c.mx, c.st, A);
+    SmallJobs small;
     for (int k = 0; k < 4; ++k) {
-        factor_products(c, k, A[k], true, fp64);
+        factor_products(c, k, A[k], true, fp64, small);
         if (!fp64) mixed_project(c.mx, c.st, k, false);
     }
+    dgemm_small_run(c.st, small);
 }
 
 // One mode update. M_k is formed in the Haug rows; returns with A[k], lam, G_k, W_k new.
@@ -617,7 +619,9 @@ thc_cpd_status mode_update(Ctx& c, double* const A[4], double* lam, int k, bool 
     }
     normalise_columns(c.st, n, R, A[k], lam, c.LinvD);  // panel buffer is free after the solve
     const bool fp64 = c.prec == THC_CPD_FP64;
-    factor_products(c, k, A[k], true, fp64);
+    SmallJobs small;
+    factor_products(c, k, A[k], true, fp64, small);
+    dgemm_small_run(c.st, small);
     if (!fp64) {
         const double* one[4] = {};
         one[k] = A[k];
@@ -646,7 +650,9 @@ thc_cpd_status sweep(Ctx& c, double* const A[4], double* lam, bool safe, bool ev
             loss_eval(c.st, c.s.Rt, c.s.R, c.Y, c.W[2], c.W[3], lam, c.G, c.red, c.sc, tol);
         } else {
             // the loss is a cancelling difference: FP64 projections and Z product
-            for (int k = 0; k < 4; ++k) factor_products(c, k, A[k], false, true);
+            SmallJobs small;
+            for (int k = 0; k < 4; ++k) factor_products(c, k, A[k], false, true, small);
+            dgemm_small_run(c.st, small);
             zgemm_fp64(c, 1);
             loss_eval(c.st, c.s.Rt, c.s.R, c.Y, c.W[2], c.W[3], lam, c.G, c.red, c.sc, tol);
         }
@@ -1385,8 +1391,10 @@ thc_cpd_status thc_cpd_mttkrp(int o, int v, int Rt, int R, const double* Xo, con
     Ctx c;
     CKS(ctx_init(c, s, Xo, Xv, Z, opts, 0));
     if (c.prec == THC_CPD_FP64) {
+        SmallJobs small;
         for (int k = 0; k < 4; ++k)
-            if (k != mode) factor_products(c, k, A[k], false, true);
+            if (k != mode) factor_products(c, k, A[k], false, true, small);
+        dgemm_small_run(c.st, small);
         zgemm_fp64(c, mode / 2);
         backproject_fp64(c, mode, M);
     } else {
@@ -1465,7 +1473,9 @@ thc_cpd_status thc_cpd_loss(int o, int v, int Rt, int R, const double* Xo, const
     CKS(ctx_init(c, s, Xo, Xv, Z, &o2, NEED_GRAM | (normG2 > 0.0 ? 0u : NEED_NORM)));
     double nG2;
     CKS(obtain_norm(c, normG2, &nG2));
-    for (int k = 0; k < 4; ++k) factor_products(c, k, A[k], true, true);
+    SmallJobs small;
+    for (int k = 0; k < 4; ++k) factor_products(c, k, A[k], true, true, small);
+    dgemm_small_run(c.st, small);
     zgemm_fp64(c, 1);
     loss_eval(c.st, Rt, R, c.Y, c.W[2], c.W[3], lam ? lam : c.ones, c.G, c.red, c.sc, 0.0);
     DevScalars h;

@@ -12,6 +12,24 @@ void dgemm(cudaStream_t st, bool trans_a, int M, int N, int K, const double* A, 
            const double* B, const double* B2, int ldb, double* C, int ldc,
            const double* E, bool symm, double* part, size_t part_cap);
 
+// Independent products C = A^T B (A K x M, B K x N, all with this list's N, ldb = ldc) that take
+// small tiles of one size, in one launch. dgemm_small_add returns false for a product that dgemm
+// would not run on tiles of the list's size (the caller then calls dgemm); the list is empty again
+// after dgemm_small_run.
+struct SmallJob {
+    const double *A, *B;
+    double* C;
+    int M, K, lda, symm, row0;  // row0: first block row of the launch
+};
+struct SmallJobs {
+    SmallJob job[8];  // a Gram and a projection for each of four factors
+    int n = 0, T = 0, N = 0, ld = 0, rows = 0;
+    double flops = 0.0;
+};
+bool dgemm_small_add(SmallJobs& js, bool symm, int M, int N, int K, const double* A, int lda, const double* B,
+                     int ld, double* C);
+void dgemm_small_run(cudaStream_t st, SmallJobs& js);
+
 // Split-K partial capacity (doubles) that dgemm may use for an M x N output.
 size_t dgemm_part_need(int M, int N, int K);
 

@@ -184,16 +184,17 @@ k_dsyrk32(int N, int K, const double* __restrict__ A, const double* __restrict__
 // tiles too few CTAs: an SM takes T^2 K / 2 clocks per tile on its FP64 pipe, so a 60 x 80 x 5
 // product on two 64 x 64 tiles (K padded to 16) costs 16 us and on 80 of 8 x 8 under 2 us. K is
 // not split and not padded; with T = 8 a K of 64 is loaded at once. SYMM: lower tiles only, mirrored.
-template <int T, bool TA, bool HADB, bool SYMM>
-__global__ void __launch_bounds__(64)
-k_dgemm_small(int M, int N, int K, const double* __restrict__ A, int lda, const double* __restrict__ B,
-              const double* __restrict__ B2, int ldb, double* __restrict__ C, int ldc) {
+template <int T, bool TA, bool HADB>
+__device__ __forceinline__ void small_tile_product(int bx, int by, bool symm, int M, int N, int K,
+                                                   const double* __restrict__ A, int lda,
+                                                   const double* __restrict__ B, const double* __restrict__ B2,
+                                                   int ldb, double* __restrict__ C, int ldc,
+                                                   const double* __restrict__ E) {
     constexpr int BK = 512 / T, Q = T / 8;  // Q x Q outputs per thread
     constexpr int PER = T * BK / 64;        // elements of each operand tile per thread
     __shared__ double As[BK][T + 1];
     __shared__ double Bs[BK][T + 1];
-    const int bx = blockIdx.x, by = blockIdx.y;
-    if (SYMM && by < bx) return;
+    if (symm && by < bx) return;
     const int m0 = by * T, n0 = bx * T, tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
     double acc[Q][Q];
 #pragma unroll
@@ -242,9 +243,29 @@ k_dgemm_small(int M, int N, int K, const double* __restrict__ A, int lda, const 
         for (int j = 0; j < Q; ++j) {
             const int m = m0 + ty + 8 * i, n = n0 + tx + 8 * j;
             if (m >= M || n >= N) continue;
-            C[(size_t)m * ldc + n] = acc[i][j];
-            if (SYMM) C[(size_t)n * ldc + m] = acc[i][j];
+            const double v = E ? acc[i][j] * E[(size_t)m * ldc + n] : acc[i][j];
+            C[(size_t)m * ldc + n] = v;
+            if (symm) C[(size_t)n * ldc + m] = v;
         }
+}
+
+template <int T, bool TA, bool HADB, bool SYMM>
+__global__ void __launch_bounds__(64)
+k_dgemm_small(int M, int N, int K, const double* __restrict__ A, int lda, const double* __restrict__ B,
+              const double* __restrict__ B2, int ldb, double* __restrict__ C, int ldc, const double* __restrict__ E) {
+    small_tile_product<T, TA, HADB>(blockIdx.x, blockIdx.y, SYMM, M, N, K, A, lda, B, B2, ldb, C, ldc, E);
+}
+
+// Several such products A^T B in one launch: a small problem's Grams and projections take 3 us each,
+// of which the arithmetic is a tenth. MTTKRP at (o, v, R_thc, R_cp) = (5, 15, 60, 80) 65 -> 57 us, ten
+// ALS sweeps 3289 -> 3152.
+template <int T>
+__global__ void __launch_bounds__(64) k_dgemm_small_jobs(const __grid_constant__ SmallJobs js) {
+    int i = 0;
+    while (i + 1 < js.n && (int)blockIdx.y >= js.job[i + 1].row0) ++i;
+    const SmallJob& J = js.job[i];
+    small_tile_product<T, true, false>(blockIdx.x, blockIdx.y - J.row0, J.symm, J.M, js.N, J.K, J.A, J.lda, J.B,
+                                       nullptr, js.ld, J.C, js.ld, nullptr);
 }
 
 namespace {
@@ -345,12 +366,12 @@ int small_tile(int M, int N, int K, bool symm, bool trans_a, const GemmPlan& p) 
 
 template <int T>
 bool launch_small(cudaStream_t st, bool ta, bool hadb, bool symm, int M, int N, int K, const double* A, int lda,
-                  const double* B, const double* B2, int ldb, double* C, int ldc) {
+                  const double* B, const double* B2, int ldb, double* C, int ldc, const double* E) {
     const dim3 grid(cdiv(N, T), cdiv(M, T));
     if (grid.y > 65535) return false;
 #define THC_S(TA_, HB_, SY_)                                                                             \
     if (ta == TA_ && hadb == HB_ && symm == SY_) {                                                       \
-        k_dgemm_small<T, TA_, HB_, SY_><<<grid, 64, 0, st>>>(M, N, K, A, lda, B, B2, ldb, C, ldc);       \
+        k_dgemm_small<T, TA_, HB_, SY_><<<grid, 64, 0, st>>>(M, N, K, A, lda, B, B2, ldb, C, ldc, E);    \
         return true;                                                                                     \
     }
     THC_S(false, false, false)
@@ -363,6 +384,36 @@ bool launch_small(cudaStream_t st, bool ta, bool hadb, bool symm, int M, int N, 
     return false;
 }
 }  // namespace
+
+bool dgemm_small_add(SmallJobs& js, bool symm, int M, int N, int K, const double* A, int lda, const double* B,
+                     int ld, double* C) {
+    if (M <= 0 || N <= 0 || K <= 0 || js.n == (int)(sizeof(js.job) / sizeof(js.job[0]))) return false;
+    const int T = small_tile(M, N, K, symm, true, plan_gemm(M, N, K, symm));
+    if (T == 0 || js.rows + cdiv(M, T) > 65535) return false;
+    if (js.n > 0 && (js.T != T || js.N != N || js.ld != ld)) return false;
+    js.T = T;
+    js.N = N;
+    js.ld = ld;
+    js.job[js.n++] = SmallJob{A, B, C, M, K, lda, symm, js.rows};
+    js.rows += cdiv(M, T);
+    js.flops += (symm ? 1.0 : 2.0) * M * (double)N * K;
+    return true;
+}
+
+void dgemm_small_run(cudaStream_t st, SmallJobs& js) {
+    if (js.n > 0) {
+        ProfScope prof(st, KC_DGEMM, js.flops);
+        const dim3 grid(cdiv(js.N, js.T), js.rows);
+        count_launch();
+        if (js.T == 8)
+            k_dgemm_small_jobs<8><<<grid, 64, 0, st>>>(js);
+        else if (js.T == 16)
+            k_dgemm_small_jobs<16><<<grid, 64, 0, st>>>(js);
+        else
+            k_dgemm_small_jobs<32><<<grid, 64, 0, st>>>(js);
+    }
+    js = SmallJobs();
+}
 
 size_t dgemm_part_need(int M, int N, int K) {
     GemmPlan p = plan_gemm(M, N, K, false);
@@ -387,16 +438,14 @@ void dgemm(cudaStream_t st, bool trans_a, int M, int N, int K, const double* A, 
     }
     const bool hadb = B2 != nullptr;
     ProfScope prof(st, KC_DGEMM, (symm ? 1.0 : 2.0) * M * (double)N * K);
-    if (!E) {
-        const int T = small_tile(M, N, K, symm, trans_a, p);
-        const bool done =
-            T == 8 ? launch_small<8>(st, trans_a, hadb, symm, M, N, K, A, lda, B, B2, ldb, C, ldc)
-            : T == 16 ? launch_small<16>(st, trans_a, hadb, symm, M, N, K, A, lda, B, B2, ldb, C, ldc)
-            : T == 32 ? launch_small<32>(st, trans_a, hadb, symm, M, N, K, A, lda, B, B2, ldb, C, ldc) : false;
-        if (done) {
-            count_launch();
-            return;
-        }
+    const int T = small_tile(M, N, K, symm, trans_a, p);
+    const bool done =
+        T == 8 ? launch_small<8>(st, trans_a, hadb, symm, M, N, K, A, lda, B, B2, ldb, C, ldc, E)
+        : T == 16 ? launch_small<16>(st, trans_a, hadb, symm, M, N, K, A, lda, B, B2, ldb, C, ldc, E)
+        : T == 32 ? launch_small<32>(st, trans_a, hadb, symm, M, N, K, A, lda, B, B2, ldb, C, ldc, E) : false;
+    if (done) {
+        count_launch();
+        return;
     }
     if (symm && trans_a && !hadb && !E && M == N && lda == ldb && K > 0) {
         const int nt = cdiv(N, SYT);

@@ -214,3 +214,26 @@ def test_fp64_mttkrp_many_columns(api, R, mode):
     M = api.thc_cpd_mttkrp(X[0], X[1], Z, A, mode)
     lim = 2 * (3 * v + 2 * Rt) * U * mttkrp([x.abs() for x in X], Z.abs(), [a.abs() for a in A])
     assert ((M - mttkrp(X, Z, A)).abs() <= lim).all()
+
+
+# Grams and projections of several factors in one launch: rows of one product end inside a tile, T of
+# 8, 16 and 32, a product that leaves the list (its tiles differ). Bound as above, in FP64.
+@pytest.mark.parametrize("o,v,Rt,R", [(1, 2, 8, 8), (3, 5, 9, 65), (5, 15, 60, 80), (9, 33, 97, 161), (12, 60, 200, 300)])
+def test_small_products_in_one_launch(api, o, v, Rt, R):
+    g = torch.Generator(device="cuda").manual_seed(o * 100 + R)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda", dtype=torch.float64)
+    X, Z = [rnd(o, Rt), rnd(v, Rt)], rnd(Rt, Rt)
+    A = [rnd(n, R) for n in (o, v, o, v)]
+    lam = rnd(R)
+
+    def parts(X, Z, A, lam):
+        W = [X[k % 2].T @ A[k] for k in range(4)]
+        G = [a.T @ a for a in A]
+        return (lam * (W[0] * W[1]) * (Z @ (W[2] * W[3]))).sum(), lam @ ((G[0] * G[1] * G[2] * G[3]) @ lam)
+
+    loss, _ = api.thc_cpd_loss(X[0], X[1], Z, A, lam=lam, normG2=1.0)
+    s1, s2 = parts(X, Z, A, lam)
+    a1, a2 = parts([x.abs() for x in X], Z.abs(), [a.abs() for a in A], lam.abs())
+    # sums of v, v, Rt terms (s1) and v of four Grams (s2), then Rt R and R^2 terms, on either side
+    lim = 2 * U * (2 * (4 * v + Rt + Rt + R) * a1 + (4 * v + 2 * R) * a2)
+    assert abs(loss - float(1.0 - 2.0 * s1 + s2)) <= float(lim) + 4 * U
