@@ -4,9 +4,31 @@
 #include <stdint.h>
 #include <stddef.h>
 
+#include <map>
+#include <mutex>
 #include <string>
 
 namespace thc {
+
+// What is set up once for each device: kernel attributes (the shared memory that a launch may ask
+// for) hold for the device that is current when they are set, so a second GPU of the same process
+// needs its own. set_up(device) runs with that device current; every thread gets its result.
+template <class T>
+class PerDevice {
+    std::mutex mu_;
+    std::map<int, T> value_;
+
+public:
+    template <class F>
+    T get(F set_up) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess) return T();
+        std::lock_guard<std::mutex> lk(mu_);
+        auto it = value_.find(dev);
+        if (it == value_.end()) it = value_.emplace(dev, set_up(dev)).first;
+        return it->second;
+    }
+};
 
 // SMs of the current device (GB300: 152), queried once per device: grids of persistent and
 // grid-stride kernels follow the part they run on.

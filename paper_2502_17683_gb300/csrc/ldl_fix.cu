@@ -591,12 +591,12 @@ void ldl_fix_carve(FixWs& w, Arena& ar, int R, int n) {
 
 bool ldl_fix_prepare() {
     if (!oz_available()) return false;
-    static const bool ok =
-        cudaFuncSetAttribute(k_fix_diag, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DiagSmem)) ==
-            cudaSuccess &&
-        cudaFuncSetAttribute(k_fix_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PanelSmem)) ==
-            cudaSuccess;
-    return ok;
+    static PerDevice<bool> ready;
+    return ready.get([](int) {
+        const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        return cudaFuncSetAttribute(k_fix_diag, attr, (int)sizeof(DiagSmem)) == cudaSuccess &&
+               cudaFuncSetAttribute(k_fix_rows, attr, (int)sizeof(PanelSmem)) == cudaSuccess;
+    });
 }
 
 cudaError_t ldl_fix(cudaStream_t st, int R, int n, double* Haug, double* dinv, DevScalars* sc, int mode,

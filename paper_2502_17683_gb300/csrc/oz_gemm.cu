@@ -3,7 +3,6 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "f64.cuh"
 #include "fixed.cuh"
@@ -578,9 +577,6 @@ __global__ void k_oz_add_parts(double* __restrict__ C, int ldc, int M, int N, co
 
 // ---- host ----------------------------------------------------------------------------
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
-std::once_flag g_once;
-bool g_ready = false;
-int g_num_sm = 148;
 // From 1e7 flops on, products run from digits. An MTTKRP at (o, v, R_thc, R_cp) in us with the line at
 // 4e6 / 8e6 / 1.6e7 / 3e7 / never: (6,30,144,216) 183 / 187 / 167 / 172 / 172, (8,40,192,288)
 // 172 / 188 / 185 / 188 / 190, (14,70,336,504) 207 / 203 / 202 / 252 / 337, (20,100,480,720)
@@ -588,31 +584,27 @@ int g_num_sm = 148;
 constexpr double kWorthFlops = 1.0e7;
 constexpr int kColsSmem = COLS_PER_BLOCK * (kColsMaxK + 4) * (int)sizeof(double);
 
+// The current device can run the kernels of this file (sm_103), their attributes set on it.
 bool oz_init() {
-    std::call_once(g_once, [] {
-        int dev = 0;
+    static PerDevice<bool> ready;
+    return ready.get([](int dev) {
         cudaDeviceProp p;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaGetDeviceProperties(&p, dev) != cudaSuccess) return;
         const int need = std::max(std::max(Tile<64>::SMEM, Tile<32>::SMEM), kColsSmem);
-        if (!(p.major == 10 && p.minor == 3) || (int)p.sharedMemPerBlockOptin < need) return;
-        g_num_sm = p.multiProcessorCount;
+        if (cudaGetDeviceProperties(&p, dev) != cudaSuccess || !(p.major == 10 && p.minor == 3) ||
+            (int)p.sharedMemPerBlockOptin < need)
+            return false;
         void* fn = nullptr;
         cudaDriverEntryPointQueryResult q;
         if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) !=
                 cudaSuccess ||
             q != cudaDriverEntryPointSuccess)
-            return;
-        g_encode = (PFN_cuTensorMapEncodeTiled_v12000)fn;
-        if (cudaFuncSetAttribute(k_oz_update<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, Tile<64>::SMEM) !=
-                cudaSuccess ||
-            cudaFuncSetAttribute(k_oz_update<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, Tile<32>::SMEM) !=
-                cudaSuccess ||
-            cudaFuncSetAttribute(k_oz_split_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, kColsSmem) !=
-                cudaSuccess)
-            return;
-        g_ready = true;
+            return false;
+        g_encode = (PFN_cuTensorMapEncodeTiled_v12000)fn;  // (the same for every device)
+        const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        return cudaFuncSetAttribute(k_oz_update<64>, attr, Tile<64>::SMEM) == cudaSuccess &&
+               cudaFuncSetAttribute(k_oz_update<32>, attr, Tile<32>::SMEM) == cudaSuccess &&
+               cudaFuncSetAttribute(k_oz_split_cols, attr, kColsSmem) == cudaSuccess;
     });
-    return g_ready;
 }
 
 // 3-D map over the digit slices [planes][rows][KP] (BF16; S planes per K chunk):
@@ -637,6 +629,7 @@ struct MulPlan {
 MulPlan plan_mul(int mA, int mB, int nch, bool lower, size_t part_cap) {
     MulPlan best{64, 1};
     double bc = 1e300;
+    const int sms = num_sms();
     for (int bn : {64, 32}) {
         const int tm = cdiv(mA, BM), tn = cdiv(mB, bn);
         long act = 0;
@@ -646,7 +639,7 @@ MulPlan plan_mul(int mA, int mB, int nch, bool lower, size_t part_cap) {
         for (int g = 1; g <= gmax; ++g) {
             const int cpg = cdiv(nch, g), gr = cdiv(nch, cpg);
             if (gr != g || (size_t)(gr - 1) * mA * mB > part_cap) continue;
-            const double waves = (double)cdiv(act * gr, g_num_sm);
+            const double waves = (double)cdiv(act * gr, sms);
             const double c = waves * (cpg * (bn == 64 ? 10.7 : 5.6) + (bn == 64 ? 2.5 : 1.5)) + (gr > 1 ? 6.0 + 0.3 * gr : 0.0);
             if (c < bc) {
                 bc = c;
@@ -669,11 +662,11 @@ cudaError_t launch_mul(cudaStream_t st, const OzMat& A, const OzMat& B, UpdArgs 
     a.cpg = cdiv(a.nchunks, std::max(1, groups));
     a.kgroups = cdiv(a.nchunks, a.cpg);
     // persistent: one CTA per SM, at most one per active (tile, K group) work item
-    const int grid = (int)std::max<long>(1, std::min<long>(active * a.kgroups, g_num_sm));
+    const int grid = (int)std::max<long>(1, std::min<long>(active * a.kgroups, num_sms()));
     k_oz_update<BN><<<grid, NTHREADS, Tile<BN>::SMEM, st>>>(ma, mb, a);
     count_launch();
     if (a.kgroups > 1) {
-        k_oz_add_parts<<<(int)std::min<long>(cdiv((long)a.mA * a.mB, 256), 4L * g_num_sm), 256, 0, st>>>(
+        k_oz_add_parts<<<(int)std::min<long>(cdiv((long)a.mA * a.mB, 256), 4L * num_sms()), 256, 0, st>>>(
             a.C, a.ldc, a.mA, a.mB, a.part, a.kgroups - 1);
         count_launch();
     }
@@ -705,7 +698,7 @@ void ozmat_carve(OzMat& m, Arena& ar, int rows, int K) {
 void oz_split_rows(cudaStream_t st, const double* src, int ld, OzMat& m) {
     if (m.rows <= 0) return;
     // up to eight rows per SM, more warps to a row (see the kernel); beyond, the rows fill the chip
-    const int wpr = m.rows > 8 * g_num_sm ? 1 : m.K > 2 * KP ? 4 : m.K > KP ? 2 : 1, grid = cdiv(m.rows, ROWS_PER_BLOCK / wpr);
+    const int wpr = m.rows > 8 * num_sms() ? 1 : m.K > 2 * KP ? 4 : m.K > KP ? 2 : 1, grid = cdiv(m.rows, ROWS_PER_BLOCK / wpr);
     if (ld % 2 == 0 && ((uintptr_t)src & 15) == 0)
         k_oz_split_rows<true><<<grid, 32 * ROWS_PER_BLOCK, 0, st>>>(src, ld, m.rows, m.K, m.d, m.e, wpr);
     else
@@ -728,7 +721,7 @@ void oz_split_cols_stack(cudaStream_t st, const double* S1, const double* S2, in
     // each other's latency better (twelve 480 x 720 matrices in a stack: the exchange energies took
     // 920 us with 1024 threads, 892 with 256)
     const long blocks = (long)cdiv(n, COLS_PER_BLOCK) * parts * g;
-    const int threads = blocks > 2L * g_num_sm ? 256 : 256 * std::min(4, kpad / KP);
+    const int threads = blocks > 2L * num_sms() ? 256 : 256 * std::min(4, kpad / KP);
     k_oz_split_cols<<<dim3(cdiv(n, COLS_PER_BLOCK), parts, g), threads,
                       COLS_PER_BLOCK * (kpad + 4) * sizeof(double), st>>>(S1, S2, ld, n, m.K, m.rows, m.d, m.e,
                                                                            parts > 1 ? 1 : 0);

@@ -341,19 +341,6 @@ __global__ void k_tc_splitk_reduce(const double* __restrict__ part, int splits, 
 
 // ---- host side ---------------------------------------------------------------------
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
-std::once_flag g_encode_once;
-
-bool load_encode() {
-    std::call_once(g_encode_once, [] {
-        void* fn = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault,
-                                             &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            g_encode = (PFN_cuTensorMapEncodeTiled_v12000)fn;
-    });
-    return g_encode != nullptr;
-}
 
 bool make_map(CUtensorMap* map, bool tf32, const void* base, int rows, int cols, int pitch,
               int box_rows) {
@@ -369,19 +356,31 @@ bool make_map(CUtensorMap* map, bool tf32, const void* base, int rows, int cols,
     return r == CUDA_SUCCESS;
 }
 
-int g_max_smem = 0;
+// Shared memory that a block may have on the current device with k_tc_gemm's attributes set on it;
+// 0 where the kernel cannot run (not sm_103).
+int tc_max_smem() {
+    static PerDevice<int> smem;
+    return smem.get([](int dev) {
+        cudaDeviceProp p;
+        if (cudaGetDeviceProperties(&p, dev) != cudaSuccess || !(p.major == 10 && p.minor == 3)) return 0;
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) !=
+                cudaSuccess ||
+            q != cudaDriverEntryPointSuccess)
+            return 0;
+        g_encode = (PFN_cuTensorMapEncodeTiled_v12000)fn;  // (the same for every device)
+        const int most = (int)p.sharedMemPerBlockOptin;
+        const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        const bool ok = cudaFuncSetAttribute(k_tc_gemm<true>, attr, most) == cudaSuccess &&
+                        cudaFuncSetAttribute(k_tc_gemm<false>, attr, most) == cudaSuccess;
+        return ok ? most : 0;
+    });
+}
 
 }  // namespace
 
-bool tc_available() {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return false;
-    cudaDeviceProp p;
-    if (cudaGetDeviceProperties(&p, dev) != cudaSuccess) return false;
-    if (!(p.major == 10 && p.minor == 3)) return false;
-    g_max_smem = (int)p.sharedMemPerBlockOptin;
-    return load_encode();
-}
+bool tc_available() { return tc_max_smem() > 0; }
 
 int tc_take_error() { return take_error_word(&g_tc_error); }
 
@@ -394,7 +393,7 @@ cudaError_t tc_launch(cudaStream_t st, bool tf32, const SplitMat& A, const Split
     const int tileB = BN * KBYTES;
     const int stage_bytes = 2 * TILE_A + 2 * tileB;
     const int nkb = std::max(1, cdiv((long)K * (tf32 ? 4 : 2), KBYTES));
-    const int avail = g_max_smem - 1024 - EPI_STAGE_BYTES - 256;
+    const int avail = tc_max_smem() - 1024 - EPI_STAGE_BYTES - 256;
     const int stages = std::max(2, std::min(6, avail / stage_bytes));
     const size_t smem = 1024 + (size_t)stages * stage_bytes + EPI_STAGE_BYTES + 256;
     CUtensorMap mAh, mAl, mBh, mBl;
@@ -437,12 +436,6 @@ cudaError_t tc_launch(cudaStream_t st, bool tf32, const SplitMat& A, const Split
     const int grid = std::min(args.ntiles, num_sms());  // persistent: at most one CTA per SM
     ProfScope prof(st, ep.prof_class, 2.0 * M * (double)N * K);
     count_launch(splits > 1 ? 2 : 1);
-    static std::once_flag attr_once;
-    std::call_once(attr_once, [] {
-        // once per process, outside any stream capture: allow the largest ring
-        cudaFuncSetAttribute(k_tc_gemm<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, g_max_smem);
-        cudaFuncSetAttribute(k_tc_gemm<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, g_max_smem);
-    });
     if (tf32)
         k_tc_gemm<true><<<grid, NTHREADS, smem, st>>>(mAh, mAl, mBh, mBl, args);
     else
@@ -499,8 +492,7 @@ int tc_tuned_entries() {
 cudaError_t tc_gemm(cudaStream_t st, bool tf32, const SplitMat& A, const SplitMat& B, int M, int N,
                     int K, const TcEpilogue& ep, double* part, size_t part_cap) {
     if (M <= 0 || N <= 0) return cudaSuccess;
-    if (!g_encode && !load_encode()) return cudaErrorNotSupported;
-    if (g_max_smem == 0) tc_available();
+    if (!tc_available()) return cudaErrorNotSupported;
     const TuneKey key{M, N, K, epi_kind(tf32, ep)};
     int BN = 0;
     {

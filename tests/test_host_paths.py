@@ -1,0 +1,47 @@
+"""The host side of the entry points, on the CPU, against a CUDA runtime that runs no kernel
+(tests/_fake_cuda.py): which kernels are launched, and what becomes of a call whose launch,
+tensor map or allocation fails."""
+import shutil
+
+import pytest
+
+from tests import _fake_cuda
+
+pytestmark = pytest.mark.skipif(shutil.which("g++") is None, reason="needs a host compiler")
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    return _fake_cuda.load(tmp_path_factory.mktemp("fake_cuda"))
+
+
+@pytest.fixture
+def calls(lib):
+    lib.fake_reset()
+    yield _fake_cuda.Calls(lib)
+    lib.fake_reset()
+
+
+LAUNCHES = {
+    "mttkrp": lambda c: c.mttkrp(20, 100, 300, 400),
+    "split": lambda c: c.mttkrp(20, 100, 300, 400, precision=1),
+    "loss": lambda c: c.loss(20, 100, 300, 400, normG2=0.0),
+    "sweep": lambda c: c.sweep(20, 100, 300, 400),
+    "emulated": lambda c: c.sweep(20, 100, 300, 1100, ldl=3),
+    "batched": lambda c: c.batched([(12, 60, 200, 420), (3, 9, 30, 40)]),
+    "exchange": lambda c: c.exchange(10, 50, 200, 300, 4),
+    "core fit": lambda c: c.core_fit(10, 50, 200, 220, loss=True),
+}
+
+
+# kernel attributes (the shared memory a launch may ask for) belong to one device
+@pytest.mark.parametrize("what", LAUNCHES)
+def test_second_device_launches_what_the_first_does(calls, what):
+    counts = []
+    for dev in (0, 1):
+        calls.lib.fake_reset()
+        calls.lib.fake_device(dev)
+        assert LAUNCHES[what](calls) == 0, calls.lib.thc_cpd_last_error()
+        counts.append({k: calls.lib.fake_launches(k) for k in (b"k_oz_update", b"k_oz_split", b"k_fix", b"k_tc_gemm",
+                                                               b"k_ldl_flow", b"")})
+    assert counts[0] == counts[1] and counts[0][b""] > 0
