@@ -200,6 +200,18 @@ struct Ctx {
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};
     int gprec[2] = {-1, -1};
     long glaunch[2] = {0, 0};
+    // The first failure among the launches of this call. A launcher that reports one has cleared
+    // CUDA's own record of it, so its value has to be kept.
+    cudaError_t err = cudaSuccess;
+    void note(cudaError_t e) {
+        if (err == cudaSuccess) err = e;
+    }
+    cudaError_t take_error() {
+        note(cudaGetLastError());
+        const cudaError_t e = err;
+        err = cudaSuccess;
+        return e;
+    }
 
     ~Ctx() {
         for (auto& g : gexec)
@@ -461,14 +473,14 @@ const OzMat& digits_XT(Ctx& c, int k) {  // rows of X_k^T
 
 void mul_digits(Ctx& c, const OzMat& A, const OzMat& B, double* C, int ldc, bool symm) {
     ProfScope prof(c.st, KC_OZ, (symm ? 1.0 : 2.0) * A.rows * (double)B.rows * A.K);
-    oz_mul(c.st, A, B, C, ldc, 1.0, symm ? OZ_SYMM : 0, c.oz.part, c.oz.part_cap);
+    c.note(oz_mul(c.st, A, B, C, ldc, 1.0, symm ? OZ_SYMM : 0, c.oz.part, c.oz.part_cap));
 }
 
 // An FP64-accuracy product of operands that are used once
 void gemm64(Ctx& c, bool trans_a, int M, int N, int K, const double* A, int lda, const double* B,
             const double* B2, int ldb, double* C, int ldc, bool symm) {
     if (c.ozp && oz_worth(M, N, K, symm) && M <= c.oz.rowsA && N <= c.oz.rowsB)
-        oz_dgemm(c.st, trans_a, M, N, K, A, lda, B, B2, ldb, C, ldc, symm, c.oz);
+        c.note(oz_dgemm(c.st, trans_a, M, N, K, A, lda, B, B2, ldb, C, ldc, symm, c.oz));
     else
         dgemm(c.st, trans_a, M, N, K, A, lda, B, B2, ldb, C, ldc, nullptr, symm, c.part, c.part_cap);
 }
@@ -571,16 +583,18 @@ void prepare_digits(Ctx& c) {
 }
 
 // W_k and G_k for every mode from the current factors (start of a run / after rollback)
-void refresh_state(Ctx& c, const double* const A[4]) {
+thc_cpd_status refresh_state(Ctx& c, const double* const A[4]) {
     prepare_digits(c);
     const bool fp64 = c.prec == THC_CPD_FP64;
     if (!fp64) mixed_split_factors(c.mx, c.st, A);
     SmallJobs small;
     for (int k = 0; k < 4; ++k) {
         factor_products(c, k, A[k], true, fp64, small);
-        if (!fp64) mixed_project(c.mx, c.st, k, false);
+        if (!fp64) c.note(mixed_project(c.mx, c.st, k, false));
     }
     dgemm_small_run(c.st, small);
+    CK(c.take_error());
+    return THC_CPD_OK;
 }
 
 // One mode update. M_k is formed in the Haug rows; returns with A[k], lam, G_k, W_k new.
@@ -600,9 +614,9 @@ thc_cpd_status mode_update(Ctx& c, double* const A[4], double* lam, int k, bool 
         CK(cudaMemcpyAsync(Mrows, c.Msave, sizeof(double) * n * R, cudaMemcpyDeviceToDevice, c.st));
         CK(cudaMemcpyAsync(c.Haug, c.Hsave, sizeof(double) * R * R, cudaMemcpyDeviceToDevice, c.st));
     }
-    chol_solve(c.st, R, n, c.Haug, A[k], c.LinvD, c.LinvD + (c.fixed ? 0 : (size_t)R * R), c.sc, k, c.counters,
-               c.dataflow ? c.flow_sync : nullptr, c.flow_ctas, c.bs_sync, c.fixed ? &c.fix : nullptr,
-               c.fixed || c.two_level ? &c.oz : nullptr, c.two_level);
+    c.note(chol_solve(c.st, R, n, c.Haug, A[k], c.LinvD, c.LinvD + (c.fixed ? 0 : (size_t)R * R), c.sc, k,
+                      c.counters, c.dataflow ? c.flow_sync : nullptr, c.flow_ctas, c.bs_sync,
+                      c.fixed ? &c.fix : nullptr, c.fixed || c.two_level ? &c.oz : nullptr, c.two_level));
     if (safe) {
         DevScalars* h = host_scalars();
         if (!h) return set_err(THC_CPD_ERR_ALLOC, "pinned host buffer allocation failed");
@@ -628,7 +642,7 @@ thc_cpd_status mode_update(Ctx& c, double* const A[4], double* lam, int k, bool 
         mixed_split_factors(c.mx, c.st, one);
         CK(mixed_project(c.mx, c.st, k, true));
     }
-    CK(cudaGetLastError());
+    CK(c.take_error());
     return THC_CPD_OK;
 }
 
@@ -657,7 +671,7 @@ thc_cpd_status sweep(Ctx& c, double* const A[4], double* lam, bool safe, bool ev
             loss_eval(c.st, c.s.Rt, c.s.R, c.Y, c.W[2], c.W[3], lam, c.G, c.red, c.sc, tol);
         }
     }
-    CK(cudaGetLastError());
+    CK(c.take_error());
     return THC_CPD_OK;
 }
 
@@ -699,7 +713,7 @@ thc_cpd_status fast_sweep(Ctx& c, double* const A[4], double* lam, bool eval, do
                 if (c.gexec[gi]) cudaGraphExecDestroy(c.gexec[gi]);
                 c.gexec[gi] = nullptr;
                 *use_graph = false;
-                cudaGetLastError();  // clear a capture error; run the sweep directly
+                c.take_error();  // clear a capture error; run the sweep directly
             }
         }
         if (*use_graph) {
@@ -733,6 +747,7 @@ thc_cpd_status obtain_norm(Ctx& c, double normG2, double* out) {
     }
     scalars_init(c.st, c.sc, 0.0);
     compute_normG2(c);
+    CK(c.take_error());
     DevScalars h;
     CKS(read_scalars(c, &h));
     *out = h.normG2;
@@ -830,6 +845,7 @@ thc_cpd_status trial_loss(Ctx& c, LearnWs& L, double* loss) {
     gemm64(c, true, Rt, R, Rt, c.Z, Rt, L.Wtr[0], L.Wtr[1], R, L.Ytr, R, false);
     CK(cudaMemcpyAsync(L.sc, c.sc, sizeof(DevScalars), cudaMemcpyDeviceToDevice, c.st));
     loss_eval(c.st, Rt, R, L.Ytr, L.Wtr[2], L.Wtr[3], L.lamT, L.Gtr, c.red, L.sc, 0.0);
+    CK(c.take_error());
     DevScalars* h = host_scalars();
     if (!h) return set_err(THC_CPD_ERR_ALLOC, "pinned host buffer allocation failed");
     CK(cudaMemcpyAsync(h, L.sc, sizeof(DevScalars), cudaMemcpyDeviceToHost, c.st));
@@ -895,7 +911,7 @@ thc_cpd_status run_als(int o, int v, int Rt, int R, const double* Xo, const doub
     CKS(ctx_init(c, s, Xo, Xv, Z, opts, NEED_ALS | (normG2 > 0.0 ? 0u : NEED_NORM)));
     double nG2 = 0.0;
     CKS(obtain_norm(c, normG2, &nG2));
-    refresh_state(c, A);
+    CKS(refresh_state(c, A));
     const bool learning = la && (la->mlp || la->nalpha > 0);
     LearnWs L;
     std::vector<double> loss_hist;
@@ -939,7 +955,7 @@ thc_cpd_status run_als(int o, int v, int Rt, int R, const double* Xo, const doub
         auto launch = [&](int sw) -> thc_cpd_status {
             if (hand_over_at(sw)) {
                 c.prec = THC_CPD_FP64;
-                refresh_state(c, A);
+                CKS(refresh_state(c, A));
                 flags |= 4;
             }
             bool eval = true;
@@ -976,7 +992,7 @@ thc_cpd_status run_als(int o, int v, int Rt, int R, const double* Xo, const doub
                 CK(cudaStreamSynchronize(c.st));
                 use_snapshot_slot(c, b);
                 CKS(restore_snapshot(c, A, lam));
-                refresh_state(c, A);
+                CKS(refresh_state(c, A));
                 CKS(ctx_safe_buffers(c));
                 CKS(sweep(c, A, lam, true, eval, tol, &used));
                 CKS(read_scalars(c, &h));
@@ -1023,7 +1039,7 @@ thc_cpd_status run_als(int o, int v, int Rt, int R, const double* Xo, const doub
             ((polish > 0 && sw > max_sweeps - polish) ||
              (tol > 0.0 && isfinite(fit1) && isfinite(fit2) && fabs(fit1 - fit2) < 10.0 * tol))) {
             c.prec = THC_CPD_FP64;
-            refresh_state(c, A);
+            CKS(refresh_state(c, A));
             flags |= 4;
         }
         bool eval = true;
@@ -1046,7 +1062,7 @@ thc_cpd_status run_als(int o, int v, int Rt, int R, const double* Xo, const doub
             // a Cholesky pivot failed somewhere in this sweep: roll back and replay the
             // sweep with a host check after every factorisation
             CKS(restore_snapshot(c, A, lam));
-            refresh_state(c, A);
+            CKS(refresh_state(c, A));
             CKS(ctx_safe_buffers(c));
             CKS(sweep(c, A, lam, true, eval, tol, &used));
             CKS(read_scalars(c, &h));
@@ -1218,7 +1234,7 @@ thc_cpd_status run_batched(int np, thc_cpd_problem* P, int max_sweeps, double to
         c.sc_snap = r.dsc + np + p;
         double nG2;
         CKS(obtain_norm(c, 0.0, &nG2));
-        refresh_state(c, P[p].A);
+        CKS(refresh_state(c, P[p].A));
     }
     for (int p = 0; p < np; ++p) CK(cudaStreamSynchronize(r.streams[p]));
     std::vector<int> active(np);
@@ -1295,7 +1311,7 @@ thc_cpd_status run_batched(int np, thc_cpd_problem* P, int max_sweeps, double to
                 CK(cudaMemcpyAsync(P[p].lam, c.lamsnap, sizeof(double) * c.s.R,
                                    cudaMemcpyDeviceToDevice, c.st));
                 CK(cudaMemcpyAsync(c.sc, c.sc_snap, sizeof(DevScalars), cudaMemcpyDeviceToDevice, c.st));
-                refresh_state(c, P[p].A);
+                CKS(refresh_state(c, P[p].A));
                 CKS(ctx_safe_buffers(c));
                 int used = 0;
                 CKS(sweep(c, P[p].A, P[p].lam, true, eval, tol, &used));
@@ -1412,7 +1428,7 @@ thc_cpd_status thc_cpd_mttkrp(int o, int v, int Rt, int R, const double* Xo, con
         if (mode == 1 || mode == 3) CK(mixed_partner(c.mx, c.st, mode));
         CK(mixed_backproject(c.mx, c.st, mode, M));
     }
-    CK(cudaGetLastError());
+    CK(c.take_error());
     CK(cudaStreamSynchronize(c.st));
     return product_errors(c);
 }
@@ -1478,6 +1494,7 @@ thc_cpd_status thc_cpd_loss(int o, int v, int Rt, int R, const double* Xo, const
     dgemm_small_run(c.st, small);
     zgemm_fp64(c, 1);
     loss_eval(c.st, Rt, R, c.Y, c.W[2], c.W[3], lam ? lam : c.ones, c.G, c.red, c.sc, 0.0);
+    CK(c.take_error());
     DevScalars h;
     CKS(read_scalars(c, &h));
     if (loss_host) *loss_host = h.loss;
@@ -1623,7 +1640,7 @@ int spd_solve(cudaStream_t st, int R, int n, const double* H, const double* M, d
         else
             CK(ldl_flow(st, R, n, Haug, P, dinv, sc, 0, fsync));
     }
-    backward_solve(st, R, n, Haug, A, bsync, ozl ? &oz : nullptr);
+    CK(backward_solve(st, R, n, Haug, A, bsync, ozl ? &oz : nullptr));
     CK(cudaGetLastError());
     DevScalars* h = host_scalars();
     if (!h) return set_err(THC_CPD_ERR_ALLOC, "pinned host buffer allocation failed");

@@ -247,6 +247,7 @@ extern "C" thc_cpd_status thc_cpd_df_als(int o, int v, int naux, int R, const do
         }
         const double* Gc[4] = {c.G[0], c.G[1], c.G[2], c.G[3]};
         loss_eval(st, naux, R, c.V12, c.V34, c.ones, lam, Gc, c.red, c.sc, tol > 0.0 ? tol : -1.0);
+        c.ck(cudaGetLastError());
         c.ck(cudaMemcpyAsync(&hs, c.sc, sizeof hs, cudaMemcpyDeviceToHost, st));
         c.ck(cudaStreamSynchronize(st));
         if (c.err != cudaSuccess) return derr(THC_CPD_ERR_CUDA, "DF sweep: %s", cudaGetErrorString(c.err));

@@ -194,6 +194,10 @@ extern "C" thc_cpd_status thc_cpd_exchange(int o, int v, int Rt, int R, int nalp
             if (tc_u[k & 1] || ((k & 1) ? (tc_n && k == 1) : tc_m)) oz_split_cols(st, A[k], nullptr, R, dA[k]);
         if (tc_z) oz_split_rows(st, Z, Rt, dZ);
     }
+    cudaError_t e = cudaSuccess;  // the first failure (a launcher that reports one has cleared CUDA's record of it)
+    auto ck = [&](cudaError_t x) {
+        if (e == cudaSuccess) e = x;
+    };
     auto scale = [&](int rows, int n, int gg, const double* s, const double* X, double* out) {
         const long total = (long)rows * n * gg;
         k_scale_rows<<<(int)std::min<long>(cdiv(total, 256), 4L * num_sms()), 256, 0, st>>>(rows, n, gg, s, X, out);
@@ -216,7 +220,7 @@ extern "C" thc_cpd_status thc_cpd_exchange(int o, int v, int Rt, int R, int nalp
                 if (tc_u[h]) oz_split_cols(st, XS, nullptr, gRt, d);
                 for (int k = h; k < 4; k += 2) {
                     if (tc_u[h])
-                        oz_mul(st, d, dA[k], U[k], R, 1.0, 0);
+                        ck(oz_mul(st, d, dA[k], U[k], R, 1.0, 0));
                     else
                         dgemm(st, true, gRt, R, n, XS, gRt, A[k], nullptr, R, U[k], R, nullptr, false, gpart, part_cap);
                 }
@@ -225,7 +229,7 @@ extern "C" thc_cpd_status thc_cpd_exchange(int o, int v, int Rt, int R, int nalp
                 OzMat d = dP;
                 d.rows = gR;
                 oz_split_cols_stack(st, U[2], U[1], R, R, gg, d);
-                oz_mul(st, dZ, d, Y, gR, 1.0, 0);
+                ck(oz_mul(st, dZ, d, Y, gR, 1.0, 0));
             } else {
                 for (int al = 0; al < gg; ++al)
                     dgemm(st, false, Rt, R, Rt, Z, Rt, U[2] + al * RtR, U[1] + al * RtR, R, Y + (size_t)al * R, gR,
@@ -242,7 +246,7 @@ extern "C" thc_cpd_status thc_cpd_exchange(int o, int v, int Rt, int R, int nalp
                     d.rows = gR;
                     d.K = n;
                     oz_split_cols(st, AS, nullptr, gR, d);
-                    oz_mul(st, dl, d, out, gR, 1.0, 0);
+                    ck(oz_mul(st, dl, d, out, gR, 1.0, 0));
                 } else {
                     dgemm(st, true, R, gR, n, Al, R, AS, nullptr, gR, out, gR, nullptr, false, gpart, part_cap);
                 }
@@ -256,8 +260,9 @@ extern "C" thc_cpd_status thc_cpd_exchange(int o, int v, int Rt, int R, int nalp
         }
     }
     std::vector<double> h(2 * (size_t)nalpha);
-    cudaError_t e = cudaMemcpyAsync(h.data(), res, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    ck(cudaGetLastError());
+    ck(cudaMemcpyAsync(h.data(), res, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, st));
+    ck(cudaStreamSynchronize(st));
     // freed after the synchronisation, which gives what the pool holds unused back to the device: the
     // next call finds the block in the pool (mapping 650 MB anew took 1.9 ms)
     cudaFreeAsync(block, st);

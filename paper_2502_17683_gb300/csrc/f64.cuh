@@ -57,14 +57,14 @@ void hadamard3(cudaStream_t st, int R, const double* Ga, const double* Gb, const
 //   oz: workspace of the split backward solve's products, or null.
 struct OzWs;
 struct FixWs;
-void chol_solve(cudaStream_t st, int R, int n, double* Haug, double* A, double* P, double* dinv,
+[[nodiscard]] cudaError_t chol_solve(cudaStream_t st, int R, int n, double* Haug, double* A, double* P, double* dinv,
                 DevScalars* sc, int mode, int* counters, int* flow_sync, int flow_ctas,
                 int* bs_sync, const FixWs* fix = nullptr, const OzWs* oz = nullptr, bool two_level = false);
 // The backward solve A L = Y of a factorised Haug (Y in its rows R..R+n): with a product
 // workspace (oz) and n >= 128, a block of >= 768 columns is split at a
 // column h0: the trailing block first, the coupling Y1 -= A2 L21 as an emulated product,
 // then the leading block, each of them split again by the same rule.
-void backward_solve(cudaStream_t st, int R, int n, double* Haug, double* A, int* bs_sync,
+[[nodiscard]] cudaError_t backward_solve(cudaStream_t st, int R, int n, double* Haug, double* A, int* bs_sync,
                     const OzWs* oz = nullptr);
 // Raises *rowsA / *rowsB (emulated-product workspace rows, oz_ws_carve) to what the split
 // backward solve of an R x R factor with up to nmax right-hand sides needs to form each
@@ -86,13 +86,13 @@ int spd_solve(cudaStream_t st, int R, int n, const double* H, const double* M, d
 // the launch; the error flag of bounded waits that gave up (read and cleared).
 size_t flow_sync_ints(int R, int nmax);
 bool flow_prepare(int R, int n);
-cudaError_t ldl_flow(cudaStream_t st, int R, int n, double* Haug, double* P, double* dinv,
+[[nodiscard]] cudaError_t ldl_flow(cudaStream_t st, int R, int n, double* Haug, double* P, double* dinv,
                      DevScalars* sc, int mode, int* sync, int max_ctas = 0);
 int flow_take_error();
 // The same launch with a caller-provided task list (host, 4 shorts per task as
 // thc_cpd_ldl_schedule writes them; dev_tasks: 8 * ntasks bytes of device memory). The list
 // is used as given: an incomplete or misordered one ends in bounded waits that give up.
-cudaError_t ldl_flow_tasks(cudaStream_t st, int R, int n, double* Haug, double* P, double* dinv,
+[[nodiscard]] cudaError_t ldl_flow_tasks(cudaStream_t st, int R, int n, double* Haug, double* P, double* dinv,
                            DevScalars* sc, int mode, int* sync, const short* host_tasks,
                            int ntasks, void* dev_tasks);
 // One panel of the two-level factorisation: columns [j0, j0 + bw) of the (R + n) x R matrix
@@ -100,7 +100,7 @@ cudaError_t ldl_flow_tasks(cudaStream_t st, int R, int n, double* Haug, double* 
 // row below the panel's diagonal block (their L, or Y for the M rows, in the panel columns).
 // The trailing update is the caller's. A plan for (bw, R + n - j0 - bw) must exist
 // (flow_prepare); the pivot threshold uses the whole order R.
-cudaError_t ldl_flow_panel(cudaStream_t st, int R, int n, int j0, int bw, double* Haug, double* P,
+[[nodiscard]] cudaError_t ldl_flow_panel(cudaStream_t st, int R, int n, int j0, int bw, double* Haug, double* P,
                            double* dinv, DevScalars* sc, int mode, int* sync, int max_ctas = 0);
 // Index of the first task whose type or tile indices are out of range, or -1.
 int flow_task_check(int R, int n, const short* tasks, int ntasks);
@@ -116,7 +116,7 @@ void copy_with_maxdiag(cudaStream_t st, int R, const double* H, double* H_out, D
 // ld: row pitch of Y, A and H (0: R), so that a diagonal block of a larger factor can be
 // solved on its own.
 size_t bsolve_sync_ints(int nmax);
-cudaError_t bsolve_slices(cudaStream_t st, int R, int n, const double* Yf, double* A,
+[[nodiscard]] cudaError_t bsolve_slices(cudaStream_t st, int R, int n, const double* Yf, double* A,
                           const double* H, int* sync, int ld = 0);
 
 // lam_r = ||A[:,r]||_2; A[:,r] /= lam_r (lam_r = 0 leaves the column); scratch >= R doubles.
@@ -124,7 +124,7 @@ void normalise_columns(cudaStream_t st, int n, int R, double* A, double* lam, do
 
 // dst[p][0 .. len[p]) = src[p][...] for p < np (np <= 8) in one launch (the state snapshot
 // taken before every sweep for a rollback).
-cudaError_t copy_many(cudaStream_t st, int np, const double* const* src, double* const* dst,
+[[nodiscard]] cudaError_t copy_many(cudaStream_t st, int np, const double* const* src, double* const* dst,
                       const long* len);
 
 // Loss in factor form after a sweep: inner = sum lam_r Y[Q,r] W3[Q,r] W4[Q,r],

@@ -752,19 +752,20 @@ int bsolve_split_point(int m, int n) {
     return (m / 2 / kOzPanel) * kOzPanel;
 }
 
-void chol_solve(cudaStream_t st, int R, int n, double* Haug, double* A, double* P, double* dinv,
+cudaError_t chol_solve(cudaStream_t st, int R, int n, double* Haug, double* A, double* P, double* dinv,
                 DevScalars* sc, int mode, int* counters, int* flow_sync, int flow_ctas,
                 int* bs_sync, const FixWs* fix, const OzWs* oz, bool two_level) {
     NvtxRange nvtx_range("thc_cpd LDL^T and solve");
     const int nrows = R + n;
     const int nJ = cdiv(R, NB);
+    cudaError_t e = cudaSuccess;
     if (fix) {
-        ldl_fix(st, R, n, Haug, dinv, sc, mode, *fix);
+        e = ldl_fix(st, R, n, Haug, dinv, sc, mode, *fix);
     } else if (two_level && oz && flow_sync) {
-        ldl_oz(st, R, n, Haug, P, dinv, sc, mode, flow_sync, *oz, flow_ctas);
+        e = ldl_oz(st, R, n, Haug, P, dinv, sc, mode, flow_sync, *oz, flow_ctas);
     } else if (flow_sync && flow_prepare(R, n)) {
         ProfScope prof(st, KC_CHOL, (double)R * R * R / 3.0 + (double)n * R * R);
-        ldl_flow(st, R, n, Haug, P, dinv, sc, mode, flow_sync, flow_ctas);
+        e = ldl_flow(st, R, n, Haug, P, dinv, sc, mode, flow_sync, flow_ctas);
     } else {
         ProfScope prof(st, KC_CHOL, (double)R * R * R / 3.0 + (double)n * R * R);
         k_ldl_diag<<<1, 128, 0, st>>>(Haug, dinv, R, std::min(NB, R), sc, mode, counters, nJ);
@@ -786,7 +787,8 @@ void chol_solve(cudaStream_t st, int R, int n, double* Haug, double* A, double* 
             }
         }
     }
-    backward_solve(st, R, n, Haug, A, bs_sync, oz);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    return e == cudaSuccess ? backward_solve(st, R, n, Haug, A, bs_sync, oz) : e;
 }
 
 namespace {
@@ -794,18 +796,18 @@ namespace {
 // applied to Y: the block as one solve, or split at h into its trailing and leading parts
 // with the coupling Y[:, c0 .. c0 + h) -= A[:, c0 + h .. c0 + m) L[c0 + h .. c0 + m, c0 .. c0 + h)
 // as an emulated product between them.
-void bsolve_block(cudaStream_t st, int R, int c0, int m, int n, double* Haug, double* A, int* bs_sync,
+cudaError_t bsolve_block(cudaStream_t st, int R, int c0, int m, int n, double* Haug, double* A, int* bs_sync,
                   const OzWs* oz) {
     double* Y = Haug + (size_t)R * R;
     const int h = oz ? bsolve_split_point(m, n) : 0;
     if (h == 0) {
         ProfScope prof(st, KC_BSOLVE, (double)n * m * m);
-        bsolve_slices(st, m, n, Y + c0, A + c0, Haug + (size_t)c0 * R + c0, bs_sync, R);
-        return;
+        return bsolve_slices(st, m, n, Y + c0, A + c0, Haug + (size_t)c0 * R + c0, bs_sync, R);
     }
-    bsolve_block(st, R, c0 + h, m - h, n, Haug, A, bs_sync, oz);
-    oz_gemm_sub(st, n, h, m - h, A + c0 + h, R, Haug + (size_t)(c0 + h) * R + c0, R, Y + c0, R, *oz);
-    bsolve_block(st, R, c0, h, n, Haug, A, bs_sync, oz);
+    cudaError_t e = bsolve_block(st, R, c0 + h, m - h, n, Haug, A, bs_sync, oz);
+    if (e == cudaSuccess)
+        e = oz_gemm_sub(st, n, h, m - h, A + c0 + h, R, Haug + (size_t)(c0 + h) * R + c0, R, Y + c0, R, *oz);
+    return e == cudaSuccess ? bsolve_block(st, R, c0, h, n, Haug, A, bs_sync, oz) : e;
 }
 }  // namespace
 
@@ -833,13 +835,13 @@ void bsolve_ws_rows(int R, int nmax, int* rowsA, int* rowsB, size_t* part_double
     *part_doubles = std::max<size_t>(*part_doubles, (size_t)part);
 }
 
-void backward_solve(cudaStream_t st, int R, int n, double* Haug, double* A, int* bs_sync, const OzWs* oz) {
+cudaError_t backward_solve(cudaStream_t st, int R, int n, double* Haug, double* A, int* bs_sync, const OzWs* oz) {
     NvtxRange nvtx_range("thc_cpd backward solve");
-    if (n <= 0) return;
+    if (n <= 0) return cudaSuccess;
     // A = [A1 A2], L = [L11 0; L21 L22]: A2 L22 = Y2, then A1 L11 = Y1 - A2 L21 with the
     // coupling term (half of the block's flops) as an emulated tensor-core product, each
     // half split again while it is large enough
-    bsolve_block(st, R, 0, R, n, Haug, A, bs_sync, oz);
+    return bsolve_block(st, R, 0, R, n, Haug, A, bs_sync, oz);
 }
 
 // ------------------------------------------------------------------------------------

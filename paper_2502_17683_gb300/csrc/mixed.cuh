@@ -35,18 +35,18 @@ size_t mixed_ws_bytes(bool tf32, int o, int v, int Rt, int R);
 void mixed_ws_carve(MixedWs& mx, Arena& ar, bool tf32, int o, int v, int Rt, int R);
 // Split the operands that stay for the call: Z and Z^T, Xo and Xv both ways; with mode >= 0 those
 // of that mode's MTTKRP alone and, with A, its three factors, all in one launch.
-cudaError_t mixed_setup(MixedWs& mx, cudaStream_t st, const double* Xo, const double* Xv,
+[[nodiscard]] cudaError_t mixed_setup(MixedWs& mx, cudaStream_t st, const double* Xo, const double* Xv,
                         const double* Z, const double* const A[4] = nullptr, int mode = -1);
 // Split the factors A[k] (null entries are passed over) for their projections.
 void mixed_split_factors(MixedWs& mx, cudaStream_t st, const double* const A[4]);
 // W_k = X_k^T A_k on tensor cores (from the split A_k) with the fused Hadamard epilogue; `in_sweep`
 // enables the E products that need the current Y.
-cudaError_t mixed_project(MixedWs& mx, cudaStream_t st, int k, bool in_sweep);
-cudaError_t mixed_zgemm(MixedWs& mx, cudaStream_t st, int half);
+[[nodiscard]] cudaError_t mixed_project(MixedWs& mx, cudaStream_t st, int k, bool in_sweep);
+[[nodiscard]] cudaError_t mixed_zgemm(MixedWs& mx, cudaStream_t st, int half);
 // E = split(W_partner o Y) for modes 1 and 3 outside a sweep
-cudaError_t mixed_partner(MixedWs& mx, cudaStream_t st, int mode);
+[[nodiscard]] cudaError_t mixed_partner(MixedWs& mx, cudaStream_t st, int mode);
 // M_k = X_k E (n_k x R, FP64)
-cudaError_t mixed_backproject(MixedWs& mx, cudaStream_t st, int k, double* M);
+[[nodiscard]] cudaError_t mixed_backproject(MixedWs& mx, cudaStream_t st, int k, double* M);
 int mixed_take_error();
 
 }  // namespace thc

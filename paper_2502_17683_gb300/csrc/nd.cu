@@ -317,6 +317,7 @@ extern "C" thc_cpd_status thc_cpd_nd_als(int d, int dL, const int* dims, int Rt,
         c.hprod((long)RR, {}, g, c.GH);
         const double* Gs[4] = {c.GH, c.ones, c.ones, c.ones};
         loss_eval(st, Rt, R, c.Y, c.P, c.ones, lam, Gs, c.red, c.sc, tol > 0.0 ? tol : -1.0);
+        c.ck(cudaGetLastError());
         c.ck(cudaMemcpyAsync(&hs, c.sc, sizeof hs, cudaMemcpyDeviceToHost, st));
         c.ck(cudaStreamSynchronize(st));
         if (c.err != cudaSuccess) return nerr(THC_CPD_ERR_CUDA, "order-d sweep: %s", cudaGetErrorString(c.err));

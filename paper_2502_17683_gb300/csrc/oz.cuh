@@ -75,7 +75,7 @@ void oz_product_ws(int M, int N, int K, int* rowsA, int* rowsB, size_t* part);
 // updated only for j <= i; symm (M == N): the lower triangle is computed and mirrored. part:
 // partial sums of a K split (used when it holds enough).
 enum { OZ_ACC = 1, OZ_LOWER = 2, OZ_SYMM = 4 };
-cudaError_t oz_mul(cudaStream_t st, const OzMat& A, const OzMat& B, double* C, int ldc, double sign,
+[[nodiscard]] cudaError_t oz_mul(cudaStream_t st, const OzMat& A, const OzMat& B, double* C, int ldc, double sign,
                    int flags, double* part = nullptr, size_t part_cap = 0);
 
 // Whether an M x N x K product (symm: only its lower triangle) is faster from digits than on the
@@ -100,7 +100,7 @@ bool oz_prepare(int R, int n);
 // kTailCols) as one dataflow factorisation of the trailing block. P: R x R (X = L D of the diagonal blocks), dinv:
 // R, sync: flow_sync_ints(R, n) ints (zero; left zero).
 // max_ctas > 0: the panels run on at most that many CTAs (problems side by side).
-cudaError_t ldl_oz(cudaStream_t st, int R, int n, double* Haug, double* P, double* dinv,
+[[nodiscard]] cudaError_t ldl_oz(cudaStream_t st, int R, int n, double* Haug, double* P, double* dinv,
                    DevScalars* sc, int mode, int* sync, const OzWs& ws, int max_ctas = 0);
 
 // LDL^T of Haug ((R + n) x R, ld R; H in the first R rows, lower triangle read, M in the rest),
@@ -117,12 +117,12 @@ size_t ldl_fix_ws_bytes(int R, int n);
 void ldl_fix_carve(FixWs& w, Arena& ar, int R, int n);
 // The kernels can run on the current device (call outside capture first).
 bool ldl_fix_prepare();
-cudaError_t ldl_fix(cudaStream_t st, int R, int n, double* Haug, double* dinv, DevScalars* sc, int mode,
+[[nodiscard]] cudaError_t ldl_fix(cudaStream_t st, int R, int n, double* Haug, double* dinv, DevScalars* sc, int mode,
                     const FixWs& ws);
 
 // C (M x N, ldc) += sign * A B^T for FP64 row-major A (M x K, lda) and B (N x K, ldb); lower:
 // rows i < N are updated only for j <= i. ws must hold M (rowsA) and N (rowsB) digit rows.
-cudaError_t oz_gemm(cudaStream_t st, int M, int N, int K, const double* A, int lda, const double* B,
+[[nodiscard]] cudaError_t oz_gemm(cudaStream_t st, int M, int N, int K, const double* A, int lda, const double* B,
                     int ldb, double* C, int ldc, double sign, bool lower, const OzWs& ws);
 
 // The FP64 GEMM of f64.cuh (dgemm) emulated on the tensor cores, same semantics:
@@ -130,13 +130,13 @@ cudaError_t oz_gemm(cudaStream_t st, int M, int N, int K, const double* A, int l
 //   op(A)[m][k] = trans_a ? A[k * lda + m] : A[m * lda + k]; B, B2 row-major (ldb);
 //   symm: C symmetric (M == N); the lower triangle is computed and mirrored.
 // ws must hold M (rowsA) and N (rowsB) digit rows.
-cudaError_t oz_dgemm(cudaStream_t st, bool trans_a, int M, int N, int K, const double* A, int lda,
+[[nodiscard]] cudaError_t oz_dgemm(cudaStream_t st, bool trans_a, int M, int N, int K, const double* A, int lda,
                      const double* B, const double* B2, int ldb, double* C, int ldc, bool symm,
                      const OzWs& ws);
 
 // C (M x N, ldc) -= A B for row-major FP64 A (M x K, lda) and B (K x N, ldb) (the coupling term
 // of a split backward solve). ws must hold M (rowsA) and N (rowsB) digit rows.
-cudaError_t oz_gemm_sub(cudaStream_t st, int M, int N, int K, const double* A, int lda, const double* B,
+[[nodiscard]] cudaError_t oz_gemm_sub(cudaStream_t st, int M, int N, int K, const double* A, int lda, const double* B,
                         int ldb, double* C, int ldc, const OzWs& ws);
 
 // Device error word of the emulated-product kernel (bounded waits that gave up); read and

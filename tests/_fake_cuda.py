@@ -29,6 +29,7 @@ def load(tmp):
     lib.fake_fail_launch.argtypes = [ctypes.c_char_p, ctypes.c_long]
     lib.fake_launches.argtypes, lib.fake_launches.restype = [ctypes.c_char_p], ctypes.c_long
     lib.fake_alloc_limit.argtypes = [ctypes.c_size_t]
+    lib.fake_launched.restype = ctypes.c_char_p
     lib.fake_largest_alloc.restype = ctypes.c_size_t
     return lib
 
@@ -55,6 +56,13 @@ class Calls:
         o = Opts()
         o.precision, o.ldl = precision, ldl
         return ctypes.byref(o)
+
+    def launched(self):
+        names, i = [], 0
+        while (n := self.lib.fake_launched(i)) is not None:
+            names.append(n)
+            i += 1
+        return names
 
     def mttkrp(self, o, v, Rt, R, mode=0, **kw):
         return self.lib.thc_cpd_mttkrp(*self._problem(o, v, Rt, R), mode, self._p(max(o, v), R), self._opts(**kw))
@@ -112,6 +120,15 @@ class Calls:
         A = (ctypes.c_void_p * d)(*[self._p(n, R) for n in dims])
         return self.lib.thc_cpd_nd_mttkrp(d, dL, (ctypes.c_int * d)(*dims), Rt, R, X, self._p(Rt, Rt), A, mode,
                                           self._p(dims[mode], R), self._opts(**kw))
+
+    def nd_als(self, dims, dL, Rt, R, sweeps=1, **kw):
+        self.keep = []
+        d = len(dims)
+        X = (ctypes.c_void_p * d)(*[self._p(n, Rt) for n in dims])
+        A = (ctypes.c_void_p * d)(*[self._p(n, R) for n in dims])
+        return self.lib.thc_cpd_nd_als(d, dL, (ctypes.c_int * d)(*dims), Rt, R, X, self._p(Rt, Rt), A, self._p(R),
+                                       sweeps, 0.0, ctypes.byref(ctypes.c_int()), ctypes.byref(ctypes.c_double()),
+                                       self._opts(**kw))
 
     def solve(self, R, n, **kw):
         self.keep = []

@@ -58,7 +58,7 @@ void fake_reset() {
     s().dev = 0;
 }
 void fake_device(int d) { s().dev = d; }
-void fake_fail_launch(const char* name, long after) {  // the launch after `after` good ones of such a kernel fails
+void fake_fail_launch(const char* name, long after) {  // launches of such kernels fail after `after` good ones
     s().fail_name = name;
     s().fail_after = after;
 }
@@ -70,6 +70,12 @@ long fake_launches(const char* name) {
     for (auto& k : s().launches)
         if (k.first.find(name) != std::string::npos) n += k.second;
     return n;
+}
+
+const char* fake_launched(int i) {  // name of the i-th kernel launched so far, null past the last
+    for (auto& k : s().launches)
+        if (i-- == 0) return k.first.c_str();
+    return nullptr;
 }
 
 // ---- registration and launches ----
@@ -112,7 +118,7 @@ cudaError_t __cudaLaunchKernel(Kernel k, dim3 g, dim3 b, void**, size_t dyn, cud
         return note(cudaErrorInvalidConfiguration);
     auto it = s().smem.find({s().dev, k});
     if (dyn > 48 * 1024 && (it == s().smem.end() || dyn > (size_t)it->second)) return note(cudaErrorInvalidValue);
-    if (!s().fail_name.empty() && n.find(s().fail_name) != std::string::npos && s().fail_after-- == 0)
+    if (!s().fail_name.empty() && n.find(s().fail_name) != std::string::npos && s().fail_after-- <= 0)
         return note(cudaErrorLaunchOutOfResources);
     ++s().launches[n];
     return cudaSuccess;

@@ -31,6 +31,10 @@ LAUNCHES = {
     "batched": lambda c: c.batched([(12, 60, 200, 420), (3, 9, 30, 40)]),
     "exchange": lambda c: c.exchange(10, 50, 200, 300, 4),
     "core fit": lambda c: c.core_fit(10, 50, 200, 220, loss=True),
+    "DF": lambda c: c.df_als(10, 50, 200, 220),
+    "order 4": lambda c: c.nd_als((5, 15, 7, 9), 2, 40, 60),
+    "order 3": lambda c: c.nd_mttkrp((10, 50, 30), 1, 200, 300),
+    "solve": lambda c: c.solve(1100, 140),
 }
 
 
@@ -45,3 +49,24 @@ def test_second_device_launches_what_the_first_does(calls, what):
         counts.append({k: calls.lib.fake_launches(k) for k in (b"k_oz_update", b"k_oz_split", b"k_fix", b"k_tc_gemm",
                                                                b"k_ldl_flow", b"")})
     assert counts[0] == counts[1] and counts[0][b""] > 0
+
+
+# every kernel of a call, its first launch and its last: the call has to report the failure
+@pytest.mark.parametrize("what", LAUNCHES)
+def test_failed_launch_is_reported(calls, what):
+    from paper_2502_17683_gb300._lib import ERR_CUDA
+    assert LAUNCHES[what](calls) == 0, calls.lib.thc_cpd_last_error()
+    kernels = {n: calls.lib.fake_launches(n) for n in calls.launched()}
+    for name, n in kernels.items():
+        for after in {0, n - 1}:
+            calls.lib.fake_reset()
+            calls.lib.fake_fail_launch(name, after)
+            assert LAUNCHES[what](calls) == ERR_CUDA, (name, after)
+
+
+# (the solve of this size and the small order-4 run use no tensor map)
+@pytest.mark.parametrize("what", [w for w in LAUNCHES if w not in ("solve", "order 4")])
+def test_failed_tensor_map_is_reported(calls, what):
+    from paper_2502_17683_gb300._lib import ERR_CUDA
+    calls.lib.fake_fail_encode(1)
+    assert LAUNCHES[what](calls) == ERR_CUDA
