@@ -347,7 +347,8 @@ thc_cpd_status ctx_init(Ctx& c, const Shape& s, const double* Xo, const double* 
         }
         if (norm) oz_product_ws(Rt, Rt, Rt, &oz_ra, &oz_rb, &oz_part);
         bytes += 2 * ozmat_bytes(Rt, Rt) + ozmat_bytes(R, Rt) + ozmat_bytes(R, nmax);
-        for (int k = 0; k < 2; ++k) bytes += ozmat_bytes(s.n[k], Rt) + ozmat_bytes(Rt, s.n[k]);
+        for (int k = 0; k < 2; ++k)
+            bytes += ozmat_bytes(s.n[k], Rt) + (s.n[k] <= kOzMaxK ? ozmat_bytes(Rt, s.n[k]) : 0);
     }
     if (ozl || ozp) bytes += oz_ws_bytes(oz_ra, oz_rb, oz_part);
     CK(cudaMallocAsync(&c.block, bytes, c.st));
@@ -399,7 +400,7 @@ thc_cpd_status ctx_init(Ctx& c, const Shape& s, const double* Xo, const double* 
         for (int h = 0; h < 2; ++h) ozmat_carve(c.dZ[h], ar, Rt, Rt);
         for (int k = 0; k < 2; ++k) {
             ozmat_carve(c.dX[k], ar, s.n[k], Rt);
-            ozmat_carve(c.dXT[k], ar, Rt, s.n[k]);
+            if (s.n[k] <= kOzMaxK) ozmat_carve(c.dXT[k], ar, Rt, s.n[k]);
         }
         ozmat_carve(c.dP, ar, R, Rt);
         ozmat_carve(c.dA, ar, R, nmax);
@@ -489,8 +490,14 @@ void compute_normG2(Ctx& c) {
     const int o = c.s.o, v = c.s.v, Rt = c.s.Rt;
     // S = (Xo^T Xo) o (Xv^T Xv); U = S Z S; ||G||^2 = sum Z o U
     if (c.ozp && oz_worth(Rt, Rt, Rt, false)) {
-        mul_digits(c, digits_XT(c, 0), digits_XT(c, 0), c.T, Rt, true);
-        mul_digits(c, digits_XT(c, 1), digits_XT(c, 1), c.S, Rt, true);
+        for (int k = 0; k < 2; ++k) {
+            double* const G = k == 0 ? c.T : c.S;
+            if (c.s.n[k] <= kOzMaxK)  // longer Grams than one digit launch sums stay on the FP64 pipes
+                mul_digits(c, digits_XT(c, k), digits_XT(c, k), G, Rt, true);
+            else
+                dgemm(c.st, true, Rt, Rt, c.s.n[k], c.X[k], Rt, c.X[k], nullptr, Rt, G, Rt, nullptr, true, c.part,
+                      c.part_cap);
+        }
         // S is symmetric: its columns, cut from the two Grams, serve as left and right operand
         OzMat s, t;
         s.d = c.oz.sB;

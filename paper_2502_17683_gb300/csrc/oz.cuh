@@ -31,6 +31,7 @@ namespace thc {
 constexpr int kOzSlices = 8;    // S: integer digits per value
 constexpr int kOzPanel = 128;   // K of one digit chunk (and the panel unit of the LDL^T)
 constexpr int kOzMaxChunks = 64;  // chunks one launch may sum (its 64-bit sums stay in range)
+constexpr int kOzMaxK = kOzMaxChunks * kOzPanel;
 
 // The digits of a matrix of `rows` rows and K columns: [chunk][S][rows][kOzPanel] BF16 and one
 // exponent per row. A view: the memory belongs to an OzWs or to the caller.

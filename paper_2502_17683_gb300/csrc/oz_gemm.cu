@@ -767,7 +767,7 @@ bool oz_available() { return oz_init(); }
 bool oz_worth_flops(double flops) { return flops >= kWorthFlops; }
 
 bool oz_worth(int M, int N, int K, bool symm) {
-    return oz_worth_flops((symm ? 1.0 : 2.0) * M * (double)N * K) && M <= 8192 && N <= 8192 && K <= kOzMaxChunks * KP;
+    return oz_worth_flops((symm ? 1.0 : 2.0) * M * (double)N * K) && M <= 8192 && N <= 8192 && K <= kOzMaxK;
 }
 
 void oz_ws_carve(OzWs& w, Arena& ar, int rowsA, int rowsB, size_t part_doubles) {

@@ -70,3 +70,11 @@ def test_failed_tensor_map_is_reported(calls, what):
     from paper_2502_17683_gb300._lib import ERR_CUDA
     calls.lib.fake_fail_encode(1)
     assert LAUNCHES[what](calls) == ERR_CUDA
+
+
+# a Gram of more terms than one digit launch sums (8192) beside products that run from digits
+@pytest.mark.parametrize("o,v", [(5, 8192), (5, 8193), (8193, 5)])
+def test_long_factors_run(calls, o, v):
+    assert calls.norm2(o, v, 220) == 0, calls.lib.thc_cpd_last_error()
+    assert calls.loss(o, v, 220, 40, normG2=0.0) == 0, calls.lib.thc_cpd_last_error()
+    assert calls.lib.fake_launches(b"k_oz_update") > 0
