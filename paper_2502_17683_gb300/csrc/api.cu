@@ -1584,12 +1584,13 @@ extern "C" thc_cpd_status thc_cpd_emulated_gemm(int M, int N, int K, const doubl
 namespace thc {
 
 int spd_solve(cudaStream_t st, int R, int n, const double* H, const double* M, double* A,
-              const short* tasks, int ntasks, int* used_pinv, int ldl) {
+              const short* tasks, int ntasks, int* used_pinv, int ldl, bool fixed) {
     if (used_pinv) *used_pinv = 0;
-    Ldl route = tasks || ldl == THC_CPD_LDL_BLOCKED ? Ldl::kDataflow : ldl_route(ldl, R, n, false);
-    if (route == Ldl::kBlocked) route = Ldl::kDataflow;  // (a solve alone has no blocked variant)
-    if (route == Ldl::kTwoLevel && !oz_prepare(R, n)) route = Ldl::kDataflow;
-    const bool fixed = route == Ldl::kFixed, two = route == Ldl::kTwoLevel, ozl = fixed || two;
+    // (a solve alone has no blocked variant: the dataflow kernel stands in for it)
+    const bool two = !fixed && !tasks && ldl_route(ldl, R, n, false) == Ldl::kTwoLevel && oz_prepare(R, n);
+    const bool ozl = fixed || two;
+    if (fixed && !ldl_fix_prepare())
+        return set_err(THC_CPD_ERR_UNSUPPORTED, "fixed-point blocks need an sm_103 device");
     if (!ozl && !flow_prepare(R, n))
         return set_err(THC_CPD_ERR_UNSUPPORTED, "no dataflow schedule for R=%d n=%d", R, n);
     const size_t RR = (size_t)R * R, nR = (size_t)n * R;
@@ -1683,6 +1684,13 @@ thc_cpd_status thc_cpd_ldl_solve(int R, int n, const double* H, const double* M,
     set_wait_limit(opts);
     return (thc_cpd_status)spd_solve(stream_of(opts), R, n, H, M, A, tasks, ntasks, used_pinv,
                                      opts ? opts->ldl : THC_CPD_LDL_AUTO);
+}
+
+// thc_cpd_ldl_solve in fixed-point blocks, the factorisation that the batched driver chooses: the
+// blocks alone, for the tests (not part of the interface).
+extern "C" thc_cpd_status thc_cpd_fixed_solve(int R, int n, const double* H, const double* M, double* A,
+                                              int* used_pinv, const thc_cpd_opts* opts) {
+    return (thc_cpd_status)spd_solve(stream_of(opts), R, n, H, M, A, nullptr, 0, used_pinv, THC_CPD_LDL_AUTO, true);
 }
 
 thc_cpd_status thc_cpd_als_batched(int nprob, thc_cpd_problem* probs, int max_sweeps,

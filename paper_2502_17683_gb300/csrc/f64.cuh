@@ -76,10 +76,11 @@ void bsolve_ws_rows(int R, int nmax, int* rowsA, int* rowsB, size_t* part_double
 // all device pointers, 1 <= R <= 2048, 1 <= n <= 4096: the solve of thc_cpd_ldl_solve (LDL^T
 // with the forward solve fused, dataflow or emulated two-level by `ldl` (thc_cpd_ldl values),
 // backward solve, pseudo-inverse when a pivot fails: *used_pinv = 1). tasks: null or a
-// caller-built dataflow task list (ntasks entries). Allocates its workspace on st and
+// caller-built dataflow task list (ntasks entries). fixed: factorise in fixed-point blocks
+// (ldl_fix.cu), as the batched driver does. Allocates its workspace on st and
 // synchronises st. Returns a thc_cpd_status; the message is set on failure.
 int spd_solve(cudaStream_t st, int R, int n, const double* H, const double* M, double* A,
-              const short* tasks, int ntasks, int* used_pinv, int ldl);
+              const short* tasks, int ntasks, int* used_pinv, int ldl, bool fixed = false);
 
 // Dataflow LDL^T (ldl_flow.cu): ints of progress state for R and n <= nmax; plan set-up
 // for (R, n) (false: too large or the task order failed its check; use the blocked path);

@@ -20,7 +20,7 @@
 // FP64 operation on numbers of the same size (backward errors measured equal to the dataflow
 // kernel's, 2e-16 .. 9e-16 for R = 80 .. 1800). A value that leaves its range proves that the matrix
 // is not positive definite (rows of H) and sets the failed-pivot bit; an appended row (M) is then
-// done again with a larger exponent.
+// done again with a larger exponent, and sets the bit once no larger one is left.
 //
 // With A = S A' S (S the diagonal of 2^e), A' = C C^T, the rows' digits are those of C; the result
 // is left in the layout of the other factorisations:
@@ -447,7 +447,9 @@ k_fix_diag(double* __restrict__ H, int ld, int nb, int R_tau, double* __restrict
 // An appended row has no bound like the diagonal of H: its exponent leaves kHeadroom bits over the
 // row's largest entry for the growth of the substitution; a value that passes 2^-3 (up to there no
 // sum of 128 terms wraps) sends the row through once more with four bits more, so the row's
-// largest value keeps at least 55 of its bits.
+// largest value keeps at least 55 of its bits. A row that has grown past 2^50 times its largest entry
+// after the last try sets the failed-pivot bit like a row of H that leaves its range: what it holds
+// has wrapped.
 constexpr int kHeadroom = 5;
 constexpr int kRowLimit = 59;
 constexpr int kRetryBits = 4;
@@ -545,7 +547,7 @@ k_fix_rows(double* __restrict__ H, int ld, int nb, int nH, int nrows, DevScalars
         }
         const unsigned vote = __ballot_sync(0xffffffffu, out && live);
         const bool row_out = (vote >> (lane & 16)) & 0xFFFFu;
-        if (row_out && hrow && l16 == 0) atomicOr(&sc->fail_mask, 1 << mode);
+        if (row_out && (hrow || tries == kMaxTries) && l16 == 0) atomicOr(&sc->fail_mask, 1 << mode);
         const bool again = row_out && !hrow;
         if (!__any_sync(0xffffffffu, again) || tries == kMaxTries) break;
         if (again) er += kRetryBits;
