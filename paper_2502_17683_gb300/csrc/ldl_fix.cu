@@ -63,6 +63,7 @@ struct DiagSmem {
     int2 ll[2][TB][NB];
     int2 xs[TB][TB];         // the diagonal tile's x' as they are finished, [column][row], 31-bit halves
     long long inv[NB], dq[NB];
+    long long dg[NB];        // what is left of each row's diagonal entry (Q61, to about 2^-22), plus kDiagSlack
     int k[NB], e[NB];
     int bad;
     volatile int done;       // columns finished by the chain warp
@@ -209,6 +210,16 @@ __device__ __forceinline__ int diag_exp(double a, bool& bad) {
 // With x_rc the entry of column c below its pivot d_c once it is final, x' = x 2^k and l = x' / d'
 // (|x'| < 1, |l| <= 2): L(r, c) = l 2^k, and the entry (r, s) loses x_rc x_sc / d_c = l_r x'_s.
 
+//
+// Range. x' and l are checked entry by entry, but the sums that they go into are held modulo 4: an
+// entry that loses more than that comes back into range and would pass. Of a positive definite
+// matrix no diagonal entry gets below zero, and while none does every sum stays below 1 (an
+// off-diagonal one by Cauchy-Schwarz). So the lane of a row also follows the row's diagonal entry,
+// column by column (each takes less than 2 from it, which cannot wrap) and from the upper halves alone
+// (one multiply-add; full products cost the batch 1.5 %): the sum of 128 such products is within
+// 2^-22, and below -2^-20 the block is not positive definite.
+constexpr long long kDiagSlack = 1LL << (61 - 20);
+
 // The chain: warp 0 factorises diagonal tile p in registers, lane (row, column parity) = (lane
 // & 15, lane >> 4) holding eight columns, with shuffles only (no barrier, no shared memory on
 // the chain), and publishes each finished column for the row warps. The pivots run one column
@@ -224,6 +235,8 @@ __device__ void chain_tile(DiagSmem& S, int p, int& bad) {
     long long x = shfl64(a[0], rr);         // its entry in this lane's row
     long long xn = shfl64(a[0], 1);         // x(c + 1, c) and a(c + 1, c + 1)
     long long an = shfl64(a[0], 17);
+    long long dg = S.dg[p * TB + rr];  // this row's diagonal entry (see the note on range above)
+    int drawn = 0;                     // negative once it has been overdrawn
     // a pivot <= 0 (not positive definite) is reported at the end, any value goes on; selections
     // instead of branches keep a column one block of code whose parts the scheduler interleaves
     bool neg = d <= 0;
@@ -248,6 +261,9 @@ __device__ void chain_tile(DiagSmem& S, int p, int& bad) {
         const long long l = mul61(xp, split31(inv));
         neg = neg || (rr > c && (beyond(x, 62 - r.k) || beyond(l, 62)));
         const int2 nl = split31(-l);
+        const long long dn = madw(nl.x, xp.x, dg);
+        dg = rr > c ? dn : dg;
+        drawn |= (int)(dg >> 32);
 #pragma unroll
         for (int i = i0; i < 8; ++i) {
             if (2 * i + 1 <= c) continue;
@@ -275,7 +291,7 @@ __device__ void chain_tile(DiagSmem& S, int p, int& bad) {
         d = d1;
         r = r1;
     }
-    if (neg) bad = 1;
+    if (neg || drawn < 0) bad = 1;
 }
 
 // Rows below diagonal tile p: a lane per row follows the chain column by column (one column
@@ -289,6 +305,8 @@ __device__ void follow_rows(DiagSmem& S, BlockTab* tab, int p, int r, int& bad) 
 #pragma unroll
     for (int s = 0; s < TB; ++s) a[s] = live ? T[s] : 0;
     int2* ct = &tab->ct[t * (t - 1) / 2 + p][0][ri];
+    long long dg = live ? S.dg[r] : 0;
+    int drawn = 0;
 #pragma unroll
     for (int c = 0; c < TB; ++c) {
         // the chain warp never waits for this one, so the wait ends; bounded all the same
@@ -300,9 +318,12 @@ __device__ void follow_rows(DiagSmem& S, BlockTab* tab, int p, int r, int& bad) 
         __threadfence_block();
         const int k = S.k[p * TB + c];
         const long long x = a[c], xk = x << k;
-        const long long l = mul61(split31(xk), split31(S.inv[p * TB + c]));
-        bad |= (beyond(x, 62 - k) || beyond(l, 62)) ? 1 : 0;
+        const int2 xp = split31(xk);
+        const long long l = mul61(xp, split31(S.inv[p * TB + c]));
         const int2 nl = split31(-l);
+        dg = madw(nl.x, xp.x, dg);
+        drawn |= (int)(dg >> 32);
+        bad |= (beyond(x, 62 - k) || beyond(l, 62)) ? 1 : 0;
 #pragma unroll
         for (int s = c + 1; s < TB; ++s) a[s] += mul61(nl, S.xs[c][s]);
         if (live) {
@@ -313,6 +334,8 @@ __device__ void follow_rows(DiagSmem& S, BlockTab* tab, int p, int r, int& bad) 
             T[c] = l;
         }
     }
+    if (live) S.dg[r] = dg;
+    if (drawn < 0) bad = 1;
 }
 
 // Eight rows (half hf) of tile (tr, tc) -= l(tr, p) x'(tc, p)^T: four entries per lane, exact
@@ -381,6 +404,7 @@ k_fix_diag(double* __restrict__ H, int ld, int nb, int R_tau, double* __restrict
                 v = fixed62(h[u], er);
             }
             S.T[t][((tid >> 4) & 15) * TP + (tid & 15)] = v;
+            if (r == c) S.dg[r] = (v >> 1) + kDiagSlack;
         }
     }
     int bad = bad0 ? 1 : 0;

@@ -111,3 +111,14 @@ def test_rows_that_outgrow_every_headroom(solve, R, fits):
     assert used == (not fits)
     if fits:
         assert _backward_ok(A, H, M)
+
+
+# entries below the bound of their block (they pass the first check) that overdraw a diagonal entry far
+# enough to wrap its 64 bits back to a positive value, inside one 16-column tile and across tiles
+@pytest.mark.parametrize("R,row,cols", [(32, 5, (0, 4)), (32, 20, (0, 4)), (128, 100, (0, 4)), (128, 127, (40, 44)),
+                                        (128, 127, (13, 19)), (200, 190, (130, 134))])
+def test_overdrawn_diagonal_is_noticed(solve, R, row, cols):
+    H = 0.25 * np.eye(R)
+    H[row, cols[0]:cols[1]] = H[cols[0]:cols[1], row] = 0.475
+    A, used = solve(H, np.random.default_rng(R).standard_normal((3, R)))
+    assert used
