@@ -508,6 +508,7 @@ void compute_normG2(Ctx& c) {
         oz_split_cols(c.st, c.T, c.S, Rt, s);
         mul_digits(c, s, digits_Z(c, 1), c.U, Rt, false);  // S Z
         oz_split_rows(c.st, c.U, Rt, t);
+        s.src = OzSrc();  // (the result takes the place of a factor of S)
         mul_digits(c, t, s, c.T, Rt, false);                // (S Z) S
         sum_hadamard_normG2(c.st, (long)Rt * Rt, c.Z, c.T, c.red, c.sc);
         return;
@@ -1573,8 +1574,7 @@ extern "C" thc_cpd_status thc_cpd_emulated_gemm(int M, int N, int K, const doubl
     ar.cap = bytes;
     OzWs oz;
     oz_ws_carve(oz, ar, rowsA, rowsB);
-    CK(cudaMemset2DAsync(C, sizeof(double) * ldc, 0, sizeof(double) * N, M, st));
-    CK(oz_gemm(st, M, N, K, A, lda, B, ldb, C, ldc, 1.0, false, oz));
+    CK(oz_gemm(st, M, N, K, A, lda, B, ldb, C, ldc, oz));
     CK(cudaStreamSynchronize(st));
     if (int e = oz_take_error())
         return set_err(THC_CPD_ERR_TIMEOUT, "emulated-product kernel wait gave up (code %d)", e);

@@ -17,7 +17,8 @@
 // FP64. The error is thus 2^-53 of |result| plus about 2^-62 of (row max)(column max)
 // sqrt(K): below that of an FP64 GEMM, which rounds at every term, at the library's operands
 // (a 1200-long product of weighted THC factors: 5e-17 of the result's norm, an FP64 FMA chain
-// 1.1e-15, seven slices 5e-15). Rows that hold a NaN or an infinity give NaN.
+// 1.1e-15, seven slices 5e-15). An element whose row or column holds an infinity or a NaN is summed in
+// FP64 from the operands themselves (OzSrc), as an FP64 GEMM does.
 // 36 BF16 MMAs per 16 of K take the place of the FP64 FMAs (GB300: 2 FP64 FMA per clock per
 // SM against ~3500 BF16 MAC).
 #pragma once
@@ -33,6 +34,15 @@ constexpr int kOzPanel = 128;   // K of one digit chunk (and the panel unit of t
 constexpr int kOzMaxChunks = 64;  // chunks one launch may sum (its 64-bit sums stay in range)
 constexpr int kOzMaxK = kOzMaxChunks * kOzPanel;
 
+// Where the digits of a matrix were cut from: entry (r, k) is s1[r ld + k], or with cols = n > 0
+// column r % n of matrix r / n of a stack, s1[((r / n) K + k) ld + r % n]; times s2's entry if given. The
+// sources have to be unchanged still when the product runs, and no part of its result.
+struct OzSrc {
+    const double *s1 = nullptr, *s2 = nullptr;
+    int ld = 0, cols = 0;
+    int k0 = 0;  // entries of a row that lie before these (earlier K of the same product), at k = -k0 .. -1
+};
+
 // The digits of a matrix of `rows` rows and K columns: [chunk][S][rows][kOzPanel] BF16 and one
 // exponent per row. A view: the memory belongs to an OzWs or to the caller.
 struct OzMat {
@@ -40,6 +50,7 @@ struct OzMat {
     int* e = nullptr;
     int rows = 0, K = 0;
     int ld_rows = 0;  // rows of the buffer (0: rows); a view of its first rows
+    OzSrc src;        // set by the cuts; none: such rows give NaN
     int chunks() const { return K > 0 ? cdiv(K, kOzPanel) : 0; }
 };
 size_t ozmat_bytes(int rows, int K);
@@ -121,10 +132,10 @@ bool ldl_fix_prepare();
 [[nodiscard]] cudaError_t ldl_fix(cudaStream_t st, int R, int n, double* Haug, double* dinv, DevScalars* sc, int mode,
                     const FixWs& ws);
 
-// C (M x N, ldc) += sign * A B^T for FP64 row-major A (M x K, lda) and B (N x K, ldb); lower:
-// rows i < N are updated only for j <= i. ws must hold M (rowsA) and N (rowsB) digit rows.
+// C (M x N, ldc) = A B^T for FP64 row-major A (M x K, lda) and B (N x K, ldb). ws must hold M (rowsA)
+// and N (rowsB) digit rows.
 [[nodiscard]] cudaError_t oz_gemm(cudaStream_t st, int M, int N, int K, const double* A, int lda, const double* B,
-                    int ldb, double* C, int ldc, double sign, bool lower, const OzWs& ws);
+                    int ldb, double* C, int ldc, const OzWs& ws);
 
 // The FP64 GEMM of f64.cuh (dgemm) emulated on the tensor cores, same semantics:
 //   C[M x N] = op(A)[M x K] (B o B2)[K x N];

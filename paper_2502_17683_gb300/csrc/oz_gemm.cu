@@ -23,7 +23,7 @@ constexpr int A_TILE = BM * 128;             // bytes of one 128 x 64 BF16 slice
 constexpr int B_STAGES = 2;                  // right operand: all S slices of one K half per stage
 constexpr int TMEM_COLS = 512;
 constexpr int EPI_WARPS = 16;                // four per TMEM lane quarter, BN / 4 columns each
-constexpr int NTHREADS = 64 + 32 * EPI_WARPS;  // warp 0 TMA, warp 1 MMA + TMEM, then the epilogue
+constexpr int NTHREADS = 64 + 32 * EPI_WARPS + 32;  // warp 0 TMA, warp 1 MMA + TMEM, the epilogue, a look-out
 constexpr int STG_BYTES = EPI_WARPS * 1024;  // per epilogue warp: 32 rows x 4 columns of FP64
 constexpr uint32_t WAIT_LIMIT = 1u << 22;
 
@@ -304,7 +304,14 @@ struct UpdArgs {
     int kgroups;      // split K: work item (group g, tile) takes chunks [g cpg, (g + 1) cpg); group 0
     int cpg;          // adds into C, group g > 0 writes its sum to part + (g - 1) mA mB (ld mB)
     double* part;     // (kgroups > 1 only without lower)
+    OzSrc srcA, srcB; // where the digits come from
+    int K;
 };
+
+__device__ __forceinline__ double src_entry(const OzSrc& s, int r, long k, int K) {
+    const long i = s.cols ? ((long)(r / s.cols) * K + k) * s.ld + r % s.cols : (long)r * s.ld + k;
+    return s.s2 ? s.s1[i] * s.s2[i] : s.s1[i];
+}
 
 // Active tiles of row block tm: on a lower-only (symmetric or LDL^T trailing) block, rows
 // that lie within the first mB stop at the diagonal; below them every tile is active.
@@ -337,6 +344,40 @@ __device__ __forceinline__ void tile_of(const UpdArgs& a, int u, int& m0, int& n
     n0 = (u % a.tiles_n) * BN;
 }
 
+// Between the epilogue's warps and the one that looks out for rows without digits.
+__device__ __forceinline__ void epi_barrier() {
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * EPI_WARPS + 32) : "memory");
+}
+
+// The elements of this CTA's tiles that have no digits (an infinity or a NaN in their row or column),
+// formed in FP64 from the operands by the look-out's lanes, over what the epilogue stored. A warp, a
+// branch and a call of its own: the epilogue's loop has no register to spare. Exchange energies at
+// (20,100,480,720), 12 points, no such element in them: 897 us without this, 904 with it, 920 with the
+// loops inlined, 925 with the elements looked for in the epilogue.
+template <int BN>
+__device__ __noinline__ void fill_undigited(const UpdArgs& args, int lane) {
+    for (int w = blockIdx.x; w < args.nactive * args.kgroups; w += gridDim.x) {
+        const int t = w % args.nactive, grp = w / args.nactive;
+        const long k0 = grp == 0 ? -(long)args.srcA.k0 : (long)grp * args.cpg * KP;
+        const long k1 = min(args.K, (grp + 1) * args.cpg * KP);
+        int m0, n0;
+        tile_of<BN>(args, t, m0, n0);
+        double* const c = grp == 0 ? args.C : args.part + (size_t)(grp - 1) * args.mA * args.mB;
+        const size_t ld = grp == 0 ? args.ldc : args.mB;
+        for (int x = lane; x < BM * BN; x += 32) {
+            const int i = m0 + x / BN, j = n0 + x % BN;
+            if (i >= args.mA || j >= args.mB || (args.lower && i < args.mB && j > i) ||
+                max(args.eA[i], args.eB[j]) < kNanExp)
+                continue;
+            double s = 0.0;
+            for (long k = k0; k < k1; ++k)
+                s = fma(src_entry(args.srcA, i, k, args.K), src_entry(args.srcB, j, k, args.K), s);
+            c[i * ld + j] = args.sign * s;
+            if (args.mirror && j < i) c[j * ld + i] = args.sign * s;
+        }
+    }
+}
+
 // C (+)= sign * A B^T from the digit slices, one 128 x BN output tile at a time, each CTA (one
 // per SM) walking tiles blockIdx.x, blockIdx.x + gridDim.x, ...: warp 0 streams, per tile and
 // K half, the right operand's S slices (one stage) and the left operand's slices (16 KB stages)
@@ -346,7 +387,8 @@ __device__ __forceinline__ void tile_of(const UpdArgs& a, int u, int& m0, int& n
 // and BN / 4 columns each) add the S integer accumulators of every K chunk into two 64-bit
 // integers per element in registers and form one FP64 value per element after the last chunk:
 // C is touched once per tile, through a shared-memory transpose that turns each warp's
-// accesses into full 32-byte sectors. Every wait is bounded.
+// accesses into full 32-byte sectors. The last warp looks over the exponents of the CTA's rows and
+// columns meanwhile, for elements without digits. Every wait is bounded.
 // Bounds: 36 MMAs of 128 x BN x 16 per K step are 9.2k tensor cycles per 128 x 64 x 128 piece;
 // per chunk the epilogue issues ~18 integer instructions per element against them (it was ~150
 // with a rounding and an FP64 read-modify-write of C per chunk, which bound the kernel: the
@@ -354,7 +396,7 @@ __device__ __forceinline__ void tile_of(const UpdArgs& a, int u, int& m0, int& n
 template <int BN>
 __global__ void __launch_bounds__(NTHREADS, 1)
 k_oz_update(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
-            const UpdArgs args) {
+            const __grid_constant__ UpdArgs args) {
     using T = Tile<BN>;
     constexpr int A_STAGES = T::A_STAGES, SETS = T::SETS;
     constexpr int NC = BN / 4;  // columns per epilogue warp
@@ -476,6 +518,20 @@ k_oz_update(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 ++i;
             }
         }
+    } else if (warp == 2 + EPI_WARPS) {
+        // ---- look-out: rows and columns without digits among this CTA's tiles ----
+        bool found = false;
+        for (int w = blockIdx.x; w < nwork; w += gridDim.x) {
+            int m0, n0;
+            tile_of<BN>(args, w % ntiles, m0, n0);
+            for (int x = lane; x < BM + BN; x += 32) {
+                const int r = x < BM ? m0 + x : n0 + x - BM;
+                if (r < (x < BM ? args.mA : args.mB)) found |= __ldg((x < BM ? args.eA : args.eB) + r) >= kNanExp;
+            }
+        }
+        found = __any_sync(0xffffffffu, found);
+        epi_barrier();  // the epilogue has stored every tile
+        if (found && args.srcA.s1) fill_undigited<BN>(args, lane);
     } else if (warp >= 2) {
         // ---- epilogue: a lane quarter q and NC columns h of each tile ----
         const int q = warp & 3, h = (warp - 2) >> 2;  // h = 0..3
@@ -554,6 +610,7 @@ k_oz_update(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 __syncwarp();
             }
         }
+        epi_barrier();
     }
     tc_fence_before();
     __syncthreads();
@@ -696,6 +753,7 @@ void ozmat_carve(OzMat& m, Arena& ar, int rows, int K) {
 }
 
 void oz_split_rows(cudaStream_t st, const double* src, int ld, OzMat& m) {
+    m.src = OzSrc{src, nullptr, ld, 0};
     if (m.rows <= 0) return;
     // up to eight rows per SM, more warps to a row (see the kernel); beyond, the rows fill the chip
     const int wpr = m.rows > 8 * num_sms() ? 1 : m.K > 2 * KP ? 4 : m.K > KP ? 2 : 1, grid = cdiv(m.rows, ROWS_PER_BLOCK / wpr);
@@ -707,6 +765,7 @@ void oz_split_rows(cudaStream_t st, const double* src, int ld, OzMat& m) {
 }
 
 void oz_split_cols_stack(cudaStream_t st, const double* S1, const double* S2, int ld, int n, int g, OzMat& m) {
+    m.src = OzSrc{S1, S2, ld, n};
     if (n <= 0 || g <= 0) return;
     const int parts = cdiv(m.K, kColsMaxK);
     if (parts > 1) {
@@ -753,6 +812,12 @@ cudaError_t oz_mul(cudaStream_t st, const OzMat& A, const OzMat& B, double* C, i
     a.khalves = kb > 64 ? 2 : 1;
     a.nchunks = nch;
     a.part = part;
+    // (where C is added to, only if it holds nothing but the earlier K of the same sources)
+    if (A.src.s1 && B.src.s1 && (!a.accumulate || A.src.k0 > 0)) {
+        a.srcA = A.src;
+        a.srcB = B.src;
+    }
+    a.K = A.K;
     const MulPlan p = plan_mul(A.rows, B.rows, nch, lower, part ? part_cap : 0);
     return p.bn == 64 ? launch_mul<64>(st, A, B, a, p.groups) : launch_mul<32>(st, A, B, a, p.groups);
 }
@@ -813,6 +878,7 @@ cudaError_t product(cudaStream_t st, int M, int N, int K, const double* A, int l
             oz_split_cols(st, B + ob, B2 ? B2 + ob : nullptr, ldb, b);
         else
             oz_split_rows(st, B + ob, ldb, b);
+        b.src.k0 = k0;
         OzMat a = b;
         if (!same_ab) {
             a = view(ws.sA, ws.eA, M, kn);
@@ -820,6 +886,7 @@ cudaError_t product(cudaStream_t st, int M, int N, int K, const double* A, int l
                 oz_split_cols(st, A + (size_t)k0 * lda, nullptr, lda, a);
             else
                 oz_split_rows(st, A + k0, lda, a);
+            a.src.k0 = k0;
         }
         const cudaError_t e = oz_mul(st, a, b, C, ldc, sign, k0 > 0 ? flags | OZ_ACC : flags, ws.part, ws.part_cap);
         if (e != cudaSuccess) return e;
@@ -902,10 +969,9 @@ cudaError_t ldl_oz(cudaStream_t st, int R, int n, double* Haug, double* P, doubl
 }
 
 cudaError_t oz_gemm(cudaStream_t st, int M, int N, int K, const double* A, int lda, const double* B,
-                    int ldb, double* C, int ldc, double sign, bool lower, const OzWs& ws) {
+                    int ldb, double* C, int ldc, const OzWs& ws) {
     if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
-    return product(st, M, N, K, A, lda, false, B, nullptr, ldb, false, C, ldc, sign,
-                   OZ_ACC | (lower ? OZ_LOWER : 0), ws);
+    return product(st, M, N, K, A, lda, false, B, nullptr, ldb, false, C, ldc, 1.0, 0, ws);
 }
 
 cudaError_t oz_dgemm(cudaStream_t st, bool trans_a, int M, int N, int K, const double* A, int lda,

@@ -34,3 +34,51 @@ def test_norm_of_long_factors(api, o, v):
 
     lim = 2 * U * (2 * (o + v) + 2 * Rt + Rt * Rt) * norm2(Xo.abs(), Xv.abs(), Z.abs())
     assert abs(api.thc_cpd_thc_norm2(Xo, Xv, Z) - norm2(Xo, Xv, Z)) <= lim
+
+
+def _pattern(x):
+    return np.where(np.isnan(x), 2, np.where(np.isposinf(x), 1, np.where(np.isneginf(x), -1, 0)))
+
+
+# infinities go through a digit product as through an FP64 one: infinite with the sign of the term, NaN
+# against a zero or an infinity of the other sign, and nothing outside their row or column
+@pytest.mark.parametrize("M,N,K", [(70, 50, 200), (129, 65, 65), (3, 2, 8200)])
+def test_infinities(api, M, N, K):
+    rng = np.random.default_rng(K)
+    A, B = rng.standard_normal((M, K)), rng.standard_normal((N, K))
+    A[1, 3], A[2, 0], A[2, K - 1] = np.inf, -np.inf, np.inf
+    B[0, 3] = 0.0
+    B[1, K // 2] = -np.inf
+    if M > 100:
+        A[128, 64], A[100, 5], B[64, 0] = np.inf, np.nan, np.inf
+    d = lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    C = api.thc_cpd_emulated_gemm(d(A), d(B)).cpu().numpy()
+    with np.errstate(invalid="ignore"):
+        ref = np.array([(a * B).sum(-1) for a in A])
+    np.testing.assert_array_equal(_pattern(C), _pattern(ref))
+    ok = np.isfinite(ref)
+    lim = 2 * K * U * (np.abs(A)[:, None, :] * np.abs(B)[None, :, :]).sum(-1) if M * N * K < 1e7 else None
+    assert lim is None or np.all(np.abs(C - ref)[ok] <= lim[ok])
+
+
+# the same through an entry point: digits of Z, of X, of a factor and of Hadamard products, split K
+@pytest.mark.parametrize("mode", [0, 3])
+@pytest.mark.parametrize("zero", [False, True])
+def test_infinities_in_an_mttkrp(api, mode, zero):
+    o, v, Rt, R = 12, 90, 200, 300
+    rng = np.random.default_rng(mode)
+    X = [rng.random((n, Rt)) + 0.1 for n in (o, v)]
+    Z, A = rng.random((Rt, Rt)) + 0.1, [rng.random((n, R)) + 0.1 for n in (o, v, o, v)]
+    A[2][5, 7] = A[1][3, 130] = np.inf
+    if zero:
+        X[0][5, 3] = X[1][3, 150] = 0.0
+    d = lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    M = api.thc_cpd_mttkrp(d(X[0]), d(X[1]), d(Z), [d(a) for a in A], mode).cpu().numpy()
+    mul = lambda a, b: np.array([(r[:, None] * b).sum(0) for r in a])
+    with np.errstate(invalid="ignore"):
+        W = [mul(X[k % 2].T, A[k]) for k in range(4)]
+        Y = mul(Z, W[2] * W[3]) if mode < 2 else mul(Z.T, W[0] * W[1])
+        ref = mul(X[mode % 2], W[mode ^ 1] * Y)
+    np.testing.assert_array_equal(_pattern(M), _pattern(ref))
+    ok = np.isfinite(ref)
+    assert np.all(np.abs(M - ref)[ok] <= 2 * (3 * v + 2 * Rt + 4) * U * ref[ok])
