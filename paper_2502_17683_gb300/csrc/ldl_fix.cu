@@ -179,21 +179,21 @@ __device__ __forceinline__ long long times_recip(long long q, const Recip& r) {
     return P + (mulw(p.x, u1) >> 10) + (mulw(p.x, u0) >> 30) + (mulw(p.y, u1) >> 41);
 }
 
-// V 2^e rounded to FP64 (|V| < 2^63; results outside the normal range do not occur here except
-// for zero: below it signed zero, above it infinity)
+// V 2^e rounded to FP64 (|V| < 2^63): infinite above the normal range, subnormal below it
 __device__ __forceinline__ double fix_to_double(long long V, int e) {
     const unsigned long long sgn = (unsigned long long)V & 0x8000000000000000ULL;
     const unsigned long long u = V < 0 ? 0ULL - (unsigned long long)V : (unsigned long long)V;
     if (u == 0) return __longlong_as_double((long long)sgn);
     const int lz = __clzll((long long)u);
     const unsigned long long m = u << lz;
-    unsigned long long mant = m >> 11;
-    const unsigned rem = (unsigned)(m & 0x7FFULL);
-    mant += (rem > 0x400u || (rem == 0x400u && (mant & 1ULL))) ? 1ULL : 0ULL;
     const int be = 1023 + 63 - lz + e;
-    if (be < 1) return __longlong_as_double((long long)sgn);
     if (be > 2046) return __longlong_as_double((long long)(sgn | 0x7FF0000000000000ULL));
-    return __longlong_as_double((long long)(sgn | (((unsigned long long)(be - 1) << 52) + mant)));
+    const int sh = 11 + max(0, 1 - be);  // bits below the result's last one
+    if (sh > 64) return __longlong_as_double((long long)sgn);
+    unsigned long long mant = sh < 64 ? m >> sh : 0;
+    const unsigned long long rem = m << (64 - sh), half = 0x8000000000000000ULL;
+    mant += (rem > half || (rem == half && (mant & 1ULL))) ? 1ULL : 0ULL;
+    return __longlong_as_double((long long)(sgn | (((unsigned long long)max(be - 1, 0) << 52) + mant)));
 }
 
 // scaling exponent of a diagonal entry a > 0: a 4^-e in [1/4, 1)

@@ -17,8 +17,9 @@
 // FP64. The error is thus 2^-53 of |result| plus about 2^-62 of (row max)(column max)
 // sqrt(K): below that of an FP64 GEMM, which rounds at every term, at the library's operands
 // (a 1200-long product of weighted THC factors: 5e-17 of the result's norm, an FP64 FMA chain
-// 1.1e-15, seven slices 5e-15). An element whose row or column holds an infinity or a NaN is summed in
-// FP64 from the operands themselves (OzSrc), as an FP64 GEMM does.
+// 1.1e-15, seven slices 5e-15). An element whose row or column holds an infinity or a NaN, or that may
+// lie below the normal range, is summed in FP64 from the operands themselves (OzSrc), as an FP64 GEMM
+// does; without sources such rows give NaN and results below the normal range zero.
 // 36 BF16 MMAs per 16 of K take the place of the FP64 FMAs (GB300: 2 FP64 FMA per clock per
 // SM against ~3500 BF16 MAC).
 #pragma once
@@ -50,7 +51,7 @@ struct OzMat {
     int* e = nullptr;
     int rows = 0, K = 0;
     int ld_rows = 0;  // rows of the buffer (0: rows); a view of its first rows
-    OzSrc src;        // set by the cuts; none: such rows give NaN
+    OzSrc src;        // set by the cuts; none: see above
     int chunks() const { return K > 0 ? cdiv(K, kOzPanel) : 0; }
 };
 size_t ozmat_bytes(int rows, int K);

@@ -59,7 +59,7 @@ __device__ __forceinline__ void store_digits4(const double (&x)[4], int erow, ui
 // (0 or the sign bit): normalised and assembled in integer arithmetic, so that of each output
 // element only the final addition runs on the FP64 pipe (an int64 conversion costs as much
 // there as an FMA). |hi| < 2^44, |lo| < 2^62. Below the normal range the term is dropped
-// (signed zero), above it the result is infinite.
+// (signed zero; see kTinyExp), above it the result is infinite.
 __device__ __forceinline__ double scaled_sum(long long hi, long long lo, int e, unsigned long long neg) {
     // V = hi 2^(40 - sh) + lo 2^-sh within 62 bits; bits below 2^-59 of V are cut only for sh > 0
     const int hb = 64 - __clzll(hi < 0 ? -hi : hi);
@@ -349,11 +349,33 @@ __device__ __forceinline__ void epi_barrier() {
     asm volatile("bar.sync 1, %0;" ::"n"(32 * EPI_WARPS + 32) : "memory");
 }
 
-// The elements of this CTA's tiles that have no digits (an infinity or a NaN in their row or column),
-// formed in FP64 from the operands by the look-out's lanes, over what the epilogue stored. A warp, a
+// Rows whose exponents add up to less may give an element below the normal range (the last unit of
+// its sum is 2^(ea + eb - 68)), where the epilogue gives zero.
+constexpr int kTinyExp = -954;
+
+// The elements of this CTA's tiles that the digits do not give (an infinity or a NaN in their row or
+// column, or next to the subnormal numbers), formed in FP64 from the operands by the look-out's lanes,
+// over what the epilogue stored. A warp, a
 // branch and a call of its own: the epilogue's loop has no register to spare. Exchange energies at
 // (20,100,480,720), 12 points, no such element in them: 897 us without this, 904 with it, 920 with the
 // loops inlined, 925 with the elements looked for in the epilogue.
+// (Tiny rows are scaled by their exponents and their products and sums carried with their errors, after
+// Ogita, Rump, Oishi, "Accurate sum and dot product", SIAM J. Sci. Comput. 26, 2005: like the digits',
+// the element's only rounding is that of the result.)
+__device__ __forceinline__ double src_dot(const UpdArgs& args, int i, int j, long k0, long k1) {
+    int ea = args.eA[i], eb = args.eB[j];
+    if (max(ea, eb) >= kNanExp) ea = eb = 0;
+    double s = 0.0, c = 0.0;
+    for (long k = k0; k < k1; ++k) {
+        const double a = scalbn(src_entry(args.srcA, i, k, args.K), -ea);
+        const double b = scalbn(src_entry(args.srcB, j, k, args.K), -eb);
+        const double p = a * b, t = s + p, z = t - s;
+        c += ((s - (t - z)) + (p - z)) + fma(a, b, -p);
+        s = t;
+    }
+    return isfinite(s) ? scalbn(s + c, ea + eb) : s;
+}
+
 template <int BN>
 __device__ __noinline__ void fill_undigited(const UpdArgs& args, int lane) {
     for (int w = blockIdx.x; w < args.nactive * args.kgroups; w += gridDim.x) {
@@ -367,13 +389,11 @@ __device__ __noinline__ void fill_undigited(const UpdArgs& args, int lane) {
         for (int x = lane; x < BM * BN; x += 32) {
             const int i = m0 + x / BN, j = n0 + x % BN;
             if (i >= args.mA || j >= args.mB || (args.lower && i < args.mB && j > i) ||
-                max(args.eA[i], args.eB[j]) < kNanExp)
+                (max(args.eA[i], args.eB[j]) < kNanExp && args.eA[i] + args.eB[j] >= kTinyExp))
                 continue;
-            double s = 0.0;
-            for (long k = k0; k < k1; ++k)
-                s = fma(src_entry(args.srcA, i, k, args.K), src_entry(args.srcB, j, k, args.K), s);
-            c[i * ld + j] = args.sign * s;
-            if (args.mirror && j < i) c[j * ld + i] = args.sign * s;
+            const double s = args.sign * src_dot(args, i, j, k0, k1);
+            c[i * ld + j] = s;
+            if (args.mirror && j < i) c[j * ld + i] = s;
         }
     }
 }
@@ -519,14 +539,16 @@ k_oz_update(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
             }
         }
     } else if (warp == 2 + EPI_WARPS) {
-        // ---- look-out: rows and columns without digits among this CTA's tiles ----
+        // ---- look-out: rows and columns without digits, or of tiny numbers, among this CTA's tiles ----
         bool found = false;
         for (int w = blockIdx.x; w < nwork; w += gridDim.x) {
             int m0, n0;
             tile_of<BN>(args, w % ntiles, m0, n0);
             for (int x = lane; x < BM + BN; x += 32) {
                 const int r = x < BM ? m0 + x : n0 + x - BM;
-                if (r < (x < BM ? args.mA : args.mB)) found |= __ldg((x < BM ? args.eA : args.eB) + r) >= kNanExp;
+                if (r >= (x < BM ? args.mA : args.mB)) continue;
+                const int e = __ldg((x < BM ? args.eA : args.eB) + r);
+                found |= e >= kNanExp || e < kTinyExp / 2;  // (of a tiny pair one at least)
             }
         }
         found = __any_sync(0xffffffffu, found);

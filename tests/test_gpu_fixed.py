@@ -122,3 +122,14 @@ def test_overdrawn_diagonal_is_noticed(solve, R, row, cols):
     H[row, cols[0]:cols[1]] = H[cols[0]:cols[1], row] = 0.475
     A, used = solve(H, np.random.default_rng(R).standard_normal((3, R)))
     assert used
+
+
+# quotients below the normal range: Y = M / 4 rounded to units of 2^-1074, and A from it
+@pytest.mark.parametrize("R", [20, 130])
+@pytest.mark.parametrize("e", [-1020, -1040, -1068, -1073])
+def test_subnormal_rows(solve, R, e):
+    M = np.random.default_rng(R).standard_normal((3, R)) * 2.0 ** (e + 20) * 2.0 ** -20
+    A, used = solve(4.0 * np.eye(R), M)
+    assert not used and np.any(A != 0.0)
+    # exact but for the reciprocal square roots (2^-52 together) and one rounding of the result
+    assert np.all(np.abs(A - M / 4) <= 2.0 ** -52 * np.abs(M / 4) + 2.0 ** -1074)

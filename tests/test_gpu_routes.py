@@ -82,3 +82,20 @@ def test_infinities_in_an_mttkrp(api, mode, zero):
     np.testing.assert_array_equal(_pattern(M), _pattern(ref))
     ok = np.isfinite(ref)
     assert np.all(np.abs(M - ref)[ok] <= 2 * (3 * v + 2 * Rt + 4) * U * ref[ok])
+
+
+# results in and below the subnormal range: a digit product rounds to the smallest unit 2^-1074 where an
+# FP64 product does (half a unit each), and gives a signed zero below
+@pytest.mark.parametrize("e", [-1010, -1030, -1040, -1060, -1068, -1071, -1074, -1076, -1080])
+def test_subnormal_results(api, e):
+    rng = np.random.default_rng(-e)
+    A, B = rng.standard_normal((70, 200)), rng.standard_normal((50, 200))
+    fine = np.longdouble(2.0) ** e
+    ref = (A.astype(np.longdouble) @ B.astype(np.longdouble).T) * fine
+    d = lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    C = api.thc_cpd_emulated_gemm(d(A * 2.0 ** (e // 2)), d(B * 2.0 ** (e - e // 2))).cpu().numpy()
+    # 2^-53 of the result, the digits' 2^-61 K max max, half a unit of the subnormal range
+    top = np.max(np.abs(A), 1)[:, None] * np.max(np.abs(B), 1)[None, :]
+    lim = U * np.abs(ref) + 2.0 ** -61 * 200 * top * fine + np.longdouble(2.0) ** -1075 * (1 + 2.0 ** -20)
+    assert np.all(np.abs(C - ref) <= lim)
+    assert e < -1074 or np.any(C != 0.0)
