@@ -64,6 +64,14 @@ struct DevScalars {
     int pad1;
 };
 
+// cudaMallocAsync whose failure leaves no error behind for the calls after it.
+inline bool alloc_block(void** p, size_t bytes, cudaStream_t st) {
+    if (cudaMallocAsync(p, bytes, st) == cudaSuccess) return true;
+    cudaGetLastError();
+    *p = nullptr;
+    return false;
+}
+
 // Bump allocator over one cudaMallocAsync block; every carve is 256-byte aligned.
 struct Arena {
     char* base = nullptr;

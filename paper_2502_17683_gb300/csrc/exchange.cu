@@ -146,24 +146,38 @@ extern "C" thc_cpd_status thc_cpd_exchange(int o, int v, int Rt, int R, int nalp
     int g = (int)std::min<size_t>(nalpha, std::max<size_t>(1, (size_t(1) << 30) / per));
     while (g > 1 && ((long)g * std::max(Rt, R) * std::max(std::max(Rt, R), nmax) >= 0x7fffffffL)) --g;
     // products from digits: all on request, else those of a group that are faster there
-    const bool ozd = oz_available() && Rt <= 8192 && R <= 8192 && nmax <= 8192;
-    const bool all = ozd && opts && opts->ldl == THC_CPD_LDL_EMULATED;
-    auto on_tc = [&](int M, int N, int K) { return all || (ozd && oz_worth_flops(2.0 * g * M * (double)N * K)); };
-    const bool tc_z = on_tc(Rt, R, Rt), tc_u[2] = {on_tc(Rt, R, o), on_tc(Rt, R, v)};
-    const bool tc_m = on_tc(R, R, o), tc_n = on_tc(R, R, v);
-    const bool emu = tc_z || tc_u[0] || tc_u[1] || tc_m || tc_n;
-    const size_t part_cap = std::max(dgemm_part_need(Rt, R, Rt),
-                                     std::max(dgemm_part_need(g * Rt, R, nmax), dgemm_part_need(R, g * R, nmax)));
-    size_t bytes = Arena::need<double>((size_t)o * g * Rt) + Arena::need<double>((size_t)v * g * Rt) +
-                   5 * Arena::need<double>(g * RtR) + 2 * Arena::need<double>((size_t)o * g * R) +
-                   Arena::need<double>((size_t)v * g * R) + 3 * Arena::need<double>(g * RR) +
-                   Arena::need<double>((size_t)XR_BLOCKS * g) + Arena::need<double>(2 * (size_t)nalpha) +
-                   Arena::need<double>(part_cap);
-    if (emu)
-        bytes += 2 * ozmat_bytes(R, o) + 2 * ozmat_bytes(R, v) + ozmat_bytes(g * Rt, o) + ozmat_bytes(g * Rt, v) +
-                 ozmat_bytes(Rt, Rt) + ozmat_bytes(g * R, Rt) + ozmat_bytes(g * R, nmax);
+    bool ozd = oz_available() && Rt <= 8192 && R <= 8192 && nmax <= 8192;
+    bool tc_z, tc_u[2], tc_m, tc_n, emu;
+    size_t part_cap, bytes;
     void* block = nullptr;
-    if (cudaMallocAsync(&block, bytes, st) != cudaSuccess) return xerr(THC_CPD_ERR_ALLOC, "workspace allocation failed");
+    // where a group's block does not fit, half the points, at last one without digits: what one point
+    // takes on the FP64 pipes is what the call needs
+    for (;;) {
+        const bool all = ozd && opts && opts->ldl == THC_CPD_LDL_EMULATED;
+        auto on_tc = [&](int M, int N, int K) { return all || (ozd && oz_worth_flops(2.0 * g * M * (double)N * K)); };
+        tc_z = on_tc(Rt, R, Rt);
+        tc_u[0] = on_tc(Rt, R, o);
+        tc_u[1] = on_tc(Rt, R, v);
+        tc_m = on_tc(R, R, o);
+        tc_n = on_tc(R, R, v);
+        emu = tc_z || tc_u[0] || tc_u[1] || tc_m || tc_n;
+        part_cap = std::max(dgemm_part_need(Rt, R, Rt),
+                            std::max(dgemm_part_need(g * Rt, R, nmax), dgemm_part_need(R, g * R, nmax)));
+        bytes = Arena::need<double>((size_t)o * g * Rt) + Arena::need<double>((size_t)v * g * Rt) +
+                5 * Arena::need<double>(g * RtR) + 2 * Arena::need<double>((size_t)o * g * R) +
+                Arena::need<double>((size_t)v * g * R) + 3 * Arena::need<double>(g * RR) +
+                Arena::need<double>((size_t)XR_BLOCKS * g) + Arena::need<double>(2 * (size_t)nalpha) +
+                Arena::need<double>(part_cap);
+        if (emu)
+            bytes += 2 * ozmat_bytes(R, o) + 2 * ozmat_bytes(R, v) + ozmat_bytes(g * Rt, o) + ozmat_bytes(g * Rt, v) +
+                     ozmat_bytes(Rt, Rt) + ozmat_bytes(g * R, Rt) + ozmat_bytes(g * R, nmax);
+        if (alloc_block(&block, bytes, st)) break;
+        if (g == 1 && !ozd) return xerr(THC_CPD_ERR_ALLOC, "workspace allocation failed");
+        if (g == 1)
+            ozd = false;
+        else
+            g = (g + 1) / 2;
+    }
     Arena ar;
     ar.base = (char*)block;
     ar.cap = bytes;

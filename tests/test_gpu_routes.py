@@ -99,3 +99,22 @@ def test_subnormal_results(api, e):
     lim = U * np.abs(ref) + 2.0 ** -61 * 200 * top * fine + np.longdouble(2.0) ** -1075 * (1 + 2.0 ** -20)
     assert np.all(np.abs(C - ref) <= lim)
     assert e < -1074 or np.any(C != 0.0)
+
+
+# more points than 1 GB of intermediates holds: two full groups and a shorter last one
+@pytest.mark.parametrize("na", [500, 301])
+def test_exchange_in_groups(api, na):
+    from oracle import exchange as X
+    from tests._util import to_dev
+    from thc_inputs import make_lt, make_problem
+    o, v, Rt, R = 20, 60, 203, 261
+    p = make_problem(o, v, Rt, R, seed=na)
+    lam = np.random.default_rng(na).uniform(0.5, 2.0, R)
+    Lam, Gam = X.lt_factors(*make_lt(o, v, na, na))
+    d, dev = to_dev(p, torch), lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    e1, e2, _ = api.thc_cpd_exchange(d["Xo"], d["Xv"], d["Z"], d["A"], dev(lam), dev(Lam), dev(Gam))
+    r1, r2, _ = X.exchange_robust(p.Xo, p.Xv, p.Z, p.A, lam, Lam, Gam)
+    # relative to the size of the terms, as for one group
+    s1 = abs(X.exchange_single(np.abs(p.Xo), np.abs(p.Xv), np.abs(p.Z), [np.abs(a) for a in p.A], lam, Lam, Gam))
+    s2 = abs(X.exchange_double([np.abs(a) for a in p.A], lam, Lam, Gam))
+    assert abs(e1 - r1) <= 1e-12 * s1 and abs(e2 - r2) <= 1e-12 * s2

@@ -78,3 +78,27 @@ def test_long_factors_run(calls, o, v):
     assert calls.norm2(o, v, 220) == 0, calls.lib.thc_cpd_last_error()
     assert calls.loss(o, v, 220, 40, normG2=0.0) == 0, calls.lib.thc_cpd_last_error()
     assert calls.lib.fake_launches(b"k_oz_update") > 0
+
+
+# a block that does not fit is asked for with fewer points, at last without digits: one point's needs on
+# the FP64 pipes are enough (five Rt x R, three R x R, the scaled factors, partial sums)
+@pytest.mark.parametrize("ldl", [0, 3])
+def test_exchange_makes_do_with_one_point(calls, ldl):
+    from paper_2502_17683_gb300._lib import ERR_ALLOC
+    o, v, Rt, R, na = 10, 50, 400, 600, 12
+    run = lambda: calls.exchange(o, v, Rt, R, na, ldl=ldl)
+    assert run() == 0
+    sizes = [calls.lib.fake_largest_alloc()]
+    while True:
+        calls.lib.fake_reset()
+        calls.lib.fake_alloc_limit(sizes[-1] - 1)
+        s = run()
+        if s != 0:
+            break
+        sizes.append(calls.lib.fake_largest_alloc())
+    assert s == ERR_ALLOC
+    # 16 split-K partial sums of the largest product at most, 256 bytes of padding a piece
+    one = 8 * ((o + v) * Rt + 5 * Rt * R + (2 * o + v) * R + 3 * R * R + 16 * Rt * R) + 65536
+    assert len(sizes) > 3 and sizes[-1] <= one
+    calls.lib.fake_alloc_limit(1 << 62)
+    assert run() == 0  # the failure leaves nothing behind
