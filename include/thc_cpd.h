@@ -21,7 +21,8 @@
  *     stream before returning.
  *   - Device workspace is allocated per call with the stream-ordered allocator
  *     (cudaMallocAsync) and released before return. The library never frees caller
- *     memory.
+ *     memory. Where the workspace of the FP64-accurate tensor-core products does not fit,
+ *     the call runs them on the FP64 pipes; THC_CPD_ERR_ALLOC when those lack room, too.
  *   - Errors: a status code is returned and thc_cpd_last_error() gives a message
  *     (per host thread). Arguments are validated before any work is enqueued; on an
  *     argument error no device memory is touched. A CUDA error leaves outputs
@@ -294,7 +295,8 @@ thc_cpd_status thc_cpd_exchange(int o, int v, int Rt, int R, int nalpha, const d
  * pipes; with opts->ldl = THC_CPD_LDL_EMULATED all run on the tensor cores (and the solve uses
  * the emulated two-level LDL^T).
  * Allocates its workspace (about 256 MiB plus 2 naux R_thc doubles, plus naux o v and naux^2
- * doubles with loss) with cudaMallocAsync on opts->stream. Synchronises. */
+ * doubles with loss; the tensor-core products take up to 512 MiB more for the digits of their
+ * operands) with cudaMallocAsync on opts->stream. Synchronises. */
 thc_cpd_status thc_cpd_core_fit(int o, int v, int Rt, int naux, const double* Xo, const double* Xv,
                                 const double* B, double* Z, double* loss, int* used_pinv,
                                 const thc_cpd_opts* opts);
@@ -308,7 +310,8 @@ thc_cpd_status thc_cpd_core_fit(int o, int v, int Rt, int naux, const double* Xo
  * opts->precision must be THC_CPD_FP64; GEMMs as for thc_cpd_core_fit, opts->ldl =
  * THC_CPD_LDL_EMULATED runs them all and the solve on the FP64-accurate tensor-core path. opts->history: NULL or 2 * max_sweeps host
  * doubles (loss, fit per sweep). opts->flags_out bit 0: a pseudo-inverse solve was used.
- * Workspace: about (2 o v + max(o, v) R + 3 R) naux + naux^2 + 5 R^2 doubles (cudaMallocAsync).
+ * Workspace: about (2 o v + max(o, v) R + 3 R) naux + naux^2 + 5 R^2 doubles and partial sums, the
+ * tensor-core products up to 512 MiB for the digits of their operands (cudaMallocAsync).
  * 1 <= R <= 2048, 1 <= o, v <= 4096. Synchronises once per sweep. */
 thc_cpd_status thc_cpd_df_als(int o, int v, int naux, int R, const double* B, double* const A[4],
                               double* lam, int max_sweeps, double tol, int* sweeps_done,

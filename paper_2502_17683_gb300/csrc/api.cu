@@ -268,7 +268,7 @@ Ldl ldl_route(int ldl, int R, int nmax, bool batched) {
 constexpr int kBatchedFlowCtas = 32;
 
 thc_cpd_status ctx_init(Ctx& c, const Shape& s, const double* Xo, const double* Xv,
-                        const double* Z, const thc_cpd_opts* opts, unsigned need) {
+                        const double* Z, const thc_cpd_opts* opts, unsigned need, bool digits = true) {
     c.s = s;
     c.X[0] = Xo;
     c.X[1] = Xv;
@@ -285,7 +285,7 @@ thc_cpd_status ctx_init(Ctx& c, const Shape& s, const double* Xo, const double* 
     const bool fp64 = !mixed || als || gram;  // FP64 projections (MTTKRP, or a split run's loss)
     // FP64 products that go to the tensor cores: room for the operands' digits and split sums
     const bool w_z = fp64 && oz_worth(Rt, R, Rt, false), w_n = norm && oz_worth(Rt, Rt, Rt, false);
-    c.ozp = oz_available() && (w_z || w_n || (fp64 && oz_worth(Rt, R, nmax, false)) ||
+    c.ozp = digits && oz_available() && (w_z || w_n || (fp64 && oz_worth(Rt, R, nmax, false)) ||
                                (gram && oz_worth(R, R, nmax, true)));
     const bool ozp = c.ozp;
     // FP64-pipe products: split-K partial sums of those that stay there
@@ -337,21 +337,36 @@ thc_cpd_status ctx_init(Ctx& c, const Shape& s, const double* Xo, const double* 
     const bool ozl = c.fixed || c.two_level;
     if (ozl) bsolve_ws_rows(R, nmax, &oz_ra, &oz_rb, &oz_part);
     if (c.two_level) oz_ldl_ws_rows(R, nmax, &oz_ra, &oz_rb);
+    // digits of what the products from digits take: X_k both ways, Z both ways, P = W o W or W o Y, a
+    // factor's columns
+    const bool d_gram = gram && oz_worth(R, R, nmax, true);
+    bool d_x[2], d_xt[2], d_p = w_z, d_a = d_gram;
+    for (int k = 0; k < 2; ++k) {
+        const int n = s.n[k];
+        d_x[k] = ozp && fp64 && oz_worth(n, R, Rt, false);
+        const bool proj = fp64 && oz_worth(Rt, R, n, false);
+        d_xt[k] = ozp && (proj || (w_n && n <= kOzMaxK));
+        d_p |= d_x[k];
+        d_a |= proj || (gram && oz_worth(R, R, n, true));
+        int left = 1, right = 1;  // (a back-projection's operands have digits of their own)
+        if (d_x[k]) oz_product_ws(n, R, Rt, &left, &right, &oz_part);
+        if (ozp && proj) oz_product_ws(Rt, R, n, &oz_ra, &oz_rb, &oz_part);
+    }
     if (ozp) {
-        if (fp64) {
-            for (int k = 0; k < 2; ++k) {
-                oz_product_ws(s.n[k], R, Rt, &oz_ra, &oz_rb, &oz_part);
-                oz_product_ws(Rt, R, s.n[k], &oz_ra, &oz_rb, &oz_part);
-            }
-            oz_product_ws(Rt, R, Rt, &oz_ra, &oz_rb, &oz_part);
-        }
-        if (norm) oz_product_ws(Rt, Rt, Rt, &oz_ra, &oz_rb, &oz_part);
-        bytes += 2 * ozmat_bytes(Rt, Rt) + ozmat_bytes(R, Rt) + ozmat_bytes(R, nmax);
+        if (w_z) oz_product_ws(Rt, R, Rt, &oz_ra, &oz_rb, &oz_part);
+        if (d_gram) oz_product_ws(R, R, 1, &oz_ra, &oz_rb, nullptr);
+        if (w_n) oz_product_ws(Rt, Rt, Rt, &oz_ra, &oz_rb, &oz_part);
+        if (w_z || w_n) bytes += 2 * ozmat_bytes(Rt, Rt);
+        if (d_p) bytes += ozmat_bytes(R, Rt);
+        if (d_a) bytes += ozmat_bytes(R, nmax);
         for (int k = 0; k < 2; ++k)
-            bytes += ozmat_bytes(s.n[k], Rt) + (s.n[k] <= kOzMaxK ? ozmat_bytes(Rt, s.n[k]) : 0);
+            bytes += (d_x[k] ? ozmat_bytes(s.n[k], Rt) : 0) + (d_xt[k] ? ozmat_bytes(Rt, s.n[k]) : 0);
     }
     if (ozl || ozp) bytes += oz_ws_bytes(oz_ra, oz_rb, oz_part);
-    CK(cudaMallocAsync(&c.block, bytes, c.st));
+    if (!alloc_block(&c.block, bytes, c.st)) {
+        if (ozp) return ctx_init(c, s, Xo, Xv, Z, opts, need, false);  // the FP64 pipes make do with less
+        return set_err(THC_CPD_ERR_ALLOC, "workspace allocation of %zu bytes failed", bytes);
+    }
     Arena ar;
     ar.base = (char*)c.block;
     ar.cap = bytes;
@@ -397,13 +412,13 @@ thc_cpd_status ctx_init(Ctx& c, const Shape& s, const double* Xo, const double* 
         if (als) CK(mixed_setup(c.mx, c.st, Xo, Xv, Z));  // a single MTTKRP splits what its mode takes
     }
     if (ozp) {
-        for (int h = 0; h < 2; ++h) ozmat_carve(c.dZ[h], ar, Rt, Rt);
+        for (int h = 0; h < 2 && (w_z || w_n); ++h) ozmat_carve(c.dZ[h], ar, Rt, Rt);
         for (int k = 0; k < 2; ++k) {
-            ozmat_carve(c.dX[k], ar, s.n[k], Rt);
-            if (s.n[k] <= kOzMaxK) ozmat_carve(c.dXT[k], ar, Rt, s.n[k]);
+            if (d_x[k]) ozmat_carve(c.dX[k], ar, s.n[k], Rt);
+            if (d_xt[k]) ozmat_carve(c.dXT[k], ar, Rt, s.n[k]);
         }
-        ozmat_carve(c.dP, ar, R, Rt);
-        ozmat_carve(c.dA, ar, R, nmax);
+        if (d_p) ozmat_carve(c.dP, ar, R, Rt);
+        if (d_a) ozmat_carve(c.dA, ar, R, nmax);
     }
     if (ozl || ozp) oz_ws_carve(c.oz, ar, oz_ra, oz_rb, oz_part);
     if (gram) fill(c.st, c.ones, R, 1.0);
@@ -428,7 +443,8 @@ thc_cpd_status ctx_safe_buffers(Ctx& c) {
     size_t bytes = 2 * Arena::need<double>(RR) + Arena::need<double>(TT) +
                    2 * Arena::need<double>((size_t)nmax * R) + Arena::need<double>(R);
     void* p = nullptr;
-    CK(cudaMallocAsync(&p, bytes, c.st));
+    if (!alloc_block(&p, bytes, c.st))
+        return set_err(THC_CPD_ERR_ALLOC, "workspace allocation of %zu bytes failed", bytes);
     Arena ar;
     ar.base = (char*)p;
     ar.cap = bytes;
@@ -806,7 +822,7 @@ thc_cpd_status learn_init(Ctx& c, LearnWs& L) {
          4 * Arena::need<double>((size_t)R * R) + Arena::need<double>(256) + Arena::need<double>(8) +
          Arena::need<float>(64) + Arena::need<DevScalars>(1);
     L.st = c.st;
-    CK(cudaMallocAsync(&L.block, b, c.st));
+    if (!alloc_block(&L.block, b, c.st)) return set_err(THC_CPD_ERR_ALLOC, "workspace allocation of %zu bytes failed", b);
     Arena ar;
     ar.base = (char*)L.block;
     for (int k = 0; k < 4; ++k) L.T[k] = ar.take<double>((size_t)c.s.n[k] * R);
@@ -1228,7 +1244,8 @@ thc_cpd_status run_batched(int np, thc_cpd_problem* P, int max_sweeps, double to
     CK(cudaEventRecord(ev_fork, caller));
     CK(cudaStreamWaitEvent(r.cap, ev_fork, 0));
     for (int p = 0; p < np; ++p) CK(cudaStreamWaitEvent(r.streams[p], ev_fork, 0));
-    CK(cudaMallocAsync((void**)&r.dsc, sizeof(DevScalars) * 2 * np, caller));
+    if (!alloc_block((void**)&r.dsc, sizeof(DevScalars) * 2 * np, caller))
+        return set_err(THC_CPD_ERR_ALLOC, "workspace allocation failed");
     CK(cudaMallocHost((void**)&r.hsc, sizeof(DevScalars) * np));
     CK(cudaStreamSynchronize(caller));
     r.ctx.resize(np);
@@ -1568,7 +1585,8 @@ extern "C" thc_cpd_status thc_cpd_emulated_gemm(int M, int N, int K, const doubl
         }
     } ws;
     ws.st = st;
-    CK(cudaMallocAsync(&ws.p, bytes, st));
+    if (!alloc_block(&ws.p, bytes, st))
+        return set_err(THC_CPD_ERR_ALLOC, "workspace allocation of %zu bytes failed", bytes);
     Arena ar;
     ar.base = (char*)ws.p;
     ar.cap = bytes;
@@ -1612,7 +1630,8 @@ int spd_solve(cudaStream_t st, int R, int n, const double* H, const double* M, d
         }
     } ws;
     ws.st = st;
-    CK(cudaMallocAsync(&ws.p, bytes, st));
+    if (!alloc_block(&ws.p, bytes, st))
+        return set_err(THC_CPD_ERR_ALLOC, "workspace allocation of %zu bytes failed", bytes);
     Arena ar;
     ar.base = (char*)ws.p;
     ar.cap = bytes;

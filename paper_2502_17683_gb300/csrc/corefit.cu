@@ -120,8 +120,8 @@ extern "C" thc_cpd_status thc_cpd_core_fit(int o, int v, int Rt, int naux, const
     cudaStream_t st = opts ? (cudaStream_t)opts->stream : (cudaStream_t)0;
     const int ldl = opts ? opts->ldl : THC_CPD_LDL_AUTO;
     // products from digits on the tensor cores: all on request, else those that are faster there
-    const bool all = ldl == THC_CPD_LDL_EMULATED && oz_available();
-    const bool emu = oz_available() && (all || oz_worth(std::min(naux * o, 8192), Rt, v, false) ||
+    bool all = ldl == THC_CPD_LDL_EMULATED && oz_available();
+    bool emu = oz_available() && (all || oz_worth(std::min(naux * o, 8192), Rt, v, false) ||
                                         oz_worth(Rt, Rt, std::max(v, naux), true));
     if (opts) {
         const double lim = opts->wait_limit_s;
@@ -146,10 +146,13 @@ extern "C" thc_cpd_status thc_cpd_core_fit(int o, int v, int Rt, int naux, const
             oz_product_ws(naux, naux, std::min<size_t>(ov, 8 * kOzPanel), &rowsA, &rowsB, nullptr);
             oz_product_ws(Rt, Rt, Rt, &rowsA, &rowsB, &oz_part);
         }
-        bytes += oz_ws_bytes(rowsA, rowsB, oz_part);
     }
     void* block = nullptr;
-    if (cudaMallocAsync(&block, bytes, st) != cudaSuccess) return cerr(THC_CPD_ERR_ALLOC, "workspace allocation failed");
+    if (emu && !alloc_block(&block, bytes + oz_ws_bytes(rowsA, rowsB, oz_part), st)) all = emu = false;
+    if (emu)
+        bytes += oz_ws_bytes(rowsA, rowsB, oz_part);
+    else if (!alloc_block(&block, bytes, st))  // (the FP64 pipes make do with less)
+        return cerr(THC_CPD_ERR_ALLOC, "workspace allocation failed");
     struct Free {
         void* p;
         cudaStream_t st;

@@ -175,9 +175,12 @@ extern "C" thc_cpd_status thc_cpd_df_als(int o, int v, int naux, int R, const do
                    3 * Arena::need<double>(nR) + 5 * Arena::need<double>(RR) + Arena::need<double>(nmax * R) +
                    Arena::need<double>(R) + Arena::need<double>(c.part_cap) + Arena::need<double>(loss_red_need()) +
                    Arena::need<double>((size_t)naux * naux) + Arena::need<DevScalars>(1);
-    if (c.emu) bytes += oz_ws_bytes(rowsA, rowsB, oz_part);
     void* block = nullptr;
-    if (cudaMallocAsync(&block, bytes, c.st) != cudaSuccess) return derr(THC_CPD_ERR_ALLOC, "workspace allocation failed");
+    if (c.emu && !alloc_block(&block, bytes + oz_ws_bytes(rowsA, rowsB, oz_part), c.st)) c.all = c.emu = false;
+    if (c.emu)
+        bytes += oz_ws_bytes(rowsA, rowsB, oz_part);
+    else if (!alloc_block(&block, bytes, c.st))  // (the FP64 pipes make do with less)
+        return derr(THC_CPD_ERR_ALLOC, "workspace allocation failed");
     struct Free {
         void* p;
         cudaStream_t st;

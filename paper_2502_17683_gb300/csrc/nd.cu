@@ -174,8 +174,11 @@ thc_cpd_status nd_alloc(NdCtx& c, int d, int dL, const int* dims, int Rt, int R,
                    Arena::need<double>(std::max(RtR, RR)) + Arena::need<double>(R) + Arena::need<double>(c.part_cap) +
                    Arena::need<double>(loss_red_need()) + Arena::need<DevScalars>(1);
     if (setup) bytes += 3 * Arena::need<double>(RtRt);
-    if (c.emu) bytes += oz_ws_bytes(rowsA, rowsB, oz_part);
-    if (cudaMallocAsync(block, bytes, c.st) != cudaSuccess) return nerr(THC_CPD_ERR_ALLOC, "workspace allocation failed");
+    if (c.emu && !alloc_block(block, bytes + oz_ws_bytes(rowsA, rowsB, oz_part), c.st)) c.all = c.emu = false;
+    if (c.emu)
+        bytes += oz_ws_bytes(rowsA, rowsB, oz_part);
+    else if (!alloc_block(block, bytes, c.st))  // (the FP64 pipes make do with less)
+        return nerr(THC_CPD_ERR_ALLOC, "workspace allocation failed");
     Arena ar;
     ar.base = (char*)*block;
     ar.cap = bytes;

@@ -78,10 +78,11 @@ struct OzWs {
 
 // Workspace for left operands of rowsA and right operands of rowsB digit rows (a product of
 // M x K by K x N takes cdiv(K, kOzPanel) x M and x N of them; with less it runs in several
-// launches over K, with at least M and N), and part_doubles doubles of partial sums.
+// launches, of at least one row of A and all of B's at a time), and part_doubles doubles of partial sums.
 size_t oz_ws_bytes(int rowsA, int rowsB, size_t part_doubles = 0);
 void oz_ws_carve(OzWs& w, Arena& ar, int rowsA, int rowsB, size_t part_doubles = 0);
-// Raises *rowsA / *rowsB / *part to what one M x N x K product takes in a single pass.
+// Raises *rowsA / *rowsB / *part to what one M x N x K product takes, in a single pass up to 256 MB of
+// digits an operand.
 void oz_product_ws(int M, int N, int K, int* rowsA, int* rowsB, size_t* part);
 
 // C (M x N, ldc) = or += sign A B^T from the operands' digits (same K). lower: rows i < N are
@@ -142,13 +143,13 @@ bool ldl_fix_prepare();
 //   C[M x N] = op(A)[M x K] (B o B2)[K x N];
 //   op(A)[m][k] = trans_a ? A[k * lda + m] : A[m * lda + k]; B, B2 row-major (ldb);
 //   symm: C symmetric (M == N); the lower triangle is computed and mirrored.
-// ws must hold M (rowsA) and N (rowsB) digit rows.
+// ws must hold N (rowsB) digit rows, and M (rowsA) of a symmetric product.
 [[nodiscard]] cudaError_t oz_dgemm(cudaStream_t st, bool trans_a, int M, int N, int K, const double* A, int lda,
                      const double* B, const double* B2, int ldb, double* C, int ldc, bool symm,
                      const OzWs& ws);
 
 // C (M x N, ldc) -= A B for row-major FP64 A (M x K, lda) and B (K x N, ldb) (the coupling term
-// of a split backward solve). ws must hold M (rowsA) and N (rowsB) digit rows.
+// of a split backward solve). ws must hold N (rowsB) digit rows.
 [[nodiscard]] cudaError_t oz_gemm_sub(cudaStream_t st, int M, int N, int K, const double* A, int lda, const double* B,
                         int ldb, double* C, int ldc, const OzWs& ws);
 

@@ -868,12 +868,13 @@ void oz_ws_carve(OzWs& w, Arena& ar, int rowsA, int rowsB, size_t part_doubles) 
     w.part_cap = part_doubles;
 }
 
+// Digit rows of one operand of a product, at most: 256 MB. A product of more runs in several launches.
+constexpr long kMaxDigitRows = 1L << 17;
+
 void oz_product_ws(int M, int N, int K, int* rowsA, int* rowsB, size_t* part) {
     const long nch = std::min(cdiv(std::max(K, 1), KP), kOzMaxChunks);
-    // at most 2^20 digit rows (2 GB) a side; beyond that the product runs in several K ranges
-    const long most = 1L << 20;
-    *rowsA = (int)std::max<long>(*rowsA, std::max<long>(M, std::min(nch * M, most)));
-    *rowsB = (int)std::max<long>(*rowsB, std::max<long>(N, std::min(nch * N, most)));
+    *rowsA = (int)std::max<long>(*rowsA, std::min(nch * M, kMaxDigitRows));
+    *rowsB = (int)std::max<long>(*rowsB, std::max<long>(N, std::min(nch * N, kMaxDigitRows)));
     if (part) {
         const long tiles = (long)cdiv(M, BM) * cdiv(N, 32);
         const long g = std::min<long>(nch, std::max<long>(1, 2L * num_sms() / tiles));
@@ -882,18 +883,25 @@ void oz_product_ws(int M, int N, int K, int* rowsA, int* rowsB, size_t* part) {
 }
 
 namespace {
-// C (+)= sign op(A) (B o B2) with both operands split into ws, in K ranges of as many chunks as
-// ws holds. a_cols / b_cols: the operand's rows are the columns of the stored matrix.
+// C (+)= sign op(A) (B o B2) with both operands split into ws, in K ranges of as many chunks as ws
+// holds of B, and of A in as many rows as it holds of those (fewer chunks where that would be less
+// than 1024). a_cols / b_cols: the operand's rows are the columns of the stored matrix.
 cudaError_t product(cudaStream_t st, int M, int N, int K, const double* A, int lda, bool a_cols, const double* B,
                     const double* B2, int ldb, bool b_cols, double* C, int ldc, double sign, int flags,
                     const OzWs& ws) {
     if (!oz_init()) return cudaErrorNotSupported;
-    if (M > ws.rowsA || N > ws.rowsB) return cudaErrorInvalidValue;
     // A^T A (a Gram): one operand split serves both sides
     const bool same_ab = a_cols && b_cols && A == B && !B2 && lda == ldb && M == N;
-    const int most = std::min(std::min(same_ab ? kOzMaxChunks : ws.rowsA / M, ws.rowsB / N), kOzMaxChunks) * KP;
-    for (int k0 = 0; k0 < K; k0 += most) {
-        const int kn = std::min(most, K - k0);
+    if (N > ws.rowsB || (!same_ab && (flags & OZ_SYMM) && M > ws.rowsA)) return cudaErrorInvalidValue;
+    int chunks = std::min(std::min(cdiv(K, KP), ws.rowsB / N), kOzMaxChunks), rows = M;
+    if (!same_ab) {
+        const int least = (flags & OZ_SYMM) ? M : std::min(M, 1024);
+        chunks = std::min(chunks, std::max(1, ws.rowsA / least));
+        rows = std::min(M, ws.rowsA / chunks);
+        if (rows < M && rows > BM) rows = rows / BM * BM;
+    }
+    for (int k0 = 0; k0 < K; k0 += chunks * KP) {
+        const int kn = std::min(chunks * KP, K - k0);
         OzMat b = view(ws.sB, ws.eB, N, kn);
         const size_t ob = b_cols ? (size_t)k0 * ldb : (size_t)k0;
         if (b_cols)
@@ -901,17 +909,20 @@ cudaError_t product(cudaStream_t st, int M, int N, int K, const double* A, int l
         else
             oz_split_rows(st, B + ob, ldb, b);
         b.src.k0 = k0;
-        OzMat a = b;
-        if (!same_ab) {
-            a = view(ws.sA, ws.eA, M, kn);
-            if (a_cols)
-                oz_split_cols(st, A + (size_t)k0 * lda, nullptr, lda, a);
-            else
-                oz_split_rows(st, A + k0, lda, a);
-            a.src.k0 = k0;
+        for (int m0 = 0; m0 < M; m0 += rows) {
+            OzMat a = b;
+            if (!same_ab) {
+                a = view(ws.sA, ws.eA, std::min(rows, M - m0), kn);
+                if (a_cols)
+                    oz_split_cols(st, A + (size_t)k0 * lda + m0, nullptr, lda, a);
+                else
+                    oz_split_rows(st, A + (size_t)m0 * lda + k0, lda, a);
+                a.src.k0 = k0;
+            }
+            const cudaError_t e = oz_mul(st, a, b, C + (size_t)m0 * ldc, ldc, sign, k0 > 0 ? flags | OZ_ACC : flags,
+                                         ws.part, ws.part_cap);
+            if (e != cudaSuccess) return e;
         }
-        const cudaError_t e = oz_mul(st, a, b, C, ldc, sign, k0 > 0 ? flags | OZ_ACC : flags, ws.part, ws.part_cap);
-        if (e != cudaSuccess) return e;
     }
     return cudaGetLastError();
 }

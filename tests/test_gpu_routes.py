@@ -118,3 +118,19 @@ def test_exchange_in_groups(api, na):
     s1 = abs(X.exchange_single(np.abs(p.Xo), np.abs(p.Xv), np.abs(p.Z), [np.abs(a) for a in p.A], lam, Lam, Gam))
     s2 = abs(X.exchange_double([np.abs(a) for a in p.A], lam, Lam, Gam))
     assert abs(e1 - r1) <= 1e-12 * s1 and abs(e2 - r2) <= 1e-12 * s2
+
+
+# a left operand of more digit rows than 256 MB holds (32000 of eight chunks): two ranges of rows
+def test_core_fit_in_row_ranges(api):
+    o, v, Rt, na = 200, 1000, 100, 160
+    rnd = _rnd(3)
+    Xo, Xv, B = rnd(o, Rt), rnd(v, Rt), rnd(na, o, v)
+    Z, _, used = api.thc_cpd_core_fit(Xo, Xv, B)
+    E = ((B.reshape(na * o, v) @ Xv).reshape(na, o, Rt) * Xo).sum(1)
+    S = (Xo.T @ Xo) * (Xv.T @ Xv)
+    F = torch.linalg.solve(S, E.T).T
+    ref = F.T @ F
+    # sums of v, o and na terms and the solve, each against its own size: the factors' norms carry them on
+    cond = float(torch.linalg.cond(S))
+    lim = 4 * (v + o + na + Rt) * U * cond * float(torch.linalg.norm(F)) ** 2
+    assert not used and float(torch.linalg.norm(Z - ref)) <= lim

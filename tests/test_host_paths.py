@@ -102,3 +102,45 @@ def test_exchange_makes_do_with_one_point(calls, ldl):
     assert len(sizes) > 3 and sizes[-1] <= one
     calls.lib.fake_alloc_limit(1 << 62)
     assert run() == 0  # the failure leaves nothing behind
+
+
+ALLOCS = {
+    "mttkrp": lambda c: c.mttkrp(20, 100, 300, 400),
+    "loss": lambda c: c.loss(20, 100, 300, 400, normG2=0.0),
+    "norm": lambda c: c.norm2(20, 100, 300),
+    "sweep": lambda c: c.sweep(20, 100, 300, 400, normG2=0.0),
+    "split": lambda c: c.sweep(20, 100, 300, 400, precision=1),
+    "batched": lambda c: c.batched([(12, 60, 200, 420), (3, 9, 30, 40)]),
+    "core fit": lambda c: c.core_fit(10, 50, 200, 220, loss=True),
+    "DF": lambda c: c.df_als(10, 50, 200, 220),
+    "order 3": lambda c: c.nd_mttkrp((10, 50, 30), 1, 200, 300),
+}
+
+
+# a call whose digits do not fit runs on the FP64 pipes; what those need is refused as before
+@pytest.mark.parametrize("what", ALLOCS)
+def test_call_makes_do_without_digits(calls, what):
+    from paper_2502_17683_gb300._lib import ERR_ALLOC
+    assert ALLOCS[what](calls) == 0, calls.lib.thc_cpd_last_error()
+    sizes = [calls.lib.fake_largest_alloc()]
+    for expect in (0, ERR_ALLOC):
+        calls.lib.fake_reset()
+        calls.lib.fake_alloc_limit(sizes[-1] - 1)
+        assert ALLOCS[what](calls) == expect, calls.lib.thc_cpd_last_error()
+        sizes.append(calls.lib.fake_largest_alloc())
+        assert what == "batched" or calls.lib.fake_launches(b"k_oz_update") == 0
+    calls.lib.fake_alloc_limit(1 << 62)
+    assert ALLOCS[what](calls) == 0, calls.lib.thc_cpd_last_error()  # the failure leaves nothing behind
+
+
+# the digits of one operand take 256 MB at most, however long or many its rows, beside what the call
+# takes without them
+@pytest.mark.parametrize("what", [lambda c: c.core_fit(200, 1000, 100, 160), lambda c: c.df_als(60, 70, 4000, 20),
+                                  lambda c: c.norm2(5, 200000, 250)], ids=["core fit", "DF", "norm"])
+def test_digit_workspace_is_bounded(calls, what):
+    assert what(calls) == 0 and calls.lib.fake_launches(b"k_oz_update") > 0
+    full = calls.lib.fake_largest_alloc()
+    calls.lib.fake_reset()
+    calls.lib.fake_alloc_limit(full - 1)
+    assert what(calls) == 0 and calls.lib.fake_launches(b"k_oz_update") == 0
+    assert full - calls.lib.fake_largest_alloc() <= 2 * ((1 << 28) + (1 << 20))
