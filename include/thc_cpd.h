@@ -82,6 +82,8 @@ typedef struct thc_cpd_opts {
                             (problems side by side fill the GPU better with short launches).
                             Both give the same factorisation up to rounding order; each is
                             bit-reproducible on its own. */
+    int products;        /* thc_cpd_products: where the FP64 products run (0: AUTO). It takes what was
+                            padding of this struct; values other than 1 count as AUTO. */
     double wait_limit_s; /* limit of every device-side wait of the dataflow LDL^T and the
                             backward solve, in seconds (0: 1 s). A wait that runs out makes
                             the launch give up and the call return THC_CPD_ERR_TIMEOUT. */
@@ -104,6 +106,24 @@ typedef enum {
                                   every value it stores (R <= 4096; dataflow otherwise) */
 } thc_cpd_ldl;
 
+/* Values of thc_cpd_opts.products: the products that run in FP64 (every product of THC_CPD_FP64; the
+ * Grams and the loss of every precision; ||G||^2; those of thc_cpd_exchange, thc_cpd_core_fit,
+ * thc_cpd_df_als and thc_cpd_nd_*). */
+typedef enum {
+    /* From 1e7 flops on as sums of exact integer digits on the BF16 tensor cores, smaller ones on the FP64
+     * pipes. A digit product keeps each row of its left and each column of its right operand to 2^-62 of
+     * the largest entry there and rounds once:
+     *     |error of C_ij| <= about 2^-53 |C_ij| + 2^-61 K max_k |A_ik| max_k |B_kj|.
+     * Against the norms of the operands that is below the error of FP64 arithmetic; but an entry that
+     * lies more than 2^-9 below the largest of its row or column has fewer than the 53 bits it has in FP64,
+     * and one below 2^-63 of it none. On operands graded so strongly (rows or columns over many
+     * decades whose large entries meet zeros) single small results lose relative accuracy. */
+    THC_CPD_PRODUCTS_AUTO = 0,
+    /* All on the FP64 pipes, each term with its own 53 bits; with ldl AUTO the normal equations as well
+     * (dataflow or, in batches, blocked LDL^T). 2 to 12 times slower from the middle sizes on. */
+    THC_CPD_PRODUCTS_FP64 = 1
+} thc_cpd_products;
+
 /* One independent problem of a batched run (thc_cpd_als_batched). Inputs as for
  * thc_cpd_als (device pointers); sweeps_done, flags_out, loss and fit are outputs. */
 typedef struct thc_cpd_problem {
@@ -120,7 +140,8 @@ typedef struct thc_cpd_problem {
 } thc_cpd_problem;
 
 /* ||G||_F^2 = sum_PQ Z[P,Q] (S Z S)[P,Q], S = (Xo^T Xo) o (Xv^T Xv): the THC norm in
- * O(Rt^3), the contraction pattern of the J term of Eq. thc_Ej. Result in *normG2_host. */
+ * O(Rt^3), the contraction pattern of the J term of Eq. thc_Ej. Result in *normG2_host. Accuracy of
+ * the products: thc_cpd_products. */
 thc_cpd_status thc_cpd_thc_norm2(int o, int v, int Rt,
                                  const double* Xo, const double* Xv, const double* Z,
                                  double* normG2_host, const thc_cpd_opts* opts);
@@ -129,14 +150,14 @@ thc_cpd_status thc_cpd_thc_norm2(int o, int v, int Rt,
  *   M1 = Xo (W2 o (Z   (W3 o W4)))     M2 = Xv (W1 o (Z   (W3 o W4)))
  *   M3 = Xo (W4 o (Z^T (W1 o W2)))     M4 = Xv (W3 o (Z^T (W1 o W2)))
  * with W_k = X_k^T A_k. lam is not applied. M (device, n_mode x R) is overwritten.
- * opts->precision selects FP64 or a split tensor-core path. */
+ * opts->precision selects FP64 (products as thc_cpd_products says) or a split tensor-core path. */
 thc_cpd_status thc_cpd_mttkrp(int o, int v, int Rt, int R,
                               const double* Xo, const double* Xv, const double* Z,
                               const double* const A[4], int mode, double* M,
                               const thc_cpd_opts* opts);
 
 /* Loss in factor form (Eq. lossF): ||G||^2 - 2 <G, Gt> + lam^T (G1 o G2 o G3 o G4) lam,
- * evaluated in FP64 for every precision. lam may be NULL (all ones). normG2 <= 0 makes
+ * evaluated in FP64 for every precision (products as thc_cpd_products says). lam may be NULL (all ones). normG2 <= 0 makes
  * the call compute ||G||^2 itself. Outputs in host memory (either may be NULL). */
 thc_cpd_status thc_cpd_loss(int o, int v, int Rt, int R,
                             const double* Xo, const double* Xv, const double* Z,
@@ -148,7 +169,8 @@ thc_cpd_status thc_cpd_loss(int o, int v, int Rt, int R,
  * (pseudo-inverse from a symmetric eigendecomposition if a pivot is <= R*eps*max H_ii),
  * then lam_r = ||A_k[:,r]||, A_k[:,r] /= lam_r. A and lam (device) are updated in place;
  * the incoming lam is absorbed by the first update. Loss and fit of the result are
- * returned (FP64). normG2 <= 0 makes the call compute ||G||^2. */
+ * returned (FP64). normG2 <= 0 makes the call compute ||G||^2. Accuracy of the FP64 products:
+ * thc_cpd_products. */
 thc_cpd_status thc_cpd_als_sweep(int o, int v, int Rt, int R,
                                  const double* Xo, const double* Xv, const double* Z,
                                  double* const A[4], double* lam, double normG2,
@@ -157,7 +179,8 @@ thc_cpd_status thc_cpd_als_sweep(int o, int v, int Rt, int R,
 /* CP-ALS: up to max_sweeps sweeps, stopping after sweep s when |fit_s - fit_{s-1}| < tol
  * (tol <= 0: run all sweeps). A holds the start point on entry and the normalised
  * factors on exit; lam receives the weights. sweeps_done, loss_host and fit_host (host,
- * may be NULL) receive the sweep count and the final FP64 loss and fit. */
+ * may be NULL) receive the sweep count and the final FP64 loss and fit. Accuracy of the FP64
+ * products: thc_cpd_products. */
 thc_cpd_status thc_cpd_als(int o, int v, int Rt, int R,
                            const double* Xo, const double* Xv, const double* Z,
                            double* const A[4], double* lam, int max_sweeps, double tol,
@@ -274,7 +297,7 @@ thc_cpd_status thc_cpd_emulated_gemm(int M, int N, int K, const double* A, int l
  * G the THC block (Eq. THC) and Gt = sum_r lam_r A1 A2 A3 A4 (Eq. cp4). Device inputs as for
  * thc_cpd_loss (lam may not be NULL); the three energies are returned in host memory (each
  * pointer may be NULL). Contractions of 1e7 flops or more (over a group of points) run as
- * FP64-accurate products on the tensor cores, smaller ones on the FP64 pipes; with
+ * digit products on the tensor cores, smaller ones on the FP64 pipes (thc_cpd_products); with
  * opts->ldl = THC_CPD_LDL_EMULATED all run on the tensor cores. The reductions run in a fixed order. 1 <= nalpha <= 1024. Synchronises. */
 thc_cpd_status thc_cpd_exchange(int o, int v, int Rt, int R, int nalpha, const double* Xo,
                                 const double* Xv, const double* Z, const double* const A[4],
@@ -291,8 +314,8 @@ thc_cpd_status thc_cpd_exchange(int o, int v, int Rt, int R, int nalpha, const d
  * Xo (o x Rt), Xv (v x Rt), B (naux x o x v, row-major), Z (Rt x Rt, written): device FP64.
  * loss: NULL, or host double receiving ||G_DF - G_THC(Z)||^2 (no 1/2) in factor form.
  * 1 <= R_thc <= 2048; o * v, naux * o, naux * R_thc and naux^2 below 2^31. GEMMs of
- * 1e7 flops or more run as FP64-accurate products on the tensor cores, smaller ones on the FP64
- * pipes; with opts->ldl = THC_CPD_LDL_EMULATED all run on the tensor cores (and the solve uses
+ * 1e7 flops or more run as digit products on the tensor cores, smaller ones on the FP64
+ * pipes (thc_cpd_products); with opts->ldl = THC_CPD_LDL_EMULATED all run on the tensor cores (and the solve uses
  * the emulated two-level LDL^T).
  * Allocates its workspace (about 256 MiB plus 2 naux R_thc doubles, plus naux o v and naux^2
  * doubles with loss; the tensor-core products take up to 512 MiB more for the digits of their

@@ -15,6 +15,7 @@ STATUS_NAMES = {0: "OK", 1: "ERR_ARG", 2: "ERR_SHAPE", 3: "ERR_CUDA", 4: "ERR_NO
                 5: "ERR_TIMEOUT", 6: "ERR_ALLOC", 7: "ERR_UNSUPPORTED"}
 PRECISIONS = {"fp64": 0, "bf16x3": 1, "tf32x3": 2}
 LDL_VARIANTS = {"auto": 0, "blocked": 1, "dataflow": 2, "emulated": 3}
+PRODUCTS = {"auto": 0, "fp64": 1}
 
 # every symbol include/thc_cpd.h declares
 EXPORTS = ("thc_cpd_thc_norm2", "thc_cpd_mttkrp", "thc_cpd_loss", "thc_cpd_als_sweep",
@@ -52,6 +53,7 @@ class Opts(ctypes.Structure):
                 ("accepted_out", ctypes.c_int),
                 ("mlp", ctypes.c_void_p),
                 ("ldl", ctypes.c_int),
+                ("products", ctypes.c_int),
                 ("wait_limit_s", ctypes.c_double),
                 ("target_fit", ctypes.c_double)]
 

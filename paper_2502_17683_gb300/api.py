@@ -10,7 +10,7 @@ import ctypes
 
 import torch
 
-from ._lib import (ERR_ARG, KCLASS_NAMES, LDL_VARIANTS, MLP_NPARAM, PRECISIONS, PTR4, KStat,
+from ._lib import (ERR_ARG, KCLASS_NAMES, LDL_VARIANTS, MLP_NPARAM, PRECISIONS, PRODUCTS, PTR4, KStat,
                    Opts, Problem, ThcCpdError, check, load)
 
 __all__ = ["thc_cpd_thc_norm2", "thc_cpd_mttkrp", "thc_cpd_loss", "thc_cpd_als_sweep",
@@ -42,8 +42,11 @@ def _fdev(t: torch.Tensor, name: str, shape=None) -> int:
 
 
 def _opts(precision="fp64", stream=None, loss_every=0, history=None, polish_sweeps=0,
-          autotune=False, ldl="auto", wait_limit_s=0.0) -> Opts:
+          autotune=False, ldl="auto", wait_limit_s=0.0, products="auto") -> Opts:
     o = Opts()
+    if products not in PRODUCTS:
+        raise ThcCpdError(ERR_ARG, f"unknown products {products!r}")
+    o.products = PRODUCTS[products]
     o.wait_limit_s = float(wait_limit_s)
     if ldl not in LDL_VARIANTS:
         raise ThcCpdError(ERR_ARG, f"unknown ldl variant {ldl!r}")
@@ -75,13 +78,13 @@ def _ptr4(A, dims, R):
     return PTR4(*[_dev(a, f"A[{k}]", (dims[k], R)) for k, a in enumerate(A)])
 
 
-def thc_cpd_exchange(Xo, Xv, Z, A, lam, Lam, Gam, emulated=False, stream=None):
+def thc_cpd_exchange(Xo, Xv, Z, A, lam, Lam, Gam, emulated=False, stream=None, products="auto"):
     """CPD+THC LT-MP2 exchange energies (single, double, robust) for the Laplace factors Lam
     (n_alpha x o) and Gam (n_alpha x v); emulated: FP64-accurate tensor-core products."""
     o, v, Rt = _dims(Xo, Xv, Z)
     R = A[0].shape[1]
     na = Lam.shape[0]
-    opts = _opts("fp64", stream, ldl="emulated" if emulated else "auto")
+    opts = _opts("fp64", stream, ldl="emulated" if emulated else "auto", products=products)
     e1, e2, er = ctypes.c_double(), ctypes.c_double(), ctypes.c_double()
     check(load().thc_cpd_exchange(o, v, Rt, R, na, _dev(Xo, "Xo", (o, Rt)), _dev(Xv, "Xv", (v, Rt)),
                                   _dev(Z, "Z", (Rt, Rt)), _ptr4(A, (o, v, o, v), R),
@@ -91,7 +94,7 @@ def thc_cpd_exchange(Xo, Xv, Z, A, lam, Lam, Gam, emulated=False, stream=None):
     return e1.value, e2.value, er.value
 
 
-def thc_cpd_core_fit(Xo, Xv, B, Z=None, loss=False, emulated=False, stream=None):
+def thc_cpd_core_fit(Xo, Xv, B, Z=None, loss=False, emulated=False, stream=None, products="auto"):
     """THC core least-squares fit: Z (R_thc x R_thc) from the grid factors Xo (o x R_thc),
     Xv (v x R_thc) and the DF tensor B (naux x o x v). Returns (Z, loss or None, used_pinv);
     emulated: FP64-accurate tensor-core products and the emulated two-level LDL^T."""
@@ -100,7 +103,7 @@ def thc_cpd_core_fit(Xo, Xv, B, Z=None, loss=False, emulated=False, stream=None)
     naux = B.shape[0]
     if Z is None:
         Z = torch.empty(Rt, Rt, dtype=torch.float64, device=Xo.device)
-    opts = _opts("fp64", stream, ldl="emulated" if emulated else "auto")
+    opts = _opts("fp64", stream, ldl="emulated" if emulated else "auto", products=products)
     lv, pinv = ctypes.c_double(), ctypes.c_int()
     check(load().thc_cpd_core_fit(o, v, Rt, naux, _dev(Xo, "Xo", (o, Rt)), _dev(Xv, "Xv", (v, Rt)),
                                   _dev(B, "B", (naux, o, v)), _dev(Z, "Z", (Rt, Rt)),
@@ -121,7 +124,7 @@ def thc_cpd_emulated_gemm(A, B, C=None, stream=None):
     return C
 
 
-def thc_cpd_ldl_solve(H, M, A=None, tasks=None, wait_limit_s=0.0, stream=None, ldl="auto"):
+def thc_cpd_ldl_solve(H, M, A=None, tasks=None, wait_limit_s=0.0, stream=None, ldl="auto", products="auto"):
     """A with A H = M (H: R x R SPD, M: n x R) by the library's dataflow LDL^T and backward
     solve, pseudo-inverse on a failed pivot. tasks: None (the library's schedule) or an
     int16 array of shape (ntasks, 4) in the format of thc_cpd_ldl_schedule. Returns
@@ -130,7 +133,7 @@ def thc_cpd_ldl_solve(H, M, A=None, tasks=None, wait_limit_s=0.0, stream=None, l
     n = M.shape[0]
     if A is None:
         A = torch.empty(n, R, dtype=torch.float64, device=H.device)
-    opts = _opts("fp64", stream, wait_limit_s=wait_limit_s, ldl=ldl)
+    opts = _opts("fp64", stream, wait_limit_s=wait_limit_s, ldl=ldl, products=products)
     used = ctypes.c_int(0)
     tp, nt = None, 0
     if tasks is not None:
@@ -155,22 +158,22 @@ def thc_cpd_version() -> str:
     return load().thc_cpd_version().decode()
 
 
-def thc_cpd_thc_norm2(Xo, Xv, Z, stream=None) -> float:
+def thc_cpd_thc_norm2(Xo, Xv, Z, stream=None, products="auto") -> float:
     o, v, Rt = _dims(Xo, Xv, Z)
     out = ctypes.c_double()
-    opts = _opts("fp64", stream)
+    opts = _opts("fp64", stream, products=products)
     check(load().thc_cpd_thc_norm2(o, v, Rt, _dev(Xo, "Xo", (o, Rt)), _dev(Xv, "Xv", (v, Rt)),
                                    _dev(Z, "Z", (Rt, Rt)), ctypes.byref(out), ctypes.byref(opts)))
     return out.value
 
 
-def thc_cpd_mttkrp(Xo, Xv, Z, A, mode: int, M=None, precision="fp64", stream=None):
+def thc_cpd_mttkrp(Xo, Xv, Z, A, mode: int, M=None, precision="fp64", stream=None, products="auto"):
     o, v, Rt = _dims(Xo, Xv, Z)
     R = A[0].shape[1]
     dims = (o, v, o, v)
     if M is None:
         M = torch.empty(dims[mode] if 0 <= mode < 4 else 1, R, dtype=torch.float64, device=Xo.device)
-    opts = _opts(precision, stream)
+    opts = _opts(precision, stream, products=products)
     check(load().thc_cpd_mttkrp(o, v, Rt, R, _dev(Xo, "Xo", (o, Rt)), _dev(Xv, "Xv", (v, Rt)),
                                 _dev(Z, "Z", (Rt, Rt)), _ptr4(A, dims, R), int(mode),
                                 _dev(M, "M"), ctypes.byref(opts)))
@@ -190,11 +193,11 @@ def thc_cpd_mttkrp_noalloc(Xo, Xv, Z, A, mode: int, M, stream=None):
     return M
 
 
-def thc_cpd_loss(Xo, Xv, Z, A, lam=None, normG2: float = 0.0, stream=None):
+def thc_cpd_loss(Xo, Xv, Z, A, lam=None, normG2: float = 0.0, stream=None, products="auto"):
     o, v, Rt = _dims(Xo, Xv, Z)
     R = A[0].shape[1]
     loss, fit = ctypes.c_double(), ctypes.c_double()
-    opts = _opts("fp64", stream)
+    opts = _opts("fp64", stream, products=products)
     lp = None if lam is None else _dev(lam, "lam", (R,))
     check(load().thc_cpd_loss(o, v, Rt, R, _dev(Xo, "Xo", (o, Rt)), _dev(Xv, "Xv", (v, Rt)),
                               _dev(Z, "Z", (Rt, Rt)), _ptr4(A, (o, v, o, v), R), lp,
@@ -204,11 +207,11 @@ def thc_cpd_loss(Xo, Xv, Z, A, lam=None, normG2: float = 0.0, stream=None):
 
 
 def thc_cpd_als_sweep(Xo, Xv, Z, A, lam, normG2: float = 0.0, precision="fp64", stream=None,
-                      ldl="auto"):
+                      ldl="auto", products="auto"):
     o, v, Rt = _dims(Xo, Xv, Z)
     R = A[0].shape[1]
     loss, fit = ctypes.c_double(), ctypes.c_double()
-    opts = _opts(precision, stream, ldl=ldl)
+    opts = _opts(precision, stream, ldl=ldl, products=products)
     check(load().thc_cpd_als_sweep(o, v, Rt, R, _dev(Xo, "Xo", (o, Rt)), _dev(Xv, "Xv", (v, Rt)),
                                    _dev(Z, "Z", (Rt, Rt)), _ptr4(A, (o, v, o, v), R),
                                    _dev(lam, "lam", (R,)), float(normG2), ctypes.byref(loss),
@@ -218,14 +221,14 @@ def thc_cpd_als_sweep(Xo, Xv, Z, A, lam, normG2: float = 0.0, precision="fp64", 
 
 def thc_cpd_als(Xo, Xv, Z, A, lam, max_sweeps: int, tol: float = 0.0, precision="fp64",
                 stream=None, loss_every: int = 0, history: bool = False, polish_sweeps: int = 0,
-                autotune: bool = False, mlp=None, ldl="auto", target_fit: float = 0.0):
+                autotune: bool = False, mlp=None, ldl="auto", target_fit: float = 0.0, products="auto"):
     o, v, Rt = _dims(Xo, Xv, Z)
     R = A[0].shape[1]
     loss, fit, done = ctypes.c_double(), ctypes.c_double(), ctypes.c_int()
     hist = (ctypes.c_double * max(1, 2 * max_sweeps))() if history else None
     opts = _opts(precision, stream, loss_every,
                  ctypes.cast(hist, ctypes.POINTER(ctypes.c_double)) if hist is not None else None,
-                 polish_sweeps, autotune, ldl)
+                 polish_sweeps, autotune, ldl, products=products)
     opts.target_fit = float(target_fit)
     if mlp is not None:
         opts.mlp = _fdev(mlp, "mlp", (MLP_NPARAM,))
@@ -244,7 +247,7 @@ def thc_cpd_als(Xo, Xv, Z, A, lam, max_sweeps: int, tol: float = 0.0, precision=
 
 
 def thc_cpd_df_als(B, A, lam, max_sweeps: int, tol: float = 0.0, emulated=False, history=False,
-                   stream=None):
+                   stream=None, products="auto"):
     """DF-driven CP-ALS of G_DF = sum_X B[X] (x) B[X] (B: naux x o x v); A (four factors) and lam
     are updated in place. emulated: FP64-accurate tensor-core GEMMs and the emulated LDL^T."""
     naux, o, v = B.shape
@@ -253,7 +256,7 @@ def thc_cpd_df_als(B, A, lam, max_sweeps: int, tol: float = 0.0, emulated=False,
     hist = (ctypes.c_double * max(1, 2 * max_sweeps))() if history else None
     opts = _opts("fp64", stream, 0,
                  ctypes.cast(hist, ctypes.POINTER(ctypes.c_double)) if hist is not None else None,
-                 ldl="emulated" if emulated else "auto")
+                 ldl="emulated" if emulated else "auto", products=products)
     check(load().thc_cpd_df_als(o, v, naux, R, _dev(B, "B", (naux, o, v)), _ptr4(A, (o, v, o, v), R),
                                 _dev(lam, "lam", (R,)), int(max_sweeps), float(tol),
                                 ctypes.byref(done), ctypes.byref(fit), ctypes.byref(opts)))
@@ -277,26 +280,26 @@ def _nd_args(X, Z, A, dL):
     return d, int(dL), dims, Rt, R, xs, _dev(Z, "Z", (Rt, Rt)), As
 
 
-def thc_cpd_nd_mttkrp(X, Z, A, dL: int, mode: int, M=None, emulated=False, stream=None):
+def thc_cpd_nd_mttkrp(X, Z, A, dL: int, mode: int, M=None, emulated=False, stream=None, products="auto"):
     """Order-d MTTKRP of the THC-like tensor (X: d grid factors, modes < dL on P, the rest on Q)."""
     d, dL, dims, Rt, R, xs, z, As = _nd_args(X, Z, A, dL)
     if M is None:
         M = torch.empty(X[mode].shape[0] if 0 <= mode < d else 1, R, dtype=torch.float64, device=Z.device)
-    opts = _opts("fp64", stream, ldl="emulated" if emulated else "auto")
+    opts = _opts("fp64", stream, ldl="emulated" if emulated else "auto", products=products)
     check(load().thc_cpd_nd_mttkrp(d, dL, dims, Rt, R, xs, z, As, int(mode), _dev(M, "M"),
                                    ctypes.byref(opts)))
     return M
 
 
 def thc_cpd_nd_als(X, Z, A, lam, dL: int, max_sweeps: int, tol: float = 0.0, emulated=False,
-                   history=False, stream=None):
+                   history=False, stream=None, products="auto"):
     """Order-d THC-driven CP-ALS; A (d factors) and lam are updated in place."""
     d, dL, dims, Rt, R, xs, z, As = _nd_args(X, Z, A, dL)
     fit, done = ctypes.c_double(), ctypes.c_int()
     hist = (ctypes.c_double * max(1, 2 * max_sweeps))() if history else None
     opts = _opts("fp64", stream, 0,
                  ctypes.cast(hist, ctypes.POINTER(ctypes.c_double)) if hist is not None else None,
-                 ldl="emulated" if emulated else "auto")
+                 ldl="emulated" if emulated else "auto", products=products)
     check(load().thc_cpd_nd_als(d, dL, dims, Rt, R, xs, z, As, _dev(lam, "lam", (R,)), int(max_sweeps),
                                 float(tol), ctypes.byref(done), ctypes.byref(fit), ctypes.byref(opts)))
     out = dict(sweeps=done.value, fit=fit.value, flags=opts.flags_out)
@@ -355,7 +358,7 @@ def thc_cpd_profile_read() -> dict:
 
 
 def thc_cpd_als_batched(problems, max_sweeps: int, tol: float = 0.0, precision="fp64",
-                        stream=None, autotune: bool = False, ldl="auto"):
+                        stream=None, autotune: bool = False, ldl="auto", products="auto"):
     """problems: list of dicts with Xo, Xv, Z, A (list of 4), lam (device tensors, updated in
     place). Returns a list of dict(sweeps, loss, fit, flags) per problem."""
     n = len(problems)
@@ -370,7 +373,7 @@ def thc_cpd_als_batched(problems, max_sweeps: int, tol: float = 0.0, precision="
         for k, a in enumerate(pr["A"]):
             arr[i].A[k] = _dev(a, f"A[{k}]", ((o, v, o, v)[k], R))
         arr[i].lam = _dev(pr["lam"], "lam", (R,))
-    opts = _opts(precision, stream, autotune=autotune, ldl=ldl)
+    opts = _opts(precision, stream, autotune=autotune, ldl=ldl, products=products)
     check(load().thc_cpd_als_batched(n, ctypes.cast(arr, ctypes.c_void_p), int(max_sweeps),
                                      float(tol), ctypes.byref(opts)))
     return [dict(sweeps=arr[i].sweeps_done, loss=arr[i].loss, fit=arr[i].fit, flags=arr[i].flags_out)
@@ -427,7 +430,7 @@ def thc_cpd_mlp_train(params, X, y, epochs: int, batch: int = 64, lr: float = 1e
 
 
 def thc_cpd_als_trajectory(Xo, Xv, Z, A, lam, sweeps: int, alphas, precision="fp64", stream=None,
-                           ldl="auto"):
+                           ldl="auto", products="auto"):
     """Plain ALS for `sweeps` sweeps, recording per sweep the 40 features and the exact losses
     of the trial points at each alpha. Returns (features (sweeps, 40), losses (sweeps, na))."""
     import numpy as np
@@ -436,7 +439,7 @@ def thc_cpd_als_trajectory(Xo, Xv, Z, A, lam, sweeps: int, alphas, precision="fp
     al = np.ascontiguousarray(np.asarray(alphas, dtype=np.float64))
     feats = np.zeros((sweeps, 40), dtype=np.float32)
     tl = np.zeros((sweeps, len(al)), dtype=np.float64)
-    opts = _opts(precision, stream, ldl=ldl)
+    opts = _opts(precision, stream, ldl=ldl, products=products)
     check(load().thc_cpd_als_trajectory(
         o, v, Rt, R, _dev(Xo, "Xo", (o, Rt)), _dev(Xv, "Xv", (v, Rt)), _dev(Z, "Z", (Rt, Rt)),
         _ptr4(A, (o, v, o, v), R), _dev(lam, "lam", (R,)), int(sweeps),

@@ -250,8 +250,8 @@ constexpr int kFixedBatchedMinR = 400;
 // On its own, a problem takes the dataflow kernel up to 1024 columns and from there dataflow panels
 // with emulated trailing updates (within their plans' range). Side by side, problems of 400 columns
 // and more take fixed-point blocks (ldl_fix.cu), which leave the FP64 pipes to the others, smaller
-// ones the blocked FP64 kernels.
-Ldl ldl_route(int ldl, int R, int nmax, bool batched) {
+// ones the blocked FP64 kernels. pipes (thc_cpd_opts.products): FP64 kernels only.
+Ldl ldl_route(int ldl, int R, int nmax, bool batched, bool pipes = false) {
     const bool two = R > kOzPanel && R <= 4096 && cdiv((long)R + nmax - kOzPanel, 16) <= 256;
     switch (ldl) {
         case THC_CPD_LDL_BLOCKED: return Ldl::kBlocked;
@@ -259,6 +259,7 @@ Ldl ldl_route(int ldl, int R, int nmax, bool batched) {
         case THC_CPD_LDL_EMULATED: return two ? Ldl::kTwoLevel : Ldl::kBlocked;
         default: break;
     }
+    if (pipes) return batched ? Ldl::kBlocked : Ldl::kDataflow;
     if (two && R >= kEmulatedMinR) return Ldl::kTwoLevel;
     if (batched && R >= kFixedBatchedMinR && ldl_fix_prepare()) return Ldl::kFixed;
     return batched ? Ldl::kBlocked : Ldl::kDataflow;
@@ -285,7 +286,8 @@ thc_cpd_status ctx_init(Ctx& c, const Shape& s, const double* Xo, const double* 
     const bool fp64 = !mixed || als || gram;  // FP64 projections (MTTKRP, or a split run's loss)
     // FP64 products that go to the tensor cores: room for the operands' digits and split sums
     const bool w_z = fp64 && oz_worth(Rt, R, Rt, false), w_n = norm && oz_worth(Rt, Rt, Rt, false);
-    c.ozp = digits && oz_available() && (w_z || w_n || (fp64 && oz_worth(Rt, R, nmax, false)) ||
+    const bool pipes = fp64_pipes(opts);
+    c.ozp = digits && !pipes && oz_available() && (w_z || w_n || (fp64 && oz_worth(Rt, R, nmax, false)) ||
                                (gram && oz_worth(R, R, nmax, true)));
     const bool ozp = c.ozp;
     // FP64-pipe products: split-K partial sums of those that stay there
@@ -304,7 +306,7 @@ thc_cpd_status ctx_init(Ctx& c, const Shape& s, const double* Xo, const double* 
     if (norm) pipe(Rt, Rt, Rt, false);
     c.part_cap = pc;
     const int ldl = opts ? opts->ldl : THC_CPD_LDL_AUTO;
-    Ldl route = als ? ldl_route(ldl, R, nmax, need & NEED_BATCHED) : Ldl::kDataflow;
+    Ldl route = als ? ldl_route(ldl, R, nmax, need & NEED_BATCHED, pipes) : Ldl::kDataflow;
     if (route == Ldl::kTwoLevel && !(oz_prepare(R, s.o) && oz_prepare(R, s.v)))
         route = (need & NEED_BATCHED) ? Ldl::kBlocked : Ldl::kDataflow;
     c.fixed = als && route == Ldl::kFixed;
@@ -1601,6 +1603,13 @@ extern "C" thc_cpd_status thc_cpd_emulated_gemm(int M, int N, int K, const doubl
 
 namespace thc {
 
+bool fp64_pipes(const thc_cpd_opts* opts) { return opts && opts->products == THC_CPD_PRODUCTS_FP64; }
+
+int solve_ldl(const thc_cpd_opts* opts) {
+    const int ldl = opts ? opts->ldl : THC_CPD_LDL_AUTO;
+    return ldl == THC_CPD_LDL_AUTO && fp64_pipes(opts) ? THC_CPD_LDL_DATAFLOW : ldl;
+}
+
 int spd_solve(cudaStream_t st, int R, int n, const double* H, const double* M, double* A,
               const short* tasks, int ntasks, int* used_pinv, int ldl, bool fixed) {
     if (used_pinv) *used_pinv = 0;
@@ -1702,7 +1711,7 @@ thc_cpd_status thc_cpd_ldl_solve(int R, int n, const double* H, const double* M,
     }
     set_wait_limit(opts);
     return (thc_cpd_status)spd_solve(stream_of(opts), R, n, H, M, A, tasks, ntasks, used_pinv,
-                                     opts ? opts->ldl : THC_CPD_LDL_AUTO);
+                                     solve_ldl(opts));
 }
 
 // thc_cpd_ldl_solve in fixed-point blocks, the factorisation that the batched driver chooses: the

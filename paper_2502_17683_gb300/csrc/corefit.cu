@@ -118,10 +118,11 @@ extern "C" thc_cpd_status thc_cpd_core_fit(int o, int v, int Rt, int naux, const
     if (!Xo || !Xv || !B || !Z) return cerr(THC_CPD_ERR_ARG, "Xo, Xv, B and Z must be non-null");
     if (used_pinv) *used_pinv = 0;
     cudaStream_t st = opts ? (cudaStream_t)opts->stream : (cudaStream_t)0;
-    const int ldl = opts ? opts->ldl : THC_CPD_LDL_AUTO;
+    const int ldl = solve_ldl(opts);
     // products from digits on the tensor cores: all on request, else those that are faster there
-    bool all = ldl == THC_CPD_LDL_EMULATED && oz_available();
-    bool emu = oz_available() && (all || oz_worth(std::min(naux * o, 8192), Rt, v, false) ||
+    const bool digits = oz_available() && !fp64_pipes(opts);
+    bool all = ldl == THC_CPD_LDL_EMULATED && digits;
+    bool emu = digits && (all || oz_worth(std::min(naux * o, 8192), Rt, v, false) ||
                                         oz_worth(Rt, Rt, std::max(v, naux), true));
     if (opts) {
         const double lim = opts->wait_limit_s;

@@ -152,9 +152,10 @@ extern "C" thc_cpd_status thc_cpd_df_als(int o, int v, int naux, int R, const do
     c.v = v;
     c.naux = naux;
     c.R = R;
-    c.ldl = opts ? opts->ldl : THC_CPD_LDL_AUTO;
-    c.all = c.ldl == THC_CPD_LDL_EMULATED && oz_available();
-    c.emu = c.all || (oz_available() && oz_worth((int)std::min<long>(naux * std::max(o, v), 8192), R, std::max(o, v), false));
+    c.ldl = solve_ldl(opts);
+    const bool digits = oz_available() && !fp64_pipes(opts);
+    c.all = c.ldl == THC_CPD_LDL_EMULATED && digits;
+    c.emu = c.all || (digits && oz_worth((int)std::min<long>(naux * std::max(o, v), 8192), R, std::max(o, v), false));
     c.B = B;
     if (opts) {
         const double lim = opts->wait_limit_s;

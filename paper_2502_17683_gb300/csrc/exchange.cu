@@ -146,7 +146,7 @@ extern "C" thc_cpd_status thc_cpd_exchange(int o, int v, int Rt, int R, int nalp
     int g = (int)std::min<size_t>(nalpha, std::max<size_t>(1, (size_t(1) << 30) / per));
     while (g > 1 && ((long)g * std::max(Rt, R) * std::max(std::max(Rt, R), nmax) >= 0x7fffffffL)) --g;
     // products from digits: all on request, else those of a group that are faster there
-    bool ozd = oz_available() && Rt <= 8192 && R <= 8192 && nmax <= 8192;
+    bool ozd = oz_available() && !fp64_pipes(opts) && Rt <= 8192 && R <= 8192 && nmax <= 8192;
     bool tc_z, tc_u[2], tc_m, tc_n, emu;
     size_t part_cap, bytes;
     void* block = nullptr;

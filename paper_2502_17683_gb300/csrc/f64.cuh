@@ -72,6 +72,14 @@ struct FixWs;
 // its split-K partial sums; with less the products run chunk by chunk / unsplit.
 void bsolve_ws_rows(int R, int nmax, int* rowsA, int* rowsB, size_t* part_doubles);
 
+// thc_cpd_opts.products: whether every product stays on the FP64 pipes; the ldl variant of a solve with
+// these options (AUTO: the dataflow kernel for those).
+}  // namespace thc
+struct thc_cpd_opts;
+namespace thc {
+bool fp64_pipes(const thc_cpd_opts* opts);
+int solve_ldl(const thc_cpd_opts* opts);
+
 // A = M H^-1 for H symmetric positive definite (R x R, lower triangle read) and M (n x R),
 // all device pointers, 1 <= R <= 2048, 1 <= n <= 4096: the solve of thc_cpd_ldl_solve (LDL^T
 // with the forward solve fused, dataflow or emulated two-level by `ldl` (thc_cpd_ldl values),

@@ -149,9 +149,10 @@ thc_cpd_status nd_alloc(NdCtx& c, int d, int dL, const int* dims, int Rt, int R,
         c.nmax = std::max(c.nmax, dims[k]);
     }
     c.Z = Z;
-    c.ldl = opts ? opts->ldl : THC_CPD_LDL_AUTO;
-    c.all = c.ldl == THC_CPD_LDL_EMULATED && oz_available();
-    c.emu = c.all || (oz_available() && (oz_worth(Rt, R, Rt, false) || oz_worth(Rt, R, c.nmax, false) ||
+    c.ldl = solve_ldl(opts);
+    const bool digits = oz_available() && !fp64_pipes(opts);
+    c.all = c.ldl == THC_CPD_LDL_EMULATED && digits;
+    c.emu = c.all || (digits && (oz_worth(Rt, R, Rt, false) || oz_worth(Rt, R, c.nmax, false) ||
                                          oz_worth(R, R, c.nmax, true) || (setup && oz_worth(Rt, Rt, Rt, false))));
     const size_t RtR = (size_t)Rt * R, RR = (size_t)R * R, RtRt = (size_t)Rt * Rt;
     c.part_cap = std::max(dgemm_part_need(Rt, R, c.nmax), dgemm_part_need(Rt, R, Rt));

@@ -51,10 +51,10 @@ class Calls:
         return [o, v, Rt, R, self._p(o, Rt), self._p(v, Rt), self._p(Rt, Rt),
                 PTR4(*[self._p(n, R) for n in (o, v, o, v)])]
 
-    def _opts(self, precision=0, ldl=0):
+    def _opts(self, precision=0, ldl=0, products=0):
         from paper_2502_17683_gb300._lib import Opts
         o = Opts()
-        o.precision, o.ldl = precision, ldl
+        o.precision, o.ldl, o.products = precision, ldl, products
         return ctypes.byref(o)
 
     def launched(self):

@@ -102,8 +102,9 @@ def test_subnormal_results(api, e):
 
 
 # more points than 1 GB of intermediates holds: two full groups and a shorter last one
+@pytest.mark.parametrize("products", ["auto", "fp64"])
 @pytest.mark.parametrize("na", [500, 301])
-def test_exchange_in_groups(api, na):
+def test_exchange_in_groups(api, na, products):
     from oracle import exchange as X
     from tests._util import to_dev
     from thc_inputs import make_lt, make_problem
@@ -112,7 +113,8 @@ def test_exchange_in_groups(api, na):
     lam = np.random.default_rng(na).uniform(0.5, 2.0, R)
     Lam, Gam = X.lt_factors(*make_lt(o, v, na, na))
     d, dev = to_dev(p, torch), lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()
-    e1, e2, _ = api.thc_cpd_exchange(d["Xo"], d["Xv"], d["Z"], d["A"], dev(lam), dev(Lam), dev(Gam))
+    e1, e2, _ = api.thc_cpd_exchange(d["Xo"], d["Xv"], d["Z"], d["A"], dev(lam), dev(Lam), dev(Gam),
+                                     products=products)
     r1, r2, _ = X.exchange_robust(p.Xo, p.Xv, p.Z, p.A, lam, Lam, Gam)
     # relative to the size of the terms, as for one group
     s1 = abs(X.exchange_single(np.abs(p.Xo), np.abs(p.Xv), np.abs(p.Z), [np.abs(a) for a in p.A], lam, Lam, Gam))
@@ -134,3 +136,24 @@ def test_core_fit_in_row_ranges(api):
     cond = float(torch.linalg.cond(S))
     lim = 4 * (v + o + na + Rt) * U * cond * float(torch.linalg.norm(F)) ** 2
     assert not used and float(torch.linalg.norm(Z - ref)) <= lim
+
+
+# Z and a factor graded over 80 binary digits, the large entries of one against zeros of the other: on the
+# FP64 pipes every entry is right to the rounding of its own terms (all positive), the tiny ones too
+@pytest.mark.parametrize("mode", [0, 2])
+def test_graded_operands_on_the_fp64_pipes(api, mode):
+    o, v, Rt, R = 10, 90, 200, 300
+    rng = np.random.default_rng(mode)
+    X, Z = [rng.random((n, Rt)) + 0.1 for n in (o, v)], rng.random((Rt, Rt)) + 0.1
+    A = [rng.random((n, R)) + 0.1 for n in (o, v, o, v)]
+    Z[:, 100:], Z[100:, :] = Z[:, 100:] * 2.0 ** -80, Z[100:, :] * 2.0 ** -80
+    X[1][:45, 100:], X[1][45:, :100] = 0.0, 0.0
+    A[1][:45, :150], A[3][:45, :150] = 0.0, 0.0   # W2, W4: rows below 100 are zero for these columns
+    d = lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    M = api.thc_cpd_mttkrp(d(X[0]), d(X[1]), d(Z), [d(a) for a in A], mode, products="fp64").cpu().numpy()
+    L = lambda x: x.astype(np.longdouble)
+    W = [L(X[k % 2]).T @ L(A[k]) for k in range(4)]
+    Y = L(Z) @ (W[2] * W[3]) if mode < 2 else L(Z).T @ (W[0] * W[1])
+    ref = L(X[mode % 2]) @ (W[mode ^ 1] * Y)
+    assert np.max(ref[:, :150]) < 1e-20 * np.min(ref[:, 150:])
+    assert np.all(np.abs(M - ref) <= (3 * v + 2 * Rt + 4) * U * ref)

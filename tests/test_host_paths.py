@@ -144,3 +144,31 @@ def test_digit_workspace_is_bounded(calls, what):
     calls.lib.fake_alloc_limit(full - 1)
     assert what(calls) == 0 and calls.lib.fake_launches(b"k_oz_update") == 0
     assert full - calls.lib.fake_largest_alloc() <= 2 * ((1 << 28) + (1 << 20))
+
+
+def test_products_option_took_padding():
+    from paper_2502_17683_gb300._lib import Opts
+    assert Opts.products.offset == Opts.ldl.offset + 4 and Opts.wait_limit_s.offset == Opts.ldl.offset + 8
+
+
+# products = 1: nothing of an FP64 call leaves the FP64 pipes, the factorisation included
+PIPES = {
+    "mttkrp": lambda c, **k: c.mttkrp(20, 100, 300, 400, **k),
+    "norm": lambda c, **k: c.norm2(20, 100, 300, **k),
+    "loss": lambda c, **k: c.loss(20, 100, 300, 400, normG2=0.0, **k),
+    "sweep": lambda c, **k: c.sweep(20, 100, 300, 1100, **k),
+    "batched": lambda c, **k: c.batched([(12, 60, 200, 420), (20, 100, 300, 1100)], **k),
+    "exchange": lambda c, **k: c.exchange(10, 50, 200, 300, 4, **k),
+    "core fit": lambda c, **k: c.core_fit(10, 50, 200, 220, loss=True, **k),
+    "DF": lambda c, **k: c.df_als(10, 50, 200, 220, **k),
+    "order 3": lambda c, **k: c.nd_mttkrp((10, 50, 30), 1, 200, 300, **k),
+    "solve": lambda c, **k: c.solve(1100, 140, **k),
+}
+
+
+@pytest.mark.parametrize("what", PIPES)
+@pytest.mark.parametrize("products", [0, 1])
+def test_products_on_the_fp64_pipes(calls, what, products):
+    assert PIPES[what](calls, products=products) == 0, calls.lib.thc_cpd_last_error()
+    digits = calls.lib.fake_launches(b"k_oz_") + calls.lib.fake_launches(b"k_fix_")
+    assert (digits == 0) == (products == 1)
