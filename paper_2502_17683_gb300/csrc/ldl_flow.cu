@@ -1112,3 +1112,18 @@ extern "C" int thc_cpd_ldl_schedule(int R, int n, short* out, int cap) {
     }
     return (int)h.size();
 }
+
+// The lists as the kernel gets them (main tasks, then the critical ones, type 2 folded): for the tests,
+// not part of the interface. Returns the number of tasks, *nmain of them main.
+extern "C" int thc_cpd_ldl_device_lists(int R, int n, short* out, int cap, int* nmain) {
+    using namespace thc;
+    std::vector<FlowTask> h;
+    int nT = 0, nM = 0;
+    if (R < 1 || n < 0 || cdiv(R, FB) > kMaxTiles || cdiv(n, FB) > kMaxTiles || !build_tasks(R, n, h, nT, nM)) return -1;
+    *nmain = device_lists(h, nT);
+    for (size_t i = 0; i < h.size() && (int)i < cap; ++i) {
+        const short x[4] = {h[i].type, h[i].t, h[i].j, h[i].k};
+        std::copy(x, x + 4, out + 4 * i);
+    }
+    return (int)h.size();
+}
