@@ -133,3 +133,25 @@ def test_subnormal_rows(solve, R, e):
     assert not used and np.any(A != 0.0)
     # exact but for the reciprocal square roots (2^-52 together) and one rounding of the result
     assert np.all(np.abs(A - M / 4) <= 2.0 ** -52 * np.abs(M / 4) + 2.0 ** -1074)
+
+
+# in the batch: two identical columns in every start factor make each H singular, so the sweep is rolled back
+# and replayed with the pseudo-inverse, beside a problem that is not
+def test_batched_problem_with_a_failed_pivot():
+    import __graft_entry__ as g
+    g.build()
+    from oracle import thc_cpd as O
+    from paper_2502_17683_gb300 import api
+    from thc_inputs import make_problem
+    dev = lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    ps = [make_problem(12, 57, 200, 420, seed=50), make_problem(12, 57, 200, 420, seed=51)]
+    As = [[a.copy() for a in p.A] for p in ps]
+    for a in As[0]:
+        a[:, 333] = a[:, 17]
+    batch = [dict(Xo=dev(p.Xo), Xv=dev(p.Xv), Z=dev(p.Z), A=[dev(a) for a in A],
+                  lam=torch.ones(420, dtype=torch.float64, device="cuda")) for p, A in zip(ps, As)]
+    res = api.thc_cpd_als_batched(batch, 2, 0.0)
+    for p, A, r, singular in zip(ps, As, res, (True, False)):
+        ref = O.als(p.Xo, p.Xv, p.Z, tuple(A), 2)
+        assert bool(r["flags"] & 1) == bool(r["flags"] & 2) == singular
+        assert abs(r["loss"] - ref["losses"][-1]) <= 1e-9 * ref["normG2"]
