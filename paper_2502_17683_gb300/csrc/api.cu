@@ -168,7 +168,7 @@ struct Ctx {
     // transpose, rows of X_k and of its transpose), those of W o W, W o Y and of a factor's
     // columns into dP / dA as they are formed.
     bool ozp = false;
-    OzMat dZ[2], dX[2], dXT[2], dP, dA;
+    OzMat dZ[2], dX[2], dXT[2], dP, dA, dS[2];  // dS: S and S Z of ||G||^2
     bool have_dZ[2] = {}, have_dX[2] = {}, have_dXT[2] = {};
     double* part = nullptr;
     size_t part_cap = 0;
@@ -357,7 +357,9 @@ thc_cpd_status ctx_init(Ctx& c, const Shape& s, const double* Xo, const double* 
     if (ozp) {
         if (w_z) oz_product_ws(Rt, R, Rt, &oz_ra, &oz_rb, &oz_part);
         if (d_gram) oz_product_ws(R, R, 1, &oz_ra, &oz_rb, nullptr);
-        if (w_n) oz_product_ws(Rt, Rt, Rt, &oz_ra, &oz_rb, &oz_part);
+        int left = 1, right = 1;  // (||G||^2 has digits of its own)
+        if (w_n) oz_product_ws(Rt, Rt, Rt, &left, &right, &oz_part);
+        if (w_n) bytes += 2 * ozmat_bytes(Rt, Rt);
         if (w_z || w_n) bytes += 2 * ozmat_bytes(Rt, Rt);
         if (d_p) bytes += ozmat_bytes(R, Rt);
         if (d_a) bytes += ozmat_bytes(R, nmax);
@@ -421,6 +423,7 @@ thc_cpd_status ctx_init(Ctx& c, const Shape& s, const double* Xo, const double* 
         }
         if (d_p) ozmat_carve(c.dP, ar, R, Rt);
         if (d_a) ozmat_carve(c.dA, ar, R, nmax);
+        for (int h = 0; h < 2 && w_n; ++h) ozmat_carve(c.dS[h], ar, Rt, Rt);
     }
     if (ozl || ozp) oz_ws_carve(c.oz, ar, oz_ra, oz_rb, oz_part);
     if (gram) fill(c.st, c.ones, R, 1.0);
@@ -517,12 +520,7 @@ void compute_normG2(Ctx& c) {
                       c.part_cap);
         }
         // S is symmetric: its columns, cut from the two Grams, serve as left and right operand
-        OzMat s, t;
-        s.d = c.oz.sB;
-        s.e = c.oz.eB;
-        t.d = c.oz.sA;
-        t.e = c.oz.eA;
-        s.rows = s.K = t.rows = t.K = Rt;
+        OzMat &s = c.dS[0], &t = c.dS[1];
         oz_split_cols(c.st, c.T, c.S, Rt, s);
         mul_digits(c, s, digits_Z(c, 1), c.U, Rt, false);  // S Z
         oz_split_rows(c.st, c.U, Rt, t);

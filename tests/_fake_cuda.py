@@ -29,6 +29,7 @@ def load(tmp):
     lib.fake_fail_launch.argtypes = [ctypes.c_char_p, ctypes.c_long]
     lib.fake_launches.argtypes, lib.fake_launches.restype = [ctypes.c_char_p], ctypes.c_long
     lib.fake_alloc_limit.argtypes = [ctypes.c_size_t]
+    lib.fake_outside.restype = ctypes.c_long
     lib.fake_launched.restype = ctypes.c_char_p
     lib.fake_largest_alloc.restype = ctypes.c_size_t
     return lib

@@ -26,6 +26,8 @@ struct State {
     long fail_after = 0;
     bool fail_encode = false;
     size_t limit = ~size_t(0), largest = 0;
+    std::map<const char*, size_t> blocks;  // of cudaMallocAsync
+    long outside = 0;                      // digit cuts and tensor maps that leave their block
     cudaError_t last = cudaSuccess;
     dim3 grid, block;
     size_t dyn = 0;
@@ -39,9 +41,22 @@ cudaError_t note(cudaError_t e) {
     if (e != cudaSuccess) s().last = e;
     return e;
 }
-CUresult encode(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                CUtensorMapL2promotion, CUtensorMapFloatOOBfill) {
+// [p, p + n) lies in one block
+void check(const void* p, size_t n) {
+    auto it = s().blocks.upper_bound((const char*)p);
+    if (it == s().blocks.begin() || (const char*)p + n > (--it)->first + it->second) ++s().outside;
+}
+// the digit planes and exponents of `rows` rows of K values
+void check_digits(const void* d, const void* e, size_t rows, size_t K) {
+    check(d, (K + 127) / 128 * 8 * rows * 128 * 2);
+    check(e, rows * 4);
+}
+CUresult encode(CUtensorMap*, CUtensorMapDataType type, cuuint32_t rank, void* base, const cuuint64_t* dims,
+                const cuuint64_t* strides, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill) {
+    size_t n = dims[0] * (type == CU_TENSOR_MAP_DATA_TYPE_FLOAT32 ? 4 : 2);
+    for (cuuint32_t i = 1; i < rank; ++i) n += (dims[i] - 1) * strides[i - 1];
+    check(base, n);
     return s().fail_encode ? CUDA_ERROR_INVALID_VALUE : CUDA_SUCCESS;
 }
 }  // namespace
@@ -54,6 +69,7 @@ void fake_reset() {
     s().fail_encode = false;
     s().limit = ~size_t(0);
     s().largest = 0;
+    s().outside = 0;
     s().last = cudaSuccess;
     s().dev = 0;
 }
@@ -65,6 +81,7 @@ void fake_fail_launch(const char* name, long after) {  // launches of such kerne
 void fake_fail_encode(int on) { s().fail_encode = on; }
 void fake_alloc_limit(size_t bytes) { s().limit = bytes; }
 size_t fake_largest_alloc() { return s().largest; }  // of those that succeeded
+long fake_outside() { return s().outside; }
 long fake_launches(const char* name) {
     long n = 0;
     for (auto& k : s().launches)
@@ -112,7 +129,7 @@ cudaError_t __cudaPopCallConfiguration(dim3* g, dim3* b, size_t* dyn, void* st) 
     *(cudaStream_t*)st = s().st;
     return cudaSuccess;
 }
-cudaError_t __cudaLaunchKernel(Kernel k, dim3 g, dim3 b, void**, size_t dyn, cudaStream_t) {
+cudaError_t __cudaLaunchKernel(Kernel k, dim3 g, dim3 b, void** a, size_t dyn, cudaStream_t) {
     const std::string& n = s().name[k];
     if (!g.x || !g.y || !g.z || !b.x || g.y > 65535 || g.z > 65535 || b.x * b.y * b.z > 1024)
         return note(cudaErrorInvalidConfiguration);
@@ -121,6 +138,14 @@ cudaError_t __cudaLaunchKernel(Kernel k, dim3 g, dim3 b, void**, size_t dyn, cud
     if (!s().fail_name.empty() && n.find(s().fail_name) != std::string::npos && s().fail_after-- <= 0)
         return note(cudaErrorLaunchOutOfResources);
     ++s().launches[n];
+    auto num = [&](int i) { return (size_t) * (int*)a[i]; };
+    auto ptr = [&](int i) { return *(void**)a[i]; };
+    if (n.find("k_oz_split_rows") != std::string::npos) check_digits(ptr(4), ptr(5), num(2), num(3));
+    if (n.find("k_oz_split_cols") != std::string::npos) check_digits(ptr(6), ptr(7), num(5), num(4));
+    if (n.find("k_oz_split_ldl") != std::string::npos) {
+        check_digits(ptr(7), ptr(8), num(2), num(4));
+        check_digits(ptr(9), ptr(10), num(3), num(4));
+    }
     return cudaSuccess;
 }
 
@@ -163,7 +188,9 @@ cudaError_t cudaMallocAsync(void** p, size_t n, cudaStream_t) {
     if (n > s().limit) return note(cudaErrorMemoryAllocation);
     if (n > s().largest) s().largest = n;
     *p = calloc(1, n);
-    return *p ? cudaSuccess : note(cudaErrorMemoryAllocation);
+    if (!*p) return note(cudaErrorMemoryAllocation);
+    s().blocks[(const char*)*p] = n;
+    return cudaSuccess;
 }
 cudaError_t cudaMalloc(void** p, size_t n) {
     *p = calloc(1, n);
@@ -171,6 +198,7 @@ cudaError_t cudaMalloc(void** p, size_t n) {
 }
 cudaError_t cudaMallocHost(void** p, size_t n) { return cudaMalloc(p, n); }
 cudaError_t cudaFreeAsync(void* p, cudaStream_t) {
+    s().blocks.erase((const char*)p);
     free(p);
     return cudaSuccess;
 }

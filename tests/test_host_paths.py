@@ -172,3 +172,39 @@ def test_products_on_the_fp64_pipes(calls, what, products):
     assert PIPES[what](calls, products=products) == 0, calls.lib.thc_cpd_last_error()
     digits = calls.lib.fake_launches(b"k_oz_") + calls.lib.fake_launches(b"k_fix_")
     assert (digits == 0) == (products == 1)
+
+
+# Every digit cut and every tensor map stays inside its block, at the sizes of the other tests and where the
+# operands are long, wide or many: as many chunks as a launch sums, more rows than 256 MB of digits hold.
+EXTENTS = {
+    **LAUNCHES, **{"alloc " + k: f for k, f in ALLOCS.items()},
+    "norm R_thc 8000": lambda c: c.norm2(3, 5, 8000),
+    "norm R_thc 8192": lambda c: c.norm2(8192, 5, 8192),
+    "norm R_thc 8193": lambda c: c.norm2(3, 5, 8193),
+    "loss wide": lambda c: c.loss(1, 1, 8000, 700, normG2=0.0),
+    "loss many columns": lambda c: c.loss(1, 1, 300, 8000, normG2=0.0),
+    "mttkrp long": lambda c: c.mttkrp(4000, 8, 700, 900, mode=1),
+    "mttkrp long factors": lambda c: c.mttkrp(9000, 8, 300, 200),
+    "mttkrp many columns": lambda c: c.mttkrp(30, 200, 400, 8192),
+    "sweep two-level": lambda c: c.sweep(50, 250, 1200, 1800, normG2=0.0),
+    "sweep of 2048": lambda c: c.sweep(5, 2100, 300, 2049),
+    "sweep split": lambda c: c.sweep(20, 100, 480, 720, precision=1, normG2=0.0),
+    "batch": lambda c: c.batched([(30, 150, 720, 1080), (20, 100, 480, 720), (5, 15, 60, 80)]),
+    "exchange groups": lambda c: c.exchange(20, 60, 203, 261, 500),
+    "exchange large": lambda c: c.exchange(50, 250, 1200, 1800, 12),
+    "exchange wide": lambda c: c.exchange(3, 4, 5000, 2000, 5),
+    "core fit long": lambda c: c.core_fit(200, 1000, 100, 160, loss=True),
+    "core fit 2048": lambda c: c.core_fit(20, 100, 2048, 300, loss=True),
+    "core fit emulated": lambda c: c.core_fit(40, 300, 128, 2000, ldl=3),
+    "DF long": lambda c: c.df_als(60, 70, 4000, 20),
+    "DF emulated": lambda c: c.df_als(30, 300, 600, 300, ldl=3),
+    "order 4 large": lambda c: c.nd_als((20, 100, 20, 100), 2, 480, 720),
+    "order 2 long": lambda c: c.nd_mttkrp((4096, 4096), 1, 500, 700),
+    "solve 1800": lambda c: c.solve(1800, 250),
+}
+
+
+@pytest.mark.parametrize("what", EXTENTS)
+def test_digits_and_maps_stay_inside_their_blocks(calls, what):
+    assert EXTENTS[what](calls) == 0, calls.lib.thc_cpd_last_error()
+    assert calls.lib.fake_outside() == 0
