@@ -77,10 +77,13 @@ typedef struct thc_cpd_opts {
     const float* mlp;    /* thc_cpd_als: device parameters of the step-proposer network
                             (THC_CPD_MLP_NPARAM floats) or NULL for plain ALS; see below */
     int ldl;             /* thc_cpd_ldl: how the LDL^T of the normal equations runs.
-                            AUTO (0): the dataflow kernel for a single problem with R <= 2048,
-                            the blocked launches for larger R and for thc_cpd_als_batched
-                            (problems side by side fill the GPU better with short launches).
-                            Both give the same factorisation up to rounding order; each is
+                            AUTO (0): from R = 1024 the two-level variant (EMULATED, to R = 4096 and
+                            about 4000 rows of M); below, the dataflow kernel for a single
+                            problem, and in thc_cpd_als_batched fixed-point blocks from R = 400
+                            (128 columns in 62-bit fixed point on the integer pipe, trailing
+                            updates as FP64-accurate tensor-core products: problems side by
+                            side compete for the FP64 pipe) and blocked launches for smaller R.
+                            All give the same factorisation up to rounding; each is
                             bit-reproducible on its own. */
     int products;        /* thc_cpd_products: where the FP64 products run (0: AUTO). It takes what was
                             padding of this struct; values other than 1 count as AUTO. */
@@ -103,7 +106,8 @@ typedef enum {
                                   tensor cores (exact integer slices, see
                                   thc_cpd_emulated_gemm), the last few hundred columns in
                                   one dataflow launch; the factorisation stays FP64 in
-                                  every value it stores (R <= 4096; dataflow otherwise) */
+                                  every value it stores (128 < R <= 4096; otherwise blocked
+                                  launches in the ALS, dataflow in a solve alone) */
 } thc_cpd_ldl;
 
 /* Values of thc_cpd_opts.products: the products that run in FP64 (every product of THC_CPD_FP64; the
@@ -196,7 +200,8 @@ thc_cpd_status thc_cpd_split_gemm(int M, int N, int K, const double* A, const do
                                   double* C, const thc_cpd_opts* opts);
 
 /* CP-ALS of many independent problems of uneven (o, v, R_thc, R_cp) at once: each problem
- * follows thc_cpd_als (same sweeps, same results bit for bit), but one sweep of every
+ * follows thc_cpd_als (same sweeps; same results bit for bit with the same factorisation, see
+ * opts->ldl), but one sweep of every
  * still-running problem is captured into a single CUDA graph whose branches run
  * concurrently, and the graph is replayed once per sweep; problems that meet
  * |fit_s - fit_{s-1}| < tol leave the graph. opts->precision applies to all problems

@@ -257,8 +257,8 @@ k_dgemm_small(int M, int N, int K, const double* __restrict__ A, int lda, const 
 }
 
 // Several such products A^T B in one launch: a small problem's Grams and projections take 3 us each,
-// of which the arithmetic is a tenth. MTTKRP at (o, v, R_thc, R_cp) = (5, 15, 60, 80) 65 -> 57 us, ten
-// ALS sweeps 3289 -> 3152.
+// of which the arithmetic is a tenth. MTTKRP at (o, v, R_thc, R_cp) = (5, 15, 60, 80) 61.7 -> 54.9 us,
+// ten ALS sweeps 3407 -> 3244.
 template <int T>
 __global__ void __launch_bounds__(64) k_dgemm_small_jobs(const __grid_constant__ SmallJobs js) {
     int i = 0;

@@ -346,6 +346,7 @@ __device__ __forceinline__ void tile_of(const UpdArgs& a, int u, int& m0, int& n
 
 // Between the epilogue's warps and the one that looks out for rows without digits.
 __device__ __forceinline__ void epi_barrier() {
+    __syncwarp();
     asm volatile("bar.sync 1, %0;" ::"n"(32 * EPI_WARPS + 32) : "memory");
 }
 
