@@ -126,8 +126,8 @@ LDL_SOURCES = [os.path.join("paper_2502_17683_gb300", "csrc", f)
 LDL_TRAFFIC = {
     # 24 launches of sweep 1: 20 panels of 256 columns and 4 tails
     # (profiles/ldl_flow_panels_o50_v250_Rt1200_R1800_emulated.md)
-    ("c3", "emulated"): {"bytes_per_launch": 2811584,
-                         "sha256": "10b282a25f98cca0edf588eb48c0df1357b2cc87ff8f414aa244c4b6ed1b4ada"},
+    ("c3", "emulated"): {"bytes_per_launch": 2819488,
+                         "sha256": "4ed550791838d03ef525f1fabff2cbd3e854bc60fb391bb0da30a2feab104e9e"},
 }
 
 
