@@ -364,9 +364,13 @@ constexpr int kTinyExp = -954;
 // Ogita, Rump, Oishi, "Accurate sum and dot product", SIAM J. Sci. Comput. 26, 2005: like the digits',
 // the element's only rounding is that of the result.)
 __device__ __forceinline__ double src_dot(const UpdArgs& args, int i, int j, long k0, long k1) {
-    int ea = args.eA[i], eb = args.eB[j];
-    if (max(ea, eb) >= kNanExp) ea = eb = 0;
+    const int ea = args.eA[i], eb = args.eB[j];
     double s = 0.0, c = 0.0;
+    if (max(ea, eb) >= kNanExp) {  // (nothing changes a NaN: a call on such data is not held up by it)
+        for (long k = k0; k < k1 && !isnan(s); ++k)
+            s = fma(src_entry(args.srcA, i, k, args.K), src_entry(args.srcB, j, k, args.K), s);
+        return s;
+    }
     for (long k = k0; k < k1; ++k) {
         const double a = scalbn(src_entry(args.srcA, i, k, args.K), -ea);
         const double b = scalbn(src_entry(args.srcB, j, k, args.K), -eb);
@@ -374,7 +378,7 @@ __device__ __forceinline__ double src_dot(const UpdArgs& args, int i, int j, lon
         c += ((s - (t - z)) + (p - z)) + fma(a, b, -p);
         s = t;
     }
-    return isfinite(s) ? scalbn(s + c, ea + eb) : s;
+    return scalbn(s + c, ea + eb);
 }
 
 template <int BN>
