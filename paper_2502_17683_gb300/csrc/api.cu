@@ -239,9 +239,9 @@ thc_cpd_status product_errors(const Ctx& c) {
     return THC_CPD_OK;
 }
 
-// What a call needs of the context: the sweeps' buffers, ||G||^2, the Grams, and whether several
-// problems run side by side.
-enum : unsigned { NEED_ALS = 1, NEED_NORM = 2, NEED_GRAM = 4, NEED_BATCHED = 8 };
+// What a call needs of the context: the sweeps' buffers, ||G||^2, the Grams, whether several
+// problems run side by side, and the losses of trial points (gemm64's digit workspace).
+enum : unsigned { NEED_ALS = 1, NEED_NORM = 2, NEED_GRAM = 4, NEED_BATCHED = 8, NEED_TRIAL = 16 };
 
 // The factorisation of an R x R normal matrix for the `ldl` option.
 enum class Ldl { kBlocked, kDataflow, kTwoLevel, kFixed };
@@ -343,6 +343,8 @@ thc_cpd_status ctx_init(Ctx& c, const Shape& s, const double* Xo, const double* 
     // factor's columns
     const bool d_gram = gram && oz_worth(R, R, nmax, true);
     bool d_x[2], d_xt[2], d_p = w_z, d_a = d_gram;
+    int own[2] = {1, 1};  // (operands with digits of their own: their product takes partial sums only)
+    int *ra = need & NEED_TRIAL ? &oz_ra : own, *rb = need & NEED_TRIAL ? &oz_rb : own + 1;
     for (int k = 0; k < 2; ++k) {
         const int n = s.n[k];
         d_x[k] = ozp && fp64 && oz_worth(n, R, Rt, false);
@@ -350,15 +352,13 @@ thc_cpd_status ctx_init(Ctx& c, const Shape& s, const double* Xo, const double* 
         d_xt[k] = ozp && (proj || (w_n && n <= kOzMaxK));
         d_p |= d_x[k];
         d_a |= proj || (gram && oz_worth(R, R, n, true));
-        int left = 1, right = 1;  // (a back-projection's operands have digits of their own)
-        if (d_x[k]) oz_product_ws(n, R, Rt, &left, &right, &oz_part);
-        if (ozp && proj) oz_product_ws(Rt, R, n, &oz_ra, &oz_rb, &oz_part);
+        if (d_x[k]) oz_product_ws(n, R, Rt, own, own + 1, &oz_part);
+        if (ozp && proj) oz_product_ws(Rt, R, n, ra, rb, &oz_part);
     }
     if (ozp) {
-        if (w_z) oz_product_ws(Rt, R, Rt, &oz_ra, &oz_rb, &oz_part);
-        if (d_gram) oz_product_ws(R, R, 1, &oz_ra, &oz_rb, nullptr);
-        int left = 1, right = 1;  // (||G||^2 has digits of its own)
-        if (w_n) oz_product_ws(Rt, Rt, Rt, &left, &right, &oz_part);
+        if (w_z) oz_product_ws(Rt, R, Rt, ra, rb, &oz_part);
+        if (d_gram) oz_product_ws(R, R, 1, ra, rb, nullptr);
+        if (w_n) oz_product_ws(Rt, Rt, Rt, own, own + 1, &oz_part);
         if (w_n) bytes += 2 * ozmat_bytes(Rt, Rt);
         if (w_z || w_n) bytes += 2 * ozmat_bytes(Rt, Rt);
         if (d_p) bytes += ozmat_bytes(R, Rt);
@@ -931,12 +931,13 @@ thc_cpd_status run_als(int o, int v, int Rt, int R, const double* Xo, const doub
     if (!lam) return set_err(THC_CPD_ERR_ARG, "lam must be non-null");
     if (max_sweeps < 0) return set_err(THC_CPD_ERR_ARG, "max_sweeps must be >= 0");
     if (opts) opts->flags_out = 0;
+    const bool learning = la && (la->mlp || la->nalpha > 0);
     Ctx c;
-    CKS(ctx_init(c, s, Xo, Xv, Z, opts, NEED_ALS | (normG2 > 0.0 ? 0u : NEED_NORM)));
+    CKS(ctx_init(c, s, Xo, Xv, Z, opts,
+                 NEED_ALS | (normG2 > 0.0 ? 0u : NEED_NORM) | (learning ? NEED_TRIAL : 0u)));
     double nG2 = 0.0;
     CKS(obtain_norm(c, normG2, &nG2));
     CKS(refresh_state(c, A));
-    const bool learning = la && (la->mlp || la->nalpha > 0);
     LearnWs L;
     std::vector<double> loss_hist;
     std::vector<std::array<double, 4>> chg_hist;

@@ -82,6 +82,11 @@ class Calls:
         return self.lib.thc_cpd_als_sweep(*self._problem(o, v, Rt, R), self._p(R), normG2, ctypes.byref(d),
                                           ctypes.byref(d), self._opts(**kw))
 
+    def trajectory(self, o, v, Rt, R, sweeps=2, **kw):
+        a, al, tl = self._problem(o, v, Rt, R), (ctypes.c_double * 2)(1.0, 1.5), (ctypes.c_double * (2 * sweeps))()
+        return self.lib.thc_cpd_als_trajectory(*a, self._p(R), sweeps, al, 2, (ctypes.c_float * (40 * sweeps))(), tl,
+                                               self._opts(**kw))
+
     def batched(self, shapes, sweeps=2, **kw):
         from paper_2502_17683_gb300._lib import Problem
         probs, keep = (Problem * len(shapes))(), []

@@ -189,6 +189,8 @@ EXTENTS = {
     "sweep two-level": lambda c: c.sweep(50, 250, 1200, 1800, normG2=0.0),
     "sweep of 2048": lambda c: c.sweep(5, 2100, 300, 2049),
     "sweep split": lambda c: c.sweep(20, 100, 480, 720, precision=1, normG2=0.0),
+    "trial points": lambda c: c.trajectory(20, 100, 480, 720),
+    "trial points split": lambda c: c.trajectory(30, 150, 720, 1080, precision=1),
     "batch": lambda c: c.batched([(30, 150, 720, 1080), (20, 100, 480, 720), (5, 15, 60, 80)]),
     "exchange groups": lambda c: c.exchange(20, 60, 203, 261, 500),
     "exchange large": lambda c: c.exchange(50, 250, 1200, 1800, 12),
@@ -208,3 +210,15 @@ EXTENTS = {
 def test_digits_and_maps_stay_inside_their_blocks(calls, what):
     assert EXTENTS[what](calls) == 0, calls.lib.thc_cpd_last_error()
     assert calls.lib.fake_outside() == 0
+
+
+# only a run with trial points reserves the workspace of their products, and those run from digits
+def test_trial_points_run_from_digits(calls):
+    assert calls.sweep(20, 100, 480, 720, normG2=0.0) == 0
+    plain, n = calls.lib.fake_largest_alloc(), calls.lib.fake_launches(b"k_oz_update")
+    calls.lib.fake_reset()
+    assert calls.trajectory(20, 100, 480, 720, sweeps=1) == 0
+    # the start point's loss and the one of alpha = 1.5: four projections, four Grams and Z each, of which the
+    # occupied Grams (1.04e7 flops) count, too
+    assert calls.lib.fake_launches(b"k_oz_update") == n + 2 * 9
+    assert calls.lib.fake_largest_alloc() > plain
