@@ -157,3 +157,22 @@ def test_graded_operands_on_the_fp64_pipes(api, mode):
     ref = L(X[mode % 2]) @ (W[mode ^ 1] * Y)
     assert np.max(ref[:, :150]) < 1e-20 * np.min(ref[:, 150:])
     assert np.all(np.abs(M - ref) <= (3 * v + 2 * Rt + 4) * U * ref)
+
+
+# two K ranges (8192 terms and the rest) of which one has tiny rows only: their exponents say nothing of the
+# other range's entries
+@pytest.mark.parametrize("big,tiny", [(slice(0, 8192), slice(8192, 8300)), (slice(8192, 8300), slice(0, 8192))])
+@pytest.mark.parametrize("scale", [1e50, 1e-120])
+def test_tiny_range_beside_another(api, big, tiny, scale):
+    rng = np.random.default_rng(9)
+    A, B = rng.standard_normal((31, 8300)), rng.standard_normal((33, 8300))
+    A[:, big], B[:, big] = A[:, big] * scale, B[:, big] * scale
+    A[:, tiny], B[:, tiny] = A[:, tiny] * 1e-200, B[:, tiny] * 1e-200
+    d = lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    C = api.thc_cpd_emulated_gemm(d(A), d(B)).cpu().numpy()
+    ref = A.astype(np.longdouble) @ B.astype(np.longdouble).T
+    K = 8300
+    top = np.max(np.abs(A), 1)[:, None] * np.max(np.abs(B), 1)[None, :]
+    # one rounding per range, the digits' bound, the longdouble sum's; what underflows lies below 1e-300
+    lim = 3 * U * np.abs(ref) + 2.0 ** -61 * K * top + K * 2.0 ** -63 * (np.abs(A) @ np.abs(B).T) + 1e-300
+    assert np.all(np.abs(C - ref) <= lim)
