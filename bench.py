@@ -126,8 +126,8 @@ LDL_SOURCES = [os.path.join("paper_2502_17683_gb300", "csrc", f)
 LDL_TRAFFIC = {
     # 24 launches of sweep 1: 20 panels of 256 columns and 4 tails
     # (profiles/ldl_flow_panels_o50_v250_Rt1200_R1800_emulated.md)
-    ("c3", "emulated"): {"bytes_per_launch": 2822464,
-                         "sha256": "31b920ff5afee447473f52f06888c47704c276ce572af88e88f0996953ce7703"},
+    ("c3", "emulated"): {"bytes_per_launch": 2808992,
+                         "sha256": "e55b6e36e449b6056d4da94baf679dbe98d627bbeca1c5fa138911da0bc06159"},
 }
 
 
